@@ -329,8 +329,8 @@ size_t adwin_lmhead_workspace_bytes(int64_t B, int64_t T, int64_t V, int64_t d_s
   if (V < 1) V = 1;
   if (d_s < 1) d_s = 1;
   if (d_t < 1) d_t = 1;
-  return lmhead_workspace_bytes(B, T, V, d_s, d_t, max_rows, with_grad != 0,
-                                (flags & ADWIN_RANGE_FULL) != 0);
+  (void)flags;
+  return lmhead_workspace_bytes(B, T, V, d_s, d_t, max_rows, with_grad != 0);
 }
 
 int adwin_opd_kl_lmhead_fwd_bwd(const void* hidden_student, const void* w_student,
@@ -363,8 +363,7 @@ int adwin_opd_kl_lmhead_fwd_bwd(const void* hidden_student, const void* w_studen
     return ADWIN_ERR_ALIGN;
   const bool want_grad = grad_hidden || grad_w;
   if (!workspace || !aligned(workspace, 1024) ||
-      workspace_bytes < lmhead_workspace_bytes(B, T, V, d_s, d_t, max_rows, want_grad,
-                                               (flags & ADWIN_RANGE_FULL) != 0))
+      workspace_bytes < lmhead_workspace_bytes(B, T, V, d_s, d_t, max_rows, want_grad))
     return ADWIN_ERR_WORKSPACE;
   const int sms = sm_count_of_current_device();
   if (sms <= 0) return ADWIN_ERR_CUDA;
@@ -437,22 +436,5 @@ int adwin_lmhead_weight_align(const void* hidden_student, const void* w_student,
     return ADWIN_ERR_CUDA;
   return ADWIN_OK;
 }
-
-#ifdef ADWIN_DEV_EXPORTS
-void adwin_dev_set_sweep_bn(int bn) { set_sweep_tile_columns(bn); }
-void adwin_dev_set_sweep_pair(int on) { set_sweep_pair(on); }
-// Development build only: the tensor-core GEMM on its own, C = A B (bf16 in, fp32 or bf16 out).
-int adwin_dev_gemm(const void* A, int64_t lda, int a_mn, const void* Bm, int64_t ldb, int b_mn,
-                   int64_t M, int64_t N, int64_t K, void* C, int64_t ldc, int c_bf16,
-                   int32_t* dev_status, void* cuda_stream) {
-  const int sms = sm_count_of_current_device();
-  if (sms <= 0) return ADWIN_ERR_CUDA;
-  return launch_tc_gemm(A, lda, a_mn != 0, Bm, ldb, b_mn != 0, M, N, K, C, ldc, c_bf16 != 0,
-                        nullptr, nullptr, nullptr, dev_status, sms,
-                        static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess
-             ? ADWIN_OK
-             : ADWIN_ERR_CUDA;
-}
-#endif
 
 }  // extern "C"

@@ -65,17 +65,14 @@ cudaError_t launch_drift_curves(const float* entropy, const int32_t* rank,
                                 double* bf_mean, int32_t* n_active, cudaStream_t s);
 
 // Fused LM-head form (lmhead.cu).
-void set_sweep_tile_columns(int bn);
-void set_sweep_pair(int on);
 size_t lmhead_workspace_bytes(int64_t B, int64_t T, int64_t V, int64_t ds, int64_t dt,
-                              int64_t max_rows, bool want_grad, bool range_full);
+                              int64_t max_rows, bool want_grad);
 cudaError_t launch_lmhead(const void* hs, const void* ws, const void* ht, const void* wt, int64_t B,
                           int64_t T, int64_t V, int64_t ds, int64_t dt, const int32_t* tokens,
                           const int32_t* window, const int32_t* rollout_len, float alpha, int mode,
                           int flags, void* dH, int dh_dtype, float* dW, float* kl, float* logratio,
                           float* gsq, float* lse_s, float* lse_t, void* workspace,
-                          int64_t max_rows, int32_t* status, int sm_count, cudaStream_t s,
-                          bool keep_G = false);
+                          int64_t max_rows, int32_t* status, int sm_count, cudaStream_t s);
 size_t lmhead_align_workspace_bytes(int64_t B, int64_t T, int64_t V, int64_t ds, int64_t dt,
                                     int64_t max_rows, int K);
 cudaError_t launch_lmhead_weight_align(const void* hs, const void* ws, const void* ht,
@@ -86,10 +83,20 @@ cudaError_t launch_lmhead_weight_align(const void* hs, const void* ws, const voi
                                        float* gsq, double* batch_stats, int32_t* L_next,
                                        int32_t* flags_out, void* workspace, int64_t max_rows,
                                        int32_t* status, int sm_count, cudaStream_t s);
+// Tensor-core GEMM (tc_gemm.cu): C[M,N] = A B, bf16 in.  A is [M,K] (K contiguous, a_mn = false) or
+// [K,M] (M contiguous, a_mn = true), B is [K,N].  scratch: tc_gemm_scratch_bytes() for split tiles,
+// or null; pace: a zeroed counter of this launch's own, or null.
+size_t tc_gemm_scratch_bytes();
 cudaError_t launch_tc_gemm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
-                           bool b_mn, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
-                           bool c_bf16, const int32_t* m_tiles_dev, const int32_t* k_tiles_dev,
-                           const int32_t* row_map, int32_t* status, int sm_count, cudaStream_t s,
-                           const int32_t* k_list = nullptr, const int32_t* k_count_dev = nullptr);
+                           int64_t M, int64_t N, int64_t K, void* C, int64_t ldc, bool c_bf16,
+                           const int32_t* m_tiles_dev, const int32_t* k_tiles_dev,
+                           const int32_t* row_map, float* scratch, unsigned int* pace,
+                           int32_t* status, int sm_count, cudaStream_t s);
+// n_bins products C_i = A^T B over consecutive ranges of the contraction (A [K,M], B [K,N]):
+// bin i takes the 64-row blocks [kblock_dev[i], kblock_dev[i+1]) and writes C + i * bin_stride.
+cudaError_t launch_tc_gemm_bins(const void* A, int64_t lda, const void* B, int64_t ldb, int64_t M,
+                                int64_t N, int64_t K, float* C, int64_t ldc, int64_t bin_stride,
+                                int n_bins, const int32_t* kblock_dev, int32_t* status,
+                                int sm_count, cudaStream_t s);
 
 }  // namespace adwin

@@ -1,23 +1,28 @@
 // Fused LM-head form of the windowed OPD divergence: the two policies of Eq. 2 are given as hidden
-// states times an output embedding, z = H_s W_s^T and u = H_t W_t^T, and the logits are never
-// written to memory.
+// states times an output embedding, z = H_s W_s^T and u = H_t W_t^T.
 //
-//   plan      tile table over the processed positions (128 consecutive positions of one sequence
-//             per tile), compact zero-padded copies of the hidden states
-//   sweep 1   per (tile, vocabulary group): 128 x 256 logit tiles of both policies from tcgen05.mma
-//             into tensor memory, read back with tcgen05.ld and folded into online log-sum-exp /
-//             KL / squared-norm moments; one partial record per (row, group, column half)
+//   plan      compact order of the processed positions: rows with gradient first, then the rest
+//             (or, for the weight-space audit, one segment per candidate bin), 128 rows per tile
+//   gather    compact zero-padded copies of the hidden states, the two logits at the sampled token
+//   sweep     per (pair of tiles, vocabulary group): 256 x 256 logit tiles of both policies from
+//             tcgen05.mma on CTA pairs into tensor memory, read back with tcgen05.ld and folded
+//             into online log-sum-exp / KL / squared-norm moments; one partial record per (row,
+//             group, column half).  For rows with gradient the fp32 logits of a block of tiles are
+//             also left in a scratch buffer
 //   merge     partial records -> per-token kl, logratio, gsq, lse (float64 combination) and the
 //             per-row coefficients of the gradient
-//   sweep 2   the same tiles again; the epilogue turns them into the logit gradient
-//             G = alpha p (d - KL)  or  alpha c (e_y - p)  (Eq. 2 / Eq. 4) in bf16
-//   dH, dW    dH_s = G W_s and dW_s = G^T H_s as two tensor-core GEMMs over G
+//   gradient  the block's logits -> G = alpha p (d - KL)  or  alpha c (e_y - p)  (Eq. 2 / Eq. 4), bf16
+//   dH, dW    dH_s = G W_s and dW_s = G^T H_s as two tensor-core GEMMs over G (tc_gemm.cu)
 //
-// Every kernel here is persistent (one CTA per SM, static round-robin over work items) and warp
-// specialised: warp 0 issues the TMA loads, warp 1 the MMAs, warps 4..11 run the epilogue.
+// The logits of a call never exist in memory as a whole: the scratch buffer holds one block of
+// tiles (at most kKeepBytes) and is overwritten by the next block.  Keeping them for those few
+// milliseconds replaces a second pass of both products: 8 bytes written and read again per logit
+// pair against 2 (d_s + d_t) operations.  A long run is bound by the board's 1 kW, so what counts is
+// energy: at 34 816 rows, V = 151 936, d = 2048 + 2560 a call takes 87 ms (sweep 38, gradient 10,
+// dH 15, dW 17) where computing the products twice on single-CTA tiles took 123 ms (40 + 43 + 17 +
+// 19).  At 225 rows, V = 32 000, d = 1024 + 1536: 254 us against 893 us (groups chosen by size, rows
+// packed across sequences, dH's contraction split).
 #include <cuda_bf16.h>
-
-#include <mutex>
 
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
@@ -31,397 +36,397 @@ using namespace tc;
 constexpr int kRecFields = 8;    // m2s, S, A, B0, B1, B2, m2t, St
 constexpr int kTokFields = 4;    // z_y, u_y, has_y, unused
 constexpr int kInfoFields = 8;   // L2s, a1, a0, gy, y (bits), unused x3
-constexpr int kTileFields = 8;   // b, t0, nvalid, ngrad, gidx, unused x3
 // Logit value given to the columns past the vocabulary in the last tile: far enough below any
 // real logit that its exponential is exactly zero against a real row maximum, and small enough
 // that the rounding residual of z*log2e against the running reference stays a fraction of one
 // (a partial that sees only such columns keeps finite sums and merges with weight 2^-huge = 0).
 constexpr float kMasked = -1.0e6f;
+// Scratch for the logits of one block of tiles.  Large enough that a block fills the GPU several
+// times over (38 tiles at V = 151 936: 8 blocks for 34 816 rows), small beside G.
+constexpr size_t kKeepBytes = size_t(6) << 30;
+constexpr int kKeepArray = kBM * kBN / 4;            // float4 of one policy's 128 x 256 tile
+constexpr size_t kKeepTileChunk = (size_t)2 * kKeepArray * 16;
+constexpr int kGradGroups = 32;                      // column groups of the gradient kernel, at most
+constexpr int kMaxCand = 16;
+constexpr int kMaxSeg = kMaxCand + 1;
 
 // ---------------------------------------------------------------------------- workspace
 struct LmLayout {
-  size_t off_rowmap, off_hdr, off_tiles, off_g2t, off_rowdst, off_info, off_tok, off_part, off_hs,
-      off_ht, off_hg, off_G, total;
-  int64_t max_tiles;
-  int n_groups, n_chunks;
+  size_t off_rowmap, off_hdr, off_seg, off_rowsrc, off_rowdst, off_info, off_tok, off_part, off_park,
+      off_hs, off_ht, off_keep, off_q, off_G, off_pieces, total;
+  int64_t max_tiles, block_tiles, part_slots;
+  int n_chunks, grad_groups;
   int64_t ldG;
 };
 
-int64_t max_tiles_for(int64_t B, int64_t T, int64_t max_rows) {
-  const int64_t per_seq = (T + kBM - 1) / kBM;
-  int64_t cap = B * per_seq;
-  if (max_rows > 0 && max_rows < B * T) {
-    const int64_t bound = (max_rows + kBM - 1) / kBM + B;   // one ragged tile per sequence
-    if (bound < cap) cap = bound;
-  }
-  return cap < 1 ? 1 : cap;
-}
-
+// n_seg segments of compact rows, each padded to a multiple of seg_pad rows.
 LmLayout lm_layout(int64_t B, int64_t T, int64_t V, int64_t ds, int64_t dt, int64_t max_rows,
-                   bool want_grad, bool range_full) {
+                   bool want_grad, int n_seg, int seg_pad, int sm_count) {
   auto up = [](size_t x) { return (x + 1023) & ~size_t(1023); };
   LmLayout L;
-  L.max_tiles = max_tiles_for(B, T, max_rows);
+  int64_t bound = B * T;
+  if (max_rows > 0 && max_rows < bound) bound = max_rows;
+  bound += (int64_t)n_seg * (seg_pad - 1);
+  L.max_tiles = (bound + kBM - 1) / kBM;
+  if (L.max_tiles < 1) L.max_tiles = 1;
   L.n_chunks = (int)((V + kBN - 1) / kBN);
-  L.n_groups = L.n_chunks < 8 ? L.n_chunks : 8;
+  L.grad_groups = L.n_chunks < kGradGroups ? L.n_chunks : kGradGroups;
   L.ldG = (V + 7) / 8 * 8;
+  // equal blocks of an even number of tiles
+  int64_t most = (int64_t)(kKeepBytes / ((size_t)L.n_chunks * kKeepTileChunk)) & ~int64_t(1);
+  if (most < 2) most = 2;
+  const int64_t blocks = (L.max_tiles + most - 1) / most;
+  L.block_tiles = ((L.max_tiles + blocks - 1) / blocks + 1) & ~int64_t(1);
+  // see lm_sweep_kernel: at most 8 groups per tile, or 8 items per pair of CTAs
+  L.part_slots = 8 * (L.max_tiles + 2) + 8 * (int64_t)sm_count;
   const size_t rows = (size_t)L.max_tiles * kBM;
   size_t o = 0;
   L.off_rowmap = o;  o = up(o + workspace_layout(B).total_ext);
-  L.off_hdr = o;     o = up(o + 256);
-  L.off_tiles = o;   o = up(o + (size_t)L.max_tiles * kTileFields * 4);
-  L.off_g2t = o;     o = up(o + (size_t)L.max_tiles * 4);
+  L.off_hdr = o;     o = up(o + 1024);
+  L.off_seg = o;     o = up(o + (size_t)n_seg * (B + 1) * 8);
+  L.off_rowsrc = o;  o = up(o + rows * 4);
   L.off_rowdst = o;  o = up(o + rows * 4);
   L.off_info = o;    o = up(o + rows * kInfoFields * 4);
   L.off_tok = o;     o = up(o + rows * kTokFields * 4);
-  L.off_part = o;    o = up(o + rows * (size_t)L.n_groups * 2 * kRecFields * 4);
+  L.off_part = o;    o = up(o + (size_t)L.part_slots * 2 * kRecFields * kBM * 4);
+  L.off_park = o;    o = up(o + (size_t)sm_count * kKeepArray * 16);
   L.off_hs = o;      o = up(o + rows * (size_t)ds * 2);
   L.off_ht = o;      o = up(o + rows * (size_t)dt * 2);
-  L.off_hg = o;      if (want_grad && range_full) o = up(o + rows * (size_t)ds * 2);
+  L.off_keep = o;    if (want_grad) o = up(o + (size_t)L.block_tiles * L.n_chunks * kKeepTileChunk);
+  L.off_q = o;       if (want_grad) o = up(o + rows * (size_t)L.grad_groups * 2 * 4);
   L.off_G = o;       if (want_grad) o = up(o + rows * (size_t)L.ldG * 2);
+  L.off_pieces = o;  if (want_grad) o = up(o + tc_gemm_scratch_bytes());
   L.total = o;
   return L;
 }
 
-// ---------------------------------------------------------------------------- tensor maps
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+// ---------------------------------------------------------------------------- plan and gather
+// Device header, filled by the gather kernel's first block (n_groups: by the sweep).
+struct LmHeader {
+  int32_t tiles;                    // tiles of processed rows
+  int32_t grad_tiles;               // the leading tiles that hold gradient rows
+  int32_t n_groups;                 // vocabulary groups of the latest sweep
+  int32_t unused;
+  uint32_t pace[60];                // one counter per tensor-core launch
+  int32_t seg_kblock[kMaxSeg + 1];  // first 64-row block of every segment
+};
+static_assert(sizeof(LmHeader) <= 1024, "header too large");
 
-EncodeTiledFn encode_tiled() {
-  static std::mutex mu;
-  static EncodeTiledFn fn = nullptr;
-  std::lock_guard<std::mutex> lock(mu);
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
+// The compact order: segment 0, segment 1, ..., each in sequence order.  Without cuts (n_seg = 2)
+// segment 0 holds the positions with gradient (t < E_b, none unless want_grad) and segment 1 the
+// rest of the processed range; with cuts segment i holds the positions in [cut[i-1], cut[i]).
+struct SegPlan {
+  int n_seg, pad, want_grad, by_cut;
+  int32_t cut[kMaxCand];
+  __device__ __forceinline__ void range(int i, int E, int P, int& lo, int& hi) const {
+    if (by_cut) {
+      lo = i == 0 ? 0 : cut[i - 1];
+      hi = i == n_seg - 1 ? P : cut[i];
+    } else {
+      const int g = want_grad ? E : 0;
+      lo = i == 0 ? 0 : g;
+      hi = i == 0 ? g : P;
+    }
+    lo = lo < P ? lo : P;
+    hi = hi < P ? hi : P;
   }
-  return fn;
-}
+};
 
-// bf16 matrix [rows, cols], row pitch in elements; boxes of 64 columns x box_rows rows with the
-// 128-byte swizzle; out-of-range elements read as zero.
-bool make_map(CUtensorMap* m, const void* base, int64_t cols, int64_t rows, int64_t pitch,
-              int box_rows) {
-  EncodeTiledFn fn = encode_tiled();
-  if (!fn || rows < 1 || cols < 1) return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)pitch * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// ---------------------------------------------------------------------------- plan kernels
-// hdr[0] = number of tiles, hdr[1] = number of tiles that hold gradient rows.
+// Exclusive prefix sums over the sequences of every segment's row counts; block i = segment i.
 __global__ void __launch_bounds__(1024) lm_plan_kernel(const int32_t* __restrict__ range,
                                                        const int32_t* __restrict__ ewin, int64_t B,
-                                                       int64_t T, int64_t max_tiles, int32_t* hdr,
-                                                       int32_t* tiles, int32_t* g2t,
-                                                       int32_t* rowdst, int32_t* status) {
-  __shared__ int64_t s_tiles;
-  if (threadIdx.x == 0) {
-    int64_t nt = 0, ng = 0;
-    for (int64_t b = 0; b < B; ++b) {
-      nt += (range[b] + kBM - 1) / kBM;
-      ng += (ewin[b] + kBM - 1) / kBM;
+                                                       const SegPlan plan, int64_t* seg) {
+  __shared__ int64_t part[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int64_t* out = seg + (int64_t)blockIdx.x * (B + 1);
+  int64_t base = 0;
+  for (int64_t b0 = 0; b0 < B; b0 += 1024) {
+    const int64_t b = b0 + tid;
+    int64_t n = 0;
+    if (b < B) {
+      int lo, hi;
+      plan.range(blockIdx.x, ewin[b], range[b], lo, hi);
+      n = hi - lo;
     }
-    if (nt > max_tiles) {   // more processed rows than the workspace was sized for
-      atomicOr(status, ADWIN_DEV_WORKSPACE);
-      nt = 0;
-      ng = 0;
-    }
-    s_tiles = nt;
-    hdr[0] = (int32_t)nt;
-    hdr[1] = (int32_t)ng;
-  }
-  __syncthreads();
-  if (s_tiles == 0) return;
-  // every thread walks the sequences it owns; the running tile counts are recomputed per thread
-  for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
-    int64_t tile = 0, gt = 0;
-    for (int64_t c = 0; c < b; ++c) {
-      tile += (range[c] + kBM - 1) / kBM;
-      gt += (ewin[c] + kBM - 1) / kBM;
-    }
-    const int P = range[b], E = ewin[b];
-    for (int t0 = 0; t0 < P; t0 += kBM, ++tile) {
-      const int nvalid = P - t0 < kBM ? P - t0 : kBM;
-      int ngrad = E - t0;
-      ngrad = ngrad < 0 ? 0 : (ngrad > kBM ? kBM : ngrad);
-      if (!ADWIN_CHK(tile < max_tiles && gt < max_tiles, status)) break;
-      int32_t* e = tiles + tile * kTileFields;
-      e[0] = (int32_t)b;
-      e[1] = t0;
-      e[2] = nvalid;
-      e[3] = ngrad;
-      e[4] = ngrad > 0 ? (int32_t)gt : -1;
-      if (ngrad > 0) {
-        g2t[gt] = (int32_t)tile;
-        for (int i = 0; i < kBM; ++i)
-          rowdst[gt * kBM + i] = i < ngrad ? (int32_t)(b * T + t0 + i) : -1;
-        ++gt;
-      }
-    }
-  }
-}
-
-// Compact, zero-padded copy of the hidden states of the processed positions: row tile*128+i of
-// dst is src[b, t0+i, :] for i < nvalid and zero otherwise.  by_gtile selects the gradient tiles.
-__global__ void __launch_bounds__(256) lm_gather_kernel(const __nv_bfloat16* __restrict__ src,
-                                                        int64_t T, int64_t d, const int32_t* hdr,
-                                                        const int32_t* __restrict__ tiles,
-                                                        const int32_t* __restrict__ g2t,
-                                                        bool by_gtile, __nv_bfloat16* dst) {
-  const int64_t n_rows = (int64_t)hdr[by_gtile ? 1 : 0] * kBM;
-  const int64_t vec_per_row = d / 8;
-  for (int64_t row = blockIdx.x; row < n_rows; row += gridDim.x) {
-    const int64_t tl = row / kBM;
-    const int i = (int)(row % kBM);
-    const int32_t* e = tiles + (by_gtile ? g2t[tl] : tl) * kTileFields;
-    const int lim = by_gtile ? e[3] : e[2];
-    uint4* o = reinterpret_cast<uint4*>(dst + row * d);
-    if (i < lim) {
-      const uint4* s = reinterpret_cast<const uint4*>(src + ((int64_t)e[0] * T + e[1] + i) * d);
-      for (int64_t v = threadIdx.x; v < vec_per_row; v += blockDim.x) o[v] = s[v];
-    } else {
-      for (int64_t v = threadIdx.x; v < vec_per_row; v += blockDim.x) o[v] = make_uint4(0, 0, 0, 0);
-    }
-  }
-}
-
-// The two logits at the sampled token of every processed position, z_y = h_s . W_s[y] and
-// u_y = h_t . W_t[y], as plain fp32 dot products (one warp per compact row).  They give the
-// sampled-token log-ratio of Section 2.3 without a search through the logit tiles, and their
-// difference is the value the sweep centres z - u on: on a peaked row the sampled token is almost
-// surely the peak, where the centred difference is then exactly zero, which keeps the
-// single-sweep squared-norm moments well conditioned.
-__device__ __forceinline__ float warp_dot_bf16(const __nv_bfloat16* a, const __nv_bfloat16* b,
-                                               int64_t d, int lane) {
-  float acc = 0.f;
-  for (int64_t v = lane; v < d / 8; v += 32) {
-    const uint4 x = reinterpret_cast<const uint4*>(a)[v], y = reinterpret_cast<const uint4*>(b)[v];
-    float xf[8], yf[8];
-    Elem<__nv_bfloat16>::unpack(x, xf);
-    Elem<__nv_bfloat16>::unpack(y, yf);
+    int64_t x = n;   // inclusive scan of the warp
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc = fmaf(xf[i], yf[i], acc);
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) part[warp] = x;
+    __syncthreads();
+    int64_t before = 0, all = 0;
+    for (int w = 0; w < 32; ++w) {
+      if (w < warp) before += part[w];
+      all += part[w];
+    }
+    if (b < B) out[b] = base + before + x - n;
+    base += all;
+    __syncthreads();
+  }
+  if (tid == 0) out[B] = base;
+}
+
+struct GatherParams {
+  const __nv_bfloat16* hs;
+  const __nv_bfloat16* ht;
+  const __nv_bfloat16* ws;
+  const __nv_bfloat16* wt;
+  const int32_t* tokens;
+  const int32_t* range;
+  const int32_t* ewin;
+  const int64_t* seg;
+  int64_t B, T, V, ds, dt, max_tiles;
+  LmHeader* hdr;
+  int32_t* rowsrc;
+  int32_t* rowdst;
+  float* tok;
+  __nv_bfloat16* hs_c;
+  __nv_bfloat16* ht_c;
+  int32_t* status;
+};
+
+// Copies one hidden-state row (d % 8 == 0) and forms its fp32 dot product with an embedding row.
+__device__ __forceinline__ float copy_dot(const __nv_bfloat16* src, const __nv_bfloat16* w,
+                                          __nv_bfloat16* dst, int64_t d, int lane) {
+  float acc = 0.f;
+#pragma unroll 4
+  for (int64_t v = lane; v < d / 8; v += 32) {
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    if (src) x = __ldg(reinterpret_cast<const uint4*>(src) + v);
+    reinterpret_cast<uint4*>(dst)[v] = x;
+    if (w) {
+      const uint4 y = __ldg(reinterpret_cast<const uint4*>(w) + v);
+      float xf[8], yf[8];
+      Elem<__nv_bfloat16>::unpack(x, xf);
+      Elem<__nv_bfloat16>::unpack(y, yf);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc = fmaf(xf[i], yf[i], acc);
+    }
   }
   return warp_sum(acc);
 }
 
-__global__ void __launch_bounds__(256) lm_token_kernel(
-    const __nv_bfloat16* __restrict__ hs_c, const __nv_bfloat16* __restrict__ ws,
-    const __nv_bfloat16* __restrict__ ht_c, const __nv_bfloat16* __restrict__ wt, int64_t T,
-    int64_t V, int64_t ds, int64_t dt, const int32_t* hdr, const int32_t* __restrict__ tiles,
-    const int32_t* __restrict__ tokens, float* tok) {
+// One warp per compact row: which position it is, copies of its two hidden-state rows (zeros past
+// the rows), and the two logits at its sampled token, z_y = h_s . W_s[y] and u_y = h_t . W_t[y].
+// They give the sampled-token log-ratio of Section 2.3 without a search through the logit tiles, and
+// their difference is the value the sweep centres z - u on: on a peaked row the sampled token is
+// almost surely the peak, where the centred difference is then exactly zero, which keeps the
+// single-sweep squared-norm moments well conditioned.
+__global__ void __launch_bounds__(256) lm_gather_kernel(const GatherParams p, const SegPlan plan) {
+  __shared__ int64_t base[kMaxSeg + 1];
+  if (threadIdx.x == 0) {
+    int64_t o = 0;
+    for (int i = 0; i < plan.n_seg; ++i) {
+      base[i] = o;
+      o += (p.seg[(int64_t)i * (p.B + 1) + p.B] + plan.pad - 1) / plan.pad * plan.pad;
+    }
+    base[plan.n_seg] = o;
+  }
+  __syncthreads();
+  const int64_t rows = base[plan.n_seg];
+  const int64_t grad_rows = plan.by_cut ? rows : base[1];
+  int64_t tiles = (rows + kBM - 1) / kBM;
+  const bool fits = tiles <= p.max_tiles;
+  if (!fits) tiles = 0;
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) {
+      if (!fits) atomicOr(p.status, ADWIN_DEV_WORKSPACE);   // more rows than the workspace is for
+      p.hdr->tiles = (int32_t)tiles;
+      p.hdr->grad_tiles = fits ? (int32_t)((grad_rows + kBM - 1) / kBM) : 0;
+    }
+    if (threadIdx.x < 60) p.hdr->pace[threadIdx.x] = 0u;
+    if (threadIdx.x <= plan.n_seg)
+      p.hdr->seg_kblock[threadIdx.x] = fits ? (int32_t)(base[threadIdx.x] / 64) : 0;
+  }
   const int lane = threadIdx.x & 31;
-  const int64_t n_rows = (int64_t)hdr[0] * kBM;
-  for (int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); row < n_rows;
-       row += (int64_t)gridDim.x * 8) {
-    const int32_t* e = tiles + (row / kBM) * kTileFields;
-    const int i = (int)(row % kBM);
-    float zy = 0.f, uy = 0.f, has = 0.f;
-    if (i < e[2]) {
-      const int y = tokens[(int64_t)e[0] * T + e[1] + i];
-      if (y >= 0 && y < V) {
-        zy = warp_dot_bf16(hs_c + row * ds, ws + (int64_t)y * ds, ds, lane);
-        uy = warp_dot_bf16(ht_c + row * dt, wt + (int64_t)y * dt, dt, lane);
-        has = 1.f;
+  for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < tiles * kBM;
+       r += (int64_t)gridDim.x * 8) {
+    int64_t src = -1;
+    if (r < rows) {
+      int i = 0;
+      while (r >= base[i + 1]) ++i;
+      const int64_t* off = p.seg + (int64_t)i * (p.B + 1);
+      const int64_t k = r - base[i];
+      if (k < off[p.B]) {
+        int64_t b = 0, e = p.B;   // the last sequence with off[b] <= k
+        while (e - b > 1) {
+          const int64_t m = (b + e) / 2;
+          if (off[m] <= k) b = m; else e = m;
+        }
+        int lo, hi;
+        plan.range(i, p.ewin[b], p.range[b], lo, hi);
+        src = b * p.T + lo + (k - off[b]);
       }
     }
+    if (!ADWIN_CHK(src < p.B * p.T && r < p.max_tiles * kBM, p.status)) continue;
+    const int y = src >= 0 ? p.tokens[src] : -1;
+    const bool has = y >= 0 && y < p.V;
+    const float zy = copy_dot(src >= 0 ? p.hs + src * p.ds : nullptr,
+                              has ? p.ws + (int64_t)y * p.ds : nullptr, p.hs_c + r * p.ds, p.ds, lane);
+    const float uy = copy_dot(src >= 0 ? p.ht + src * p.dt : nullptr,
+                              has ? p.wt + (int64_t)y * p.dt : nullptr, p.ht_c + r * p.dt, p.dt, lane);
     if (lane == 0) {
-      float* o = tok + row * kTokFields;
-      o[0] = zy;
-      o[1] = uy;
-      o[2] = has;
-      o[3] = 0.f;
+      p.rowsrc[r] = (int32_t)src;
+      p.rowdst[r] = r < grad_rows ? (int32_t)src : -1;
+      *reinterpret_cast<float4*>(p.tok + r * kTokFields) =
+          make_float4(has ? zy : 0.f, has ? uy : 0.f, has ? 1.f : 0.f, 0.f);
     }
   }
 }
 
 // ---------------------------------------------------------------------------- sweep kernel
 struct SweepParams {
-  const int32_t* hdr;
-  const int32_t* tiles;
-  const int32_t* g2t;
-  const float* tok;             // sweep 1 in: z_y, u_y per compact row
-  int64_t T, V;
+  LmHeader* hdr;
+  const float* tok;             // z_y, u_y per compact row
+  int64_t V;
   int ks_blocks, kt_blocks;     // k-blocks of the student / teacher contraction
-  int n_chunks, n_groups;
-  float* part;                  // sweep 1 out: partial records; sweep 2 out: partial sum g^2
-  const float* info;            // sweep 2 in
-  __nv_bfloat16* G;             // sweep 2 out
-  int64_t ldG;
-  int64_t max_tiles;            // capacity of the per-tile buffers (checked flavour)
+  int n_chunks;
+  int64_t tile0;                // first tile of this launch (unused with rest = 1)
+  int64_t tile_cap;             // tiles of this launch, at most
+  int rest;                     // 0: gradient tiles, 1: the tiles behind them, 2: all tiles
+  float4* keep;                 // logits of the launch's tiles (null: not kept)
+  int keep_u;                   // the teacher's as well
+  float4* park;                 // one student tile per CTA (when nothing is kept)
+  float* part;                  // partial records
+  int64_t part_slots;
+  unsigned int* pace;
   uint64_t limit_ns;            // limit of the handshake waits
   int32_t* status;
 };
 
-// chunk range of vocabulary group g
-__device__ __forceinline__ void group_chunks(const SweepParams& p, int g, int& c0, int& c1) {
-  const int per = (p.n_chunks + p.n_groups - 1) / p.n_groups;
-  c0 = g * per;
-  c1 = c0 + per < p.n_chunks ? c0 + per : p.n_chunks;
-  if (c0 > c1) c0 = c1;
+// The tiles [lo, hi) of a launch.
+__device__ __forceinline__ void launch_tiles(const LmHeader* hdr, int64_t tile0, int64_t cap, int rest,
+                                             int64_t& lo, int64_t& hi) {
+  const int64_t all = rest ? hdr->tiles : hdr->grad_tiles;
+  lo = rest == 1 ? hdr->grad_tiles : tile0;
+  hi = lo + cap < all ? lo + cap : all;
+  if (hi < lo) hi = lo;
 }
 
-// MOMENTS = false drops the squared-norm moments from sweep 1 (when every processed row gets its
-// gsq from sweep 2, or no gsq is asked for).
-// GRAD = false: sweep 1 (statistics).  GRAD = true: sweep 2 (logit gradient); NEED_U = false
-// skips the teacher product there (the sampled-token estimator of Eq. 4 does not need it).
-template <bool GRAD, bool NEED_U, int BN, bool MOMENTS = true, bool PAIR = false>
+// Cost of cutting the vocabulary into g groups, in quarter chunks: rounds of items over the pairs
+// of CTAs times the chunks of an item (plus a quarter for its records).
+__device__ __forceinline__ unsigned int group_cost(int64_t units, int n_chunks, int pairs, int g) {
+  return (unsigned int)((units * g + pairs - 1) / pairs * (4 * ((n_chunks + g - 1) / g) + 1));
+}
+
+// chunk range of vocabulary group g
+__device__ __forceinline__ void group_chunks(int n_chunks, int n_groups, int g, int& c0, int& c1) {
+  c0 = (int)((int64_t)n_chunks * g / n_groups);
+  c1 = (int)((int64_t)n_chunks * (g + 1) / n_groups);
+}
+
+// Statistics of 256 x 256 logit tiles on CTA pairs (this CTA: 128 of the rows).  The student
+// product of a chunk goes to accumulator slot 0, the teacher product to slot 1.  The epilogue takes
+// the student tile out of tensor memory as soon as it is complete, while the teacher product runs,
+// and parks it in global memory (L2; the same thread reads it back), so the MMAs never wait for
+// the arithmetic, which runs on the teacher tile during the next chunk's student product.
+// MOMENTS = false drops the squared-norm moments (when every processed row gets its gsq from the
+// gradient entries, or no gsq is asked for).
+template <bool MOMENTS>
 __global__ void __launch_bounds__(kThreads, 1)
 lm_sweep_kernel(const __grid_constant__ CUtensorMap map_hs, const __grid_constant__ CUtensorMap map_ws,
                 const __grid_constant__ CUtensorMap map_ht, const __grid_constant__ CUtensorMap map_wt,
                 const SweepParams p) {
-  // BN = 256: one accumulator pair (student + teacher tile) fills the 512 TMEM columns, the
-  // epilogue and the MMAs of the next chunk alternate.  BN = 128: two pairs, so the epilogue of a
-  // chunk overlaps the MMAs of the next, at 1.5x the operand bytes per flop.
-  // PAIR: two CTAs of a cluster form one MMA unit (cta_group::2): a 256-row tile pair, each CTA
-  // stages its own A tile and half of the B tile (32 KB per stage instead of 48) and reads its own
-  // 128 rows of the accumulators; the even CTA issues the MMAs.
-  static_assert(!PAIR || BN == 256, "the pair form uses 256-column tiles");
-  constexpr int kBrows = PAIR ? BN / 2 : BN;        // rows of the B tile this CTA stages
-  constexpr int kStB = kABytes + kBrows * kBK * 2;  // bytes per stage
-  constexpr int kSt = (kStages * kStageBytes) / kStB < kMaxStages ? (kStages * kStageBytes) / kStB
-                                                                  : kMaxStages;   // pipeline stages
-  constexpr int kAcc = kTmemCols / (2 * BN);        // accumulator pairs
-  constexpr int kHalf = BN / 2;                     // columns per epilogue warpgroup
-  static_assert(kSt <= kMaxStages && kSt * kStB <= kStages * kStageBytes, "stage budget");
   extern __shared__ uint8_t smem_raw[];
+  __shared__ unsigned long long s_best;
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(smem_raw);
   const uint32_t stage0 = (smem_addr(smem_raw) + kCtrlBytes + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort = &ctrl->abort;
-  const uint32_t rank = PAIR ? cluster_ctarank() : 0u;   // 0: the CTA that issues the MMAs
+  const uint32_t rank = cluster_ctarank();   // 0: the CTA that issues the MMAs
+  const int pair = blockIdx.x / 2, pairs = gridDim.x / 2;
 
+  int64_t lo, hi;
+  launch_tiles(p.hdr, p.tile0, p.tile_cap, p.rest, lo, hi);
+  const int64_t units = (hi - lo + 1) / 2;   // pairs of tiles
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kSt; ++s) {
-      bar_init(smem_addr(&ctrl->full[s]), 1);
-      bar_init(smem_addr(&ctrl->empty[s]), 1);
-    }
-    for (int s = 0; s < kAcc; ++s) {
-      bar_init(smem_addr(&ctrl->acc_full[s]), 1);
-      bar_init(smem_addr(&ctrl->acc_empty[s]), PAIR ? 2 * (kEpiThreads / 32) : kEpiThreads);
-    }
-    bar_init(smem_addr(&ctrl->drain), 1);
-    ctrl->abort = 0;
-    bar_init_fence();
+    s_best = ~0ull;
+    pair_bars_init(ctrl);
   }
   if (warp == 2) {
-    if (PAIR) {
-      tmem_alloc_pair(smem_addr(&ctrl->tmem_base), kTmemCols);
-      tmem_relinquish_pair();
-    } else {
-      tmem_alloc(smem_addr(&ctrl->tmem_base), kTmemCols);
-      tmem_relinquish();
-    }
+    tmem_alloc_pair(smem_addr(&ctrl->tmem_base), kTmemCols);
+    tmem_relinquish_pair();
     tc_fence_before_sync();
   }
   __syncthreads();
-  if (PAIR) cluster_sync();   // the partner's barriers exist before anything signals them
+  // The number of vocabulary groups: the cheapest cut within the record buffer.  (With 8 groups
+  // throughout, a call of 225 rows at V = 32 000 had 24 items for 148 SMs.)
+  if (units > 0) {
+    int64_t most = 4 * pairs / units;
+    if (most < 8) most = 8;
+    if (most > p.n_chunks) most = p.n_chunks;
+    for (int g = 1 + (int)threadIdx.x; g <= most; g += kThreads)
+      atomicMin(&s_best, ((unsigned long long)group_cost(units, p.n_chunks, pairs, g) << 32) | (unsigned)g);
+  }
+  __syncthreads();
+  cluster_sync();   // the partner's barriers exist before anything signals them
   tc_fence_after_sync();
   const uint32_t tmem_base = ctrl->tmem_base;
-
-  // Work items: (tile, vocabulary group), or (pair of consecutive tiles, group) for a CTA pair,
-  // in which CTA `rank` owns tile 2*pair + rank (the second tile of the last pair may not exist).
-  const int n_tiles = p.hdr[GRAD ? 1 : 0];
-  const int64_t n_units = PAIR ? (n_tiles + 1) / 2 : n_tiles;
-  const int64_t n_items = n_units * p.n_groups;
-  const int64_t first_item = PAIR ? blockIdx.x / 2 : blockIdx.x;
-  const int64_t item_step = PAIR ? gridDim.x / 2 : gridDim.x;
+  const int n_groups = units > 0 ? (int)(s_best & 0xffffffffu) : 1;
+  if (blockIdx.x == 0 && threadIdx.x == 0) p.hdr->n_groups = n_groups;
+  const int64_t n_items = units * n_groups;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int64_t item = first_item; ok && item < n_items; item += item_step) {
-        const int tile = (PAIR ? 2 : 1) * (int)(item / p.n_groups) + (int)rank;
-        const int g = (int)(item % p.n_groups);
-        const int row0 = tile * kBM;          // compact row of the tile (tile or gradient-tile order)
+      Pace pace(rank == 0 ? p.pace : nullptr, pairs);
+      for (int64_t item = pair; ok && item < n_items; item += pairs) {
+        const int row0 = (int)(lo + 2 * (item / n_groups) + rank) * kBM;
         int c0, c1;
-        group_chunks(p, g, c0, c1);
+        group_chunks(p.n_chunks, n_groups, (int)(item % n_groups), c0, c1);
         for (int c = c0; ok && c < c1; ++c) {
-          for (int pass = 0; ok && pass < (NEED_U ? 2 : 1); ++pass) {
+          for (int pass = 0; ok && pass < 2; ++pass) {
             const CUtensorMap* ma = pass ? &map_ht : &map_hs;
             const CUtensorMap* mb = pass ? &map_wt : &map_ws;
             const int nk = pass ? p.kt_blocks : p.ks_blocks;
             for (int kb = 0; kb < nk; ++kb, ++it) {
-              const uint32_t s = it % kSt, ph = (it / kSt) & 1;
+              const uint32_t s = it % kPairStages, ph = (it / kPairStages) & 1;
+              pace.kblock(it);
               if (!bar_wait(smem_addr(&ctrl->empty[s]), ph ^ 1, abort, p.limit_ns)) { ok = false; break; }
               const uint32_t bar = smem_addr(&ctrl->full[s]);
-              const uint32_t a = stage0 + s * kStB, b = a + kABytes;
-              if (PAIR) {
-                // both CTAs' bytes are counted by the even CTA's barrier
-                if (rank == 0) bar_expect_tx(bar, 2 * kStB);
-                const uint32_t bar0 = map_to_cta(bar, 0);
-                tma_load_2d_pair(a, ma, kb * kBK, row0, bar0);
-                tma_load_2d_pair(b, mb, kb * kBK, c * BN + (int)rank * kBrows, bar0);
-              } else {
-                bar_expect_tx(bar, kStB);
-                tma_load_2d(a, ma, kb * kBK, row0, bar);
-                tma_load_2d(b, mb, kb * kBK, c * BN, bar);
-              }
+              const uint32_t a = stage0 + s * kPairStageBytes, b = a + kABytes;
+              if (rank == 0) bar_expect_tx(bar, 2 * kPairStageBytes);   // both CTAs' bytes
+              const uint32_t bar0 = map_to_cta(bar, 0);
+              load_operand_pair<false>(a, ma, row0, kb * kBK, bar0);
+              load_operand_pair<false>(b, mb, c * kBN + (int)rank * (kBN / 2), kb * kBK, bar0);
             }
           }
         }
       }
-      // give up: let the copies in flight land before the CTA's shared memory goes (in a pair the
-      // even CTA's barriers count both CTAs' copies, and the final cluster barrier holds the odd
-      // CTA until the even one has waited for them)
-      if (!ok && rank == 0) {
-        const uint32_t n_out = it < (uint32_t)kSt ? it : (uint32_t)kSt;
-        for (uint32_t j = it - n_out; j < it; ++j)
-          bar_wait_drain(smem_addr(&ctrl->full[j % kSt]), (j / kSt) & 1);
-      }
+      pace.done();
+      if (!ok && rank == 0) pair_drain_loads(ctrl, it);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0 && rank == 0) {
       uint32_t it = 0, acc_it = 0;
       bool ok = true;
-      for (int64_t item = first_item; ok && item < n_items; item += item_step) {
+      for (int64_t item = pair; ok && item < n_items; item += pairs) {
         int c0, c1;
-        group_chunks(p, (int)(item % p.n_groups), c0, c1);
+        group_chunks(p.n_chunks, n_groups, (int)(item % n_groups), c0, c1);
         for (int c = c0; ok && c < c1; ++c, ++acc_it) {
-          const uint32_t slot = acc_it % kAcc, aph = (acc_it / kAcc) & 1;
-          if (!bar_wait(smem_addr(&ctrl->acc_empty[slot]), aph ^ 1, abort, p.limit_ns)) { ok = false; break; }
-          tc_fence_after_sync();
-          for (int pass = 0; ok && pass < (NEED_U ? 2 : 1); ++pass) {
+          for (int pass = 0; ok && pass < 2; ++pass) {
+            if (!bar_wait(smem_addr(&ctrl->acc_empty[pass]), (acc_it & 1) ^ 1, abort, p.limit_ns)) { ok = false; break; }
+            tc_fence_after_sync();
             const int nk = pass ? p.kt_blocks : p.ks_blocks;
-            const uint32_t tmem_d = tmem_base + slot * (2 * BN) + (pass ? BN : 0);
             for (int kb = 0; kb < nk; ++kb, ++it) {
-              const uint32_t s = it % kSt, ph = (it / kSt) & 1;
+              const uint32_t s = it % kPairStages, ph = (it / kPairStages) & 1;
               if (!bar_wait(smem_addr(&ctrl->full[s]), ph, abort, p.limit_ns)) { ok = false; break; }
               tc_fence_after_sync();
-              const uint32_t a = stage0 + s * kStB, b = a + kABytes;
-              if (PAIR) {
-                issue_kblock_pair<BN>(tmem_d, a, b, kb == 0);
-                umma_commit_pair(smem_addr(&ctrl->empty[s]));
-              } else {
-                issue_kblock<false, false, BN>(tmem_d, a, b, kb == 0);
-                umma_commit(smem_addr(&ctrl->empty[s]));
-              }
+              const uint32_t a = stage0 + s * kPairStageBytes, b = a + kABytes;
+              issue_kblock_pair<false, false>(tmem_base + pass * kBN, a, b, kb == 0);
+              umma_commit_pair(smem_addr(&ctrl->empty[s]));
             }
-          }
-          if (ok) {
-            if (PAIR) umma_commit_pair(smem_addr(&ctrl->acc_full[slot]));
-            else umma_commit(smem_addr(&ctrl->acc_full[slot]));
+            if (ok) umma_commit_pair(smem_addr(&ctrl->acc_full[pass]));
           }
         }
       }
       if (!ok) {   // give up: wait until the MMAs already issued have retired
-        if (PAIR) umma_commit_pair(smem_addr(&ctrl->drain));
-        else umma_commit(smem_addr(&ctrl->drain));
+        umma_commit_pair(smem_addr(&ctrl->drain));
         bar_wait_drain(smem_addr(&ctrl->drain), 0);
       }
     }
@@ -431,59 +436,83 @@ lm_sweep_kernel(const __grid_constant__ CUtensorMap map_hs, const __grid_constan
     const int quad = warp & 3;               // TMEM lanes 32*quad .. 32*quad+31
     const int half = ew >> 2;                // columns half*128 .. half*128+127 of the tile
     const int row = quad * 32 + lane;
-    const uint32_t t_quad = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * kHalf);
+    const uint32_t t_lane = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * 128);
     uint32_t acc_it = 0;
     bool ok = true;
-    for (int64_t item = first_item; ok && item < n_items; item += item_step) {
-      const int tile_c = (PAIR ? 2 : 1) * (int)(item / p.n_groups) + (int)rank;
-      const int g = (int)(item % p.n_groups);
-      const bool live = tile_c < n_tiles;     // the last pair's second tile may not exist
-      const int tile = !live ? 0 : (GRAD ? p.g2t[tile_c] : tile_c);
+    for (int64_t item = pair; ok && item < n_items; item += pairs) {
+      const int64_t tile = lo + 2 * (item / n_groups) + rank;
+      const int g = (int)(item % n_groups);
+      const bool live = tile < hi;     // the last pair's second tile may not exist
       int c0, c1;
-      group_chunks(p, g, c0, c1);
-
-      int y = -1;
+      group_chunks(p.n_chunks, n_groups, g, c0, c1);
       RowAcc acc;
-      float dref = 0.f, q = 0.f;   // q: this thread's share of the row's sum g^2 (sweep 2)
-      float L2s = 0.f, a1 = 0.f, a0 = 0.f, gy = 0.f;
       acc.reset();
-      if (!live) {
-        // nothing to read: the tile's accumulators hold products of whatever the loads returned
-      } else if (!GRAD) {
-        const float* tk = p.tok + ((int64_t)tile * kBM + row) * kTokFields;
+      float dref = 0.f;
+      if (live) {
+        const float* tk = p.tok + (tile * kBM + row) * kTokFields;
         dref = tk[0] - tk[1];      // centre of z - u for this row: the sampled token's difference
-      } else {
-        const float* inf = p.info + ((int64_t)tile * kBM + row) * kInfoFields;
-        L2s = inf[0];
-        a1 = inf[1];
-        a0 = inf[2];
-        gy = inf[3];
-        y = __float_as_int(inf[4]);
       }
       for (int c = c0; ok && c < c1; ++c, ++acc_it) {
-        const uint32_t slot = acc_it % kAcc, aph = (acc_it / kAcc) & 1;
-        const uint32_t t_lane = t_quad + slot * (2 * BN);
-        if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&ctrl->acc_full[slot]), aph, abort, p.limit_ns))) {
+        // this thread's place in the 128 x 256 tile: [64 groups of 4 columns][128 rows]
+        float4* zp = (p.keep ? p.keep + ((tile - lo) * p.n_chunks + c) * (2 * kKeepArray)
+                             : p.park + (int64_t)blockIdx.x * kKeepArray) +
+                     (half * 32) * kBM + row;
+        if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&ctrl->acc_full[0]), acc_it & 1, abort, p.limit_ns))) {
           ok = false;   // the same decision in every lane: tcgen05.ld below is warp-collective
           break;
         }
         tc_fence_after_sync();
-        const int64_t col_base = (int64_t)c * BN + half * kHalf;
-        const bool ragged = col_base + kHalf > p.V;
 #pragma unroll 1
-        for (int j = 0; live && j < kHalf / 32; ++j) {
-          uint32_t zr[32], ur[32];
-          tmem_ld32(t_lane + j * 32, zr);
-          if (NEED_U) tmem_ld32(t_lane + BN + j * 32, ur);
+        for (int j = 0; j < 4; ++j) {
+          uint32_t r[32];
+          tmem_ld32(t_lane + j * 32, r);
           tmem_ld_wait();
-          const int64_t col = col_base + j * 32;
-          float z[32], u[32];
+          if (live) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            z[i] = __uint_as_float(zr[i]);
-            u[i] = NEED_U ? __uint_as_float(ur[i]) : 0.f;
+            for (int i = 0; i < 8; ++i)
+              zp[(j * 8 + i) * kBM] =
+                  make_float4(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1]),
+                              __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3]));
+          }
+        }
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) pair_release(&ctrl->acc_empty[0], rank);
+
+        if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&ctrl->acc_full[1]), acc_it & 1, abort, p.limit_ns))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after_sync();
+        const int64_t col_base = (int64_t)c * kBN + half * 128;
+        const bool ragged = col_base + 128 > p.V;
+#pragma unroll 1
+        for (int j = 0; j < 4; ++j) {
+          uint32_t ur[32];
+          float z[32], u[32];
+          if (live) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float4 x = zp[(j * 8 + i) * kBM];
+              z[4 * i] = x.x;
+              z[4 * i + 1] = x.y;
+              z[4 * i + 2] = x.z;
+              z[4 * i + 3] = x.w;
+            }
+          }
+          tmem_ld32(t_lane + kBN + j * 32, ur);
+          tmem_ld_wait();
+          if (!live) continue;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) u[i] = __uint_as_float(ur[i]);
+          if (p.keep && p.keep_u) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              zp[kKeepArray + (j * 8 + i) * kBM] =
+                  make_float4(u[4 * i], u[4 * i + 1], u[4 * i + 2], u[4 * i + 3]);
           }
           if (ragged) {   // columns past the vocabulary: exp -> 0, z - u -> 0
+            const int64_t col = col_base + j * 32;
 #pragma unroll
             for (int i = 0; i < 32; ++i)
               if (col + i >= p.V) {
@@ -491,60 +520,15 @@ lm_sweep_kernel(const __grid_constant__ CUtensorMap map_hs, const __grid_constan
                 u[i] = kMasked;
               }
           }
-          if (!GRAD) {
-            acc_piece<32, MOMENTS>(z, u, dref, acc);
-          } else {
-            uint32_t pk[16];
-#pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-              float gv[2];
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const float pz = ex2f(fmaf(z[i + e], kLog2e, -L2s));
-                const float w = NEED_U ? fmaf(a1, z[i + e] - u[i + e], a0) : a0;
-                gv[e] = pz * w;
-                q = fmaf(gv[e], gv[e], q);
-              }
-              pk[i >> 1] = pack_bf16x2(gv[0], gv[1]);
-            }
-            if ((unsigned)(y - (int)col) < 32u) {   // the sampled token's own entry (Eq. 4)
-              const int yi = y - (int)col;
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (i == yi) {
-                  const float pz = ex2f(fmaf(z[i], kLog2e, -L2s));
-                  const float w = NEED_U ? fmaf(a1, z[i] - u[i], a0) : a0;
-                  const float gv = fmaf(pz, w, gy);
-                  q += gv * gv - (pz * w) * (pz * w);
-                  const uint32_t h = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(gv));
-                  pk[i >> 1] = (i & 1) ? ((pk[i >> 1] & 0x0000ffffu) | (h << 16))
-                                       : ((pk[i >> 1] & 0xffff0000u) | h);
-                }
-            }
-            __nv_bfloat16* gp = p.G + ((int64_t)tile_c * kBM + row) * p.ldG + col;
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-              if (col + v * 8 < p.V &&
-                  ADWIN_CHK(tile_c < p.max_tiles && col + v * 8 + 8 <= p.ldG, p.status))
-                *reinterpret_cast<uint4*>(gp + v * 8) =
-                    make_uint4(pk[v * 4], pk[v * 4 + 1], pk[v * 4 + 2], pk[v * 4 + 3]);
-          }
+          acc_piece<32, MOMENTS>(z, u, dref, acc);
         }
         tc_fence_before_sync();
-        if (PAIR) {   // one arrival per warp: the odd CTA's arrivals cross to the even CTA
-          __syncwarp();
-          if (lane == 0) {
-            if (rank != 0) bar_arrive_cluster(map_to_cta(smem_addr(&ctrl->acc_empty[slot]), 0));
-            else bar_arrive(smem_addr(&ctrl->acc_empty[slot]));
-          }
-        } else {
-          bar_arrive(smem_addr(&ctrl->acc_empty[slot]));
-        }
+        __syncwarp();
+        if (lane == 0) pair_release(&ctrl->acc_empty[1], rank);
       }
-      if (GRAD && ok && live && ADWIN_CHK(tile_c < p.max_tiles && g < p.n_groups, p.status))
-        p.part[(((int64_t)tile_c * p.n_groups + g) * 2 + half) * kBM + row] = q;
-      if (!GRAD && ok && live && ADWIN_CHK(tile < p.max_tiles && g < p.n_groups && row < kBM, p.status)) {
-        float* o = p.part + ((((int64_t)tile * p.n_groups + g) * 2 + half) * kRecFields) * kBM + row;
+      const int64_t slot = (tile - lo) * n_groups + g;
+      if (ok && live && ADWIN_CHK(slot < p.part_slots, p.status)) {
+        float* o = p.part + ((slot * 2 + half) * kRecFields) * kBM + row;
         o[0 * kBM] = acc.m2s;
         o[1 * kBM] = acc.S;
         o[2 * kBM] = acc.A;
@@ -558,28 +542,28 @@ lm_sweep_kernel(const __grid_constant__ CUtensorMap map_hs, const __grid_constan
   }
   if (*abort && threadIdx.x == 0) {
     atomicOr(p.status, ADWIN_DEV_TIMEOUT);
-    if (PAIR) store_cluster_u32(map_to_cta(smem_addr(&ctrl->abort), rank ^ 1u), 1u);   // partner too
+    store_cluster_u32(map_to_cta(smem_addr(&ctrl->abort), rank ^ 1u), 1u);   // partner too
   }
   tc_fence_before_sync();
   __syncthreads();
-  if (PAIR) cluster_sync();   // neither CTA leaves while the other may still use its memory
+  cluster_sync();   // neither CTA leaves while the other may still use its memory
   if (warp == 2) {
     tc_fence_after_sync();
-    if (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
-    else tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc_pair(tmem_base, kTmemCols);
   }
 }
 
 // ---------------------------------------------------------------------------- merge kernel
 struct MergeParams {
-  const int32_t* hdr;
-  const int32_t* tiles;
+  const LmHeader* hdr;
+  const int32_t* rowsrc;
+  const int32_t* rowdst;
   const int32_t* tokens;
   const float* part;
   const float* tok;
   float* info;
-  int64_t T, V;
-  int n_groups;
+  int64_t tile0, tile_cap;
+  int rest;
   float alpha;
   int mode;
   float* kl;
@@ -590,46 +574,74 @@ struct MergeParams {
   int32_t* status;
 };
 
-// One thread per compact row: combine the partial records of the row in float64 against common
-// references and derive the per-token outputs and the gradient coefficients of sweep 2:
+// One block per tile, kMergeWays threads per compact row: combine the partial records of the row in
+// float64 against common references (fixed order) and derive the per-token outputs and the
+// gradient coefficients:
 //   g_k = p_k (a1 (z_k - u_k) + a0) (+ gy at k = y),   p_k = 2^(z_k log2e - L2s).
-__global__ void __launch_bounds__(kBM) lm_merge_kernel(const MergeParams p) {
-  const int tile = blockIdx.x;
-  if (tile >= p.hdr[0]) return;
-  const int row = threadIdx.x;
-  const int32_t* te = p.tiles + (int64_t)tile * kTileFields;
-  float* inf = p.info + ((int64_t)tile * kBM + row) * kInfoFields;
-  if (row >= te[2]) {
-    inf[0] = 0.f; inf[1] = 0.f; inf[2] = 0.f; inf[3] = 0.f; inf[4] = __int_as_float(-1);
-    return;
-  }
-  const int n = p.n_groups * 2;
-  const float* rec = p.part + ((int64_t)tile * n * kRecFields) * kBM + row;
+constexpr int kMergeWays = 8;
+__global__ void __launch_bounds__(kBM * kMergeWays) lm_merge_kernel(const MergeParams p) {
+  __shared__ double red[kMergeWays][kBM];
+  __shared__ double tot[kBM];
+  int64_t lo, hi;
+  launch_tiles(p.hdr, p.tile0, p.tile_cap, p.rest, lo, hi);
+  const int64_t tile = lo + blockIdx.x;
+  if (tile >= hi) return;
+  const int row = threadIdx.x % kBM, way = threadIdx.x / kBM;
+  const int64_t crow = tile * kBM + row;
+  const int n = p.hdr->n_groups * 2;
+  const float* rec = p.part + ((tile - lo) * n * kRecFields) * kBM + row;
   auto f = [&](int i, int k) { return (double)rec[((int64_t)i * kRecFields + k) * kBM]; };
+  // the sum (or maximum) of one value over the ways, in order; valid in every thread of the row
+  auto all_ways = [&](double v, bool max) {
+    __syncthreads();
+    red[way][row] = v;
+    __syncthreads();
+    if (way == 0) {
+      double a = red[0][row];
+      for (int i = 1; i < kMergeWays; ++i) a = max ? fmax(a, red[i][row]) : a + red[i][row];
+      tot[row] = a;
+    }
+    __syncthreads();
+    return tot[row];
+  };
   double M2s = -INFINITY, M2t = -INFINITY;
-  for (int i = 0; i < n; ++i) {
+  for (int i = way; i < n; i += kMergeWays) {
     M2s = fmax(M2s, f(i, 0));
     M2t = fmax(M2t, f(i, 6));
   }
-  const float* tk = p.tok + ((int64_t)tile * kBM + row) * kTokFields;
+  M2s = all_ways(M2s, true);
+  M2t = all_ways(M2t, true);
+  double S = 0, St = 0, Ac = 0, B0 = 0, B1 = 0, B2 = 0;
+  for (int i = way; i < n; i += kMergeWays) {
+    const double w = exp2(f(i, 0) - M2s), w2 = w * w;
+    S += w * f(i, 1);
+    Ac += w * f(i, 2);
+    B0 += w2 * f(i, 3);
+    B1 += w2 * f(i, 4);
+    B2 += w2 * f(i, 5);
+    St += exp2(f(i, 6) - M2t) * f(i, 7);
+  }
+  S = all_ways(S, false);
+  Ac = all_ways(Ac, false);
+  B0 = all_ways(B0, false);
+  B1 = all_ways(B1, false);
+  B2 = all_ways(B2, false);
+  St = all_ways(St, false);
+  if (way != 0) return;
+
+  float* inf = p.info + crow * kInfoFields;
+  const int64_t r = p.rowsrc[crow];
+  if (r < 0) {
+    inf[0] = 0.f; inf[1] = 0.f; inf[2] = 0.f; inf[3] = 0.f; inf[4] = __int_as_float(-1);
+    return;
+  }
+  const float* tk = p.tok + crow * kTokFields;
   const bool has_y = tk[2] != 0.f;
   const double zy = tk[0], uy = tk[1];
   const double dref = (double)(tk[0] - tk[1]);   // the centre the sweep used (an fp32 difference)
-  double S = 0, St = 0, Ac = 0;
-  for (int i = 0; i < n; ++i) {
-    const double w = exp2(f(i, 0) - M2s);
-    S += w * f(i, 1);
-    Ac += w * f(i, 2);
-    St += exp2(f(i, 6) - M2t) * f(i, 7);
-  }
   const double sh = -Ac / S;                   // centre minus E_p[z - u]
   const double c0 = dref - sh;                 // E_p[z - u]
-  double B0 = 0, B2c = 0;
-  for (int i = 0; i < n; ++i) {
-    const double w = exp2(f(i, 0) - M2s), w2 = w * w;
-    B0 += w2 * f(i, 3);
-    B2c += w2 * (f(i, 5) + 2.0 * sh * f(i, 4) + sh * sh * f(i, 3));
-  }
+  const double B2c = B2 + 2.0 * sh * B1 + sh * sh * B0;
   constexpr double kLn2 = 0.69314718055994530942;
   const double lse_s = (M2s + log2(S)) * kLn2, lse_t = (M2t + log2(St)) * kLn2;
   const double delta = lse_s - lse_t;
@@ -650,13 +662,12 @@ __global__ void __launch_bounds__(kBM) lm_merge_kernel(const MergeParams p) {
     a0 = -alpha * c;
     gy = alpha * c;
   }
-  const int64_t r = (int64_t)te[0] * p.T + te[1] + row;
   p.kl[r] = (float)kl;
   p.logratio[r] = (float)c;
   if (p.gsq) p.gsq[r] = (float)gsq;
   if (p.lse_s) p.lse_s[r] = (float)lse_s;
   if (p.lse_t) p.lse_t[r] = (float)lse_t;
-  const bool in_grad = row < te[3];
+  const bool in_grad = p.rowdst[crow] >= 0;
   inf[0] = in_grad ? (float)(lse_s * 1.4426950408889634074) : 0.f;
   inf[1] = in_grad ? (float)a1 : 0.f;
   inf[2] = in_grad ? (float)a0 : 0.f;
@@ -666,285 +677,282 @@ __global__ void __launch_bounds__(kBM) lm_merge_kernel(const MergeParams p) {
   if (!(isfinite(lse_s) && isfinite(lse_t))) atomicOr(p.status, ADWIN_DEV_NONFINITE);
 }
 
-// Squared gradient norm of the rows whose gradient sweep 2 formed: the sum of g_k^2 over the
-// entries themselves (fixed order, float64), which replaces the single-sweep moment value there.
-__global__ void __launch_bounds__(kBM) lm_gsq_kernel(const int32_t* hdr, const float* __restrict__ part,
+// ---------------------------------------------------------------------------- gradient kernel
+struct GradParams {
+  const LmHeader* hdr;
+  const float4* keep;
+  const float* info;
+  int64_t tile0, tile_cap, V;
+  int n_chunks, n_groups;       // column groups of this kernel
+  __nv_bfloat16* G;
+  int64_t ldG;
+  float* q;                     // per-row partial sums of g^2: [tile][group][half][128]
+  int64_t max_tiles;
+  int32_t* status;
+};
+
+// Streams a block's kept logits once and writes G.  One item = (tile, column group); a thread owns
+// one row of one 128-column half, so loads are coalesced over rows and every 32 columns of G leave
+// as two full 32-byte sectors.  Bound by memory: 8 bytes read and 2 written per entry.
+template <bool NEED_U>
+__global__ void __launch_bounds__(256, 2) lm_grad_kernel(const GradParams p) {
+  int64_t lo, hi;
+  launch_tiles(p.hdr, p.tile0, p.tile_cap, 0, lo, hi);
+  const int64_t tile = lo + blockIdx.x / p.n_groups;
+  const int g = blockIdx.x % p.n_groups;
+  if (tile >= hi) return;
+  const int row = threadIdx.x % kBM, half = threadIdx.x / kBM;
+  const int64_t crow = tile * kBM + row;
+  const float* inf = p.info + crow * kInfoFields;
+  const float L2s = inf[0], a1 = inf[1], a0 = inf[2], gy = inf[3];
+  const int y = __float_as_int(inf[4]);
+  int c0, c1;
+  group_chunks(p.n_chunks, p.n_groups, g, c0, c1);
+  float q = 0.f;
+  for (int c = c0; c < c1; ++c) {
+    const float4* zp = p.keep + ((tile - lo) * p.n_chunks + c) * (2 * kKeepArray) +
+                       (half * 32) * kBM + row;
+    const int64_t col_base = (int64_t)c * kBN + half * 128;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      const int64_t col = col_base + j * 32;
+      if (col >= p.V) break;
+      float4 z4[8], u4[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        z4[i] = __ldcs(zp + (j * 8 + i) * kBM);
+        if (NEED_U) u4[i] = __ldcs(zp + kKeepArray + (j * 8 + i) * kBM);
+      }
+      float v[32];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float z[4] = {z4[i].x, z4[i].y, z4[i].z, z4[i].w};
+        const float u[4] = {u4[i].x, u4[i].y, u4[i].z, u4[i].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float pz = ex2f(fmaf(z[e], kLog2e, -L2s));
+          v[4 * i + e] = pz * (NEED_U ? fmaf(a1, z[e] - u[e], a0) : a0);
+        }
+      }
+      if ((unsigned)(y - (int)col) < 32u) {   // the sampled token's own entry (Eq. 4)
+        const int yi = y - (int)col;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (i == yi) v[i] += gy;
+      }
+      uint32_t pk[16];
+#pragma unroll
+      for (int i = 0; i < 32; ++i)
+        if (col + i < p.V) q = fmaf(v[i], v[i], q);
+#pragma unroll
+      for (int i = 0; i < 32; i += 2) pk[i >> 1] = pack_bf16x2(v[i], v[i + 1]);
+      __nv_bfloat16* gp = p.G + crow * p.ldG + col;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (col + i * 8 < p.V && ADWIN_CHK(tile < p.max_tiles && col + i * 8 + 8 <= p.ldG, p.status))
+          *reinterpret_cast<uint4*>(gp + i * 8) =
+              make_uint4(pk[i * 4], pk[i * 4 + 1], pk[i * 4 + 2], pk[i * 4 + 3]);
+    }
+  }
+  p.q[((tile * p.n_groups + g) * 2 + half) * kBM + row] = q;
+}
+
+// Squared gradient norm of the rows whose gradient was formed: the sum of g_k^2 over the entries
+// themselves (fixed order, float64), which replaces the single-sweep moment value there.
+__global__ void __launch_bounds__(kBM) lm_gsq_kernel(const LmHeader* hdr, const float* __restrict__ q,
                                                      const int32_t* __restrict__ rowdst,
                                                      int n_groups, float* gsq) {
-  const int gt = blockIdx.x;
-  if (gt >= hdr[1]) return;
+  const int tile = blockIdx.x;
+  if (tile >= hdr->grad_tiles) return;
   const int row = threadIdx.x;
-  const int32_t dst = rowdst[(int64_t)gt * kBM + row];
+  const int32_t dst = rowdst[(int64_t)tile * kBM + row];
   if (dst < 0) return;
   double acc = 0.0;
+#pragma unroll 8
   for (int i = 0; i < n_groups * 2; ++i)
-    acc += (double)part[((int64_t)gt * n_groups * 2 + i) * kBM + row];
+    acc += (double)q[((int64_t)tile * n_groups * 2 + i) * kBM + row];
   gsq[dst] = (float)acc;
 }
 
-// ---------------------------------------------------------------------------- GEMM kernel
-// C[M,N] = A B with A[m,k], B[n,k] read through TMA in either major, fp32 accumulation in tensor
-// memory (two accumulator slots, so the epilogue of a tile overlaps the MMAs of the next one).
-struct GemmParams {
-  int64_t M, N;                 // extents of C (rows beyond M / columns beyond N are not stored)
-  int m_tiles, n_tiles, k_blocks;
-  const int32_t* m_tiles_dev;   // optional device-side override of m_tiles (index into hdr)
-  const int32_t* k_tiles_dev;   // optional: k_blocks = 2 * (*k_tiles_dev) (128 rows per tile)
-  const int32_t* k_list;        // optional: contraction row of every k-block (instead of kb*64)
-  const int32_t* k_count_dev;   // with k_list: number of k-blocks
-  const int32_t* row_map;       // optional: destination row of every C row, or -1 (skip)
-  void* C;
-  int64_t ldc;
-  int c_is_bf16;
+// The pass as the plain call and the weight-space audit use it.
+struct LmCall {
+  const void *hs, *ws, *ht, *wt;
+  int64_t B, T, V, ds, dt;
+  const int32_t *tokens, *window, *rollout_len;
+  float alpha;
+  int mode, flags;
+  void* dH;
+  int dh_dtype;
+  float* dW;
+  bool want_grad;               // G is formed (for dH, dW or the audit)
+  float *kl, *logratio, *gsq, *lse_s, *lse_t;
+  char* ws_base;
   int32_t* status;
-  uint64_t limit_ns;            // limit of the handshake waits
+  int sm_count;
 };
 
-template <bool A_MN, bool B_MN>
-__global__ void __launch_bounds__(kThreads, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const GemmParams p) {
-  extern __shared__ uint8_t smem_raw[];
-  Ctrl* ctrl = reinterpret_cast<Ctrl*>(smem_raw);
-  const uint32_t stage0 = (smem_addr(smem_raw) + kCtrlBytes + 1023u) & ~1023u;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  volatile int* abort = &ctrl->abort;
+cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, cudaStream_t s) {
+  char* wb = a.ws_base;
+  const bool range_full = (a.flags & ADWIN_RANGE_FULL) != 0;
+  LmHeader* hdr = reinterpret_cast<LmHeader*>(wb + L.off_hdr);
+  int64_t* seg = reinterpret_cast<int64_t*>(wb + L.off_seg);
+  int32_t* rowsrc = reinterpret_cast<int32_t*>(wb + L.off_rowsrc);
+  int32_t* rowdst = reinterpret_cast<int32_t*>(wb + L.off_rowdst);
+  float* info = reinterpret_cast<float*>(wb + L.off_info);
+  float* tok = reinterpret_cast<float*>(wb + L.off_tok);
+  float* part = reinterpret_cast<float*>(wb + L.off_part);
+  float* q = reinterpret_cast<float*>(wb + L.off_q);
+  float4* keep = reinterpret_cast<float4*>(wb + L.off_keep);
+  __nv_bfloat16* hs_c = reinterpret_cast<__nv_bfloat16*>(wb + L.off_hs);
+  __nv_bfloat16* ht_c = reinterpret_cast<__nv_bfloat16*>(wb + L.off_ht);
+  __nv_bfloat16* G = reinterpret_cast<__nv_bfloat16*>(wb + L.off_G);
+  float* pieces = reinterpret_cast<float*>(wb + L.off_pieces);
+  const int64_t rows_cap = L.max_tiles * kBM;
+  const int64_t ds = a.ds, dt = a.dt, V = a.V;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      bar_init(smem_addr(&ctrl->full[s]), 1);
-      bar_init(smem_addr(&ctrl->empty[s]), 1);
-    }
-    for (int s = 0; s < 2; ++s) {
-      bar_init(smem_addr(&ctrl->acc_full[s]), 1);
-      bar_init(smem_addr(&ctrl->acc_empty[s]), kEpiThreads);
-    }
-    bar_init(smem_addr(&ctrl->drain), 1);
-    ctrl->abort = 0;
-    bar_init_fence();
-  }
-  if (warp == 2) {
-    tmem_alloc(smem_addr(&ctrl->tmem_base), kTmemCols);
-    tmem_relinquish();
-    tc_fence_before_sync();
-  }
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem_base = ctrl->tmem_base;
-
-  const int m_tiles = p.m_tiles_dev ? *p.m_tiles_dev : p.m_tiles;
-  const int nk = p.k_list ? *p.k_count_dev : (p.k_tiles_dev ? 2 * (*p.k_tiles_dev) : p.k_blocks);
-  const int64_t n_items = (int64_t)m_tiles * p.n_tiles;
-
-  if (warp == 0) {
-    if (lane == 0 && nk > 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int64_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-        const int m0 = (int)(item / p.n_tiles) * kBM, n0 = (int)(item % p.n_tiles) * kBN;
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const uint32_t s = it % kStages, ph = (it / kStages) & 1;
-          if (!bar_wait(smem_addr(&ctrl->empty[s]), ph ^ 1, abort, p.limit_ns)) { ok = false; break; }
-          const uint32_t bar = smem_addr(&ctrl->full[s]);
-          const uint32_t a = stage0 + s * kStageBytes, b = a + kABytes;
-          bar_expect_tx(bar, kStageBytes);
-          const int k0 = p.k_list ? p.k_list[kb] : kb * kBK;
-          load_operand<A_MN, kBM>(a, &map_a, m0, k0, bar);
-          load_operand<B_MN, kBN>(b, &map_b, n0, k0, bar);
-        }
-      }
-      if (!ok) {
-        const uint32_t n_out = it < (uint32_t)kStages ? it : (uint32_t)kStages;
-        for (uint32_t j = it - n_out; j < it; ++j)
-          bar_wait_drain(smem_addr(&ctrl->full[j % kStages]), (j / kStages) & 1);
-      }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      uint32_t it = 0, acc_it = 0;
-      bool ok = true;
-      for (int64_t item = blockIdx.x; ok && item < n_items; item += gridDim.x, ++acc_it) {
-        const uint32_t slot = acc_it & 1, aph = (acc_it >> 1) & 1;
-        if (!bar_wait(smem_addr(&ctrl->acc_empty[slot]), aph ^ 1, abort, p.limit_ns)) { ok = false; break; }
-        tc_fence_after_sync();
-        const uint32_t tmem_d = tmem_base + slot * kBN;
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const uint32_t s = it % kStages, ph = (it / kStages) & 1;
-          if (!bar_wait(smem_addr(&ctrl->full[s]), ph, abort, p.limit_ns)) { ok = false; break; }
-          tc_fence_after_sync();
-          const uint32_t a = stage0 + s * kStageBytes, b = a + kABytes;
-          issue_kblock<A_MN, B_MN>(tmem_d, a, b, kb == 0);
-          umma_commit(smem_addr(&ctrl->empty[s]));
-        }
-        if (ok) {
-          if (nk > 0) umma_commit(smem_addr(&ctrl->acc_full[slot]));
-          else bar_arrive(smem_addr(&ctrl->acc_full[slot]));
-        }
-      }
-      if (!ok) {
-        umma_commit(smem_addr(&ctrl->drain));
-        bar_wait_drain(smem_addr(&ctrl->drain), 0);
-      }
-    }
-  } else if (warp >= kEpiWarp0) {
-    const int ew = warp - kEpiWarp0;
-    const int quad = warp & 3, half = ew >> 2;
-    const int row = quad * 32 + lane;
-    uint32_t acc_it = 0;
-    bool ok = true;
-    for (int64_t item = blockIdx.x; ok && item < n_items; item += gridDim.x, ++acc_it) {
-      const uint32_t slot = acc_it & 1, aph = (acc_it >> 1) & 1;
-      const int64_t m = (int64_t)(item / p.n_tiles) * kBM + row;
-      const int64_t n0 = (int64_t)(item % p.n_tiles) * kBN + half * 128;
-      if (!__all_sync(0xffffffffu, bar_wait(smem_addr(&ctrl->acc_full[slot]), aph, abort, p.limit_ns))) {
-        ok = false;
-        break;
-      }
-      tc_fence_after_sync();
-      int64_t dst = m;
-      if (p.row_map) dst = (m < p.M) ? p.row_map[m] : -1;
-      const bool store = m < p.M && dst >= 0 && ADWIN_CHK(n0 >= 0 && n0 < (int64_t)p.n_tiles * kBN, p.status);
-      const uint32_t t_lane =
-          tmem_base + ((uint32_t)(quad * 32) << 16) + slot * kBN + (uint32_t)(half * 128);
-#pragma unroll 1
-      for (int j = 0; j < 4; ++j) {
-        uint32_t r[32];
-        if (nk > 0) {
-          tmem_ld32(t_lane + j * 32, r);
-          tmem_ld_wait();
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) r[i] = 0u;
-        }
-        const int64_t n = n0 + j * 32;
-        if (store) {
-          if (p.c_is_bf16) {
-            __nv_bfloat16* cp = static_cast<__nv_bfloat16*>(p.C) + dst * p.ldc + n;
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-              if (n + v * 8 < p.N)
-                *reinterpret_cast<uint4*>(cp + v * 8) = make_uint4(
-                    pack_bf16x2(__uint_as_float(r[v * 8]), __uint_as_float(r[v * 8 + 1])),
-                    pack_bf16x2(__uint_as_float(r[v * 8 + 2]), __uint_as_float(r[v * 8 + 3])),
-                    pack_bf16x2(__uint_as_float(r[v * 8 + 4]), __uint_as_float(r[v * 8 + 5])),
-                    pack_bf16x2(__uint_as_float(r[v * 8 + 6]), __uint_as_float(r[v * 8 + 7])));
-          } else {
-            float* cp = static_cast<float*>(p.C) + dst * p.ldc + n;
-#pragma unroll
-            for (int v = 0; v < 8; ++v)
-              if (n + v * 4 < p.N)
-                *reinterpret_cast<uint4*>(cp + v * 4) =
-                    make_uint4(r[v * 4], r[v * 4 + 1], r[v * 4 + 2], r[v * 4 + 3]);
-          }
-        }
-      }
-      tc_fence_before_sync();
-      bar_arrive(smem_addr(&ctrl->acc_empty[slot]));
-    }
-  }
-  if (*abort && threadIdx.x == 0) atomicOr(p.status, ADWIN_DEV_TIMEOUT);
-  tc_fence_before_sync();
-  __syncthreads();
-  if (warp == 2) {
-    tc_fence_after_sync();
-    tmem_dealloc(tmem_base, kTmemCols);
-  }
-}
-
-// One sweep launch: single CTAs, or clusters of two for the pair form.
-template <bool GRAD, bool NEED_U, int BN, bool MOM, bool PAIR>
-cudaError_t launch_sweep(const CUtensorMap& m_hs, const CUtensorMap& m_ws, const CUtensorMap& m_ht,
-                         const CUtensorMap& m_wt, const SweepParams& sp, int sm_count,
-                         cudaStream_t s) {
-  auto kernel = lm_sweep_kernel<GRAD, NEED_U, BN, MOM, PAIR>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+  cudaError_t e = launch_rowmap(a.window, a.rollout_len, a.B, a.T, a.flags & ADWIN_RANGE_FULL,
+                                wb + L.off_rowmap, false, a.kl, a.logratio, a.gsq, a.lse_s, a.lse_t,
+                                a.status, s);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(PAIR ? (sm_count & ~1) : sm_count);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = PAIR ? 2 : 1;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, m_hs, m_ws, m_ht, m_wt, sp);
+  const WorkspaceLayout wl = workspace_layout(a.B);
+  GatherParams gp;
+  gp.hs = static_cast<const __nv_bfloat16*>(a.hs);
+  gp.ht = static_cast<const __nv_bfloat16*>(a.ht);
+  gp.ws = static_cast<const __nv_bfloat16*>(a.ws);
+  gp.wt = static_cast<const __nv_bfloat16*>(a.wt);
+  gp.tokens = a.tokens;
+  gp.range = reinterpret_cast<const int32_t*>(wb + L.off_rowmap + wl.off_range);
+  gp.ewin = reinterpret_cast<const int32_t*>(wb + L.off_rowmap + wl.off_ewin);
+  gp.seg = seg;
+  gp.B = a.B; gp.T = a.T; gp.V = V; gp.ds = ds; gp.dt = dt;
+  gp.max_tiles = L.max_tiles;
+  gp.hdr = hdr;
+  gp.rowsrc = rowsrc;
+  gp.rowdst = rowdst;
+  gp.tok = tok;
+  gp.hs_c = hs_c;
+  gp.ht_c = ht_c;
+  gp.status = a.status;
+  lm_plan_kernel<<<plan.n_seg, 1024, 0, s>>>(gp.range, gp.ewin, a.B, plan, seg);
+  const int64_t gather_blocks = rows_cap / 8;
+  lm_gather_kernel<<<(int)(gather_blocks < 8192 ? gather_blocks : 8192), 256, 0, s>>>(gp, plan);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+
+  CUtensorMap m_hs, m_ws, m_ht, m_wt;
+  if (!make_map(&m_hs, hs_c, ds, rows_cap, ds, kBM) || !make_map(&m_ws, a.ws, ds, V, ds, kBN / 2) ||
+      !make_map(&m_ht, ht_c, dt, rows_cap, dt, kBM) || !make_map(&m_wt, a.wt, dt, V, dt, kBN / 2))
+    return cudaErrorInvalidValue;
+
+  SweepParams sp;
+  sp.hdr = hdr;
+  sp.tok = tok;
+  sp.V = V;
+  sp.ks_blocks = (int)((ds + kBK - 1) / kBK);
+  sp.kt_blocks = (int)((dt + kBK - 1) / kBK);
+  sp.n_chunks = L.n_chunks;
+  sp.keep_u = a.mode == ADWIN_GRAD_FULL_KL ? 1 : 0;
+  sp.park = reinterpret_cast<float4*>(wb + L.off_park);
+  sp.part = part;
+  sp.part_slots = L.part_slots;
+  sp.limit_ns = handshake_wait_limit_ns();
+  sp.status = a.status;
+
+  MergeParams mp;
+  mp.hdr = hdr;
+  mp.rowsrc = rowsrc;
+  mp.rowdst = rowdst;
+  mp.tokens = a.tokens;
+  mp.part = part;
+  mp.tok = tok;
+  mp.info = info;
+  mp.alpha = a.alpha;
+  mp.mode = a.mode;
+  mp.kl = a.kl;
+  mp.logratio = a.logratio;
+  mp.gsq = a.gsq;
+  mp.lse_s = a.lse_s;
+  mp.lse_t = a.lse_t;
+  mp.status = a.status;
+
+  int launch = 0;
+  // statistics of the tiles [tile0, tile0 + cap) (rest: see SweepParams)
+  auto statistics = [&](int64_t tile0, int64_t cap, int rest, bool kept, bool moments) {
+    sp.tile0 = mp.tile0 = tile0;
+    sp.tile_cap = mp.tile_cap = cap;
+    sp.rest = mp.rest = rest;
+    sp.keep = kept ? keep : nullptr;
+    sp.pace = launch < 58 ? &hdr->pace[2 + launch] : nullptr;
+    ++launch;
+    const cudaError_t r =
+        moments ? launch_pairs(lm_sweep_kernel<true>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp)
+                : launch_pairs(lm_sweep_kernel<false>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp);
+    if (r != cudaSuccess) return r;
+    lm_merge_kernel<<<(unsigned)cap, kBM * kMergeWays, 0, s>>>(mp);
+    return cudaGetLastError();
+  };
+  if (!a.want_grad) return statistics(0, L.max_tiles, 2, false, a.gsq != nullptr);
+
+  GradParams gr;
+  gr.hdr = hdr;
+  gr.keep = keep;
+  gr.info = info;
+  gr.V = V;
+  gr.n_chunks = L.n_chunks;
+  gr.n_groups = L.grad_groups;
+  gr.G = G;
+  gr.ldG = L.ldG;
+  gr.q = q;
+  gr.max_tiles = L.max_tiles;
+  gr.status = a.status;
+  // the moments are only needed for rows whose gsq does not come from the gradient entries
+  const bool moments = a.gsq != nullptr && range_full;
+  for (int64_t t0 = 0; t0 < L.max_tiles; t0 += L.block_tiles) {
+    const int64_t cap = L.block_tiles < L.max_tiles - t0 ? L.block_tiles : L.max_tiles - t0;
+    if ((e = statistics(t0, cap, 0, true, moments)) != cudaSuccess) return e;
+    gr.tile0 = t0;
+    gr.tile_cap = cap;
+    const unsigned grid = (unsigned)(cap * L.grad_groups);
+    if (a.mode == ADWIN_GRAD_FULL_KL) lm_grad_kernel<true><<<grid, 256, 0, s>>>(gr);
+    else lm_grad_kernel<false><<<grid, 256, 0, s>>>(gr);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  if (range_full && (e = statistics(0, L.max_tiles, 1, false, moments)) != cudaSuccess) return e;
+  if (a.gsq) lm_gsq_kernel<<<(unsigned)L.max_tiles, kBM, 0, s>>>(hdr, q, rowdst, L.grad_groups, a.gsq);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+
+  if (a.dH) {
+    if (a.flags & ADWIN_ZERO_TAIL) {
+      e = cudaMemsetAsync(a.dH, 0, (size_t)a.B * a.T * ds * (a.dh_dtype == ADWIN_F32 ? 4 : 2), s);
+      if (e != cudaSuccess) return e;
+    }
+    // dH_s[rows, d_s] = G[rows, V] W_s[V, d_s]: A K-major; rows scattered to [B,T]
+    e = launch_tc_gemm(G, L.ldG, false, a.ws, ds, rows_cap, ds, V, a.dH, ds,
+                       a.dh_dtype == ADWIN_BF16, &hdr->grad_tiles, nullptr, rowdst, pieces,
+                       &hdr->pace[0], a.status, a.sm_count, s);
+    if (e != cudaSuccess) return e;
+  }
+  if (a.dW) {
+    // dW_s[V, d_s] = G^T[V, rows] H_s[rows, d_s]: A MN-major, the contraction runs over rows
+    e = launch_tc_gemm(G, L.ldG, true, hs_c, ds, V, ds, rows_cap, a.dW, ds, false, nullptr,
+                       &hdr->grad_tiles, nullptr, pieces, &hdr->pace[1], a.status, a.sm_count, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-template <typename K>
-cudaError_t opt_in_smem(K kernel) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+int current_sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 148;
+  return n;
 }
 
 }  // namespace
 
-// C[M,N] = A B on the tensor cores.  A is [M,K] (K contiguous, a_mn = false) or [K,M] (M
-// contiguous, a_mn = true); B is [N,K] or [K,N] likewise; bf16 in, fp32 accumulation.
-cudaError_t launch_tc_gemm(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
-                           bool b_mn, int64_t M, int64_t N, int64_t K, void* C, int64_t ldc,
-                           bool c_bf16, const int32_t* m_tiles_dev, const int32_t* k_tiles_dev,
-                           const int32_t* row_map, int32_t* status, int sm_count, cudaStream_t s,
-                           const int32_t* k_list, const int32_t* k_count_dev) {
-  CUtensorMap ma, mb;
-  const bool oka = a_mn ? make_map(&ma, A, M, K, lda, 64) : make_map(&ma, A, K, M, lda, kBM);
-  const bool okb = b_mn ? make_map(&mb, B, N, K, ldb, 64) : make_map(&mb, B, K, N, ldb, kBN);
-  if (!oka || !okb) return cudaErrorInvalidValue;
-  GemmParams p;
-  p.M = M;
-  p.N = N;
-  p.m_tiles = (int)((M + kBM - 1) / kBM);
-  p.n_tiles = (int)((N + kBN - 1) / kBN);
-  p.k_blocks = (int)((K + kBK - 1) / kBK);
-  p.m_tiles_dev = m_tiles_dev;
-  p.k_tiles_dev = k_tiles_dev;
-  p.k_list = k_list;
-  p.k_count_dev = k_count_dev;
-  p.row_map = row_map;
-  p.C = C;
-  p.ldc = ldc;
-  p.c_is_bf16 = c_bf16 ? 1 : 0;
-  p.status = status;
-  p.limit_ns = handshake_wait_limit_ns();
-  cudaError_t e;
-#define ADWIN_LAUNCH_GEMM(AM, BM_)                                                    \
-  do {                                                                                \
-    e = opt_in_smem(tc_gemm_kernel<AM, BM_>);                                         \
-    if (e != cudaSuccess) return e;                                                   \
-    tc_gemm_kernel<AM, BM_><<<sm_count, kThreads, kSmemBytes, s>>>(ma, mb, p);        \
-  } while (0)
-  if (!a_mn && !b_mn) ADWIN_LAUNCH_GEMM(false, false);
-  else if (!a_mn && b_mn) ADWIN_LAUNCH_GEMM(false, true);
-  else if (a_mn && !b_mn) ADWIN_LAUNCH_GEMM(true, false);
-  else ADWIN_LAUNCH_GEMM(true, true);
-#undef ADWIN_LAUNCH_GEMM
-  return cudaGetLastError();
-}
-
-// Column width of the sweeps' logit tiles.  256 is what the library runs: one accumulator pair
-// fills the tensor memory and the epilogue alternates with the MMAs.  The 128-column form (two
-// pairs, epilogue overlapped) is correct but measured 1.5x slower at the paper-scale shape -- its
-// MMAs are bound by operand traffic -- and is only instantiated in development builds.
-#ifdef ADWIN_DEV_EXPORTS
-#define ADWIN_SWEEP_128 1
-#else
-#define ADWIN_SWEEP_128 0
-#endif
-// CTA pairs (tcgen05 cta_group::2: a 256-row tile pair per MMA, each CTA staging half of the B
-// tile).  Correct (the whole test-suite passes with it) and it cuts the operand bytes a CTA pulls
-// through L2 by a third, but at the paper-scale shape it measured no faster than single CTAs
-// (44.4 ms against 42.2 ms for the statistics sweep): the partner CTAs' epilogues have to meet
-// before the next chunk's MMAs start.  Instantiated in development builds only.
-static int g_sweep_pair = 0;
-void set_sweep_pair(int on) { g_sweep_pair = (ADWIN_SWEEP_128 && on) ? 1 : 0; }
-static int g_sweep_bn = 256;
-void set_sweep_tile_columns(int bn) { g_sweep_bn = (ADWIN_SWEEP_128 && bn == 128) ? 128 : 256; }
-
 size_t lmhead_workspace_bytes(int64_t B, int64_t T, int64_t V, int64_t ds, int64_t dt,
-                              int64_t max_rows, bool want_grad, bool range_full) {
-  return lm_layout(B, T, V, ds, dt, max_rows, want_grad, range_full).total;
+                              int64_t max_rows, bool want_grad) {
+  return lm_layout(B, T, V, ds, dt, max_rows, want_grad, 2, 1, current_sm_count()).total;
 }
 
 // The whole fused pass; arguments validated by the caller.
@@ -953,168 +961,16 @@ cudaError_t launch_lmhead(const void* hs, const void* ws, const void* ht, const 
                           const int32_t* window, const int32_t* rollout_len, float alpha, int mode,
                           int flags, void* dH, int dh_dtype, float* dW, float* kl, float* logratio,
                           float* gsq, float* lse_s, float* lse_t, void* workspace,
-                          int64_t max_rows, int32_t* status, int sm_count, cudaStream_t s,
-                          bool keep_G) {
-  const bool want_grad = dH != nullptr || dW != nullptr || keep_G;
-  const bool range_full = (flags & ADWIN_RANGE_FULL) != 0;
-  const LmLayout L = lm_layout(B, T, V, ds, dt, max_rows, want_grad, range_full);
-  char* wb = static_cast<char*>(workspace);
-  int32_t* hdr = reinterpret_cast<int32_t*>(wb + L.off_hdr);
-  int32_t* tiles = reinterpret_cast<int32_t*>(wb + L.off_tiles);
-  int32_t* g2t = reinterpret_cast<int32_t*>(wb + L.off_g2t);
-  int32_t* rowdst = reinterpret_cast<int32_t*>(wb + L.off_rowdst);
-  float* info = reinterpret_cast<float*>(wb + L.off_info);
-  float* tok = reinterpret_cast<float*>(wb + L.off_tok);
-  float* part = reinterpret_cast<float*>(wb + L.off_part);
-  __nv_bfloat16* hs_c = reinterpret_cast<__nv_bfloat16*>(wb + L.off_hs);
-  __nv_bfloat16* ht_c = reinterpret_cast<__nv_bfloat16*>(wb + L.off_ht);
-  __nv_bfloat16* hs_g = range_full ? reinterpret_cast<__nv_bfloat16*>(wb + L.off_hg) : hs_c;
-  __nv_bfloat16* G = reinterpret_cast<__nv_bfloat16*>(wb + L.off_G);
-  const int64_t rows_cap = L.max_tiles * kBM;
-
-  cudaError_t e = launch_rowmap(window, rollout_len, B, T, flags & ADWIN_RANGE_FULL, wb + L.off_rowmap,
-                                false, kl, logratio, gsq, lse_s, lse_t, status, s);
-  if (e != cudaSuccess) return e;
-  const WorkspaceLayout wl = workspace_layout(B);
-  const int32_t* range = reinterpret_cast<const int32_t*>(wb + L.off_rowmap + wl.off_range);
-  const int32_t* ewin = reinterpret_cast<const int32_t*>(wb + L.off_rowmap + wl.off_ewin);
-  lm_plan_kernel<<<1, 1024, 0, s>>>(range, ewin, B, T, L.max_tiles, hdr, tiles, g2t, rowdst, status);
-  const int gather_blocks = (int)(rows_cap < 8192 ? rows_cap : 8192);
-  lm_gather_kernel<<<gather_blocks, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(hs), T, ds, hdr,
-                                                 tiles, g2t, false, hs_c);
-  lm_gather_kernel<<<gather_blocks, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(ht), T, dt, hdr,
-                                                 tiles, g2t, false, ht_c);
-  if (want_grad && range_full)
-    lm_gather_kernel<<<gather_blocks, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(hs), T, ds,
-                                                   hdr, tiles, g2t, true, hs_g);
-  lm_token_kernel<<<gather_blocks, 256, 0, s>>>(hs_c, static_cast<const __nv_bfloat16*>(ws), ht_c,
-                                                static_cast<const __nv_bfloat16*>(wt), T, V, ds, dt,
-                                                hdr, tiles, tokens, tok);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-
-  const int bn = g_sweep_bn;
-  CUtensorMap m_hs, m_ws, m_ht, m_wt;
-  if (!make_map(&m_hs, hs_c, ds, rows_cap, ds, kBM) || !make_map(&m_ws, ws, ds, V, ds, bn) ||
-      !make_map(&m_ht, ht_c, dt, rows_cap, dt, kBM) || !make_map(&m_wt, wt, dt, V, dt, bn))
-    return cudaErrorInvalidValue;
-
-  SweepParams sp;
-  sp.hdr = hdr;
-  sp.tiles = tiles;
-  sp.g2t = g2t;
-  sp.tok = tok;
-  sp.T = T;
-  sp.V = V;
-  sp.ks_blocks = (int)((ds + kBK - 1) / kBK);
-  sp.kt_blocks = (int)((dt + kBK - 1) / kBK);
-  sp.n_chunks = (int)((V + bn - 1) / bn);
-  sp.n_groups = L.n_groups;
-  sp.part = part;
-  sp.info = info;
-  sp.G = G;
-  sp.ldG = L.ldG;
-  sp.max_tiles = L.max_tiles;
-  sp.limit_ns = handshake_wait_limit_ns();
-  sp.status = status;
-  // 128-row boxes of the output embeddings for the pair form (each CTA stages half a B tile)
-  const bool pair = ADWIN_SWEEP_128 && g_sweep_pair && bn == 256 && sm_count >= 2;
-  CUtensorMap m_ws_h = m_ws, m_wt_h = m_wt;
-  if (pair && (!make_map(&m_ws_h, ws, ds, V, ds, kBN / 2) || !make_map(&m_wt_h, wt, dt, V, dt, kBN / 2)))
-    return cudaErrorInvalidValue;
-  // the single-sweep moments are only needed for rows whose gsq does not come from sweep 2
-  const bool moments = gsq != nullptr && (!want_grad || range_full);
-  if (bn != 256) {
-#if ADWIN_SWEEP_128
-    e = launch_sweep<false, true, 128, true, false>(m_hs, m_ws, m_ht, m_wt, sp, sm_count, s);
-#endif
-#if ADWIN_SWEEP_128
-  } else if (pair) {
-    e = moments ? launch_sweep<false, true, 256, true, true>(m_hs, m_ws_h, m_ht, m_wt_h, sp, sm_count, s)
-                : launch_sweep<false, true, 256, false, true>(m_hs, m_ws_h, m_ht, m_wt_h, sp, sm_count, s);
-#endif
-  } else {
-    e = moments ? launch_sweep<false, true, 256, true, false>(m_hs, m_ws, m_ht, m_wt, sp, sm_count, s)
-                : launch_sweep<false, true, 256, false, false>(m_hs, m_ws, m_ht, m_wt, sp, sm_count, s);
-  }
-  if (e != cudaSuccess) return e;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-
-  MergeParams mp;
-  mp.hdr = hdr;
-  mp.tiles = tiles;
-  mp.tokens = tokens;
-  mp.part = part;
-  mp.tok = tok;
-  mp.info = info;
-  mp.T = T;
-  mp.V = V;
-  mp.n_groups = L.n_groups;
-  mp.alpha = alpha;
-  mp.mode = mode;
-  mp.kl = kl;
-  mp.logratio = logratio;
-  mp.gsq = gsq;
-  mp.lse_s = lse_s;
-  mp.lse_t = lse_t;
-  mp.status = status;
-  lm_merge_kernel<<<(unsigned)L.max_tiles, kBM, 0, s>>>(mp);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (!want_grad) return cudaSuccess;
-
-  // sweep 2: the gradient tiles' logits again, written out as G (bf16, one row per compact row)
-  CUtensorMap m_hg = m_hs;
-  if (range_full && !make_map(&m_hg, hs_g, ds, rows_cap, ds, kBM)) return cudaErrorInvalidValue;
-  if (mode == ADWIN_GRAD_FULL_KL) {
-    // With ADWIN_RANGE_FULL the compact teacher copy is in tile order and sweep 1 is done with it:
-    // gather the gradient tiles' rows into the same buffer.
-    if (range_full)
-      lm_gather_kernel<<<gather_blocks, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(ht), T, dt,
-                                                     hdr, tiles, g2t, true, ht_c);
-    if (bn != 256) {
-#if ADWIN_SWEEP_128
-      e = launch_sweep<true, true, 128, true, false>(m_hg, m_ws, m_ht, m_wt, sp, sm_count, s);
-#endif
-#if ADWIN_SWEEP_128
-    } else if (pair) {
-      e = launch_sweep<true, true, 256, true, true>(m_hg, m_ws_h, m_ht, m_wt_h, sp, sm_count, s);
-#endif
-    } else {
-      e = launch_sweep<true, true, 256, true, false>(m_hg, m_ws, m_ht, m_wt, sp, sm_count, s);
-    }
-  } else {
-    if (bn != 256) {
-#if ADWIN_SWEEP_128
-      e = launch_sweep<true, false, 128, true, false>(m_hg, m_ws, m_ht, m_wt, sp, sm_count, s);
-#endif
-#if ADWIN_SWEEP_128
-    } else if (pair) {
-      e = launch_sweep<true, false, 256, true, true>(m_hg, m_ws_h, m_ht, m_wt_h, sp, sm_count, s);
-#endif
-    } else {
-      e = launch_sweep<true, false, 256, true, false>(m_hg, m_ws, m_ht, m_wt, sp, sm_count, s);
-    }
-  }
-  if (e != cudaSuccess) return e;
-  if (gsq) lm_gsq_kernel<<<(unsigned)L.max_tiles, kBM, 0, s>>>(hdr, part, rowdst, L.n_groups, gsq);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-
-  if (dH) {
-    if (flags & ADWIN_ZERO_TAIL) {
-      e = cudaMemsetAsync(dH, 0, (size_t)B * T * ds * (dh_dtype == ADWIN_F32 ? 4 : 2), s);
-      if (e != cudaSuccess) return e;
-    }
-    // dH_s[rows, d_s] = G[rows, V] W_s[V, d_s]: A K-major, B MN-major; rows scattered to [B,T]
-    e = launch_tc_gemm(G, L.ldG, false, ws, ds, true, rows_cap, ds, V, dH, ds,
-                       dh_dtype == ADWIN_BF16, hdr + 1, nullptr, rowdst, status, sm_count, s);
-    if (e != cudaSuccess) return e;
-  }
-  if (dW) {
-    // dW_s[V, d_s] = G^T[V, rows] H_s[rows, d_s]: both MN-major, the contraction runs over rows
-    e = launch_tc_gemm(G, L.ldG, true, hs_g, ds, true, V, ds, rows_cap, dW, ds, false, nullptr,
-                       hdr + 1, nullptr, status, sm_count, s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+                          int64_t max_rows, int32_t* status, int sm_count, cudaStream_t s) {
+  const bool want_grad = dH != nullptr || dW != nullptr;
+  const LmCall a = {hs, ws, ht, wt, B, T, V, ds, dt, tokens, window, rollout_len, alpha, mode, flags,
+                    dH, dh_dtype, dW, want_grad, kl, logratio, gsq, lse_s, lse_t,
+                    static_cast<char*>(workspace), status, sm_count};
+  SegPlan plan = {};
+  plan.n_seg = 2;
+  plan.pad = 1;
+  plan.want_grad = want_grad ? 1 : 0;
+  return run_lmhead(a, lm_layout(B, T, V, ds, dt, max_rows, want_grad, 2, 1, sm_count), plan, s);
 }
 
 // ---------------------------------------------------------------------------- weight-space audit
@@ -1123,32 +979,12 @@ cudaError_t launch_lmhead(const void* hs, const void* ws, const void* ht, const 
 // positions; dW_bin[i] = G[bin i]^T H_s[bin i] is one GEMM per bin over that bin's 64-row k-blocks,
 // the prefix gradient of candidate j is the sum of bins 0..j and the full-horizon reference the sum
 // of all bins, so the K cosines come from one pass over the K+1 bin matrices.
-constexpr int kMaxCand = 16;
 struct CandList {
   int32_t K;
   int32_t L[kMaxCand];
 };
 
 namespace {
-
-// k-block lists per bin: entry = first compact gradient row of a 64-row block.
-__global__ void lm_bins_kernel(const int32_t* hdr, const int32_t* __restrict__ tiles,
-                               const int32_t* __restrict__ g2t, CandList cand, int64_t list_stride,
-                               int32_t* lists, int32_t* counts) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int i = 0; i <= cand.K; ++i) counts[i] = 0;
-  const int n_gt = hdr[1];
-  for (int g = 0; g < n_gt; ++g) {
-    const int32_t* e = tiles + (int64_t)g2t[g] * kTileFields;
-    for (int h = 0; h < 2; ++h) {
-      if (64 * h >= e[3]) continue;          // no gradient row in this half
-      const int t = e[1] + 64 * h;
-      int bin = 0;
-      while (bin < cand.K && cand.L[bin] <= t) ++bin;
-      lists[bin * list_stride + counts[bin]++] = g * kBM + 64 * h;
-    }
-  }
-}
 
 // Per block: sums over its share of the elements of  pre_j * full,  pre_j^2  (j < K)  and full^2,
 // where pre_j = sum of bins 0..j and full = sum of all bins.  Fixed order inside the block.
@@ -1242,19 +1078,15 @@ __global__ void lm_align_finish_kernel(const double* __restrict__ partial, int n
 }
 
 struct AlignLayout {
-  size_t off_lists, off_counts, off_bins, off_partial, total;
-  int64_t list_stride;
+  size_t off_bins, off_partial, total;
   int gram_blocks;
 };
 
 AlignLayout align_layout(const LmLayout& L, int64_t V, int64_t ds, int K) {
   auto up = [](size_t x) { return (x + 1023) & ~size_t(1023); };
   AlignLayout A;
-  A.list_stride = 2 * L.max_tiles;
   A.gram_blocks = 1184;
   size_t o = L.total;
-  A.off_lists = o;    o = up(o + (size_t)(K + 1) * A.list_stride * 4);
-  A.off_counts = o;   o = up(o + (size_t)(K + 1) * 4);
   A.off_bins = o;     o = up(o + (size_t)(K + 1) * (size_t)V * ds * 4);
   A.off_partial = o;  o = up(o + (size_t)A.gram_blocks * (2 * kMaxCand + 1) * 8);
   A.total = o;
@@ -1265,7 +1097,8 @@ AlignLayout align_layout(const LmLayout& L, int64_t V, int64_t ds, int K) {
 
 size_t lmhead_align_workspace_bytes(int64_t B, int64_t T, int64_t V, int64_t ds, int64_t dt,
                                     int64_t max_rows, int K) {
-  return align_layout(lm_layout(B, T, V, ds, dt, max_rows, true, false), V, ds, K).total;
+  return align_layout(lm_layout(B, T, V, ds, dt, max_rows, true, K + 1, 64, current_sm_count()), V,
+                      ds, K).total;
 }
 
 cudaError_t launch_lmhead_weight_align(const void* hs, const void* ws, const void* ht,
@@ -1276,36 +1109,32 @@ cudaError_t launch_lmhead_weight_align(const void* hs, const void* ws, const voi
                                        float* gsq, double* batch_stats, int32_t* L_next,
                                        int32_t* flags_out, void* workspace, int64_t max_rows,
                                        int32_t* status, int sm_count, cudaStream_t s) {
-  const LmLayout L = lm_layout(B, T, V, ds, dt, max_rows, true, false);
+  const LmLayout L = lm_layout(B, T, V, ds, dt, max_rows, true, K + 1, 64, sm_count);
   const AlignLayout A = align_layout(L, V, ds, K);
   char* wb = static_cast<char*>(workspace);
   // every position of every rollout carries gradient here: the window is the rollout itself
   // (window == NULL stands for W_b = T in the row map, so E_b = R_b)
-  cudaError_t e = launch_lmhead(hs, ws, ht, wt, B, T, V, ds, dt, tokens, nullptr, rollout_len, 1.0f,
-                                mode, 0, nullptr, ADWIN_F32, nullptr, kl, logratio, gsq, nullptr,
-                                nullptr, workspace, max_rows, status, sm_count, s, true);
-  if (e != cudaSuccess) return e;
-  const int32_t* hdr = reinterpret_cast<const int32_t*>(wb + L.off_hdr);
-  const int32_t* tiles = reinterpret_cast<const int32_t*>(wb + L.off_tiles);
-  const int32_t* g2t = reinterpret_cast<const int32_t*>(wb + L.off_g2t);
-  const __nv_bfloat16* hs_c = reinterpret_cast<const __nv_bfloat16*>(wb + L.off_hs);
-  const __nv_bfloat16* G = reinterpret_cast<const __nv_bfloat16*>(wb + L.off_G);
-  int32_t* lists = reinterpret_cast<int32_t*>(wb + A.off_lists);
-  int32_t* counts = reinterpret_cast<int32_t*>(wb + A.off_counts);
-  float* bins = reinterpret_cast<float*>(wb + A.off_bins);
-  double* partial = reinterpret_cast<double*>(wb + A.off_partial);
+  const LmCall a = {hs, ws, ht, wt, B, T, V, ds, dt, tokens, nullptr, rollout_len, 1.0f, mode, 0,
+                    nullptr, ADWIN_F32, nullptr, true, kl, logratio, gsq, nullptr, nullptr, wb, status,
+                    sm_count};
   CandList cand;
   cand.K = K;
-  for (int i = 0; i < kMaxCand; ++i) cand.L[i] = i < K ? cand_host[i] : 0;
-  lm_bins_kernel<<<1, 32, 0, s>>>(hdr, tiles, g2t, cand, A.list_stride, lists, counts);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const int64_t rows_cap = L.max_tiles * kBM;
-  for (int i = 0; i <= K; ++i) {
-    e = launch_tc_gemm(G, L.ldG, true, hs_c, ds, true, V, ds, rows_cap,
-                       bins + (size_t)i * V * ds, ds, false, nullptr, nullptr, nullptr, status,
-                       sm_count, s, lists + (size_t)i * A.list_stride, counts + i);
-    if (e != cudaSuccess) return e;
-  }
+  SegPlan plan = {};
+  plan.n_seg = K + 1;
+  plan.pad = 64;          // a 64-row k-block never straddles two bins
+  plan.want_grad = 1;
+  plan.by_cut = 1;
+  for (int i = 0; i < kMaxCand; ++i) plan.cut[i] = cand.L[i] = i < K ? cand_host[i] : 0;
+  cudaError_t e = run_lmhead(a, L, plan, s);
+  if (e != cudaSuccess) return e;
+  const LmHeader* hdr = reinterpret_cast<const LmHeader*>(wb + L.off_hdr);
+  const __nv_bfloat16* hs_c = reinterpret_cast<const __nv_bfloat16*>(wb + L.off_hs);
+  const __nv_bfloat16* G = reinterpret_cast<const __nv_bfloat16*>(wb + L.off_G);
+  float* bins = reinterpret_cast<float*>(wb + A.off_bins);
+  double* partial = reinterpret_cast<double*>(wb + A.off_partial);
+  e = launch_tc_gemm_bins(G, L.ldG, hs_c, ds, V, ds, L.max_tiles * kBM, bins, ds, V * ds, K + 1,
+                          hdr->seg_kblock, status, sm_count, s);
+  if (e != cudaSuccess) return e;
   lm_gram_kernel<<<A.gram_blocks, kGramThreads, 0, s>>>(bins, V * ds, K, partial);
   lm_align_finish_kernel<<<1, 32, 0, s>>>(partial, A.gram_blocks, cand, rho_star, rollout_len, B, T,
                                           batch_stats, L_next, flags_out);

@@ -2,9 +2,9 @@
 // memory, tcgen05.mma with the accumulator in tensor memory, tcgen05.ld for the epilogue, and
 // mbarrier waits that give up after a time limit instead of spinning for ever.
 //
-// Tile shapes are fixed: an MMA tile is 128 rows (M) x 256 columns (N), one k-block is 64 bf16
-// (128 bytes, the span of the 128-byte swizzle), one tcgen05.mma covers K = 16.  A shared-memory
-// stage holds the A tile (16 KB) and the B tile (32 KB) of one k-block.
+// Tile shapes are fixed: an MMA tile is 256 rows (M, 128 per CTA of a pair) x 256 columns (N), one
+// k-block is 64 bf16 (128 bytes, the span of the 128-byte swizzle), one tcgen05.mma covers K = 16.
+// A CTA's shared-memory stage holds its 128 rows of A (16 KB) and its half of B (16 KB).
 //
 // Operand layouts in shared memory (what the TMA boxes below produce and the matrix descriptors
 // describe):
@@ -23,15 +23,13 @@
 namespace adwin {
 namespace tc {
 
-constexpr int kBM = 128;            // rows of an MMA tile (TMEM lanes)
+constexpr int kBM = 128;            // rows of a CTA's share of an MMA tile (TMEM lanes)
 constexpr int kBN = 256;            // columns of an MMA tile (TMEM columns of one accumulator)
 constexpr int kBK = 64;             // bf16 per k-block (one 128-byte swizzle span)
 constexpr int kUmmaK = 16;          // K of one tcgen05.mma (bf16)
-constexpr int kStages = 4;
-constexpr int kMaxStages = 6;        // barrier arrays are sized for the deepest pipeline in use
 constexpr int kABytes = kBM * kBK * 2;            // 16384
-constexpr int kBBytes = kBN * kBK * 2;            // 32768
-constexpr int kStageBytes = kABytes + kBBytes;    // 49152
+constexpr int kPairStageBytes = 2 * kABytes;      // 128 rows of A and 128 of the 256 columns of B
+constexpr int kPairStages = 6;
 constexpr int kBoxBytesMN = 64 * kBK * 2;         // 8192: one {64 mn, 64 k} box
 constexpr int kTmemCols = 512;
 constexpr int kThreads = 384;       // warp 0: TMA producer, warp 1: MMA issuer, warp 2: TMEM
@@ -43,8 +41,8 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
 // Control block at the start of dynamic shared memory; the stages follow at the next 1024-byte
 // boundary.
 struct Ctrl {
-  unsigned long long full[kMaxStages];   // TMA -> MMA: the stage's tiles have landed
-  unsigned long long empty[kMaxStages];  // MMA -> TMA: the stage's tiles have been consumed
+  unsigned long long full[kPairStages];   // TMA -> MMA: the stage's tiles have landed
+  unsigned long long empty[kPairStages];  // MMA -> TMA: the stage's tiles have been consumed
   unsigned long long acc_full[2];      // MMA -> epilogue: accumulator slot complete
   unsigned long long acc_empty[2];     // epilogue -> MMA: accumulator slot read out
   unsigned long long drain;            // give-up path: all issued MMAs have retired
@@ -52,7 +50,7 @@ struct Ctrl {
   int abort;
 };
 constexpr int kCtrlBytes = 1024;
-constexpr int kSmemBytes = kCtrlBytes + 1024 + kStages * kStageBytes;   // + alignment slack
+constexpr int kSmemBytes = kCtrlBytes + 1024 + kPairStages * kPairStageBytes;   // + alignment slack
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -138,34 +136,7 @@ __device__ __forceinline__ bool bar_wait_drain(uint32_t bar, uint32_t parity) {
   }
 }
 
-// ---------------------------------------------------------------------------- TMA
-// 2-D tiled load: c0 is the coordinate along the contiguous dimension (elements), c1 the row.
-// c0 times the element size must be a multiple of 16 bytes (here always a multiple of 64 bf16).
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int32_t c0,
-                                            int32_t c1, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-      "l"(map), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
-}
-__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
-}
-
 // ---------------------------------------------------------------------------- tensor memory
-__device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
-               "r"(ncols)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
-               : "memory");
-}
 __device__ __forceinline__ void tc_fence_before_sync() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -207,64 +178,22 @@ __device__ __forceinline__ uint64_t desc_mn_major(uint32_t saddr) {
 constexpr uint32_t kStepKMajor = (kUmmaK * 2) >> 4;        // 32 bytes along the swizzled row
 constexpr uint32_t kStepMNMajor = (kUmmaK * 128) >> 4;     // 16 k-rows of 128 bytes
 
-// Instruction descriptor of tcgen05.mma.kind::f16 for bf16 x bf16 -> fp32, M = 128, N = 256:
+// Instruction descriptor of tcgen05.mma.kind::f16 for bf16 x bf16 -> fp32, M = 256, N = 256:
 // accumulator format fp32 (bits 4..5 = 1), A and B format bf16 (bits 7..9, 10..12 = 1), operand
 // majors in bits 15 / 16 (0 = K-major, 1 = MN-major), N >> 3 in bits 17..22, M >> 4 in bits 24..28.
-__host__ __device__ constexpr uint32_t instr_desc(bool a_mn, bool b_mn, int n = kBN) {
+__host__ __device__ constexpr uint32_t instr_desc(bool a_mn, bool b_mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) |
-         ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-}
-__device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
-                                     uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// Arrive on an mbarrier once every tcgen05.mma issued so far by this thread has retired.
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   bar)
-               : "memory");
-}
-
-// The four MMAs of one k-block.  `first` clears the accumulator on the very first MMA of a tile.
-template <bool A_MN, bool B_MN, int N = kBN>
-__device__ __forceinline__ void issue_kblock(uint32_t tmem_d, uint32_t a_saddr, uint32_t b_saddr,
-                                             bool first) {
-  constexpr uint32_t idesc = instr_desc(A_MN, B_MN, N);
-  const uint64_t ad = A_MN ? desc_mn_major(a_saddr) : desc_k_major(a_saddr);
-  const uint64_t bd = B_MN ? desc_mn_major(b_saddr) : desc_k_major(b_saddr);
-#pragma unroll
-  for (int k = 0; k < kBK / kUmmaK; ++k) {
-    umma(tmem_d, ad + (uint64_t)(k * (A_MN ? kStepMNMajor : kStepKMajor)),
-         bd + (uint64_t)(k * (B_MN ? kStepMNMajor : kStepKMajor)), idesc,
-         (first && k == 0) ? 0u : 1u);
-  }
-}
-
-// One stage's TMA loads.  Coordinates: (k0, row0) for a K-major operand; (mn0, k0) for an MN-major
-// one, where the tile is fetched as 64-wide boxes.
-template <bool MN, int ROWS>
-__device__ __forceinline__ void load_operand(uint32_t dst, const CUtensorMap* map, int32_t mn0,
-                                             int32_t k0, uint32_t bar) {
-  if (!MN) {
-    tma_load_2d(dst, map, k0, mn0, bar);
-  } else {
-#pragma unroll
-    for (int i = 0; i < ROWS / 64; ++i) tma_load_2d(dst + i * kBoxBytesMN, map, mn0 + 64 * i, k0, bar);
-  }
+         ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(2 * kBM >> 4) << 24);
 }
 
 // ---------------------------------------------------------------------------- CTA pairs
-// Forms used when two CTAs of a cluster work as one MMA unit (cta_group::2): an MMA tile is then
-// 256 rows (128 per CTA, each CTA's rows accumulate in its own tensor memory) x 256 columns, and
-// each CTA stages only half of the B tile, so the operand bytes per flop that a CTA pulls through
-// L2 drop by a third.  The even CTA of the pair (cluster rank 0) issues the MMAs; TMA loads of both
-// CTAs report their bytes to its `full` barrier; tcgen05.commit signals barriers at the same
-// shared-memory offset in both CTAs.  No load is multicast: each CTA fetches its own tiles.
+// Two CTAs of a cluster work as one MMA unit (cta_group::2): an MMA tile is 256 rows (128 per CTA,
+// each CTA's rows accumulate in its own tensor memory) x 256 columns, and each CTA stages only half
+// of the B tile, so the operand bytes per flop that a CTA pulls through L2 are a third lower than
+// for 128 x 256 tiles of single CTAs.  The even CTA of the pair (cluster rank 0) issues the MMAs;
+// TMA loads of both CTAs report their bytes to its `full` barrier; tcgen05.commit signals barriers
+// at the same shared-memory offset in both CTAs.  No load is multicast: each CTA fetches its own
+// tiles.
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -298,7 +227,8 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
                : "memory");
 }
-// TMA load of a CTA of a pair; `bar_cluster` is the shared::cluster address of the barrier that
+// 2-D tiled TMA load of a CTA of a pair: c0 is the coordinate along the contiguous dimension
+// (elements; always a multiple of 64 bf16 here, 16 bytes are required), c1 the row; `bar_cluster` is the shared::cluster address of the barrier that
 // receives the bytes (the even CTA's).
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int32_t c0,
                                                  int32_t c1, uint32_t bar_cluster) {
@@ -327,17 +257,119 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
       "h"(mask)
       : "memory");
 }
-// The four MMAs of one k-block of a pair tile (K-major operands, M = 256).
-template <int N>
+// The four MMAs of one k-block of a pair tile.  `first` clears the accumulator on the first MMA.
+template <bool A_MN, bool B_MN>
 __device__ __forceinline__ void issue_kblock_pair(uint32_t tmem_d, uint32_t a_saddr,
                                                   uint32_t b_saddr, bool first) {
-  constexpr uint32_t idesc = (instr_desc(false, false, N) & ~(0x1fu << 24)) | ((256u >> 4) << 24);
-  const uint64_t ad = desc_k_major(a_saddr), bd = desc_k_major(b_saddr);
+  constexpr uint32_t idesc = instr_desc(A_MN, B_MN);
+  const uint64_t ad = A_MN ? desc_mn_major(a_saddr) : desc_k_major(a_saddr);
+  const uint64_t bd = B_MN ? desc_mn_major(b_saddr) : desc_k_major(b_saddr);
 #pragma unroll
   for (int k = 0; k < kBK / kUmmaK; ++k)
-    umma_pair(tmem_d, ad + (uint64_t)(k * kStepKMajor), bd + (uint64_t)(k * kStepKMajor), idesc,
+    umma_pair(tmem_d, ad + (uint64_t)(k * (A_MN ? kStepMNMajor : kStepKMajor)),
+              bd + (uint64_t)(k * (B_MN ? kStepMNMajor : kStepKMajor)), idesc,
               (first && k == 0) ? 0u : 1u);
 }
 
+// One CTA's 128 rows (A) or columns (B) of a k-block.  Coordinates: (k0, row0) for a K-major operand;
+// (mn0, k0) for an MN-major one, which is fetched as two 64-wide boxes.
+template <bool MN>
+__device__ __forceinline__ void load_operand_pair(uint32_t dst, const CUtensorMap* map, int32_t mn0,
+                                                  int32_t k0, uint32_t bar_cluster) {
+  if (!MN) {
+    tma_load_2d_pair(dst, map, k0, mn0, bar_cluster);
+  } else {
+    tma_load_2d_pair(dst, map, mn0, k0, bar_cluster);
+    tma_load_2d_pair(dst + kBoxBytesMN, map, mn0 + 64, k0, bar_cluster);
+  }
+}
+
+// Keeps the pairs of a launch in step.  Pairs that work on neighbouring tiles read the same operand
+// slabs at about the same time, so all but the first read should hit L2; but a pipeline that is
+// never short of operands has nothing that pulls a pair back once it is ahead, and after a few
+// tiles the pairs had drifted further apart than L2 holds: 72 GB read from DRAM instead of 20 for
+// G W_s at 34 816 rows, V = 151 936, d_s = 2048 (28 GB with this; 1105 -> 1202 TFLOP/s sustained,
+// because DRAM traffic costs clock under the power limit).  Every kPaceStep k-blocks a pair adds to
+// a common counter and, if it is more than kPaceSlack steps ahead of the average, waits a little.
+// The wait is a courtesy: it ends by itself after kPaceTries looks, nothing depends on it.
+constexpr uint32_t kPaceStep = 16;     // k-blocks per step
+constexpr int kPaceSlack = 2;          // steps ahead of the average
+constexpr int kPaceTries = 64;
+struct Pace {
+  unsigned int* total;   // null: no pacing
+  int pairs;
+  unsigned int mine;
+  __device__ __forceinline__ Pace(unsigned int* t, int n) : total(t), pairs(n), mine(0) {}
+  __device__ __forceinline__ bool ahead() const {
+    const unsigned int sum = *reinterpret_cast<volatile unsigned int*>(total);
+    return (int)(mine * (unsigned int)pairs - sum) > kPaceSlack * pairs;
+  }
+  __device__ __forceinline__ void kblock(uint32_t it) {
+    if (!total || it % kPaceStep != 0) return;
+    ++mine;
+    atomicAdd(total, 1u);
+    for (int i = 0; i < kPaceTries && ahead(); ++i) __nanosleep(250);
+  }
+  // a pair without further work no longer holds the average back
+  __device__ __forceinline__ void done() {
+    if (total) atomicAdd(total, 1u << 24);
+  }
+};
+
+// Barriers of a pair pipeline; one thread of each CTA.  acc_empty counts one arrival per epilogue
+// warp of both CTAs and is only used in the even CTA.
+__device__ __forceinline__ void pair_bars_init(Ctrl* ctrl) {
+  for (int s = 0; s < kPairStages; ++s) {
+    bar_init(smem_addr(&ctrl->full[s]), 1);
+    bar_init(smem_addr(&ctrl->empty[s]), 1);
+  }
+  for (int s = 0; s < 2; ++s) {
+    bar_init(smem_addr(&ctrl->acc_full[s]), 1);
+    bar_init(smem_addr(&ctrl->acc_empty[s]), 2 * (kEpiThreads / 32));
+  }
+  bar_init(smem_addr(&ctrl->drain), 1);
+  ctrl->abort = 0;
+  bar_init_fence();
+}
+// One epilogue warp hands an accumulator slot back to the MMA issuer (one lane calls).
+__device__ __forceinline__ void pair_release(unsigned long long* acc_empty, uint32_t rank) {
+  if (rank != 0) bar_arrive_cluster(map_to_cta(smem_addr(acc_empty), 0));
+  else bar_arrive(smem_addr(acc_empty));
+}
+// Give-up path of the even CTA's producer after `it` k-blocks: let the copies in flight land (its
+// barriers count both CTAs' bytes; the final cluster barrier holds the odd CTA meanwhile).
+__device__ __forceinline__ void pair_drain_loads(Ctrl* ctrl, uint32_t it) {
+  const uint32_t n_out = it < (uint32_t)kPairStages ? it : (uint32_t)kPairStages;
+  for (uint32_t j = it - n_out; j < it; ++j)
+    bar_wait_drain(smem_addr(&ctrl->full[j % kPairStages]), (j / kPairStages) & 1);
+}
+
 }  // namespace tc
+
+// bf16 matrix [rows, cols], row pitch in elements; boxes of 64 columns x box_rows rows with the
+// 128-byte swizzle; out-of-range elements read as zero.
+bool make_map(CUtensorMap* m, const void* base, int64_t cols, int64_t rows, int64_t pitch,
+              int box_rows);
+
+// Launches a pair kernel: clusters of two CTAs on all SMs.
+template <typename K, typename... Args>
+cudaError_t launch_pairs(K kernel, int sm_count, cudaStream_t s, const Args&... args) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       tc::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(sm_count & ~1);
+  cfg.blockDim = dim3(tc::kThreads);
+  cfg.dynamicSmemBytes = tc::kSmemBytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 }  // namespace adwin

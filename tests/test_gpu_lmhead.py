@@ -375,3 +375,17 @@ def test_weight_space_alignment_rejects_bad_candidate_lists():
                                           batch.hidden_teacher, batch.w_teacher, batch.tokens,
                                           batch.rollout_len, bad)
         assert e.value.code == 2
+
+
+@pytest.mark.parametrize("windows", [[127], [128, 1], [60, 69, 0, 128], [100, 156], [1] * 9, [257, 3]])
+def test_rows_packed_across_sequences_at_tile_edges(windows):
+    """Compact rows fill the 128-row tiles across sequences (and tiles pair up): row counts on both
+    sides of one and two tiles, rows without gradient behind those with, a split contraction (2048
+    entries over 8 or more pieces) for dH."""
+    B, T = len(windows), max(windows) + 5
+    batch = synth.make_lmhead_batch(DEV, B=B, T=T, V=2048, d_s=128, d_t=72, w_std=0.12)
+    batch.window = torch.tensor(windows, dtype=torch.int32, device=DEV)
+    rows = int(sum(windows))
+    for flags, bound in ((0, rows), (api.RANGE_FULL, 0)):
+        got = run(batch, flags=flags, max_rows=bound)
+        check_all(batch, got, oracle(batch, api.GRAD_FULL_KL, flags), flags)
