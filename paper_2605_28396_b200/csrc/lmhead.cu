@@ -20,7 +20,7 @@
 // pair against 2 (d_s + d_t) operations.  A long run is bound by the board's 1 kW, so what counts is
 // energy: at 34 816 rows, V = 151 936, d = 2048 + 2560 a call takes 87 ms (sweep 38, gradient 10,
 // dH 15, dW 17) where computing the products twice on single-CTA tiles took 123 ms (40 + 43 + 17 +
-// 19).  At 225 rows, V = 32 000, d = 1024 + 1536: 254 us against 893 us (groups chosen by size, rows
+// 19).  At 225 rows, V = 32 000, d = 1024 + 1536: 212 us against 893 us (groups chosen by size, rows
 // packed across sequences, dH's contraction split).
 #include <cuda_bf16.h>
 
@@ -46,7 +46,6 @@ constexpr float kMasked = -1.0e6f;
 constexpr size_t kKeepBytes = size_t(6) << 30;
 constexpr int kKeepArray = kBM * kBN / 4;            // float4 of one policy's 128 x 256 tile
 constexpr size_t kKeepTileChunk = (size_t)2 * kKeepArray * 16;
-constexpr int kGradGroups = 32;                      // column groups of the gradient kernel, at most
 constexpr int kMaxCand = 16;
 constexpr int kMaxSeg = kMaxCand + 1;
 
@@ -70,13 +69,16 @@ LmLayout lm_layout(int64_t B, int64_t T, int64_t V, int64_t ds, int64_t dt, int6
   L.max_tiles = (bound + kBM - 1) / kBM;
   if (L.max_tiles < 1) L.max_tiles = 1;
   L.n_chunks = (int)((V + kBN - 1) / kBN);
-  L.grad_groups = L.n_chunks < kGradGroups ? L.n_chunks : kGradGroups;
   L.ldG = (V + 7) / 8 * 8;
   // equal blocks of an even number of tiles
   int64_t most = (int64_t)(kKeepBytes / ((size_t)L.n_chunks * kKeepTileChunk)) & ~int64_t(1);
   if (most < 2) most = 2;
   const int64_t blocks = (L.max_tiles + most - 1) / most;
   L.block_tiles = ((L.max_tiles + blocks - 1) / blocks + 1) & ~int64_t(1);
+  // column groups of the gradient kernel: four blocks per SM and more, 32 groups at least
+  int64_t gg = (4 * (int64_t)sm_count + L.block_tiles - 1) / L.block_tiles;
+  if (gg < 32) gg = 32;
+  L.grad_groups = (int)(gg < L.n_chunks ? gg : L.n_chunks);
   // see lm_sweep_kernel: at most 8 groups per tile, or 8 items per pair of CTAs
   L.part_slots = 8 * (L.max_tiles + 2) + 8 * (int64_t)sm_count;
   const size_t rows = (size_t)L.max_tiles * kBM;
@@ -187,15 +189,17 @@ struct GatherParams {
   int32_t* status;
 };
 
-// Copies one hidden-state row (d % 8 == 0) and forms its fp32 dot product with an embedding row.
+constexpr int kGatherThreads = 128;
+
+// Copies one hidden-state row (d % 8 == 0) and forms this thread's share of its fp32 dot product
+// with an embedding row.
 __device__ __forceinline__ float copy_dot(const __nv_bfloat16* src, const __nv_bfloat16* w,
-                                          __nv_bfloat16* dst, int64_t d, int lane) {
+                                          __nv_bfloat16* dst, int64_t d) {
   float acc = 0.f;
-#pragma unroll 4
-  for (int64_t v = lane; v < d / 8; v += 32) {
+#pragma unroll 2
+  for (int64_t v = threadIdx.x; v < d / 8; v += kGatherThreads) {
     uint4 x = make_uint4(0u, 0u, 0u, 0u);
     if (src) x = __ldg(reinterpret_cast<const uint4*>(src) + v);
-    reinterpret_cast<uint4*>(dst)[v] = x;
     if (w) {
       const uint4 y = __ldg(reinterpret_cast<const uint4*>(w) + v);
       float xf[8], yf[8];
@@ -204,18 +208,20 @@ __device__ __forceinline__ float copy_dot(const __nv_bfloat16* src, const __nv_b
 #pragma unroll
       for (int i = 0; i < 8; ++i) acc = fmaf(xf[i], yf[i], acc);
     }
+    reinterpret_cast<uint4*>(dst)[v] = x;
   }
-  return warp_sum(acc);
+  return acc;
 }
 
-// One warp per compact row: which position it is, copies of its two hidden-state rows (zeros past
+// One block per compact row: which position it is, copies of its two hidden-state rows (zeros past
 // the rows), and the two logits at its sampled token, z_y = h_s . W_s[y] and u_y = h_t . W_t[y].
 // They give the sampled-token log-ratio of Section 2.3 without a search through the logit tiles, and
 // their difference is the value the sweep centres z - u on: on a peaked row the sampled token is
 // almost surely the peak, where the centred difference is then exactly zero, which keeps the
 // single-sweep squared-norm moments well conditioned.
-__global__ void __launch_bounds__(256) lm_gather_kernel(const GatherParams p, const SegPlan plan) {
+__global__ void __launch_bounds__(kGatherThreads) lm_gather_kernel(const GatherParams p, const SegPlan plan) {
   __shared__ int64_t base[kMaxSeg + 1];
+  __shared__ float red[2][kGatherThreads / 32];
   if (threadIdx.x == 0) {
     int64_t o = 0;
     for (int i = 0; i < plan.n_seg; ++i) {
@@ -240,9 +246,7 @@ __global__ void __launch_bounds__(256) lm_gather_kernel(const GatherParams p, co
     if (threadIdx.x <= plan.n_seg)
       p.hdr->seg_kblock[threadIdx.x] = fits ? (int32_t)(base[threadIdx.x] / 64) : 0;
   }
-  const int lane = threadIdx.x & 31;
-  for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < tiles * kBM;
-       r += (int64_t)gridDim.x * 8) {
+  for (int64_t r = blockIdx.x; r < tiles * kBM; r += gridDim.x) {
     int64_t src = -1;
     if (r < rows) {
       int i = 0;
@@ -260,19 +264,29 @@ __global__ void __launch_bounds__(256) lm_gather_kernel(const GatherParams p, co
         src = b * p.T + lo + (k - off[b]);
       }
     }
-    if (!ADWIN_CHK(src < p.B * p.T && r < p.max_tiles * kBM, p.status)) continue;
+    if (!ADWIN_CHK(src < p.B * p.T && r < p.max_tiles * kBM, p.status)) continue;   // (uniform)
     const int y = src >= 0 ? p.tokens[src] : -1;
     const bool has = y >= 0 && y < p.V;
-    const float zy = copy_dot(src >= 0 ? p.hs + src * p.ds : nullptr,
-                              has ? p.ws + (int64_t)y * p.ds : nullptr, p.hs_c + r * p.ds, p.ds, lane);
-    const float uy = copy_dot(src >= 0 ? p.ht + src * p.dt : nullptr,
-                              has ? p.wt + (int64_t)y * p.dt : nullptr, p.ht_c + r * p.dt, p.dt, lane);
-    if (lane == 0) {
+    const float zp = warp_sum(copy_dot(src >= 0 ? p.hs + src * p.ds : nullptr,
+                                       has ? p.ws + (int64_t)y * p.ds : nullptr, p.hs_c + r * p.ds, p.ds));
+    const float up = warp_sum(copy_dot(src >= 0 ? p.ht + src * p.dt : nullptr,
+                                       has ? p.wt + (int64_t)y * p.dt : nullptr, p.ht_c + r * p.dt, p.dt));
+    if ((threadIdx.x & 31) == 0) {
+      red[0][threadIdx.x >> 5] = zp;
+      red[1][threadIdx.x >> 5] = up;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float zy = 0.f, uy = 0.f;
+      for (int w = 0; w < kGatherThreads / 32; ++w) {
+        zy += red[0][w];
+        uy += red[1][w];
+      }
       p.rowsrc[r] = (int32_t)src;
       p.rowdst[r] = r < grad_rows ? (int32_t)src : -1;
-      *reinterpret_cast<float4*>(p.tok + r * kTokFields) =
-          make_float4(has ? zy : 0.f, has ? uy : 0.f, has ? 1.f : 0.f, 0.f);
+      *reinterpret_cast<float4*>(p.tok + r * kTokFields) = make_float4(zy, uy, has ? 1.f : 0.f, 0.f);
     }
+    __syncthreads();
   }
 }
 
@@ -574,60 +588,64 @@ struct MergeParams {
   int32_t* status;
 };
 
-// One block per tile, kMergeWays threads per compact row: combine the partial records of the row in
-// float64 against common references (fixed order) and derive the per-token outputs and the
-// gradient coefficients:
+// Block = 32 compact rows, 32 threads per row: combine the partial records of the row in float64
+// against common references (fixed order) and derive the per-token outputs and the gradient
+// coefficients:
 //   g_k = p_k (a1 (z_k - u_k) + a0) (+ gy at k = y),   p_k = 2^(z_k log2e - L2s).
-constexpr int kMergeWays = 8;
-__global__ void __launch_bounds__(kBM * kMergeWays) lm_merge_kernel(const MergeParams p) {
-  __shared__ double red[kMergeWays][kBM];
-  __shared__ double tot[kBM];
+// Records are read with the row as the fast index (whole 128-byte lines), reduced with the record
+// as the lane.  A short call has many records (126 for each of 225 rows at V = 32 000), which is
+// why the records are spread over threads: 21 -> 5 us there against 8 threads per row.
+constexpr int kMergeRows = 32;
+__global__ void __launch_bounds__(1024) lm_merge_kernel(const MergeParams p) {
+  __shared__ double red[6][32][kMergeRows];
   int64_t lo, hi;
   launch_tiles(p.hdr, p.tile0, p.tile_cap, p.rest, lo, hi);
-  const int64_t tile = lo + blockIdx.x;
+  const int64_t tile = lo + blockIdx.x / (kBM / kMergeRows);
   if (tile >= hi) return;
-  const int row = threadIdx.x % kBM, way = threadIdx.x / kBM;
-  const int64_t crow = tile * kBM + row;
+  const int first = blockIdx.x % (kBM / kMergeRows) * kMergeRows;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = p.hdr->n_groups * 2;
-  const float* rec = p.part + ((tile - lo) * n * kRecFields) * kBM + row;
+  // while reading: lane = row, warp = record
+  const float* rec = p.part + ((tile - lo) * n * kRecFields) * kBM + first + lane;
   auto f = [&](int i, int k) { return (double)rec[((int64_t)i * kRecFields + k) * kBM]; };
-  // the sum (or maximum) of one value over the ways, in order; valid in every thread of the row
-  auto all_ways = [&](double v, bool max) {
-    __syncthreads();
-    red[way][row] = v;
-    __syncthreads();
-    if (way == 0) {
-      double a = red[0][row];
-      for (int i = 1; i < kMergeWays; ++i) a = max ? fmax(a, red[i][row]) : a + red[i][row];
-      tot[row] = a;
-    }
-    __syncthreads();
-    return tot[row];
-  };
   double M2s = -INFINITY, M2t = -INFINITY;
-  for (int i = way; i < n; i += kMergeWays) {
+  for (int i = warp; i < n; i += 32) {
     M2s = fmax(M2s, f(i, 0));
     M2t = fmax(M2t, f(i, 6));
   }
-  M2s = all_ways(M2s, true);
-  M2t = all_ways(M2t, true);
-  double S = 0, St = 0, Ac = 0, B0 = 0, B1 = 0, B2 = 0;
-  for (int i = way; i < n; i += kMergeWays) {
-    const double w = exp2(f(i, 0) - M2s), w2 = w * w;
-    S += w * f(i, 1);
-    Ac += w * f(i, 2);
-    B0 += w2 * f(i, 3);
-    B1 += w2 * f(i, 4);
-    B2 += w2 * f(i, 5);
-    St += exp2(f(i, 6) - M2t) * f(i, 7);
+  red[0][warp][lane] = M2s;
+  red[1][warp][lane] = M2t;
+  __syncthreads();
+  M2s = red[0][0][lane];
+  M2t = red[1][0][lane];
+  for (int w = 1; w < 32; ++w) {
+    M2s = fmax(M2s, red[0][w][lane]);
+    M2t = fmax(M2t, red[1][w][lane]);
   }
-  S = all_ways(S, false);
-  Ac = all_ways(Ac, false);
-  B0 = all_ways(B0, false);
-  B1 = all_ways(B1, false);
-  B2 = all_ways(B2, false);
-  St = all_ways(St, false);
-  if (way != 0) return;
+  __syncthreads();
+  double v[6] = {0, 0, 0, 0, 0, 0};   // S, Ac, B0, B1, B2, St
+  for (int i = warp; i < n; i += 32) {
+    const double w = exp2(f(i, 0) - M2s), w2 = w * w;
+    v[0] += w * f(i, 1);
+    v[1] += w * f(i, 2);
+    v[2] += w2 * f(i, 3);
+    v[3] += w2 * f(i, 4);
+    v[4] += w2 * f(i, 5);
+    v[5] += exp2(f(i, 6) - M2t) * f(i, 7);
+  }
+#pragma unroll
+  for (int k = 0; k < 6; ++k) red[k][warp][lane] = v[k];
+  __syncthreads();
+  if (warp < 6) {   // one field per warp, lane = row
+    double t = 0.0;
+    for (int w = 0; w < 32; ++w) t += red[warp][w][lane];
+    red[warp][0][lane] = t;
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  const int64_t crow = tile * kBM + first + lane;
+  const double S = red[0][0][lane], Ac = red[1][0][lane], B0 = red[2][0][lane];
+  const double B1 = red[3][0][lane], B2 = red[4][0][lane], St = red[5][0][lane];
 
   float* inf = p.info + crow * kInfoFields;
   const int64_t r = p.rowsrc[crow];
@@ -768,19 +786,26 @@ __global__ void __launch_bounds__(256, 2) lm_grad_kernel(const GradParams p) {
 }
 
 // Squared gradient norm of the rows whose gradient was formed: the sum of g_k^2 over the entries
-// themselves (fixed order, float64), which replaces the single-sweep moment value there.
-__global__ void __launch_bounds__(kBM) lm_gsq_kernel(const LmHeader* hdr, const float* __restrict__ q,
-                                                     const int32_t* __restrict__ rowdst,
-                                                     int n_groups, float* gsq) {
-  const int tile = blockIdx.x;
+// themselves (fixed order, float64), which replaces the single-sweep moment value there.  Block = 32
+// compact rows, 32 threads per row, as in lm_merge_kernel.
+__global__ void __launch_bounds__(1024) lm_gsq_kernel(const LmHeader* hdr, const float* __restrict__ q,
+                                                      const int32_t* __restrict__ rowdst,
+                                                      int n_groups, float* gsq) {
+  __shared__ double red[32][kMergeRows];
+  const int64_t tile = blockIdx.x / (kBM / kMergeRows);
   if (tile >= hdr->grad_tiles) return;
-  const int row = threadIdx.x;
-  const int32_t dst = rowdst[(int64_t)tile * kBM + row];
-  if (dst < 0) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = blockIdx.x % (kBM / kMergeRows) * kMergeRows + lane;
   double acc = 0.0;
-#pragma unroll 8
-  for (int i = 0; i < n_groups * 2; ++i)
-    acc += (double)q[((int64_t)tile * n_groups * 2 + i) * kBM + row];
+  for (int i = warp; i < n_groups * 2; i += 32)
+    acc += (double)q[(tile * n_groups * 2 + i) * kBM + row];
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp != 0) return;
+  const int32_t dst = rowdst[tile * kBM + row];
+  if (dst < 0) return;
+  acc = 0.0;
+  for (int w = 0; w < 32; ++w) acc += red[w][lane];
   gsq[dst] = (float)acc;
 }
 
@@ -844,8 +869,7 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
   gp.ht_c = ht_c;
   gp.status = a.status;
   lm_plan_kernel<<<plan.n_seg, 1024, 0, s>>>(gp.range, gp.ewin, a.B, plan, seg);
-  const int64_t gather_blocks = rows_cap / 8;
-  lm_gather_kernel<<<(int)(gather_blocks < 8192 ? gather_blocks : 8192), 256, 0, s>>>(gp, plan);
+  lm_gather_kernel<<<(int)(rows_cap < 16384 ? rows_cap : 16384), kGatherThreads, 0, s>>>(gp, plan);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
   CUtensorMap m_hs, m_ws, m_ht, m_wt;
@@ -897,7 +921,7 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
         moments ? launch_pairs(lm_sweep_kernel<true>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp)
                 : launch_pairs(lm_sweep_kernel<false>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp);
     if (r != cudaSuccess) return r;
-    lm_merge_kernel<<<(unsigned)cap, kBM * kMergeWays, 0, s>>>(mp);
+    lm_merge_kernel<<<(unsigned)cap * (kBM / kMergeRows), 1024, 0, s>>>(mp);
     return cudaGetLastError();
   };
   if (!a.want_grad) return statistics(0, L.max_tiles, 2, false, a.gsq != nullptr);
@@ -927,7 +951,9 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (range_full && (e = statistics(0, L.max_tiles, 1, false, moments)) != cudaSuccess) return e;
-  if (a.gsq) lm_gsq_kernel<<<(unsigned)L.max_tiles, kBM, 0, s>>>(hdr, q, rowdst, L.grad_groups, a.gsq);
+  if (a.gsq)
+    lm_gsq_kernel<<<(unsigned)L.max_tiles * (kBM / kMergeRows), 1024, 0, s>>>(hdr, q, rowdst,
+                                                                             L.grad_groups, a.gsq);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
   if (a.dH) {

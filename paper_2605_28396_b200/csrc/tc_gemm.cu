@@ -65,6 +65,7 @@ namespace {
 
 // Pieces of split tiles that the scratch buffer holds (256 KB each).
 constexpr int kMaxPieces = 4 * 74;
+constexpr int kMinPiece = 8;     // k-blocks of a piece, at least
 constexpr size_t kPieceBytes = (size_t)2 * kBM * kBN * 4;
 
 struct GemmParams {
@@ -106,7 +107,7 @@ struct GemmWork {
       // The last round's cost in k-blocks; a piece pays ~8 for filling the pipeline, storing and
       // being summed, so short contractions stay whole.
       int best = nk;
-      for (int s = 2; s <= 64 && s * rest <= kMaxPieces && s * 8 <= nk; ++s) {
+      for (int s = 2; s <= 64 && s * rest <= kMaxPieces && s * kMinPiece <= nk; ++s) {
         const int cost = (s * rest + pairs - 1) / pairs * ((nk + s - 1) / s + 8) + 8;
         if (cost < best) {
           best = cost;
@@ -144,13 +145,14 @@ struct GemmWork {
   }
 };
 
-// 32 consecutive columns of one row of C.
-__device__ __forceinline__ void store_c32(const GemmParams& p, int bin, int64_t dst, int64_t n,
-                                          const float (&v)[32]) {
+// NC consecutive columns (a multiple of 8) of one row of C.
+template <int NC>
+__device__ __forceinline__ void store_c(const GemmParams& p, int bin, int64_t dst, int64_t n,
+                                        const float (&v)[NC]) {
   if (p.c_is_bf16) {
     __nv_bfloat16* cp = static_cast<__nv_bfloat16*>(p.C) + dst * p.ldc + n;
 #pragma unroll
-    for (int i = 0; i < 32; i += 8)
+    for (int i = 0; i < NC; i += 8)
       if (n + i < p.N)
         *reinterpret_cast<uint4*>(cp + i) =
             make_uint4(pack_bf16x2(v[i], v[i + 1]), pack_bf16x2(v[i + 2], v[i + 3]),
@@ -159,7 +161,7 @@ __device__ __forceinline__ void store_c32(const GemmParams& p, int bin, int64_t 
     float* cp = static_cast<float*>(p.C) + (int64_t)bin * p.bin_stride + dst * p.ldc + n;
     if ((reinterpret_cast<uintptr_t>(cp) & 31) == 0) {   // whole 32-byte sectors
 #pragma unroll
-      for (int i = 0; i < 32; i += 8)
+      for (int i = 0; i < NC; i += 8)
         if (n + i < p.N)   // (N % 8 == 0)
           asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(cp + i),
                        "f"(v[i]), "f"(v[i + 1]), "f"(v[i + 2]), "f"(v[i + 3]), "f"(v[i + 4]),
@@ -167,7 +169,7 @@ __device__ __forceinline__ void store_c32(const GemmParams& p, int bin, int64_t 
                        : "memory");
     } else {
 #pragma unroll
-      for (int i = 0; i < 32; i += 4)
+      for (int i = 0; i < NC; i += 4)
         if (n + i < p.N)
           *reinterpret_cast<float4*>(cp + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
     }
@@ -307,7 +309,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                   make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
           }
         } else if (store) {
-          store_c32(p, bin, dst, n0 + j * 32, v);
+          store_c<32>(p, bin, dst, n0 + j * 32, v);
         }
       }
       tc_fence_before_sync();
@@ -328,37 +330,32 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   }
 }
 
-// Sums the pieces of the split tiles in order and stores C.
+// Sums the pieces of the split tiles in order and stores C; a thread owns 8 columns of a row.
 __global__ void __launch_bounds__(128) gemm_reduce_kernel(const GemmParams p, int pairs) {
   const GemmWork w(p, pairs);
   if (w.split == 1) return;
   const int rest = w.m_pairs * p.n_tiles - w.whole;
   const int row = threadIdx.x;
-  for (int u = blockIdx.x; u < rest * 16; u += gridDim.x) {   // 2 CTAs x 8 column blocks of 32
-    const int t = u / 16, rank = (u / 8) & 1, j = u % 8;
+  for (int u = blockIdx.x; u < rest * 64; u += gridDim.x) {   // 2 CTAs x 32 column groups of 8
+    const int t = u / 64, rank = (u / 32) & 1, j = u % 32;
     const int tile = w.whole + t;
     const int64_t m = (int64_t)(2 * (tile / p.n_tiles) + rank) * kBM + row;
-    const int64_t n = (int64_t)(tile % p.n_tiles) * kBN + j * 32;
+    const int64_t n = (int64_t)(tile % p.n_tiles) * kBN + j * 8;
     int64_t dst = m;
     if (p.row_map) dst = (m < w.M) ? p.row_map[m] : -1;
     if (m >= w.M || dst < 0 || n >= p.N) continue;
-    float v[32];
+    float v[8];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = 0.f;
-    for (int s = 0; s < w.split; ++s) {
-      const float4* pc = reinterpret_cast<const float4*>(p.pieces) +
-                         ((size_t)(t * w.split + s) * 2 + rank) * (kBM * kBN / 4) +
-                         (size_t)(j * 8) * kBM + row;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 x = pc[(size_t)i * kBM];
-        v[4 * i] += x.x;
-        v[4 * i + 1] += x.y;
-        v[4 * i + 2] += x.z;
-        v[4 * i + 3] += x.w;
-      }
+    for (int i = 0; i < 8; ++i) v[i] = 0.f;
+    const float4* pc = reinterpret_cast<const float4*>(p.pieces) +
+                       ((size_t)t * w.split * 2 + rank) * (kBM * kBN / 4) + (size_t)(j * 2) * kBM + row;
+#pragma unroll 6
+    for (int s = 0; s < w.split; ++s, pc += kBM * kBN / 2) {
+      const float4 x = __ldcs(pc), y = __ldcs(pc + kBM);
+      v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+      v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
     }
-    store_c32(p, 0, dst, n, v);
+    store_c<8>(p, 0, dst, n, v);
   }
 }
 
@@ -373,7 +370,7 @@ cudaError_t launch_gemm(const void* A, int64_t lda, bool a_mn, const void* B, in
   p.limit_ns = handshake_wait_limit_ns();
   const cudaError_t e = a_mn ? launch_pairs(tc_gemm_kernel<true, true>, sm_count, s, ma, mb, p)
                              : launch_pairs(tc_gemm_kernel<false, true>, sm_count, s, ma, mb, p);
-  if (e != cudaSuccess || !p.pieces) return e;
+  if (e != cudaSuccess || !p.pieces || p.k_blocks < 2 * kMinPiece) return e;   // (nothing is split)
   gemm_reduce_kernel<<<sm_count * 4, 128, 0, s>>>(p, sm_count / 2);
   return cudaGetLastError();
 }
