@@ -142,9 +142,9 @@ int adwin_teacher_drift(const void* teacher_logits, int dtype, int64_t B, int64_
     return ADWIN_ERR_ALIGN;
   const int sms = sm_count_of_current_device();
   if (sms <= 0) return ADWIN_ERR_CUDA;
-  const bool vec16 = aligned(teacher_logits, 16) && (ld * es) % 16 == 0 && (V * es) % 16 == 0;
+  // (element-aligned rows always reach a 16-byte boundary; rows of a few entries are read singly)
   if (launch_teacher_drift(teacher_logits, dtype, B, T, V, ld, tokens, rollout_len, entropy, rank,
-                           dev_status, vec16, sms,
+                           dev_status, V * (int64_t)es >= 64, sms,
                            static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess)
     return ADWIN_ERR_CUDA;
   return ADWIN_OK;
@@ -226,17 +226,30 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
   p.row_coef = row_coef;
   p.skip_below = nullptr;
 
-  // 16-byte layout test shared by the vectorised streaming path and the staged kernel.
+  // Layout.  vec: row r of every array has the same offset from a 16-byte boundary (the gradient in
+  // units of its own entries), so 16 bytes move at a time except at a row's ends (V = 50 257 bf16,
+  // rows packed, 2283 rows with gradient: 739 us entry by entry, 249 us through the staged kernel).  whole: rows also
+  // start and end on boundaries.  The staged kernel takes arrays that start on a boundary.  (Rows of
+  // a few entries are not worth it.)
   const int gd = grad_student ? grad_dtype : dtype;
-  bool vec16 = aligned(student_logits, 16) && aligned(teacher_logits, 16) &&
-               (ld * es) % 16 == 0 && (V * es) % 16 == 0;
-  if (grad_student)
-    vec16 = vec16 && aligned(grad_student, 16) && (ld_grad * elem_size(gd)) % 16 == 0 &&
-            (V * elem_size(gd)) % 16 == 0;
+  const size_t gs = elem_size(gd);
+  const uintptr_t zb = reinterpret_cast<uintptr_t>(student_logits), ub = reinterpret_cast<uintptr_t>(teacher_logits),
+                  gb = reinterpret_cast<uintptr_t>(grad_student);
+  const bool rows16 = (ld * es) % 16 == 0;
+  bool vec = zb % 16 == ub % 16 && V * (int64_t)es >= 64, whole = rows16 && (V * es) % 16 == 0;
+  bool start16 = zb % 16 == 0 && ub % 16 == 0;
+  if (grad_student) {
+    // a piece of N input entries is N output entries, 8 to 32 bytes
+    const bool grad_rows16 = (ld_grad * gs) % 16 == 0;
+    start16 = start16 && gb % 16 == 0;
+    vec = vec && start16 && (ld_grad == ld || (rows16 && grad_rows16));
+    whole = whole && grad_rows16 && (V * gs) % 16 == 0;
+  }
+  const bool staged_ok = vec && start16;
   // Scalars over the whole rollout with the gradient inside the window: the window rows need the
   // staged kernel's two sweeps, the rows past the window are a single read, which the streaming
   // kernel does faster.  With the extended workspace the call runs them as two launches.
-  const bool split = vec16 && grad_student && (flags & ADWIN_RANGE_FULL) &&
+  const bool split = staged_ok && grad_student && (flags & ADWIN_RANGE_FULL) &&
                      !(flags & (ADWIN_FORCE_GENERIC | ADWIN_FORCE_STAGED)) &&
                      workspace_bytes >= wl.total_ext;
 
@@ -251,13 +264,13 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
     KlParams pw = p;          // window rows: the compact list built from the effective windows
     pw.offsets = reinterpret_cast<const int64_t*>(wbase + wl.off_offsets_win);
     pw.range = p.ewin;
-    const cudaError_t e = launch_kl_staged(pw, dtype, gd, sms, s);
+    const cudaError_t e = launch_kl_staged(pw, dtype, gd, !whole, sms, s);
     if (e == cudaSuccess) {
       KlParams pr = p;        // the rest of every rollout, without gradient
       pr.grad = nullptr;
       pr.ld_grad = 0;
       pr.skip_below = p.ewin;
-      if (launch_kl_generic(pr, dtype, dtype, true, sms, s) != cudaSuccess) return ADWIN_ERR_CUDA;
+      if (launch_kl_generic(pr, dtype, dtype, vec, sms, s) != cudaSuccess) return ADWIN_ERR_CUDA;
       return ADWIN_OK;
     }
     if (e != cudaErrorNotSupported) return ADWIN_ERR_CUDA;
@@ -266,12 +279,12 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
   // staged cluster kernel.  A call without gradient is a single read of every row, which the
   // row-per-CTA streaming kernel does faster (90 % against 74 % of the copy bandwidth, measured).
   const bool want_staged = (flags & ADWIN_FORCE_STAGED) || grad_student != nullptr;
-  if (vec16 && want_staged && !(flags & ADWIN_FORCE_GENERIC)) {
-    const cudaError_t e = launch_kl_staged(p, dtype, gd, sms, s);
+  if (staged_ok && want_staged && !(flags & ADWIN_FORCE_GENERIC)) {
+    const cudaError_t e = launch_kl_staged(p, dtype, gd, !whole, sms, s);
     if (e == cudaSuccess) return ADWIN_OK;
     if (e != cudaErrorNotSupported) return ADWIN_ERR_CUDA;
   }
-  if (launch_kl_generic(p, dtype, gd, vec16, sms, s) != cudaSuccess) return ADWIN_ERR_CUDA;
+  if (launch_kl_generic(p, dtype, gd, vec, sms, s) != cudaSuccess) return ADWIN_ERR_CUDA;
   return ADWIN_OK;
 }
 

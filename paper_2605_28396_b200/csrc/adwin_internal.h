@@ -36,8 +36,9 @@ cudaError_t launch_kl_generic(const KlParams& p, int dtype, int grad_dtype, bool
                               cudaStream_t s);
 
 // Staged cluster kernel.  Returns cudaErrorNotSupported when the shape does not fit its plan
-// (the caller then falls back to the generic kernel).
-cudaError_t launch_kl_staged(const KlParams& p, int dtype, int grad_dtype, int sm_count,
+// (the caller then falls back to the generic kernel).  ragged: rows that do not all start and end on
+// 16-byte boundaries.
+cudaError_t launch_kl_staged(const KlParams& p, int dtype, int grad_dtype, bool ragged, int sm_count,
                              cudaStream_t s);
 
 cudaError_t launch_window_reduce(const float* kl, const float* logratio, const float* gsq,

@@ -3,8 +3,10 @@
 // Sweep 1 streams z and u once and accumulates the online log-sum-exp statistics, sum e*delta
 // (reverse KL) and the moments of the single-sweep gradient norm.  Sweep 2 (only for rows whose
 // gradient is written) re-reads the row and writes g.  Any V, any row stride, any element
-// alignment; 16-byte vector loads when the layout allows.  This is the fallback for layouts the
-// staged cluster kernel does not take, and the reference point it is measured against.
+// alignment.  VEC: the rows of all arrays share one offset from a 16-byte boundary (always so when
+// the arrays start on one and have one stride), and everything but the at most N - 1 entries before
+// the first boundary and after the last is moved 16 bytes at a time; otherwise entry by entry.
+// Calls without gradient come here, and layouts that the staged cluster kernel does not take.
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
 
@@ -206,19 +208,31 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
 
     RowAcc a;
     a.reset();
-    const int64_t pieces = (p.V + N - 1) / N;  // VEC requires V % N == 0
+    // VEC: `head` entries up to the first boundary, whole pieces, `tail` entries
+    int head = 0, tail = 0;
+    if (VEC) {
+      const int shift = (int)((reinterpret_cast<uintptr_t>(zrow) & 15) / sizeof(TIn));
+      head = shift ? N - shift : 0;
+      if (head > p.V) head = (int)p.V;
+      tail = (int)((p.V - head) % N);
+    }
+    const int64_t pieces = VEC ? (p.V - head) / N : p.V;
+    // the entry before or after the pieces that this thread looks after, or -1
+    const int64_t edge = !VEC ? -1
+                         : tid < head ? tid
+                         : (tid >= 32 && tid - 32 < tail) ? p.V - tail + (tid - 32) : -1;
     if (VEC) {
       PairAcc pa;
       pa.reset();
       // kGenericUnroll pairs of 16-byte loads in flight per thread; a row that is read only once
       // (no gradient) is streamed past the caches, otherwise sweep 2 should find it in L2
-      const uint4* zs = reinterpret_cast<const uint4*>(zrow);
-      const uint4* us = reinterpret_cast<const uint4*>(urow);
+      const uint4* zs = reinterpret_cast<const uint4*>(zrow + head * sizeof(TIn));
+      const uint4* us = reinterpret_cast<const uint4*>(urow + head * sizeof(TIn));
       int64_t i = tid;
       for (; i + (kGenericUnroll - 1) * kGenericThreads < pieces;
            i += kGenericUnroll * kGenericThreads) {
         uint4 zv[kGenericUnroll], uv[kGenericUnroll];
-        if (!ADWIN_CHK(i + (kGenericUnroll - 1) * kGenericThreads < pieces && (i + (kGenericUnroll - 1) * kGenericThreads + 1) * N <= p.ld, p.status)) break;
+        if (!ADWIN_CHK(head + (i + (kGenericUnroll - 1) * kGenericThreads + 1) * N <= p.V, p.status)) break;
 #pragma unroll
         for (int h = 0; h < kGenericUnroll; ++h) {
           zv[h] = write_grad ? __ldg(zs + i + h * kGenericThreads) : __ldcs(zs + i + h * kGenericThreads);
@@ -234,7 +248,7 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
       }
       for (; i < pieces; i += kGenericThreads) {
         float z[N], u[N];
-        if (!ADWIN_CHK((i + 1) * N <= p.ld, p.status)) break;
+        if (!ADWIN_CHK(head + (i + 1) * N <= p.V, p.status)) break;
         const uint4 zv = write_grad ? __ldg(zs + i) : __ldcs(zs + i);
         const uint4 uv = write_grad ? __ldg(us + i) : __ldcs(us + i);
         Elem<TIn>::unpack(zv, reinterpret_cast<float(&)[Elem<TIn>::N]>(z));
@@ -242,6 +256,10 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
         acc_piece_pairs<N>(z, u, dref, pa);
       }
       a = pa.fold();
+      if (edge >= 0) {
+        const float z[1] = {Elem<TIn>::load1(zrow, edge)}, u[1] = {Elem<TIn>::load1(urow, edge)};
+        acc_piece<1, true>(z, u, dref, a);
+      }
     } else {
       for (int64_t i = tid; i < pieces; i += kGenericThreads) {
         float z[N], u[N];
@@ -262,12 +280,23 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
     if (write_grad) {
       char* grow = static_cast<char*>(p.grad) + (size_t)r * p.ld_grad * sizeof(TOut);
       const bool full = (p.mode == ADWIN_GRAD_FULL_KL);
+      auto gradient = [&](float z, float u, int64_t k) {
+        const float e = ex2f(fmaf(z, kLog2e, -tot.M2s));
+        if (full) return e * (rs.coef * (((z - u) - dref) - rs.c0));
+        return (y_valid && k == yi) ? rs.gy : e * rs.coef;
+      };
+      if (edge >= 0) {
+        const float g = gradient(Elem<TIn>::load1(zrow, edge), Elem<TIn>::load1(urow, edge), edge);
+        q = fmaf(g, g, q);
+        Elem<TOut>::store1(grow, edge, g);
+      }
+      char* gbody = grow + head * sizeof(TOut);
       for (int64_t i = tid; i < pieces; i += kGenericThreads) {
         float z[N], u[N], g[N];
-        if (!ADWIN_CHK((i + 1) * N <= p.V && (i + 1) * N <= p.ld_grad && (i + 1) * N <= p.ld, p.status)) break;
+        if (!ADWIN_CHK(head + (i + 1) * N <= p.V && head + (i + 1) * N <= p.ld_grad, p.status)) break;
         if (VEC) {
-          const uint4 zv = __ldg(reinterpret_cast<const uint4*>(zrow) + i);
-          const uint4 uv = __ldg(reinterpret_cast<const uint4*>(urow) + i);
+          const uint4 zv = __ldg(reinterpret_cast<const uint4*>(zrow + head * sizeof(TIn)) + i);
+          const uint4 uv = __ldg(reinterpret_cast<const uint4*>(urow + head * sizeof(TIn)) + i);
           Elem<TIn>::unpack(zv, reinterpret_cast<float(&)[Elem<TIn>::N]>(z));
           Elem<TIn>::unpack(uv, reinterpret_cast<float(&)[Elem<TIn>::N]>(u));
         } else {
@@ -276,17 +305,12 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
         }
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-          const float e = ex2f(fmaf(z[j], kLog2e, -tot.M2s));
-          if (full) {
-            g[j] = e * (rs.coef * (((z[j] - u[j]) - dref) - rs.c0));
-          } else {
-            g[j] = (y_valid && i * N + j == yi) ? rs.gy : e * rs.coef;
-          }
+          g[j] = gradient(z[j], u[j], head + i * N + j);
           q = fmaf(g[j], g[j], q);
         }
         if (VEC) {
           if (sizeof(TOut) == 4) {
-            float4* o = reinterpret_cast<float4*>(grow) + i * (N / 4);
+            float4* o = reinterpret_cast<float4*>(gbody) + i * (N / 4);
 #pragma unroll
             for (int j = 0; j < N / 4; ++j)
               o[j] = make_float4(g[4 * j], g[4 * j + 1], g[4 * j + 2], g[4 * j + 3]);
@@ -297,12 +321,12 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
               o.y = pack_bf16x2(g[2], g[3]);
               o.z = pack_bf16x2(g[4], g[5]);
               o.w = pack_bf16x2(g[6], g[7]);
-              reinterpret_cast<uint4*>(grow)[i] = o;
+              reinterpret_cast<uint4*>(gbody)[i] = o;
             } else {  // fp32 logits, bf16 gradient: 4 entries = 8 bytes
               uint2 o;
               o.x = pack_bf16x2(g[0], g[1]);
               o.y = pack_bf16x2(g[2], g[3]);
-              reinterpret_cast<uint2*>(grow)[i] = o;
+              reinterpret_cast<uint2*>(gbody)[i] = o;
             }
           }
         } else {

@@ -504,7 +504,40 @@ __device__ __forceinline__ float lane_sum(float v) {
   return v;
 }
 
-template <typename TIn, typename TOut, bool TM>
+// Rows that do not start or end on a 16-byte boundary (RAG): the pieces are those of the aligned
+// span that covers the row, `shift` entries of the first piece belong to the row before (or to
+// padding) and so may the end of the last one.  Reading them is harmless -- a 16-byte granule that
+// holds an entry of the row is always readable -- and their values are replaced by one whose
+// exponential is zero on both sides.
+template <typename TIn>
+__device__ __forceinline__ void mask_piece(uint4& z, uint4& u, int e0, int e1) {
+  constexpr int N = Elem<TIn>::N;
+  uint32_t zw[4] = {z.x, z.y, z.z, z.w}, uw[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int e = 0; e < N; ++e) {
+    if (e >= e0 && e < e1) continue;
+    if (sizeof(TIn) == 4) {
+      zw[e % 4] = uw[e % 4] = 0xf149f2cau;             // -1e30f
+    } else {
+      const uint32_t keep = (e & 1) ? 0x0000ffffu : 0xffff0000u, put = (e & 1) ? 0xf1490000u : 0xf149u;
+      zw[(e / 2) % 4] = (zw[(e / 2) % 4] & keep) | put;  // bf16 -1e30
+      uw[(e / 2) % 4] = (uw[(e / 2) % 4] & keep) | put;
+    }
+  }
+  z = make_uint4(zw[0], zw[1], zw[2], zw[3]);
+  u = make_uint4(uw[0], uw[1], uw[2], uw[3]);
+}
+
+// Where a row lies in this CTA's slice.
+struct RowSpan {
+  int pieces;        // pieces of the slice
+  int shift;         // entries of piece 0 that precede the row
+  int first, last;   // slice-relative index of the row's first / last piece if it is partial, else -1
+  int last_n;        // entries of the row in its last piece (counted from the piece's start)
+  __device__ __forceinline__ int e0(int piece) const { return piece == first ? shift : 0; }
+};
+
+template <typename TIn, typename TOut, bool TM, bool RAG>
 __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, StagedPlan plan) {
   constexpr int N = Elem<TIn>::N;
   constexpr int NP = Pairs<TIn>::NP;
@@ -523,7 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
   const uint32_t u_off = (uint32_t)plan.chunk_pieces * 16u;
 
   // slice of this CTA, in 16-byte pieces
-  const int64_t pieces_total = p.V / N;
+  const int64_t pieces_total = RAG ? (p.V + 2 * N - 2) / N : p.V / N;   // of any row, at most
   const int64_t piece0 = (int64_t)rank * plan.per_rank_pieces;
   int64_t my_pieces = pieces_total - piece0;
   my_pieces = my_pieces < 0 ? 0 : (my_pieces > plan.per_rank_pieces ? plan.per_rank_pieces : my_pieces);
@@ -561,26 +594,41 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   cluster_sync_all();  // peers' barriers exist before any remote arrive
 
-  // pieces of this CTA's slice that fall into chunk j (<= 0 for chunks past the slice end)
-  auto pieces_in_chunk = [&](int j) -> int {
-    const int left = (int)my_pieces - j * plan.chunk_pieces;
+  // where row r lies in the slice (base pointers are 16-byte aligned, so the shift is r*ld mod N)
+  auto span_of = [&](int64_t r) -> RowSpan {
+    RowSpan a = {(int)my_pieces, 0, -1, -1, N};
+    if (RAG) {
+      a.shift = (int)((r * p.ld) & (N - 1));
+      const int64_t end = a.shift + p.V, total = (end + N - 1) / N;
+      const int64_t left = total - piece0;
+      a.pieces = (int)(left < 0 ? 0 : (left > plan.per_rank_pieces ? plan.per_rank_pieces : left));
+      a.first = (a.shift > 0 && piece0 == 0) ? 0 : -1;
+      a.last_n = (int)(end - (total - 1) * N);
+      a.last = (a.last_n < N && left > 0 && left <= plan.per_rank_pieces) ? (int)left - 1 : -1;
+    }
+    return a;
+  };
+  // pieces of a slice of `mine` pieces that fall into chunk j (<= 0 for chunks past its end)
+  auto pieces_in_chunk = [&](int j, int mine) -> int {
+    const int left = mine - j * plan.chunk_pieces;
     return left < plan.chunk_pieces ? left : plan.chunk_pieces;
   };
   // issue the two bulk copies of chunk j of row r into a slot
   auto issue_chunk = [&](int64_t r, int j, char* slot, unsigned long long* full, uint64_t pol) {
-    int np = pieces_in_chunk(j);
+    const RowSpan span = span_of(r);
+    int np = pieces_in_chunk(j, span.pieces);
     np = np < 0 ? 0 : np;
     const uint32_t bytes = (uint32_t)np * 16u;
     const uint32_t bar = smem_u32(full);
     if (bytes == 0) {
       mbar_arrive(bar);
     } else {
-      const size_t goff = ((size_t)r * p.ld + (size_t)piece0 * N) * sizeof(TIn) +
+      const size_t goff = ((size_t)r * p.ld - span.shift + (size_t)piece0 * N) * sizeof(TIn) +
                           (size_t)j * plan.chunk_pieces * 16;
       // checked flavour: the copy lies inside the row's V elements and inside one slot
       if (!ADWIN_CHK(r >= 0 && r < p.B * p.T &&
                          ((size_t)piece0 * N) * sizeof(TIn) + (size_t)j * plan.chunk_pieces * 16 + bytes <=
-                             (size_t)p.V * sizeof(TIn) &&
+                             ((size_t)(span.shift + p.V) * sizeof(TIn) + (RAG ? 15 : 0)) &&
                          bytes <= u_off && 2u * u_off <= plan.slot_bytes &&
                          slot >= res_base &&
                          slot + plan.slot_bytes <= res_base + (size_t)(nres + nring) * plan.slot_bytes,
@@ -764,6 +812,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
       const bool y_valid = (yC >= 0) && ((int64_t)yC < p.V);
       const float ref_s = zyC * kLog2e, ref_t = uyC * kLog2e;   // shared references of the row
       const float dref = wgC ? 0.f : zyC - uyC;                 // delta is centred on probe rows
+      const RowSpan spanC = span_of(rC);
       const uint32_t rpar = (uint32_t)(i & 1);                  // fill parity of resident slots
 
       // ---------------------------------------------------------------- sweep 1
@@ -776,6 +825,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
         const int vend = (real && i + 1 < my_rows) ? nch + plan.lead : nch;
         bool wgv = wgC;
         f2_t nrefs = splat2(-ref_s), nreft = splat2(-ref_t), ndref = splat2(-dref);
+        RowSpan spanv = spanC;
         for (int v = v0;; ++v) {
           if (v == nch) {
             if (TM) tm_wait_st();
@@ -806,6 +856,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
             const RowMeta& mn = ctrl.meta[msn];
             wgv = mn.wg != 0;
             const float zyN = mn.zy, uyN = mn.uy;
+            if (RAG) spanv = span_of(mn.r);
             nrefs = splat2(-zyN * kLog2e);
             nreft = splat2(-uyN * kLog2e);
             ndref = splat2(-(wgv ? 0.f : zyN - uyN));
@@ -828,7 +879,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
           if (timed_out) break;
           // The thread's pieces go to registers first and the slot is handed back at once, so
           // the refill is in flight while the arithmetic runs.
-          const int np = pieces_in_chunk(j);
+          const int np = pieces_in_chunk(j, spanv.pieces);
           uint4 zr[kP], ur[kP];
 #pragma unroll
           for (int h = 0; h < kP; ++h) {
@@ -836,6 +887,14 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
                 ADWIN_CHK(k < nres && toff + (uint32_t)(h * kGT * 16) + 16u <= u_off, p.status)) {
               zr[h] = *reinterpret_cast<const uint4*>(sl + h * kGT * 16);
               ur[h] = *reinterpret_cast<const uint4*>(sl + u_off + h * kGT * 16);
+            }
+          }
+          if (RAG) {
+#pragma unroll
+            for (int h = 0; h < kP; ++h) {
+              const int lp = j * plan.chunk_pieces + gt + h * kGT;
+              if (gt + h * kGT < np && (lp == spanv.first || lp == spanv.last))
+                mask_piece<TIn>(zr[h], ur[h], spanv.e0(lp), lp == spanv.last ? spanv.last_n : N);
             }
           }
           if (k < 0 || !wgv) {
@@ -907,12 +966,15 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
       if (!(t.S < kSumLimit) || !(t.St < kSumLimit) || !(t.B0 < kSumLimit)) {
         RowAcc ra;
         ra.reset();
-        const char* zrow = static_cast<const char*>(p.student) + ((size_t)rC * p.ld + (size_t)piece0 * N) * sizeof(TIn);
-        const char* urow = static_cast<const char*>(p.teacher) + ((size_t)rC * p.ld + (size_t)piece0 * N) * sizeof(TIn);
-        for (int64_t pc = tid; pc < my_pieces; pc += kNT) {
+        const size_t off = ((size_t)rC * p.ld - spanC.shift + (size_t)piece0 * N) * sizeof(TIn);
+        const char* zrow = static_cast<const char*>(p.student) + off;
+        const char* urow = static_cast<const char*>(p.teacher) + off;
+        for (int64_t pc = tid; pc < spanC.pieces; pc += kNT) {
           float z[N], u[N];
-          const uint4 zv = __ldg(reinterpret_cast<const uint4*>(zrow) + pc);
-          const uint4 uv = __ldg(reinterpret_cast<const uint4*>(urow) + pc);
+          uint4 zv = __ldg(reinterpret_cast<const uint4*>(zrow) + pc);
+          uint4 uv = __ldg(reinterpret_cast<const uint4*>(urow) + pc);
+          if (RAG && (pc == spanC.first || pc == spanC.last))
+            mask_piece<TIn>(zv, uv, spanC.e0((int)pc), pc == spanC.last ? spanC.last_n : N);
           Elem<TIn>::unpack(zv, z);
           Elem<TIn>::unpack(uv, u);
           acc_piece<N, true>(z, u, dref, ra);
@@ -982,9 +1044,10 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
         // bf16 logits: g = e * (coef*delta - coef*c0) saves one operation per pair; its rounding
         // (relative to coef*delta, not to the difference) is far inside that dtype's tolerance.
         const f2_t ncc0 = splat2(-rs.coef * rs.c0);
-        const int64_t ypiece = y_valid ? ((int64_t)yC / N - piece0) : -1;   // slice-relative
+        const int64_t yat = (int64_t)yC + spanC.shift;                // counted from piece 0
+        const int64_t ypiece = y_valid ? (yat / N - piece0) : -1;     // slice-relative
         char* gthread = static_cast<char*>(p.grad) +
-                        ((size_t)rC * p.ld_grad + (size_t)(piece0 + gt) * N) * sizeof(TOut);
+                        ((size_t)rC * p.ld_grad - spanC.shift + (size_t)(piece0 + gt) * N) * sizeof(TOut);
         const size_t gstep = (size_t)plan.chunk_pieces * N * sizeof(TOut);
         f2_t Q = 0ull;
         for (int j = 0; j < nch; ++j) {
@@ -999,7 +1062,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
               sl = ring_base + (size_t)rc_slot * plan.slot_bytes + toff;
             }
             if (timed_out) break;
-            const int np = pieces_in_chunk(j);
+            const int np = pieces_in_chunk(j, spanC.pieces);
             uint4 zr[kP], ur[kP];
             if (from_tm) {   // back from tensor memory (every lane takes part)
               const int o = ctrl.ord[j];
@@ -1025,6 +1088,10 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
 #pragma unroll
             for (int h = 0; h < kP; ++h) {
               if (gt + h * kGT < np) {
+                const int lp = j * plan.chunk_pieces + gt + h * kGT;
+                const bool partial = RAG && (lp == spanC.first || lp == spanC.last);
+                const int e1 = lp == spanC.last ? spanC.last_n : N;
+                if (partial) mask_piece<TIn>(zr[h], ur[h], spanC.e0(lp), e1);
                 f2_t Z[NP], U[NP], G[NP];
                 Pairs<TIn>::make(zr[h], Z);
                 Pairs<TIn>::make(ur[h], U);
@@ -1042,8 +1109,8 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
                     G[e] = mul2(E, coef2);
                   }
                 }
-                if (!full_mode && (int64_t)j * plan.chunk_pieces + gt + h * kGT == ypiece) {
-                  const int e = (int)((int64_t)yC - ((int64_t)yC / N) * N);
+                if (!full_mode && lp == ypiece) {
+                  const int e = (int)(yat - (yat / N) * N);
 #pragma unroll
                   for (int w = 0; w < NP; ++w) {
                     float lo, hi;
@@ -1056,9 +1123,21 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
 #pragma unroll
                 for (int e = 0; e < NP; ++e) Q = fma2(G[e], G[e], Q);
                 // checked flavour: the 16-byte (or 32-byte) store lies inside the row's V entries
-                if (ADWIN_CHK((piece0 + (int64_t)j * plan.chunk_pieces + gt + h * kGT + 1) * N <= p.V &&
-                                  rC >= 0 && rC < p.B * p.T, p.status))
-                  store_pairs<TOut, NP>(gthread + (size_t)j * gstep + (size_t)h * kGT * N * sizeof(TOut), G);
+                if (ADWIN_CHK((piece0 + lp + (RAG ? 0 : 1)) * N <= p.V + spanC.shift &&
+                                  rC >= 0 && rC < p.B * p.T, p.status)) {
+                  char* dst = gthread + (size_t)j * gstep + (size_t)h * kGT * N * sizeof(TOut);
+                  if (partial) {   // the row's own entries only
+#pragma unroll
+                    for (int w = 0; w < NP; ++w) {
+                      float lo, hi;
+                      upk2(G[w], lo, hi);
+                      if (2 * w >= spanC.e0(lp) && 2 * w < e1) Elem<TOut>::store1(dst, 2 * w, lo);
+                      if (2 * w + 1 >= spanC.e0(lp) && 2 * w + 1 < e1) Elem<TOut>::store1(dst, 2 * w + 1, hi);
+                    }
+                  } else {
+                    store_pairs<TOut, NP>(dst, G);
+                  }
+                }
               }
             }
           } else if (k < 0 && !TM) {
@@ -1173,9 +1252,17 @@ int plan_smem_bytes(const StagedPlan& plan) {
   return kCtrlBytes + (plan.nres + plan.nring) * (int)plan.slot_bytes;
 }
 
+typedef void (*StagedKernel)(KlParams, StagedPlan);
 template <typename TIn, typename TOut>
-cudaError_t max_clusters_for(const StagedPlan& plan, int sm_count, int& max_clusters) {
-  auto kernel = plan.tm ? kl_staged_kernel<TIn, TOut, true> : kl_staged_kernel<TIn, TOut, false>;
+StagedKernel staged_kernel(const StagedPlan& plan, bool ragged) {
+  if (ragged)
+    return plan.tm ? kl_staged_kernel<TIn, TOut, true, true> : kl_staged_kernel<TIn, TOut, false, true>;
+  return plan.tm ? kl_staged_kernel<TIn, TOut, true, false> : kl_staged_kernel<TIn, TOut, false, false>;
+}
+
+template <typename TIn, typename TOut>
+cudaError_t max_clusters_for(const StagedPlan& plan, bool ragged, int sm_count, int& max_clusters) {
+  StagedKernel kernel = staged_kernel<TIn, TOut>(plan, ragged);
   const int smem = plan_smem_bytes(plan);
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -1197,11 +1284,11 @@ cudaError_t max_clusters_for(const StagedPlan& plan, int sm_count, int& max_clus
 // (cluster sizes that do not divide a GPC's SM count leave SMs idle) among those whose streamed
 // bytes fit the L2 budget, else the one with the fewest streamed bytes.
 struct PlanKey {
-  int dev, dtype, grad_dtype, has_grad;
+  int dev, dtype, grad_dtype, has_grad, ragged;
   int64_t pieces_total;
   bool operator==(const PlanKey& o) const {
     return dev == o.dev && dtype == o.dtype && grad_dtype == o.grad_dtype &&
-           has_grad == o.has_grad && pieces_total == o.pieces_total;
+           has_grad == o.has_grad && ragged == o.ragged && pieces_total == o.pieces_total;
   }
 };
 struct PlanEntry {
@@ -1211,13 +1298,13 @@ struct PlanEntry {
 };
 
 template <typename TIn, typename TOut>
-bool choose_plan(int64_t pieces_total, bool has_grad, int sm_count, StagedPlan& best) {
+bool choose_plan(int64_t pieces_total, bool has_grad, bool ragged, int sm_count, StagedPlan& best) {
   double best_score = -1.0;
   for (int cl = 1; cl <= kMaxCL; ++cl) {
     StagedPlan plan = {};
     if (!plan_for_cluster(pieces_total, cl, has_grad, plan)) continue;
     int clusters = 0;
-    if (max_clusters_for<TIn, TOut>(plan, sm_count, clusters) != cudaSuccess) {
+    if (max_clusters_for<TIn, TOut>(plan, ragged, sm_count, clusters) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -1237,7 +1324,7 @@ bool choose_plan(int64_t pieces_total, bool has_grad, int sm_count, StagedPlan& 
 }
 
 template <typename TIn, typename TOut>
-cudaError_t launch_staged_t(const KlParams& p, int dtype, int grad_dtype, int sm_count,
+cudaError_t launch_staged_t(const KlParams& p, int dtype, int grad_dtype, bool ragged, int sm_count,
                             cudaStream_t s) {
   static std::mutex mu;
   static std::vector<PlanEntry> cache;
@@ -1245,7 +1332,8 @@ cudaError_t launch_staged_t(const KlParams& p, int dtype, int grad_dtype, int sm
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const int N = dtype == ADWIN_F32 ? 4 : 8;
-  const PlanKey key = {dev, dtype, grad_dtype, p.grad != nullptr ? 1 : 0, p.V / N};
+  const PlanKey key = {dev, dtype, grad_dtype, p.grad != nullptr ? 1 : 0, ragged ? 1 : 0,
+                       ragged ? (p.V + 2 * N - 2) / N : p.V / N};
   if (key.pieces_total < 1) return cudaErrorNotSupported;
   StagedPlan plan = {};
   bool ok = false, found = false;
@@ -1259,13 +1347,13 @@ cudaError_t launch_staged_t(const KlParams& p, int dtype, int grad_dtype, int sm
         break;
       }
     if (!found) {
-      ok = choose_plan<TIn, TOut>(key.pieces_total, key.has_grad != 0, sm_count, plan);
+      ok = choose_plan<TIn, TOut>(key.pieces_total, key.has_grad != 0, ragged, sm_count, plan);
       cache.push_back({key, ok, plan});
     }
   }
   if (!ok) return cudaErrorNotSupported;
 
-  auto kernel = plan.tm ? kl_staged_kernel<TIn, TOut, true> : kl_staged_kernel<TIn, TOut, false>;
+  StagedKernel kernel = staged_kernel<TIn, TOut>(plan, ragged);
   const int smem = plan_smem_bytes(plan);
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -1289,16 +1377,16 @@ cudaError_t launch_staged_t(const KlParams& p, int dtype, int grad_dtype, int sm
 
 }  // namespace
 
-cudaError_t launch_kl_staged(const KlParams& p, int dtype, int grad_dtype, int sm_count,
+cudaError_t launch_kl_staged(const KlParams& p, int dtype, int grad_dtype, bool ragged, int sm_count,
                              cudaStream_t s) {
   if (dtype == ADWIN_F32) {
     return grad_dtype == ADWIN_F32
-               ? launch_staged_t<float, float>(p, dtype, grad_dtype, sm_count, s)
-               : launch_staged_t<float, __nv_bfloat16>(p, dtype, grad_dtype, sm_count, s);
+               ? launch_staged_t<float, float>(p, dtype, grad_dtype, ragged, sm_count, s)
+               : launch_staged_t<float, __nv_bfloat16>(p, dtype, grad_dtype, ragged, sm_count, s);
   }
   return grad_dtype == ADWIN_F32
-             ? launch_staged_t<__nv_bfloat16, float>(p, dtype, grad_dtype, sm_count, s)
-             : launch_staged_t<__nv_bfloat16, __nv_bfloat16>(p, dtype, grad_dtype, sm_count, s);
+             ? launch_staged_t<__nv_bfloat16, float>(p, dtype, grad_dtype, ragged, sm_count, s)
+             : launch_staged_t<__nv_bfloat16, __nv_bfloat16>(p, dtype, grad_dtype, ragged, sm_count, s);
 }
 
 }  // namespace adwin

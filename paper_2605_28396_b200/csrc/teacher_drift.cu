@@ -92,13 +92,26 @@ __global__ void __launch_bounds__(kDriftThreads) teacher_drift_kernel(
 
     DriftAcc a;
     a.reset();
-    const int64_t pieces = (V + N - 1) / N;   // VEC requires V % N == 0
+    // VEC: `head` entries up to the first 16-byte boundary, whole pieces, `tail` entries
+    int head = 0, tail = 0;
     if (VEC) {
-      const uint4* src = reinterpret_cast<const uint4*>(urow);
+      const int shift = (int)((reinterpret_cast<uintptr_t>(urow) & 15) / sizeof(TIn));
+      head = shift ? N - shift : 0;
+      if (head > V) head = (int)V;
+      tail = (int)((V - head) % N);
+    }
+    const int64_t pieces = VEC ? (V - head) / N : V;
+    if (VEC) {
+      const int64_t edge = tid < head ? tid : (tid >= 32 && tid - 32 < tail) ? V - tail + (tid - 32) : -1;
+      if (edge >= 0) {
+        const float u[1] = {Elem<TIn>::load1(urow, edge)};
+        drift_piece<1>(u, uy, a);
+      }
+      const uint4* src = reinterpret_cast<const uint4*>(urow + head * sizeof(TIn));
       int64_t i = tid;
       for (; i + (kDriftUnroll - 1) * kDriftThreads < pieces; i += kDriftUnroll * kDriftThreads) {
         uint4 v[kDriftUnroll];
-        if (!ADWIN_CHK((i + (kDriftUnroll - 1) * kDriftThreads + 1) * N <= ld, status)) break;
+        if (!ADWIN_CHK(head + (i + (kDriftUnroll - 1) * kDriftThreads + 1) * N <= V, status)) break;
 #pragma unroll
         for (int k = 0; k < kDriftUnroll; ++k) v[k] = __ldcs(src + i + k * kDriftThreads);
 #pragma unroll
@@ -110,7 +123,7 @@ __global__ void __launch_bounds__(kDriftThreads) teacher_drift_kernel(
       }
       for (; i < pieces; i += kDriftThreads) {
         float u[Elem<TIn>::N];
-        if (!ADWIN_CHK((i + 1) * N <= ld, status)) break;
+        if (!ADWIN_CHK(head + (i + 1) * N <= V, status)) break;
         Elem<TIn>::unpack(__ldcs(src + i), u);
         drift_piece<Elem<TIn>::N>(u, uy, a);
       }

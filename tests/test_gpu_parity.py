@@ -437,3 +437,75 @@ def test_config4_full_size_probe_pass_on_sampled_rows():
     assert int(al.L_next.item()) == same["L_next"] and int(al.flags.item()) == same["flags"]
     rho = al.batch_stats[:, 0].cpu().numpy()
     assert (np.diff(rho[:-1]) >= -1e-12).all() and (rho <= 1 + 1e-12).all()
+
+
+@pytest.mark.parametrize("path", PATHS)
+@pytest.mark.parametrize("in_dt,g_dt", [(1, torch.float32), (1, torch.bfloat16), (2, torch.bfloat16),
+                                        (2, torch.float32), (2, None)])
+@pytest.mark.parametrize("V", [33, 1001, 11523, 23046, 50257])
+def test_rows_that_start_and_end_off_16_byte_boundaries(path, in_dt, g_dt, V):
+    """Packed rows of an odd length: every row has another offset from a 16-byte boundary, its first
+    and last pieces are shared with its neighbours (rows past the window must keep their sentinel),
+    and the pieces end just before, on and after a chunk or a cluster slice (11 520 and 23 040
+    bf16 entries are one and two full chunks).  Tokens in the partial pieces, and a row whose sampled
+    token is far below the maximum (redone with a running maximum)."""
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=7, V=V)
+    batch.window = torch.tensor([7, 4], dtype=torch.int32, device=DEV)
+    batch.tokens[0, 1], batch.tokens[0, 2], batch.tokens[1, 3] = 0, V - 1, V - 2
+    # (both policies: z - u is centred on the sampled token's difference, whose magnitude times 2^-24
+    # is the fp32 error of every centred difference -- 7e-6 for 120, most of the fp32 tolerance)
+    y = int(batch.tokens[0, 4])
+    batch.student[0, 4, y] = batch.student[0, 4].float().max() - 120.0
+    batch.teacher[0, 4, y] = batch.teacher[0, 4].float().max() - 120.0
+    flags = PATHS[path] | (api.RANGE_FULL if V == 1001 else 0)
+    for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
+        run_and_check(batch, grad_dtype=g_dt, grad_mode=mode, flags=flags)
+
+
+@pytest.mark.parametrize("path", PATHS)
+@pytest.mark.parametrize("V,ld,ld_grad", [(1001, 1008, 1008), (1001, 1008, 1024), (1001, 1003, 1003),
+                                          (1001, 1003, 1005), (12000, 12004, 12004)])
+def test_odd_rows_at_a_padded_stride(path, V, ld, ld_grad):
+    """Odd vocabularies in padded rows, whole and off the boundaries, the gradient at the same
+    stride and at another one; the padding is never written."""
+    B, T = 2, 5
+    base = synth.make_batch(2, device=DEV, B=B, T=T, V=ld)
+    s, t = base.student[..., :V], base.teacher[..., :V]
+    tok = torch.randint(0, V, (B, T), dtype=torch.int32, device=DEV)
+    win = torch.tensor([5, 3], dtype=torch.int32, device=DEV)
+    grad = torch.full((B, T, ld_grad), 3.0, dtype=torch.bfloat16, device=DEV)
+    got = api.adwin_opd_kl_fwd_bwd(s, t, tok, win, None, grad=grad[..., :V], flags=PATHS[path])
+    torch.cuda.synchronize()
+    api.raise_on_dev_status(got.dev_status)
+    ref = O.opd_kl_fwd_bwd(synth.bits_for_oracle(s.contiguous()), synth.bits_for_oracle(t.contiguous()),
+                           tok.cpu().numpy(), win.cpu().numpy(), None)
+    mask = P.processed_mask(win.cpu().numpy(), np.array([T, T]), T)
+    P.check_scalars(got, ref, 2e-3, mask)
+    g = grad.double().cpu().numpy()
+    P.check_grad_rows(g[..., :V][mask], ref["grad"][mask], 2e-3, store=2.0 ** -8)
+    assert (g[..., V:] == 3.0).all() and (g[~mask] == 3.0).all()
+
+
+def test_arrays_that_start_off_a_16_byte_boundary():
+    """Student, teacher and gradient as views that begin two bytes into a piece, and the teacher at
+    another offset than the student."""
+    B, T, V = 2, 3, 1000
+    base = synth.make_batch(2, device=DEV, B=B, T=T, V=V)
+    n = B * T * V
+    for off_s, off_t, off_g in ((1, 1, 1), (0, 1, 0), (3, 3, 0)):
+        def view(x, off):
+            buf = torch.zeros(n + 8, dtype=torch.bfloat16, device=DEV)
+            v = buf[off:off + n].view(B, T, V)
+            v.copy_(x)
+            return v
+        s, t = view(base.student, off_s), view(base.teacher, off_t)
+        batch = synth.Batch(s, t, base.tokens, torch.tensor([3, 2], dtype=torch.int32, device=DEV),
+                            base.rollout_len, 2)
+        run_and_check(batch, grad_dtype=None)
+        grad = view(torch.zeros_like(base.student), off_g)
+        got = api.adwin_opd_kl_fwd_bwd(s, t, batch.tokens, batch.window, batch.rollout_len, grad=grad)
+        torch.cuda.synchronize()
+        api.raise_on_dev_status(got.dev_status)
+        ref = P.oracle_batch(batch)
+        mask = P.processed_mask([3, 2], batch.rollout_len.cpu().numpy(), T)
+        P.check_grad_rows(grad.double().cpu().numpy()[mask], ref["grad"][mask], 2e-3, store=2.0 ** -8)
