@@ -68,9 +68,12 @@ enum {
   ADWIN_RANGE_FULL = 2,    /* per-token scalars for every t < R_b (delayed full-rollout probe,
                               Section 4.2); the gradient is still written only for t < E_b */
   ADWIN_FORCE_GENERIC = 4, /* use the row-per-CTA streaming kernel for every row */
-  ADWIN_FORCE_STAGED = 8   /* use the staged cluster kernel wherever the 16-byte layout allows,
+  ADWIN_FORCE_STAGED = 8,  /* use the staged cluster kernel wherever the 16-byte layout allows,
                               also for calls without gradient (which by default go to the
                               streaming kernel: one sweep, nothing to keep on chip) */
+  ADWIN_STATUS_INIT = 32   /* *dev_status starts at zero for this call instead of collecting bits
+                              over calls: saves a caller with a fresh status word its own clearing
+                              of it (a call that processes nothing, B = 0 or T = 0, leaves it alone) */
 };
 
 /* Flags returned by adwin_probe_align in *flags_out. */

@@ -18,7 +18,7 @@ LIB_PATH = _PKG / "libadwin_b200.so"
 OK = 0
 F32, BF16 = 0, 1
 GRAD_FULL_KL, GRAD_SAMPLED = 0, 1
-ZERO_TAIL, RANGE_FULL, FORCE_GENERIC, FORCE_STAGED = 1, 2, 4, 8
+ZERO_TAIL, RANGE_FULL, FORCE_GENERIC, FORCE_STAGED, STATUS_INIT = 1, 2, 4, 8, 32
 DEV_TOKEN_RANGE, DEV_NONFINITE, DEV_TIMEOUT, DEV_BOUNDS, DEV_WINDOW, DEV_WORKSPACE = 1, 2, 4, 8, 16, 32
 ALIGN_DEGENERATE, ALIGN_NONE_ADMISSIBLE = 1, 2
 DEFAULT_CANDIDATES = (64, 128, 256, 512, 1024, 2048)   # Section 5.1, Training Details
@@ -118,12 +118,16 @@ def lib():
     return _lib
 
 
+# A small call is bound by what happens on the host, so the helpers below avoid the objects that the
+# obvious forms create (a ctypes pointer per argument, a torch Stream per call: 12 of the 55 us of a
+# 2 x 64 x 4096 update); pointers and the stream handle travel as plain integers.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(device):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+    i = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
 
 
 def _dtype_code(dt):
@@ -143,6 +147,28 @@ def adwin_workspace_bytes(B, T, V, dtype=BF16, flags=0) -> int:
     return int(lib().adwin_workspace_bytes(B, T, V, dtype, flags))
 
 
+def _scalars(n, B, T, device):
+    """n [B,T] float32 tensors from one allocation."""
+    return torch.empty((n, B, T), dtype=torch.float32, device=device).unbind(0)
+
+
+def _row_stride(x):
+    """Uniform row stride of a [B,T,V] tensor whose last dim is contiguous."""
+    B, T, V = x.shape
+    sb, st, sv = x.stride()
+    assert sv == 1 or V == 1, "last dim must be contiguous"
+    ld = st if T > 1 else (sb if B > 1 else V)
+    assert B <= 1 or T <= 1 or sb == T * ld, "rows must sit at one uniform stride"
+    return ld
+
+
+def _new_status(device, n_rows, flags):
+    """A fresh status word and the flags that make the call clear it (nothing runs on no rows)."""
+    if n_rows == 0:
+        return torch.zeros(1, dtype=torch.int32, device=device), flags
+    return torch.empty(1, dtype=torch.int32, device=device), flags | STATUS_INIT
+
+
 def adwin_opd_kl_fwd_bwd(student, teacher, tokens, window, rollout_len=None, *, grad_scale=1.0,
                          grad_mode=GRAD_FULL_KL, flags=0, grad=None, grad_dtype=None,
                          want_gsq=True, want_lse=False, out=None, workspace=None, dev_status=None,
@@ -160,32 +186,23 @@ def adwin_opd_kl_fwd_bwd(student, teacher, tokens, window, rollout_len=None, *, 
     assert student.dim() == 3 and student.dtype == teacher.dtype
     B, T, V = student.shape
     dev = student.device
-
-    def row_stride(x):
-        assert x.stride(2) == 1 or V == 1, "last dim must be contiguous"
-        ld = x.stride(1) if T > 1 else (x.stride(0) if B > 1 else V)
-        assert B <= 1 or T <= 1 or x.stride(0) == T * ld, "rows must sit at one uniform stride"
-        return ld
-
-    ld = row_stride(student)
-    assert row_stride(teacher) == ld, "student and teacher must share the row stride"
+    ld = _row_stride(student)
+    assert _row_stride(teacher) == ld, "student and teacher must share the row stride"
     if grad is None and grad_dtype is not None:
         grad = torch.empty((B, T, V), dtype=grad_dtype, device=dev)
-    ld_grad = row_stride(grad) if grad is not None else 0
+    ld_grad = _row_stride(grad) if grad is not None else 0
     o = out if out is not None else SimpleNamespace()
-    f32 = dict(dtype=torch.float32, device=dev)
     if getattr(o, "kl", None) is None:
-        o.kl = torch.empty((B, T), **f32)
-        o.logratio = torch.empty((B, T), **f32)
-        o.gsq = torch.empty((B, T), **f32) if want_gsq else None
-        o.lse_s = torch.empty((B, T), **f32) if want_lse else None
-        o.lse_t = torch.empty((B, T), **f32) if want_lse else None
+        s = _scalars(2 + (1 if want_gsq else 0) + (2 if want_lse else 0), B, T, dev)
+        o.kl, o.logratio = s[0], s[1]
+        o.gsq = s[2] if want_gsq else None
+        o.lse_s, o.lse_t = (s[-2], s[-1]) if want_lse else (None, None)
     o.grad = grad
-    wsb = adwin_workspace_bytes(B, T, V, _dtype_code(student.dtype), flags)
     if workspace is None:
+        wsb = adwin_workspace_bytes(B, T, V, _dtype_code(student.dtype), flags)
         workspace = torch.empty(wsb, dtype=torch.uint8, device=dev)
     if dev_status is None:
-        dev_status = torch.zeros(1, dtype=torch.int32, device=dev)
+        dev_status, flags = _new_status(dev, B * T, flags)
     o.dev_status = dev_status
     o.workspace = workspace
     gdt = _dtype_code(grad.dtype) if grad is not None else 0
@@ -242,8 +259,8 @@ def adwin_window_reduce(kl, logratio, gsq, window, rollout_len=None):
     """Per-sequence and per-batch windowed sums: returns (seq_out [B,4], batch_out [4]) float64."""
     B, T = kl.shape
     dev = kl.device
-    seq = torch.empty((B, 4), dtype=torch.float64, device=dev)
-    batch = torch.empty(4, dtype=torch.float64, device=dev)
+    sums = torch.empty((B + 1, 4), dtype=torch.float64, device=dev)   # the batch's behind the sequences'
+    seq, batch = sums[:B], sums[B]
     _check(lib().adwin_window_reduce(_ptr(kl), _ptr(logratio), _ptr(gsq), _ptr(window),
                                      _ptr(rollout_len), B, T, _ptr(seq), _ptr(batch),
                                      _stream(dev)))
@@ -256,11 +273,12 @@ def adwin_probe_align(kl, logratio, gsq, window, rollout_len=None, candidates=No
     dev = kl.device
     K = 6 if candidates is None else int(candidates.numel())
     f64 = dict(dtype=torch.float64, device=dev)
+    # (the call writes L_next and flags whatever the batch)
     o = SimpleNamespace(
         seq_stats=torch.empty((B, K + 1, 4), **f64), seq_full=torch.empty((B, 3), **f64),
         batch_stats=torch.empty((K + 1, 5), **f64),
-        L_next=torch.zeros(1, dtype=torch.int32, device=dev),
-        flags=torch.zeros(1, dtype=torch.int32, device=dev))
+        L_next=torch.empty(1, dtype=torch.int32, device=dev),
+        flags=torch.empty(1, dtype=torch.int32, device=dev))
     _check(lib().adwin_probe_align(_ptr(kl), _ptr(logratio), _ptr(gsq), _ptr(window),
                                    _ptr(rollout_len), B, T, _ptr(candidates), K, float(rho_star),
                                    _ptr(o.seq_stats), _ptr(o.seq_full), _ptr(o.batch_stats),
@@ -405,20 +423,19 @@ def adwin_opd_kl_lmhead_fwd_bwd(hidden_student, w_student, hidden_teacher, w_tea
     for g in (grad_hidden, grad_w):
         if g is not None and not g.is_contiguous():
             raise ValueError("gradient tensors must be contiguous")
-    kl = torch.empty((B, T), dtype=torch.float32, device=dev)
-    logratio = torch.empty((B, T), dtype=torch.float32, device=dev)
-    gsq = torch.empty((B, T), dtype=torch.float32, device=dev) if want_gsq else None
-    lse_s = torch.empty((B, T), dtype=torch.float32, device=dev) if want_lse else None
-    lse_t = torch.empty((B, T), dtype=torch.float32, device=dev) if want_lse else None
+    s = _scalars(2 + (1 if want_gsq else 0) + (2 if want_lse else 0), B, T, dev)
+    kl, logratio = s[0], s[1]
+    gsq = s[2] if want_gsq else None
+    lse_s, lse_t = (s[-2], s[-1]) if want_lse else (None, None)
     with_grad = grad_hidden is not None or grad_w is not None
     need = adwin_lmhead_workspace_bytes(B, T, V, ds, dt, max_rows, flags, with_grad)
     if workspace is None:
         workspace = torch.empty(need + 1024, dtype=torch.uint8, device=dev)
     off = (-workspace.data_ptr()) % 1024
-    ws_ptr = ctypes.c_void_p(workspace.data_ptr() + off)
+    ws_ptr = workspace.data_ptr() + off
     ws_bytes = workspace.numel() - off
     if dev_status is None:
-        dev_status = torch.zeros(1, dtype=torch.int32, device=dev)
+        dev_status, flags = _new_status(dev, B * T, flags)
     gh_dtype = _dtype_code(grad_hidden.dtype) if grad_hidden is not None else F32
     if grad_w is not None and grad_w.dtype != torch.float32:
         raise TypeError("grad_w must be float32")

@@ -14,7 +14,7 @@ uint64_t handshake_wait_limit_ns() { return g_handshake_limit_ns.load(); }
 namespace {
 
 constexpr int kKnownFlags =
-    ADWIN_ZERO_TAIL | ADWIN_RANGE_FULL | ADWIN_FORCE_GENERIC | ADWIN_FORCE_STAGED;
+    ADWIN_ZERO_TAIL | ADWIN_RANGE_FULL | ADWIN_FORCE_GENERIC | ADWIN_FORCE_STAGED | ADWIN_STATUS_INIT;
 constexpr int64_t kMaxB = int64_t(1) << 24;
 constexpr int64_t kMaxT = int64_t(1) << 24;
 constexpr int64_t kMaxV = int64_t(1) << 28;
@@ -356,7 +356,7 @@ int adwin_opd_kl_lmhead_fwd_bwd(const void* hidden_student, const void* w_studen
                                 float* lse_teacher, int64_t max_rows, void* workspace,
                                 size_t workspace_bytes, int32_t* dev_status, void* cuda_stream) {
   if (grad_mode != ADWIN_GRAD_FULL_KL && grad_mode != ADWIN_GRAD_SAMPLED) return ADWIN_ERR_DTYPE;
-  if (flags & ~(ADWIN_RANGE_FULL | ADWIN_ZERO_TAIL)) return ADWIN_ERR_DTYPE;
+  if (flags & ~(ADWIN_RANGE_FULL | ADWIN_ZERO_TAIL | ADWIN_STATUS_INIT)) return ADWIN_ERR_DTYPE;
   if (grad_hidden && grad_hidden_dtype != ADWIN_F32 && grad_hidden_dtype != ADWIN_BF16)
     return ADWIN_ERR_DTYPE;
   if (B < 0 || T < 0 || B > 65536 || T > kMaxT || V < 1 || V > kMaxV || d_s < 1 || d_t < 1 ||

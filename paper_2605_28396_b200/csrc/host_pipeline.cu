@@ -123,6 +123,9 @@ int adwin_opd_kl_fwd_bwd_host(const void* student_host, const void* teacher_host
   std::memset(logratio_host, 0, (size_t)B * T * 4);
   if (gsq_host) std::memset(gsq_host, 0, (size_t)B * T * 4);
 
+  if ((flags & ADWIN_STATUS_INIT) && cudaMemsetAsync(dev_status, 0, 4, user) != cudaSuccess)
+    return ADWIN_ERR_CUDA;
+
   // The copy streams start after whatever the caller already enqueued.
   if (cudaEventRecord(pl->start, user) != cudaSuccess) return ADWIN_ERR_CUDA;
   cudaStreamWaitEvent(pl->in, pl->start, 0);
@@ -168,7 +171,7 @@ int adwin_opd_kl_fwd_bwd_host(const void* student_host, const void* teacher_host
           reinterpret_cast<const int32_t*>(base + L.off_tok),
           reinterpret_cast<const int32_t*>(base + L.off_win),
           reinterpret_cast<const int32_t*>(base + L.off_rl), grad_scale, grad_mode,
-          flags & ~ADWIN_ZERO_TAIL, has_grad ? base + L.off_grad : nullptr, gd, L.pitch_out,
+          flags & ~(ADWIN_ZERO_TAIL | ADWIN_STATUS_INIT), has_grad ? base + L.off_grad : nullptr, gd, L.pitch_out,
           reinterpret_cast<float*>(base + L.off_kl), reinterpret_cast<float*>(base + L.off_c),
           reinterpret_cast<float*>(base + L.off_q), nullptr, nullptr, base + L.off_ws,
           workspace_layout(1).total, dev_status, user);

@@ -1264,7 +1264,8 @@ template <typename TIn, typename TOut>
 cudaError_t max_clusters_for(const StagedPlan& plan, bool ragged, int sm_count, int& max_clusters) {
   StagedKernel kernel = staged_kernel<TIn, TOut>(plan, ragged);
   const int smem = plan_smem_bytes(plan);
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // (once per kernel and device, for the largest plan: launches of a cached plan do not repeat it)
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemOptin);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads);
@@ -1355,8 +1356,6 @@ cudaError_t launch_staged_t(const KlParams& p, int dtype, int grad_dtype, bool r
 
   StagedKernel kernel = staged_kernel<TIn, TOut>(plan, ragged);
   const int smem = plan_smem_bytes(plan);
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = (size_t)smem;

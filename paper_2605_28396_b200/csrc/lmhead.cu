@@ -845,9 +845,9 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
   const int64_t rows_cap = L.max_tiles * kBM;
   const int64_t ds = a.ds, dt = a.dt, V = a.V;
 
-  cudaError_t e = launch_rowmap(a.window, a.rollout_len, a.B, a.T, a.flags & ADWIN_RANGE_FULL,
-                                wb + L.off_rowmap, false, a.kl, a.logratio, a.gsq, a.lse_s, a.lse_t,
-                                a.status, s);
+  cudaError_t e = launch_rowmap(a.window, a.rollout_len, a.B, a.T,
+                                a.flags & (ADWIN_RANGE_FULL | ADWIN_STATUS_INIT), wb + L.off_rowmap,
+                                false, a.kl, a.logratio, a.gsq, a.lse_s, a.lse_t, a.status, s);
   if (e != cudaSuccess) return e;
   const WorkspaceLayout wl = workspace_layout(a.B);
   GatherParams gp;

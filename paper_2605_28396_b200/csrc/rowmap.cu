@@ -71,7 +71,12 @@ __global__ void __launch_bounds__(kMapThreads) rowmap_kernel(
       run += range[b];
     }
     if (tid == kMapThreads - 1) offsets[B] = part[tid];
-    if (any_bad) atomicOr(status, ADWIN_DEV_WINDOW);
+    // the first kernel of a call: later kernels OR their bits into what this leaves
+    const bool bad_lengths = __syncthreads_or(any_bad ? 1 : 0) != 0;
+    if (tid == 0) {
+      if (flags & ADWIN_STATUS_INIT) *status = bad_lengths ? ADWIN_DEV_WINDOW : 0;
+      else if (bad_lengths) atomicOr(status, ADWIN_DEV_WINDOW);
+    }
     if (offsets_win) {   // the same scan over the effective windows
       __syncthreads();
       part[tid] = sum_win;

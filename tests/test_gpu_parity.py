@@ -509,3 +509,43 @@ def test_arrays_that_start_off_a_16_byte_boundary():
         ref = P.oracle_batch(batch)
         mask = P.processed_mask([3, 2], batch.rollout_len.cpu().numpy(), T)
         P.check_grad_rows(grad.double().cpu().numpy()[mask], ref["grad"][mask], 2e-3, store=2.0 ** -8)
+
+
+@pytest.mark.parametrize("B", [1, 3, 8, 9, 64, 65])
+@pytest.mark.parametrize("K", [1, 6, 7, 8, 20])
+def test_reductions_over_batch_and_candidate_counts(B, K):
+    """One cluster up to 64 sequences, two launches beyond; eight prefix lengths per pass over a
+    sequence (the rollout, the candidates, the window): counts on both sides of each line."""
+    T = 700
+    rng = np.random.default_rng(100 * B + K)
+    kl, c, q = (rng.random((B, T), dtype=np.float32) for _ in range(3))
+    r = rng.integers(0, T + 1, B).astype(np.int32)
+    w = rng.integers(0, T + 1, B).astype(np.int32)
+    cand = rng.permutation(np.arange(1, K + 1) * (T // K)).astype(np.int32)
+    dev = [torch.from_numpy(x).to(DEV) for x in (kl, c, q, w, r, cand)]
+    seq, tot = api.adwin_window_reduce(*dev[:5])
+    al = api.adwin_probe_align(*dev)
+    torch.cuda.synchronize()
+    e = np.minimum(w, r)
+    ref = np.array([[x[b, :e[b]].astype(np.float64).sum() for x in (kl, c, q)] + [e[b]] for b in range(B)])
+    np.testing.assert_allclose(seq.cpu().numpy(), ref, rtol=1e-12)
+    np.testing.assert_allclose(tot.cpu().numpy(), ref.sum(axis=0), rtol=1e-12)
+    want = O.probe_align(kl, c, q, w, r, cand, math.sqrt(2) / 2)
+    np.testing.assert_allclose(al.seq_stats.cpu().numpy(), want["seq_stats"], rtol=1e-12, atol=1e-12)
+    np.testing.assert_allclose(al.seq_full.cpu().numpy(), want["seq_full"], rtol=1e-12, atol=1e-12)
+    np.testing.assert_allclose(al.batch_stats.cpu().numpy(), want["batch_stats"], rtol=1e-12)
+    assert int(al.L_next.item()) == want["L_next"] and int(al.flags.item()) == want["flags"]
+
+
+def test_status_word_collects_or_starts_fresh():
+    batch = synth.make_batch(2, device=DEV, B=2, T=6, V=4096)
+    batch.tokens[0, 1] = -1
+    args = (batch.student, batch.teacher, batch.tokens, batch.window, batch.rollout_len)
+    for flags, start, want in ((0, 1 << 20, (1 << 20) | api.DEV_TOKEN_RANGE),
+                               (api.STATUS_INIT, 1 << 20, api.DEV_TOKEN_RANGE)):
+        status = torch.full((1,), start, dtype=torch.int32, device=DEV)
+        api.adwin_opd_kl_fwd_bwd(*args, flags=flags | api.RANGE_FULL, dev_status=status)
+        assert int(status.item()) == want
+    batch.rollout_len[1] = 7                                     # longer than T
+    o = api.adwin_opd_kl_fwd_bwd(*args, flags=api.RANGE_FULL)
+    assert int(o.dev_status.item()) == api.DEV_TOKEN_RANGE | api.DEV_WINDOW
