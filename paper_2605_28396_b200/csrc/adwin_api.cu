@@ -264,7 +264,8 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
     KlParams pw = p;          // window rows: the compact list built from the effective windows
     pw.offsets = reinterpret_cast<const int64_t*>(wbase + wl.off_offsets_win);
     pw.range = p.ewin;
-    const cudaError_t e = launch_kl_staged(pw, dtype, gd, !whole, sms, s);
+    cudaError_t e = launch_kl_rows(pw, dtype, gd, !whole, sms, s);
+    if (e == cudaErrorNotSupported) e = launch_kl_staged(pw, dtype, gd, !whole, sms, s);
     if (e == cudaSuccess) {
       KlParams pr = p;        // the rest of every rollout, without gradient
       pr.grad = nullptr;
@@ -279,6 +280,12 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
   // staged cluster kernel.  A call without gradient is a single read of every row, which the
   // row-per-CTA streaming kernel does faster (90 % against 74 % of the copy bandwidth, measured).
   const bool want_staged = (flags & ADWIN_FORCE_STAGED) || grad_student != nullptr;
+  if (staged_ok && grad_student &&
+      !(flags & (ADWIN_FORCE_GENERIC | ADWIN_FORCE_STAGED | ADWIN_RANGE_FULL))) {
+    const cudaError_t e = launch_kl_rows(p, dtype, gd, !whole, sms, s);
+    if (e == cudaSuccess) return ADWIN_OK;
+    if (e != cudaErrorNotSupported) return ADWIN_ERR_CUDA;
+  }
   if (staged_ok && want_staged && !(flags & ADWIN_FORCE_GENERIC)) {
     const cudaError_t e = launch_kl_staged(p, dtype, gd, !whole, sms, s);
     if (e == cudaSuccess) return ADWIN_OK;

@@ -41,6 +41,11 @@ cudaError_t launch_kl_generic(const KlParams& p, int dtype, int grad_dtype, bool
 cudaError_t launch_kl_staged(const KlParams& p, int dtype, int grad_dtype, bool ragged, int sm_count,
                              cudaStream_t s);
 
+// Row kernel for calls whose processed rows all get a gradient.  Returns cudaErrorNotSupported when
+// the row does not fit its plans.
+cudaError_t launch_kl_rows(const KlParams& p, int dtype, int grad_dtype, bool ragged, int sm_count,
+                           cudaStream_t s);
+
 cudaError_t launch_window_reduce(const float* kl, const float* logratio, const float* gsq,
                                  const int32_t* window, const int32_t* rollout_len, int64_t B,
                                  int64_t T, double* seq_out, double* batch_out, cudaStream_t s);

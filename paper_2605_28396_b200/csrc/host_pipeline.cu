@@ -60,7 +60,7 @@ StageLayout stage_layout(int64_t rows, int64_t V, int dtype, int grad_dtype, boo
   L.off_tok = o; o = up256(o + (size_t)rows * 4);
   L.off_win = o; o = up256(o + 4);
   L.off_rl = o;  o = up256(o + 4);
-  L.off_ws = o;  o = up256(o + workspace_layout(1).total);
+  L.off_ws = o;  o = up256(o + workspace_layout(1).total_ext);
   L.off_grad = o; o = up256(o + (has_grad ? (size_t)rows * L.pitch_out * gs : 0));
   L.off_kl = o;  o = up256(o + (size_t)rows * 4);
   L.off_c = o;   o = up256(o + (size_t)rows * 4);
@@ -174,7 +174,7 @@ int adwin_opd_kl_fwd_bwd_host(const void* student_host, const void* teacher_host
           flags & ~(ADWIN_ZERO_TAIL | ADWIN_STATUS_INIT), has_grad ? base + L.off_grad : nullptr, gd, L.pitch_out,
           reinterpret_cast<float*>(base + L.off_kl), reinterpret_cast<float*>(base + L.off_c),
           reinterpret_cast<float*>(base + L.off_q), nullptr, nullptr, base + L.off_ws,
-          workspace_layout(1).total, dev_status, user);
+          workspace_layout(1).total_ext, dev_status, user);
       if (rc != ADWIN_OK) return rc;
       cudaEventRecord(pl->comp_done[s], user);
 

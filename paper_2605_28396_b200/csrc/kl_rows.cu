@@ -1,0 +1,600 @@
+// Row kernel for calls with gradient: a row (or a cluster's slice of it) is read from HBM once, kept on
+// chip between the two sweeps, several CTAs per SM.
+//
+// Two to eight small CTAs share an SM, each on a row of its own, so that one CTA's exchange and
+// row scalars overlap the other CTAs' streaming.  There are no roles and no hand-shakes: every
+// thread loads its own 16-byte pieces with plain coalesced loads, folds them into its sums and
+// puts them where only it will look for them again -- shared memory, or the otherwise idle tensor
+// memory (tcgen05.st / tcgen05.ld) -- so between the sweeps there is one barrier for the row's sums
+// and none for the data.  One more warp looks ahead: it fetches the next row's metadata, and while
+// the others are in the second sweep of a row it has the next row brought into L2
+// (cp.async.bulk.prefetch.L2), so that HBM stays busy during both sweeps and the loads of the first
+// sweep come from L2.
+//
+// Exponentials are taken against a reference that the whole row shares (the logit of the sampled
+// token), so partial sums add without rescaling.  If the sums overflow it (a sampled token more than
+// ~69 nats below the row maximum) the row is summed once more, from its on-chip copy, against
+// running maxima.  Rows too long for one CTA are split over a cluster; the warps' records then go
+// to every CTA of the cluster and the barrier is the cluster's.
+#include <mutex>
+#include <type_traits>
+#include <vector>
+#ifdef ADWIN_ROWS_TUNE
+#include <cstdio>
+#include <cstdlib>
+#endif
+
+#include "adwin_common.cuh"
+#include "adwin_internal.h"
+#include "kl_pairs.cuh"
+
+namespace adwin {
+namespace {
+
+constexpr int kRowsThreads = 352;     // threads of a CTA that hold pieces, at most
+#ifndef ROWS_U
+#define ROWS_U 2
+#endif
+constexpr int kU = ROWS_U;            // piece pairs in flight per thread
+constexpr int kRowsMaxCl = 4;
+constexpr int kRowsMaxRec = kRowsMaxCl * kRowsThreads / 32;
+constexpr float kSumLimit = 1.2676506e30f;   // 2^100: beyond it the shared reference is unsafe
+constexpr int kMetaDepth = 4;
+
+struct RowsPlan {
+  int cl;             // CTAs per row
+  int nt;             // threads per CTA that hold pieces (one more warp looks ahead)
+  int ctas;           // CTAs per SM
+  int per_rank;       // 16-byte pieces of a slice (per array)
+  int steps;          // piece pairs per thread, rounded up to a multiple of kU
+  int tm_steps;       // of these, in tensor memory (a multiple of kU; the first ones)
+  int tm_cols;        // tensor-memory columns per CTA (0: none)
+  int num_clusters;
+};
+
+struct __align__(16) RowsMeta {
+  int64_t r;
+  int y;
+  float w;            // caller-supplied row coefficient (0 when there is none)
+  float zy, uy;
+};
+
+struct __align__(16) RowsCtrl {
+  float rec[2][kRowsMaxRec][4];    // per row parity, one record per (rank, warp): S, A, St, q
+  float safe[kRowsMaxRec][8];      // records of the running-maximum pass
+  RowsMeta meta[kMetaDepth];
+  uint32_t tmem_base;
+};
+constexpr int kRowsCtrlBytes = (int)((sizeof(RowsCtrl) + 127) / 128 * 128);
+
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// NT: threads that hold pieces, a template constant so that the strides between a thread's pieces are
+// offsets in the instructions.  A group of kU steps in which every thread has a piece takes the path
+// without tests (FULL below).
+template <typename TIn, typename TOut, int NT, bool TM, bool RAG>
+__global__ void __launch_bounds__(NT + 32, 65536 / 80 / (NT + 32))
+kl_rows_kernel(const KlParams p, const RowsPlan plan) {
+  constexpr int N = Elem<TIn>::N;
+  constexpr int NP = Pairs<TIn>::NP;
+  constexpr int nt = NT, nw = NT / 32;
+  constexpr uint32_t array = NT * 16u;
+  extern __shared__ __align__(128) char smem[];
+  RowsCtrl& ctrl = *reinterpret_cast<RowsCtrl*>(smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cl = plan.cl;
+  char* stash = smem + kRowsCtrlBytes + tid * 16;   // [step][array][thread] 16 bytes
+  const uint32_t rank = cl > 1 ? cluster_rank() : 0u;
+  const int64_t cluster_id = blockIdx.x / cl;
+  const int piece0 = (int)rank * plan.per_rank;
+  const int64_t total_rows = p.offsets[p.B];
+  const int64_t my_rows =
+      cluster_id < total_rows ? (total_rows - cluster_id + plan.num_clusters - 1) / plan.num_clusters : 0;
+
+  if (TM && warp == nw) tm_alloc(smem_u32(&ctrl.tmem_base), (uint32_t)plan.tm_cols);
+
+  // where row r lies in this CTA's slice (base pointers are 16-byte aligned)
+  auto span_of = [&](int64_t r) -> RowSpan {
+    RowSpan a = {0, 0, -1, -1, N};
+    if (RAG) a.shift = (int)((r * p.ld) & (N - 1));
+    const int64_t end = a.shift + p.V, total = (end + N - 1) / N, left = total - piece0;
+    a.pieces = (int)(left < 0 ? 0 : (left > plan.per_rank ? plan.per_rank : left));
+    if (RAG) {
+      a.first = (a.shift > 0 && piece0 == 0) ? 0 : -1;
+      a.last_n = (int)(end - (total - 1) * N);
+      a.last = (a.last_n < N && left > 0 && left <= plan.per_rank) ? (int)left - 1 : -1;
+    }
+    return a;
+  };
+
+  if (TM) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (cl > 1) cluster_sync_all();   // peers run before anything is stored into them
+  __syncthreads();
+  if (TM) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const int64_t iters = my_rows > 0 ? my_rows + 1 : 0;   // + one exchange for the last norm
+  const int nrec = cl * nw;
+  auto row_barrier = [&]() {
+    if (cl == 1) __syncthreads();
+    else cluster_sync_all();
+  };
+  // fixed-order sum of field f of the row's records; every lane of every warp gets the same bits
+  auto record_sum = [&](int par, int f) {
+    float s = 0.f;
+    for (int j = lane; j < nrec; j += 32) s += ctrl.rec[par][j][f];
+    return lane_sum(s);
+  };
+
+  if (warp == nw) {
+    // ------------------------------------------------------------------ look-ahead warp
+    RowCursor cur;
+    cur.init(p);
+    bool wg_unused;
+    int64_t r = 0;     // row i, then row i+1
+    auto fetch = [&](int64_t i) {   // metadata of row i into its slot
+      r = cur.locate(p, cluster_id + i * plan.num_clusters, wg_unused);
+      if (lane == 0) {
+        RowsMeta& m = ctrl.meta[i % kMetaDepth];
+        const int y = p.tokens[r];
+        m.r = r;
+        m.y = y;
+        fetch_logits_at<TIn>(p, r, y, m.zy, m.uy);
+        m.w = p.row_coef ? p.row_coef[r] : 0.f;
+      }
+    };
+    if (my_rows > 0) fetch(0);
+    __syncthreads();
+    for (int64_t i = 0; i < iters; ++i) {
+      const bool more = i + 1 < my_rows;
+      if (more) fetch(i + 1);
+      row_barrier();
+      if (i == my_rows) break;
+      if (more && lane == 0) {
+        const RowSpan sn = span_of(r);
+        const size_t off = ((size_t)r * p.ld - sn.shift + (size_t)piece0 * N) * sizeof(TIn);
+        if (sn.pieces > 0) {
+          prefetch_l2(static_cast<const char*>(p.student) + off, (uint32_t)sn.pieces * 16u);
+          prefetch_l2(static_cast<const char*>(p.teacher) + off, (uint32_t)sn.pieces * 16u);
+        }
+      }
+      __syncwarp();
+      // the decision that the other warps take as well
+      const float S = record_sum((int)(i & 1), 0), St = record_sum((int)(i & 1), 2);
+      if (!(S < kSumLimit) || !(St < kSumLimit)) row_barrier();
+    }
+  } else {
+    __syncthreads();   // the first row's metadata
+    // this thread's tensor-memory columns: its lane, the columns split between the warps of a lane group
+    const uint32_t tm_lane = TM ? ctrl.tmem_base + ((uint32_t)((warp & 3) * 32) << 16) +
+                                      (uint32_t)((warp >> 2) * plan.tm_steps * 8)
+                                : 0u;
+    const bool full_mode = (p.mode == ADWIN_GRAD_FULL_KL);
+    float q_prev = 0.f;       // this warp's share of the previous row's squared norm
+    int64_t r_prev = 0;
+    for (int64_t i = 0; i < iters; ++i) {
+      const bool real = i < my_rows;
+      const int par = (int)(i & 1);
+      const RowsMeta& m = ctrl.meta[real ? i % kMetaDepth : 0];
+      const float ref_s = m.zy * kLog2e, ref_t = m.uy * kLog2e;
+      RowSpan span = {0, 0, -1, -1, N};
+      Acc2 a;
+      a.reset();
+      if (real) {
+        // ------------------------------------------------------------ sweep 1
+        span = span_of(m.r);
+        const size_t off = ((size_t)m.r * p.ld - span.shift + (size_t)piece0 * N) * sizeof(TIn);
+        const uint4* zp = reinterpret_cast<const uint4*>(static_cast<const char*>(p.student) + off) + tid;
+        const uint4* up = reinterpret_cast<const uint4*>(static_cast<const char*>(p.teacher) + off) + tid;
+        const f2_t nrefs = splat2(-ref_s), nreft = splat2(-ref_t);
+        char* st = stash;
+        int lp0 = tid;     // this thread's piece in the group's first step
+        auto group = [&](auto full, int k0) {
+          constexpr bool FULL = decltype(full)::value;
+          uint4 z[kU], u[kU];
+#pragma unroll
+          for (int h = 0; h < kU; ++h) {
+            if ((FULL || lp0 + h * nt < span.pieces) &&
+                ADWIN_CHK(((int64_t)piece0 + lp0 + h * nt + (RAG ? 0 : 1)) * N <= p.V + span.shift, p.status)) {
+              z[h] = __ldcs(zp + h * nt);
+              u[h] = __ldcs(up + h * nt);
+            }
+          }
+          if (RAG) {
+#pragma unroll
+            for (int h = 0; h < kU; ++h) {
+              const int lp = lp0 + h * nt;
+              if (lp == span.first || lp == span.last)
+                mask_piece<TIn>(z[h], u[h], span.e0(lp), lp == span.last ? span.last_n : N);
+            }
+          }
+          if (TM && k0 < plan.tm_steps) {   // (every lane takes part)
+#pragma unroll
+            for (int h = 0; h < kU; ++h) tm_store8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
+          } else {
+#pragma unroll
+            for (int h = 0; h < kU; ++h) {
+              if (FULL || lp0 + h * nt < span.pieces) {
+                *reinterpret_cast<uint4*>(st + 2 * h * array) = z[h];
+                *reinterpret_cast<uint4*>(st + (2 * h + 1) * array) = u[h];
+              }
+            }
+            st += 2 * kU * array;
+          }
+#pragma unroll
+          for (int h = 0; h < kU; ++h) {
+            if (FULL || lp0 + h * nt < span.pieces) {
+              f2_t Z[NP], U[NP];
+              Pairs<TIn>::make(z[h], Z);
+              Pairs<TIn>::make(u[h], U);
+              acc_grad<NP, 0>(Z, U, nrefs, nreft, a);
+            }
+          }
+          zp += kU * nt;
+          up += kU * nt;
+          lp0 += kU * nt;
+        };
+        int k0 = 0;
+        for (; (k0 + kU) * nt <= span.pieces; k0 += kU) group(std::true_type{}, k0);
+        for (; k0 < plan.steps; k0 += kU) group(std::false_type{}, k0);
+        if (TM) tm_wait_st();
+      }
+
+      // -------------------------------------------------------------- exchange
+      {
+        const float v0 = lane_sum(hsum2(a.S)), v1 = lane_sum(hsum2(a.A)), v2 = lane_sum(hsum2(a.St));
+        float* rec = ctrl.rec[par][rank * nw + warp];
+        if (cl == 1) {
+          if (lane == 0) *reinterpret_cast<float4*>(rec) = make_float4(v0, v1, v2, q_prev);
+        } else if (lane < cl) {
+          remote_store4(map_to_rank(smem_u32(rec), (uint32_t)lane), v0, v1, v2, q_prev);
+        }
+      }
+      row_barrier();
+      RowTotals t;
+      t.M2s = ref_s;
+      t.M2t = ref_t;
+      t.S = record_sum(par, 0);
+      t.A = record_sum(par, 1);
+      t.St = record_sum(par, 2);
+      t.B0 = t.B1 = t.B2 = 0.f;
+      if (warp == 0) {
+        const float qtot = record_sum(par, 3);
+        if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = qtot;
+      }
+      if (!real) break;
+
+      // -------------------------------------------------------------- overflow: running maxima
+      // (the totals are identical in every warp of the cluster, so this branch is uniform)
+      if (!(t.S < kSumLimit) || !(t.St < kSumLimit)) {
+        RowAcc ra;
+        ra.reset();
+        const char* st = stash;
+        for (int k = 0; k < plan.steps; ++k) {
+          uint4 zv, uv;
+          if (TM && k < plan.tm_steps) {
+            tm_load8(tm_lane + (uint32_t)(k * 8), zv, uv);
+            tm_wait_ld();
+          } else {
+            zv = *reinterpret_cast<const uint4*>(st);
+            uv = *reinterpret_cast<const uint4*>(st + array);
+            st += 2 * array;
+          }
+          if (tid + k * nt < span.pieces) {
+            float z[N], u[N];
+            Elem<TIn>::unpack(zv, z);
+            Elem<TIn>::unpack(uv, u);
+            acc_piece<N, false>(z, u, 0.f, ra);
+          }
+        }
+        const float wms = warp_max(ra.m2s), wmt = warp_max(ra.m2t);
+        const float fs = (ra.m2s == -INFINITY) ? 0.f : ex2f(ra.m2s - wms);
+        const float ft = (ra.m2t == -INFINITY) ? 0.f : ex2f(ra.m2t - wmt);
+        const float w1 = lane_sum(ra.S * fs), w2 = lane_sum(ra.A * fs), w3 = lane_sum(ra.St * ft);
+        float* rec = ctrl.safe[rank * nw + warp];
+        if (lane < cl) {
+          const uint32_t dst = cl == 1 ? smem_u32(rec) : map_to_rank(smem_u32(rec), (uint32_t)lane);
+          remote_store4(dst, wms, wmt, w1, w2);
+          remote_store4(dst + 16, w3, 0.f, 0.f, 0.f);
+        }
+        row_barrier();
+        float ms = -INFINITY, mt = -INFINITY;
+        for (int j = lane; j < nrec; j += 32) {
+          ms = fmaxf(ms, ctrl.safe[j][0]);
+          mt = fmaxf(mt, ctrl.safe[j][1]);
+        }
+        t.M2s = warp_max(ms);
+        t.M2t = warp_max(mt);
+        float s[3] = {0.f, 0.f, 0.f};
+        for (int j = lane; j < nrec; j += 32) {
+          const float* x = ctrl.safe[j];
+          const float gs = (x[0] == -INFINITY) ? 0.f : ex2f(x[0] - t.M2s);
+          const float gt = (x[1] == -INFINITY) ? 0.f : ex2f(x[1] - t.M2t);
+          s[0] += x[2] * gs;
+          s[1] += x[3] * gs;
+          s[2] += x[4] * gt;
+        }
+        t.S = lane_sum(s[0]);
+        t.A = lane_sum(s[1]);
+        t.St = lane_sum(s[2]);
+      }
+
+      // -------------------------------------------------------------- row scalars
+      const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
+      const RowScalars rs = finish_row(t, m.zy, m.uy, y_valid, 0.f, p.alpha, p.mode,
+                                       p.row_coef ? &m.w : nullptr);
+      if (rank == 0 && tid == 0) {
+        p.kl[m.r] = rs.kl;
+        p.logratio[m.r] = rs.c;
+        if (p.lse_s) p.lse_s[m.r] = rs.lse_s;
+        if (p.lse_t) p.lse_t[m.r] = rs.lse_t;
+        int bits = 0;
+        if (!y_valid) bits |= ADWIN_DEV_TOKEN_RANGE;
+        if (rs.nonfinite) bits |= ADWIN_DEV_NONFINITE;
+        if (bits) atomicOr(p.status, bits);
+      }
+
+      // -------------------------------------------------------------- sweep 2
+      const f2_t L2 = splat2(kLog2e), NEG1 = splat2(-1.f);
+      const f2_t nM2s = splat2(-t.M2s), coef2 = splat2(rs.coef);
+      // bf16 logits: g = e * (coef*delta - coef*c0) saves one operation per pair; its rounding
+      // (relative to coef*delta, not to the difference) is far inside that dtype's tolerance.
+      const f2_t nc0 = splat2(sizeof(TIn) == 2 ? -rs.coef * rs.c0 : -rs.c0);
+      const int64_t yat = (int64_t)m.y + span.shift;                     // counted from piece 0
+      const int ypiece = y_valid ? (int)(yat / N - piece0) : -1;         // slice-relative
+      char* gp = static_cast<char*>(p.grad) +
+                 ((size_t)m.r * p.ld_grad - span.shift + (size_t)(piece0 + tid) * N) * sizeof(TOut);
+      f2_t Q = 0ull;
+      const char* st = stash;
+      int lp0 = tid;
+      auto group = [&](auto full, int k0) {
+        constexpr bool FULL = decltype(full)::value;
+        uint4 z[kU], u[kU];
+        if (TM && k0 < plan.tm_steps) {
+#pragma unroll
+          for (int h = 0; h < kU; ++h) tm_load8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
+          tm_wait_ld();
+        } else {
+#pragma unroll
+          for (int h = 0; h < kU; ++h) {
+            if (FULL || lp0 + h * nt < span.pieces) {
+              z[h] = *reinterpret_cast<const uint4*>(st + 2 * h * array);
+              u[h] = *reinterpret_cast<const uint4*>(st + (2 * h + 1) * array);
+            }
+          }
+          st += 2 * kU * array;
+        }
+#pragma unroll
+        for (int h = 0; h < kU; ++h) {
+          const int lp = lp0 + h * nt;
+          if (FULL || lp < span.pieces) {
+            f2_t Z[NP], U[NP], G[NP];
+            Pairs<TIn>::make(z[h], Z);
+            Pairs<TIn>::make(u[h], U);
+#pragma unroll
+            for (int e = 0; e < NP; ++e) {
+              const f2_t E = ex2_2(fma2(Z[e], L2, nM2s));
+              if (full_mode) {
+                if (sizeof(TIn) == 2) G[e] = mul2(E, fma2(fma2(U[e], NEG1, Z[e]), coef2, nc0));
+                else G[e] = mul2(E, mul2(add2(fma2(U[e], NEG1, Z[e]), nc0), coef2));
+              } else {
+                G[e] = mul2(E, coef2);
+              }
+            }
+            if (!full_mode && lp == ypiece) {
+              const int ye = (int)(yat % N);
+#pragma unroll
+              for (int e = 0; e < NP; ++e) {
+                float lo, hi;
+                upk2(G[e], lo, hi);
+                if (ye == 2 * e) lo = rs.gy;
+                if (ye == 2 * e + 1) hi = rs.gy;
+                G[e] = pk2(lo, hi);
+              }
+            }
+#pragma unroll
+            for (int e = 0; e < NP; ++e) Q = fma2(G[e], G[e], Q);
+            if (ADWIN_CHK(((int64_t)piece0 + lp + (RAG ? 0 : 1)) * N <= p.V + span.shift && m.r < p.B * p.T, p.status)) {
+              char* dst = gp + (size_t)h * nt * N * sizeof(TOut);
+              if (RAG && (lp == span.first || lp == span.last)) {   // the row's own entries only
+                const int e0 = span.e0(lp), e1 = lp == span.last ? span.last_n : N;
+#pragma unroll
+                for (int e = 0; e < NP; ++e) {
+                  float lo, hi;
+                  upk2(G[e], lo, hi);
+                  if (2 * e >= e0 && 2 * e < e1) Elem<TOut>::store1(dst, 2 * e, lo);
+                  if (2 * e + 1 >= e0 && 2 * e + 1 < e1) Elem<TOut>::store1(dst, 2 * e + 1, hi);
+                }
+              } else {
+                store_pairs<TOut, NP>(dst, G);
+              }
+            }
+          }
+        }
+        gp += (size_t)kU * nt * N * sizeof(TOut);
+        lp0 += kU * nt;
+      };
+      int k0 = 0;
+      for (; (k0 + kU) * nt <= span.pieces; k0 += kU) group(std::true_type{}, k0);
+      for (; k0 < plan.steps; k0 += kU) group(std::false_type{}, k0);
+      q_prev = lane_sum(hsum2(Q));
+      r_prev = m.r;
+    }
+  }
+  if (TM) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (cl > 1) cluster_sync_all();   // no CTA leaves while a peer may still store into it
+  __syncthreads();
+  if (TM && warp == nw) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tm_dealloc(ctrl.tmem_base, (uint32_t)plan.tm_cols);
+  }
+}
+
+// ---------------------------------------------------------------------------- host side
+constexpr int kSmemPerSm = 233472, kSmemReserved = 1024;   // bytes per SM, and taken by every CTA
+
+struct RowsShape {
+  int ctas, nt, tm_cols, cl;
+};
+// From many small CTAs to two large ones, then clusters; the first that holds the row is taken: the
+// most CTAs per SM, because their number is what hides one row's exchange behind the others'
+// streaming.  Tensor memory is shared out in powers of two.  Measured over 2.4 GB of logits and
+// gradient (367 us at the copy rate; staged kernel / two sweeps over memory / this kernel):
+//   bf16  V =   4 096  2488 /  993 / 622 us  {8, 64}       fp32  V =   4 096  1247 / 599 / 439 us  {5, 128}
+//             16 384   993 /  625 / 555     {3, 224}              16 384   600 / 679 / 433      {2, 352}
+//             32 000   726 /  822 / 513     {2, 352}              32 000   510 / 733 / 444      {3, 224} x 2
+//             50 264   638 /  980 / 529     {2, 352}              50 264   597 / 772 / 478      {2, 352} x 2
+//            100 000   656 / 1019 / 547     {2, 352} x 2         100 000   547 / 781 / 485      {2, 352} x 4
+//            151 936   573 / 1012 / 586 (x 3), 595 (x 4)
+// bf16 rows are bound by arithmetic (28 issue slots per entry), fp32 rows by memory.  Clusters beyond
+// two CTAs leave SMs over, which costs bf16 rows more than the overlap gives: those go to the staged
+// kernel.
+constexpr RowsShape kShapes[] = {{8, 64, 0, 1}, {5, 128, 0, 1}, {3, 224, 128, 1}, {2, 352, 256, 1},
+                                 {3, 224, 128, 2}, {2, 352, 256, 2}, {2, 352, 256, 4}};
+constexpr int kMaxClBf16 = 2;
+
+bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
+  plan.cl = sh.cl;
+  plan.nt = sh.nt;
+  plan.ctas = sh.ctas;
+  plan.per_rank = (int)((pieces + sh.cl - 1) / sh.cl);
+  const int need = (plan.per_rank + sh.nt - 1) / sh.nt;
+  plan.steps = (need + kU - 1) / kU * kU;
+  const int smem = kSmemPerSm / sh.ctas - kSmemReserved - kRowsCtrlBytes;
+  const int sm_steps = smem / (32 * sh.nt) / kU * kU;
+  // a lane group's columns are shared by its warps (every fourth); a piece pair takes 8 columns
+  const int tm_most = sh.tm_cols ? sh.tm_cols / ((sh.nt + 127) / 128) / 8 / kU * kU : 0;
+  plan.tm_steps = plan.steps < tm_most ? plan.steps : tm_most;
+  plan.tm_cols = plan.tm_steps ? sh.tm_cols : 0;
+  return plan.steps - plan.tm_steps <= sm_steps;
+}
+
+int rows_smem(const RowsPlan& plan) {
+  return kRowsCtrlBytes + (plan.steps - plan.tm_steps) * 32 * plan.nt;
+}
+
+bool rows_plan(int64_t pieces, bool bf16, RowsPlan& plan) {
+  if (pieces < 1 || pieces > (int64_t)1 << 24) return false;
+#ifdef ADWIN_ROWS_TUNE
+  if (getenv("ROWS_SHAPE")) {
+    RowsShape sh;
+    sscanf(getenv("ROWS_SHAPE"), "%d,%d,%d,%d", &sh.ctas, &sh.nt, &sh.tm_cols, &sh.cl);
+    return shape_plan(sh, pieces, plan);
+  }
+#endif
+  for (const RowsShape& sh : kShapes)
+    if ((!bf16 || sh.cl <= kMaxClBf16) && shape_plan(sh, pieces, plan)) return true;
+  return false;
+}
+
+typedef void (*RowsKernel)(KlParams, RowsPlan);
+template <typename TIn, typename TOut, int NT>
+RowsKernel rows_kernel_nt(bool tm, bool ragged) {
+#ifdef ADWIN_ROWS_TUNE
+  if (ragged || sizeof(TIn) != sizeof(TOut)) return nullptr;
+  return tm ? kl_rows_kernel<TIn, TOut, NT, true, false> : kl_rows_kernel<TIn, TOut, NT, false, false>;
+#else
+  if (tm) return ragged ? kl_rows_kernel<TIn, TOut, NT, true, true> : kl_rows_kernel<TIn, TOut, NT, true, false>;
+  return ragged ? kl_rows_kernel<TIn, TOut, NT, false, true> : kl_rows_kernel<TIn, TOut, NT, false, false>;
+#endif
+}
+template <typename TIn, typename TOut>
+RowsKernel rows_kernel(int nt, bool tm, bool ragged) {
+  switch (nt) {
+    case 64: return rows_kernel_nt<TIn, TOut, 64>(tm, ragged);
+    case 128: return rows_kernel_nt<TIn, TOut, 128>(tm, ragged);
+    case 224: return rows_kernel_nt<TIn, TOut, 224>(tm, ragged);
+    case 352: return rows_kernel_nt<TIn, TOut, 352>(tm, ragged);
+    default: return nullptr;
+  }
+}
+
+// Clusters of `cl` CTAs that the GPU holds at a time (some SMs of a GPC are left over when `cl` does
+// not divide their number).  The occupancy query counts one CTA per SM for kernels that allocate
+// tensor memory, so it is asked about the same kernel without.
+cudaError_t resident_clusters(RowsKernel like, const RowsPlan& plan, int smem, int sm_count, int& n) {
+  struct Key {
+    int dev, nt, ctas, cl, n;
+  };
+  static std::mutex mu;
+  static std::vector<Key> seen;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  for (const Key& k : seen)
+    if (k.dev == dev && k.nt == plan.nt && k.ctas == plan.ctas && k.cl == plan.cl) {
+      n = k.n;
+      return cudaSuccess;
+    }
+  e = cudaFuncSetAttribute(like, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(plan.cl * sm_count * plan.ctas);
+  cfg.blockDim = dim3(plan.nt + 32);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = plan.cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaOccupancyMaxActiveClusters(&n, like, &cfg);
+  if (e != cudaSuccess) return e;
+  if (n < 1) return cudaErrorNotSupported;
+  seen.push_back({dev, plan.nt, plan.ctas, plan.cl, n});
+  return cudaSuccess;
+}
+
+template <typename TIn, typename TOut>
+cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStream_t s) {
+  constexpr int N = Elem<TIn>::N;
+  RowsPlan plan = {};
+  if (!rows_plan(ragged ? (p.V + 2 * N - 2) / N : p.V / N, sizeof(TIn) == 2, plan))
+    return cudaErrorNotSupported;
+  const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, plan.tm_cols > 0, ragged);
+  if (!kernel) return cudaErrorNotSupported;
+  const int smem = rows_smem(plan);
+  const int most = kSmemPerSm / plan.ctas - kSmemReserved;
+  plan.num_clusters = plan.ctas * sm_count;
+  cudaError_t e;
+  if (plan.cl > 1) {
+    e = resident_clusters(rows_kernel<TIn, TOut>(plan.nt, false, ragged), plan, most, sm_count,
+                          plan.num_clusters);
+    if (e != cudaSuccess) return e;
+  }
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int64_t rows = p.B * p.T;
+  if (plan.num_clusters > rows) plan.num_clusters = (int)rows;
+#ifdef ADWIN_ROWS_TUNE
+  if (getenv("ROWS_DBG")) fprintf(stderr, "rows cl %d nt %d ctas %d per %d steps %d tm %d cols %d clusters %d smem %d\n", plan.cl, plan.nt, plan.ctas, plan.per_rank, plan.steps, plan.tm_steps, plan.tm_cols, plan.num_clusters, smem);
+#endif
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(plan.cl * plan.num_clusters);
+  cfg.blockDim = dim3(plan.nt + 32);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = plan.cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = plan.cl > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, p, plan);
+}
+
+}  // namespace
+
+cudaError_t launch_kl_rows(const KlParams& p, int dtype, int grad_dtype, bool ragged, int sm_count,
+                           cudaStream_t s) {
+  if (dtype == ADWIN_F32)
+    return grad_dtype == ADWIN_F32 ? launch_rows_t<float, float>(p, ragged, sm_count, s)
+                                   : launch_rows_t<float, __nv_bfloat16>(p, ragged, sm_count, s);
+  return grad_dtype == ADWIN_F32 ? launch_rows_t<__nv_bfloat16, float>(p, ragged, sm_count, s)
+                                 : launch_rows_t<__nv_bfloat16, __nv_bfloat16>(p, ragged, sm_count, s);
+}
+
+}  // namespace adwin

@@ -40,6 +40,7 @@
 
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
+#include "kl_pairs.cuh"
 
 namespace adwin {
 
@@ -54,6 +55,8 @@ constexpr int kChunkMax = kGT * kP;  // 16-byte pieces per chunk (per array), at
 constexpr int kMaxChunks = 256;
 constexpr int kProducerWarp = kNW;   // lane 0 feeds the stream ring, lane 1 refills the resident slots
 constexpr int kThreads = kNT + 32;
+constexpr int kTmCols = 512;
+constexpr int kTmColsPerThread = 128;   // four consumer warps share the 512 columns of a lane group
 constexpr int kMaxRes = 16;
 constexpr int kMaxRing = 16;
 constexpr int kMaxCL = 4;
@@ -110,9 +113,6 @@ struct __align__(16) Ctrl {
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 
 // ---------------------------------------------------------------------------- PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -157,16 +157,6 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t local_addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void remote_store4(uint32_t addr, float a, float b, float c, float d) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b),
-               "f"(c), "f"(d)
-               : "memory");
-}
 __device__ __forceinline__ void remote_store_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -202,46 +192,11 @@ __device__ __forceinline__ void bulk_load_hint(uint32_t dst, const void* src, ui
       "l"(src), "r"(bytes), "r"(bar), "l"(pol)
       : "memory");
 }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                   : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 __device__ __forceinline__ uint64_t global_timer() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-
-// Tensor memory as a scratchpad (TM mode): 512 columns x 128 lanes x 32 bit = 256 KB per SM that a
-// kernel without MMAs leaves idle.  A consumer thread parks the 16-byte pieces it has read in
-// sweep 1 in its own lane (lane = 32*(warp%4) + laneid, the only lanes a warp may touch) and gets
-// them back in sweep 2, so the streamed chunks are neither kept in shared memory nor fetched again.
-constexpr int kTmCols = 512;
-constexpr int kTmColsPerThread = 128;      // four consumer warps share the 512 columns of a lane group
-__device__ __forceinline__ void tm_alloc(uint32_t dst_smem) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(kTmCols) : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tm_dealloc(uint32_t taddr) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(kTmCols) : "memory");
-}
-__device__ __forceinline__ void tm_store8(uint32_t taddr, const uint4& a, const uint4& b) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-               "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
-}
-__device__ __forceinline__ void tm_load8(uint32_t taddr, uint4& a, uint4& b) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-               : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tm_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Bounded wait of one thread.  Returns immediately (false) once the CTA has given up.
 template <bool CLUSTER>
@@ -275,165 +230,6 @@ __device__ __forceinline__ bool bounded_wait(uint32_t bar, uint32_t parity, vola
   return __all_sync(0xffffffffu, bounded_wait_lane<CLUSTER>(bar, parity, abort, limit_ns)) != 0;
 }
 
-// Walks the compact list of processed rows.  The prefix sums of the current sequence are cached
-// in registers, so locating a row touches global memory only when it crosses into a new sequence.
-struct RowCursor {
-  int64_t b, lo, hi;   // sequence, offsets[b], offsets[b+1]
-  int32_t ew;          // effective window of sequence b
-  __device__ __forceinline__ void init(const KlParams& p) {
-    b = 0;
-    lo = 0;
-    hi = p.B > 0 ? p.offsets[1] : 0;
-    ew = p.B > 0 ? p.ewin[0] : 0;
-  }
-  // Global row of processed-row ordinal n (ordinals must not decrease) and whether its gradient
-  // is written.
-  __device__ __forceinline__ int64_t locate(const KlParams& p, int64_t n, bool& wg) {
-    while (n >= hi && b + 1 < p.B) {
-      ++b;
-      lo = hi;
-      hi = p.offsets[b + 1];
-      ew = p.ewin[b];
-    }
-    const int64_t t = n - lo;
-    wg = (p.grad != nullptr) && (t < ew);
-    return b * p.T + t;
-  }
-  __device__ __forceinline__ void fetch_row(const KlParams& p, int64_t ordinal, bool in_range,
-                                            int64_t& r, int& y, bool& wg) {
-    if (in_range) {
-      r = locate(p, ordinal, wg);
-      y = p.tokens[r];
-    }
-  }
-};
-
-// ---------------------------------------------------------------------------- packed fp32 pairs
-// sm_100 issues add/mul/fma on two fp32 lanes held in a 64-bit register pair in one slot
-// (add.f32x2 / mul.f32x2 / fma.f32x2).  The sweeps are issue- and MUFU-bound, so all element-wise
-// arithmetic is done on pairs; only ex2 (MUFU) is per lane.
-typedef unsigned long long f2_t;
-
-__device__ __forceinline__ f2_t pk2(float lo, float hi) {
-  f2_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(f2_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f2_t fma2(f2_t a, f2_t b, f2_t c) {
-  f2_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f2_t add2(f2_t a, f2_t b) {
-  f2_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2_t mul2(f2_t a, f2_t b) {
-  f2_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2_t ex2_2(f2_t x) {
-  float a, b;
-  upk2(x, a, b);
-  return pk2(ex2f(a), ex2f(b));
-}
-__device__ __forceinline__ f2_t splat2(float v) { return pk2(v, v); }
-__device__ __forceinline__ f2_t sub2(f2_t a, f2_t b) {
-  f2_t d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-// 2^x of a pair on the FMA pipe, to relieve the MUFU unit that bounds sweep 1.  x is clamped to
-// [-120, 105] (below that the term is nil against a sum >= 1; at the upper end the result exceeds
-// the limit that sends the row to the safe path), rounded to the nearest integer n by adding
-// 1.5*2^23, 2^(x-n) comes from a degree-4 polynomial on [-1/2, 1/2] (relative error < 2.7e-6,
-// mean 4e-8) and n is added to the exponent field.  A NaN comes out as a finite number: callers
-// keep a second, unclamped use of the input so that it still poisons the row.
-__device__ __forceinline__ f2_t ex2_poly2(f2_t x) {
-  float a, b;
-  upk2(x, a, b);
-  a = fminf(fmaxf(a, -120.f), 105.f);
-  b = fminf(fmaxf(b, -120.f), 105.f);
-  const f2_t xc = pk2(a, b);
-  const f2_t MG = splat2(12582912.f);
-  const f2_t t = add2(xc, MG);
-  const f2_t f = sub2(xc, sub2(t, MG));
-  f2_t q = fma2(splat2(9.570101276e-03f), f, splat2(5.591785908e-02f));
-  q = fma2(q, f, splat2(2.402474433e-01f));
-  q = fma2(q, f, splat2(6.931217909e-01f));
-  q = fma2(q, f, splat2(9.999992847e-01f));
-  float tl, th, ql, qh;
-  upk2(t, tl, th);
-  upk2(q, ql, qh);
-  const uint32_t rl = __float_as_uint(ql) + (__float_as_uint(tl) << 23);
-  const uint32_t rh = __float_as_uint(qh) + (__float_as_uint(th) << 23);
-  return pk2(__uint_as_float(rl), __uint_as_float(rh));
-}
-__device__ __forceinline__ float hsum2(f2_t v) {
-  float a, b;
-  upk2(v, a, b);
-  return a + b;
-}
-
-// A 16-byte piece as NP pairs of consecutive vocabulary entries.
-template <typename T>
-struct Pairs;
-template <>
-struct Pairs<__nv_bfloat16> {
-  static constexpr int NP = 4;
-  __device__ static __forceinline__ void make(const uint4& v, f2_t (&o)[4]) {
-    o[0] = pk2(bf16lo(v.x), bf16hi(v.x));
-    o[1] = pk2(bf16lo(v.y), bf16hi(v.y));
-    o[2] = pk2(bf16lo(v.z), bf16hi(v.z));
-    o[3] = pk2(bf16lo(v.w), bf16hi(v.w));
-  }
-};
-template <>
-struct Pairs<float> {
-  static constexpr int NP = 2;
-  __device__ static __forceinline__ void make(const uint4& v, f2_t (&o)[2]) {
-    o[0] = pk2(__uint_as_float(v.x), __uint_as_float(v.y));
-    o[1] = pk2(__uint_as_float(v.z), __uint_as_float(v.w));
-  }
-};
-
-// Per-thread accumulators of one row slice, as pairs (even / odd entries).
-struct Acc2 {
-  f2_t S, A, St, B0, B1, B2;
-  __device__ __forceinline__ void reset() {
-    S = A = St = B0 = B1 = B2 = 0ull;   // the bit pattern of {0.f, 0.f}
-  }
-};
-
-// Teacher pairs per 16-byte piece whose exponential is evaluated on the FMA pipe: one of the four
-// pairs of a bf16 piece (more than that and the FMA/ALU pipes become the limit, measured); none
-// for fp32 logits, whose sweep has half the exponentials per byte and a 1e-5 tolerance.
-template <typename T>
-__host__ __device__ constexpr int kPolyPairs() { return sizeof(T) == 2 ? 1 : 0; }
-
-// Sweep 1, rows whose gradient is written: e = 2^(z log2e - ref_s), delta = z - u uncentred.
-// The first PT teacher pairs of a piece take their exponential from the polynomial (the teacher
-// sum only enters through its logarithm, and delta still sees the unclamped logits).
-template <int NP, int PT>
-__device__ __forceinline__ void acc_grad(const f2_t (&Z)[NP], const f2_t (&U)[NP], f2_t nrefs,
-                                         f2_t nreft, Acc2& a) {
-  const f2_t L2 = splat2(kLog2e), NEG1 = splat2(-1.f);
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    const f2_t E = ex2_2(fma2(Z[i], L2, nrefs));
-    const f2_t D = fma2(U[i], NEG1, Z[i]);
-    a.S = add2(a.S, E);
-    a.A = fma2(E, D, a.A);
-    const f2_t xt = fma2(U[i], L2, nreft);
-    a.St = add2(a.St, (i < PT) ? ex2_poly2(xt) : ex2_2(xt));
-  }
-}
-
 // Sweep 1, rows whose gradient is not written (probe rows): additionally the moments
 // sum e^2 {1, delta, delta^2} of the single-sweep squared gradient norm, delta centred on dref.
 template <int NP>
@@ -455,87 +251,12 @@ __device__ __forceinline__ void acc_probe(const f2_t (&Z)[NP], const f2_t (&U)[N
   }
 }
 
-template <typename TOut, int NP>
-__device__ __forceinline__ void store_pairs(char* dst, const f2_t (&G)[NP]) {
-  float g[2 * NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) upk2(G[i], g[2 * i], g[2 * i + 1]);
-  if (sizeof(TOut) == 4) {
-    float4* o = reinterpret_cast<float4*>(dst);
-#pragma unroll
-    for (int j = 0; j < NP / 2; ++j)
-      __stcs(o + j, make_float4(g[4 * j], g[4 * j + 1], g[4 * j + 2], g[4 * j + 3]));
-  } else if (NP == 4) {
-    uint4 o;
-    o.x = pack_bf16x2(g[0], g[1]);
-    o.y = pack_bf16x2(g[2], g[3]);
-    o.z = pack_bf16x2(g[4], g[5]);
-    o.w = pack_bf16x2(g[6], g[7]);
-    __stcs(reinterpret_cast<uint4*>(dst), o);
-  } else {
-    uint2 o;
-    o.x = pack_bf16x2(g[0], g[1]);
-    o.y = pack_bf16x2(g[2], g[3]);
-    __stcs(reinterpret_cast<uint2*>(dst), o);
-  }
-}
-
-// The two logits at the sampled token (at element 0 when the token is out of range).
-template <typename TIn>
-__device__ __forceinline__ void fetch_logits_at(const KlParams& p, int64_t r, int y, float& zy,
-                                                float& uy) {
-  const bool ok = (y >= 0) && ((int64_t)y < p.V);
-  const int64_t yi = ok ? y : 0;
-  zy = Elem<TIn>::load1(static_cast<const char*>(p.student) + (size_t)r * p.ld * sizeof(TIn), yi);
-  uy = Elem<TIn>::load1(static_cast<const char*>(p.teacher) + (size_t)r * p.ld * sizeof(TIn), yi);
-}
-
 // Chunk j of a slice is resident iff the running count floor(j*nres/nch) steps at j: the nres
 // resident chunks are spread evenly along the slice.  Returns the resident slot or -1.
 __device__ __forceinline__ int resident_slot(int j, int nres, int nch) {
   const int a = (j * nres) / nch, b = ((j + 1) * nres) / nch;
   return b > a ? a : -1;
 }
-
-// Fixed-order sum over the lanes of a warp; every lane returns the same bits.
-__device__ __forceinline__ float lane_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Rows that do not start or end on a 16-byte boundary (RAG): the pieces are those of the aligned
-// span that covers the row, `shift` entries of the first piece belong to the row before (or to
-// padding) and so may the end of the last one.  Reading them is harmless -- a 16-byte granule that
-// holds an entry of the row is always readable -- and their values are replaced by one whose
-// exponential is zero on both sides.
-template <typename TIn>
-__device__ __forceinline__ void mask_piece(uint4& z, uint4& u, int e0, int e1) {
-  constexpr int N = Elem<TIn>::N;
-  uint32_t zw[4] = {z.x, z.y, z.z, z.w}, uw[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-  for (int e = 0; e < N; ++e) {
-    if (e >= e0 && e < e1) continue;
-    if (sizeof(TIn) == 4) {
-      zw[e % 4] = uw[e % 4] = 0xf149f2cau;             // -1e30f
-    } else {
-      const uint32_t keep = (e & 1) ? 0x0000ffffu : 0xffff0000u, put = (e & 1) ? 0xf1490000u : 0xf149u;
-      zw[(e / 2) % 4] = (zw[(e / 2) % 4] & keep) | put;  // bf16 -1e30
-      uw[(e / 2) % 4] = (uw[(e / 2) % 4] & keep) | put;
-    }
-  }
-  z = make_uint4(zw[0], zw[1], zw[2], zw[3]);
-  u = make_uint4(uw[0], uw[1], uw[2], uw[3]);
-}
-
-// Where a row lies in this CTA's slice.
-struct RowSpan {
-  int pieces;        // pieces of the slice
-  int shift;         // entries of piece 0 that precede the row
-  int first, last;   // slice-relative index of the row's first / last piece if it is partial, else -1
-  int last_n;        // entries of the row in its last piece (counted from the piece's start)
-  __device__ __forceinline__ int e0(int piece) const { return piece == first ? shift : 0; }
-};
 
 template <typename TIn, typename TOut, bool TM, bool RAG>
 __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, StagedPlan plan) {
@@ -589,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
     ctrl.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (TM && warp == kProducerWarp) tm_alloc(smem_u32(&ctrl.tmem_base));   // the whole warp
+  if (TM && warp == kProducerWarp) tm_alloc(smem_u32(&ctrl.tmem_base), kTmCols);   // the whole warp
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   cluster_sync_all();  // peers' barriers exist before any remote arrive
@@ -1176,7 +897,7 @@ __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, Stag
     __syncthreads();   // every consumer of this CTA is done with tensor memory
     if (warp == kProducerWarp) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      tm_dealloc(ctrl.tmem_base);
+      tm_dealloc(ctrl.tmem_base, kTmCols);
     }
   }
 }

@@ -549,3 +549,24 @@ def test_status_word_collects_or_starts_fresh():
     batch.rollout_len[1] = 7                                     # longer than T
     o = api.adwin_opd_kl_fwd_bwd(*args, flags=api.RANGE_FULL)
     assert int(o.dev_status.item()) == api.DEV_TOKEN_RANGE | api.DEV_WINDOW
+
+
+@pytest.mark.parametrize("in_dt,V", [(2, 3584), (2, 3592), (2, 17920), (2, 36000), (2, 58880), (2, 70001),
+                                     (2, 117760), (1, 1792), (1, 33003), (1, 58900), (1, 118001)])
+def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
+    """The row kernel's shapes: rows of a few hundred pieces, rows that fill a CTA's shared memory and
+    run over into tensor memory, rows split over two and four CTAs; piece counts that fill every
+    group of steps and one more piece; a sampled token in every slice, and rows whose token is far
+    below the maximum (summed again from the copy on chip)."""
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=6, V=V)
+    batch.window = torch.tensor([6, 3], dtype=torch.int32, device=DEV)
+    for t, y in enumerate((0, V // 4 + 1, V // 2 + 1, 3 * V // 4 + 1, V - 1)):
+        batch.tokens[0, t] = y
+    for b, t in ((0, 1), (0, 4), (1, 2)):     # (both policies, see the test of odd rows)
+        y = int(batch.tokens[b, t])
+        batch.student[b, t, y] = batch.student[b, t].float().max() - 100.0
+        batch.teacher[b, t, y] = batch.teacher[b, t].float().max() - 100.0
+    g_dt = torch.float32 if in_dt == 1 else torch.bfloat16
+    for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
+        run_and_check(batch, grad_dtype=g_dt, grad_mode=mode)
+    run_and_check(batch, grad_dtype=g_dt, flags=api.RANGE_FULL)
