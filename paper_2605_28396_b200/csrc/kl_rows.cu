@@ -5,17 +5,18 @@
 // row scalars overlap the other CTAs' streaming.  There are no roles and no hand-shakes: every
 // thread loads its own 16-byte pieces with plain coalesced loads, folds them into its sums and
 // puts them where only it will look for them again -- shared memory, or the otherwise idle tensor
-// memory (tcgen05.st / tcgen05.ld) -- so between the sweeps there is one barrier for the row's sums
-// and none for the data.  One more warp looks ahead: it fetches the next row's metadata, and while
-// the others are in the second sweep of a row it has the next row brought into L2
-// (cp.async.bulk.prefetch.L2), so that HBM stays busy during both sweeps and the loads of the first
-// sweep come from L2.
+// memory (tcgen05.st / tcgen05.ld) -- so between the sweeps the threads only exchange sums.  One more
+// warp does what is done once per row: it adds up the threads' sums, derives the row's scalars and
+// hands them back (the others would otherwise each spend ~300 issue slots on it, as much as a
+// tenth of a row of 32 000 entries), fetches the next row's metadata, and while the others are
+// in the second sweep it has the next row brought into L2 (cp.async.bulk.prefetch.L2), so that HBM
+// stays busy during both sweeps and the loads of the first sweep come from L2.
 //
 // Exponentials are taken against a reference that the whole row shares (the logit of the sampled
 // token), so partial sums add without rescaling.  If the sums overflow it (a sampled token more than
 // ~69 nats below the row maximum) the row is summed once more, from its on-chip copy, against
-// running maxima.  Rows too long for one CTA are split over a cluster; the warps' records then go
-// to every CTA of the cluster and the barrier is the cluster's.
+// running maxima.  Rows too long for one CTA are split over a cluster; the CTAs' sums then go to every
+// CTA of the cluster.
 #include <mutex>
 #include <type_traits>
 #include <vector>
@@ -37,7 +38,6 @@ constexpr int kRowsThreads = 352;     // threads of a CTA that hold pieces, at m
 #endif
 constexpr int kU = ROWS_U;            // piece pairs in flight per thread
 constexpr int kRowsMaxCl = 4;
-constexpr int kRowsMaxRec = kRowsMaxCl * kRowsThreads / 32;
 constexpr float kSumLimit = 1.2676506e30f;   // 2^100: beyond it the shared reference is unsafe
 constexpr int kMetaDepth = 4;
 
@@ -59,13 +59,33 @@ struct __align__(16) RowsMeta {
   float zy, uy;
 };
 
+// What sweep 2 needs of a row.
+struct __align__(16) RowsScalars {
+  float m2s, coef, c0, gy;
+  int again;          // the sums overflowed: sum the row once more against running maxima
+};
+
 struct __align__(16) RowsCtrl {
-  float rec[2][kRowsMaxRec][4];    // per row parity, one record per (rank, warp): S, A, St, q
-  float safe[kRowsMaxRec][8];      // records of the running-maximum pass
+  float safe[kRowsThreads / 32][8];    // the warps' records of the running-maximum pass
+  float xrec[2][kRowsMaxCl][4];    // per row parity, one record per CTA of the cluster
+  float xsafe[kRowsMaxCl][8];
+  RowsScalars out;
   RowsMeta meta[kMetaDepth];
   uint32_t tmem_base;
 };
-constexpr int kRowsCtrlBytes = (int)((sizeof(RowsCtrl) + 127) / 128 * 128);
+// Shared memory: RowsCtrl, a float4 record per thread (its S, A, St of the row and q of the row
+// before), then the threads' pieces.
+constexpr int kRowsRec = (int)((sizeof(RowsCtrl) + 127) / 128 * 128);
+__host__ __device__ constexpr int rows_ctrl_bytes(int nt) { return kRowsRec + nt * 16; }
+
+// Named barriers of a CTA: the threads with pieces report on kPosted and wait on kReady.
+constexpr int kPosted = 1, kReady = 2;
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+  asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -79,13 +99,14 @@ __global__ void __launch_bounds__(NT + 32, 65536 / 80 / (NT + 32))
 kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   constexpr int N = Elem<TIn>::N;
   constexpr int NP = Pairs<TIn>::NP;
-  constexpr int nt = NT, nw = NT / 32;
+  constexpr int nt = NT, nw = NT / 32, all = NT + 32;
   constexpr uint32_t array = NT * 16u;
   extern __shared__ __align__(128) char smem[];
   RowsCtrl& ctrl = *reinterpret_cast<RowsCtrl*>(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cl = plan.cl;
-  char* stash = smem + kRowsCtrlBytes + tid * 16;   // [step][array][thread] 16 bytes
+  float4* rec = reinterpret_cast<float4*>(smem + kRowsRec);
+  char* stash = smem + rows_ctrl_bytes(NT) + tid * 16;   // [step][array][thread] 16 bytes
   const uint32_t rank = cl > 1 ? cluster_rank() : 0u;
   const int64_t cluster_id = blockIdx.x / cl;
   const int piece0 = (int)rank * plan.per_rank;
@@ -114,20 +135,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   __syncthreads();
   if (TM) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const int64_t iters = my_rows > 0 ? my_rows + 1 : 0;   // + one exchange for the last norm
-  const int nrec = cl * nw;
-  auto row_barrier = [&]() {
-    if (cl == 1) __syncthreads();
-    else cluster_sync_all();
-  };
-  // fixed-order sum of field f of the row's records; every lane of every warp gets the same bits
-  auto record_sum = [&](int par, int f) {
-    float s = 0.f;
-    for (int j = lane; j < nrec; j += 32) s += ctrl.rec[par][j][f];
-    return lane_sum(s);
-  };
-
   if (warp == nw) {
-    // ------------------------------------------------------------------ look-ahead warp
+    // ------------------------------------------------------------------ the row's own warp
     RowCursor cur;
     cur.init(p);
     bool wg_unused;
@@ -145,23 +154,111 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     };
     if (my_rows > 0) fetch(0);
     __syncthreads();
+    int64_t r_prev = 0;
     for (int64_t i = 0; i < iters; ++i) {
-      const bool more = i + 1 < my_rows;
+      const bool real = i < my_rows, more = i + 1 < my_rows;
+      const int par = (int)(i & 1);
+      const int64_t ri = r;
       if (more) fetch(i + 1);
-      row_barrier();
-      if (i == my_rows) break;
-      if (more && lane == 0) {
-        const RowSpan sn = span_of(r);
-        const size_t off = ((size_t)r * p.ld - sn.shift + (size_t)piece0 * N) * sizeof(TIn);
-        if (sn.pieces > 0) {
-          prefetch_l2(static_cast<const char*>(p.student) + off, (uint32_t)sn.pieces * 16u);
-          prefetch_l2(static_cast<const char*>(p.teacher) + off, (uint32_t)sn.pieces * 16u);
+      named_sync(kPosted, all);
+      // fixed-order sums over the threads, then over the CTAs
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int w = 0; w < nw; ++w) {
+        const float4 x = rec[w * 32 + lane];
+        v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+      }
+#pragma unroll
+      for (int f = 0; f < 4; ++f) v[f] = lane_sum(v[f]);
+      if (cl > 1) {
+        if (lane < cl)
+          remote_store4(map_to_rank(smem_u32(ctrl.xrec[par][rank]), (uint32_t)lane), v[0], v[1], v[2], v[3]);
+        cluster_sync_all();
+        v[0] = v[1] = v[2] = v[3] = 0.f;
+        for (int j = 0; j < cl; ++j) {
+          const float4 x = *reinterpret_cast<const float4*>(ctrl.xrec[par][j]);
+          v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+        }
+      }
+      if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = v[3];
+      if (!real) break;
+      const RowsMeta& m = ctrl.meta[i % kMetaDepth];
+      RowTotals t;
+      t.M2s = m.zy * kLog2e;
+      t.M2t = m.uy * kLog2e;
+      t.S = v[0];
+      t.A = v[1];
+      t.St = v[2];
+      t.B0 = t.B1 = t.B2 = 0.f;
+      // (the totals are identical in every CTA of the cluster, so this branch is too)
+      if (!(t.S < kSumLimit) || !(t.St < kSumLimit)) {
+        if (lane == 0) ctrl.out.again = 1;
+        named_sync(kReady, all);
+        named_sync(kPosted, all);
+        float x[5] = {-INFINITY, -INFINITY, 0.f, 0.f, 0.f};   // m2s, m2t, S, A, St of the CTA
+        if (lane < nw) {
+#pragma unroll
+          for (int f = 0; f < 5; ++f) x[f] = ctrl.safe[lane][f];
+        }
+        auto combine = [&]() {
+          t.M2s = warp_max(x[0]);
+          t.M2t = warp_max(x[1]);
+          const float gs = (x[0] == -INFINITY) ? 0.f : ex2f(x[0] - t.M2s);
+          const float gt = (x[1] == -INFINITY) ? 0.f : ex2f(x[1] - t.M2t);
+          t.S = lane_sum(x[2] * gs);
+          t.A = lane_sum(x[3] * gs);
+          t.St = lane_sum(x[4] * gt);
+        };
+        combine();
+        if (cl > 1) {
+          if (lane < cl) {
+            const uint32_t dst = map_to_rank(smem_u32(ctrl.xsafe[rank]), (uint32_t)lane);
+            remote_store4(dst, t.M2s, t.M2t, t.S, t.A);
+            remote_store4(dst + 16, t.St, 0.f, 0.f, 0.f);
+          }
+          cluster_sync_all();
+          x[0] = x[1] = -INFINITY;
+          x[2] = x[3] = x[4] = 0.f;
+          if (lane < cl) {
+#pragma unroll
+            for (int f = 0; f < 5; ++f) x[f] = ctrl.xsafe[lane][f];
+          }
+          combine();
+        }
+      }
+      const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
+      const RowScalars rs = finish_row(t, m.zy, m.uy, y_valid, 0.f, p.alpha, p.mode,
+                                       p.row_coef ? &m.w : nullptr);
+      if (lane == 0) {
+        ctrl.out.m2s = t.M2s;
+        ctrl.out.coef = rs.coef;
+        ctrl.out.c0 = rs.c0;
+        ctrl.out.gy = rs.gy;
+        ctrl.out.again = 0;
+      }
+      named_sync(kReady, all);
+      if (lane == 0) {
+        if (more) {
+          const RowSpan sn = span_of(r);
+          const size_t off = ((size_t)r * p.ld - sn.shift + (size_t)piece0 * N) * sizeof(TIn);
+          if (sn.pieces > 0) {
+            prefetch_l2(static_cast<const char*>(p.student) + off, (uint32_t)sn.pieces * 16u);
+            prefetch_l2(static_cast<const char*>(p.teacher) + off, (uint32_t)sn.pieces * 16u);
+          }
+        }
+        if (rank == 0) {
+          p.kl[ri] = rs.kl;
+          p.logratio[ri] = rs.c;
+          if (p.lse_s) p.lse_s[ri] = rs.lse_s;
+          if (p.lse_t) p.lse_t[ri] = rs.lse_t;
+          int bits = 0;
+          if (!y_valid) bits |= ADWIN_DEV_TOKEN_RANGE;
+          if (rs.nonfinite) bits |= ADWIN_DEV_NONFINITE;
+          if (bits) atomicOr(p.status, bits);
         }
       }
       __syncwarp();
-      // the decision that the other warps take as well
-      const float S = record_sum((int)(i & 1), 0), St = record_sum((int)(i & 1), 2);
-      if (!(S < kSumLimit) || !(St < kSumLimit)) row_barrier();
+      r_prev = ri;
     }
   } else {
     __syncthreads();   // the first row's metadata
@@ -170,13 +267,10 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
                                       (uint32_t)((warp >> 2) * plan.tm_steps * 8)
                                 : 0u;
     const bool full_mode = (p.mode == ADWIN_GRAD_FULL_KL);
-    float q_prev = 0.f;       // this warp's share of the previous row's squared norm
-    int64_t r_prev = 0;
+    float q_prev = 0.f;       // this thread's share of the previous row's squared norm
     for (int64_t i = 0; i < iters; ++i) {
       const bool real = i < my_rows;
-      const int par = (int)(i & 1);
       const RowsMeta& m = ctrl.meta[real ? i % kMetaDepth : 0];
-      const float ref_s = m.zy * kLog2e, ref_t = m.uy * kLog2e;
       RowSpan span = {0, 0, -1, -1, N};
       Acc2 a;
       a.reset();
@@ -186,7 +280,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         const size_t off = ((size_t)m.r * p.ld - span.shift + (size_t)piece0 * N) * sizeof(TIn);
         const uint4* zp = reinterpret_cast<const uint4*>(static_cast<const char*>(p.student) + off) + tid;
         const uint4* up = reinterpret_cast<const uint4*>(static_cast<const char*>(p.teacher) + off) + tid;
-        const f2_t nrefs = splat2(-ref_s), nreft = splat2(-ref_t);
+        const f2_t nrefs = splat2(-m.zy * kLog2e), nreft = splat2(-m.uy * kLog2e);
         char* st = stash;
         int lp0 = tid;     // this thread's piece in the group's first step
         auto group = [&](auto full, int k0) {
@@ -241,32 +335,14 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       }
 
       // -------------------------------------------------------------- exchange
-      {
-        const float v0 = lane_sum(hsum2(a.S)), v1 = lane_sum(hsum2(a.A)), v2 = lane_sum(hsum2(a.St));
-        float* rec = ctrl.rec[par][rank * nw + warp];
-        if (cl == 1) {
-          if (lane == 0) *reinterpret_cast<float4*>(rec) = make_float4(v0, v1, v2, q_prev);
-        } else if (lane < cl) {
-          remote_store4(map_to_rank(smem_u32(rec), (uint32_t)lane), v0, v1, v2, q_prev);
-        }
-      }
-      row_barrier();
-      RowTotals t;
-      t.M2s = ref_s;
-      t.M2t = ref_t;
-      t.S = record_sum(par, 0);
-      t.A = record_sum(par, 1);
-      t.St = record_sum(par, 2);
-      t.B0 = t.B1 = t.B2 = 0.f;
-      if (warp == 0) {
-        const float qtot = record_sum(par, 3);
-        if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = qtot;
-      }
+      rec[tid] = make_float4(hsum2(a.S), hsum2(a.A), hsum2(a.St), q_prev);
+      named_arrive(kPosted, all);
+      if (cl > 1) cluster_sync_all();
       if (!real) break;
+      named_sync(kReady, all);
 
       // -------------------------------------------------------------- overflow: running maxima
-      // (the totals are identical in every warp of the cluster, so this branch is uniform)
-      if (!(t.S < kSumLimit) || !(t.St < kSumLimit)) {
+      if (ctrl.out.again) {
         RowAcc ra;
         ra.reset();
         const char* st = stash;
@@ -291,56 +367,24 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         const float fs = (ra.m2s == -INFINITY) ? 0.f : ex2f(ra.m2s - wms);
         const float ft = (ra.m2t == -INFINITY) ? 0.f : ex2f(ra.m2t - wmt);
         const float w1 = lane_sum(ra.S * fs), w2 = lane_sum(ra.A * fs), w3 = lane_sum(ra.St * ft);
-        float* rec = ctrl.safe[rank * nw + warp];
-        if (lane < cl) {
-          const uint32_t dst = cl == 1 ? smem_u32(rec) : map_to_rank(smem_u32(rec), (uint32_t)lane);
-          remote_store4(dst, wms, wmt, w1, w2);
-          remote_store4(dst + 16, w3, 0.f, 0.f, 0.f);
+        if (lane == 0) {
+          float* x = ctrl.safe[warp];
+          x[0] = wms; x[1] = wmt; x[2] = w1; x[3] = w2; x[4] = w3;
         }
-        row_barrier();
-        float ms = -INFINITY, mt = -INFINITY;
-        for (int j = lane; j < nrec; j += 32) {
-          ms = fmaxf(ms, ctrl.safe[j][0]);
-          mt = fmaxf(mt, ctrl.safe[j][1]);
-        }
-        t.M2s = warp_max(ms);
-        t.M2t = warp_max(mt);
-        float s[3] = {0.f, 0.f, 0.f};
-        for (int j = lane; j < nrec; j += 32) {
-          const float* x = ctrl.safe[j];
-          const float gs = (x[0] == -INFINITY) ? 0.f : ex2f(x[0] - t.M2s);
-          const float gt = (x[1] == -INFINITY) ? 0.f : ex2f(x[1] - t.M2t);
-          s[0] += x[2] * gs;
-          s[1] += x[3] * gs;
-          s[2] += x[4] * gt;
-        }
-        t.S = lane_sum(s[0]);
-        t.A = lane_sum(s[1]);
-        t.St = lane_sum(s[2]);
-      }
-
-      // -------------------------------------------------------------- row scalars
-      const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
-      const RowScalars rs = finish_row(t, m.zy, m.uy, y_valid, 0.f, p.alpha, p.mode,
-                                       p.row_coef ? &m.w : nullptr);
-      if (rank == 0 && tid == 0) {
-        p.kl[m.r] = rs.kl;
-        p.logratio[m.r] = rs.c;
-        if (p.lse_s) p.lse_s[m.r] = rs.lse_s;
-        if (p.lse_t) p.lse_t[m.r] = rs.lse_t;
-        int bits = 0;
-        if (!y_valid) bits |= ADWIN_DEV_TOKEN_RANGE;
-        if (rs.nonfinite) bits |= ADWIN_DEV_NONFINITE;
-        if (bits) atomicOr(p.status, bits);
+        named_arrive(kPosted, all);
+        if (cl > 1) cluster_sync_all();
+        named_sync(kReady, all);
       }
 
       // -------------------------------------------------------------- sweep 2
       const f2_t L2 = splat2(kLog2e), NEG1 = splat2(-1.f);
-      const f2_t nM2s = splat2(-t.M2s), coef2 = splat2(rs.coef);
+      const float coef = ctrl.out.coef, c0 = ctrl.out.c0, gy = ctrl.out.gy;
+      const f2_t nM2s = splat2(-ctrl.out.m2s), coef2 = splat2(coef);
       // bf16 logits: g = e * (coef*delta - coef*c0) saves one operation per pair; its rounding
       // (relative to coef*delta, not to the difference) is far inside that dtype's tolerance.
-      const f2_t nc0 = splat2(sizeof(TIn) == 2 ? -rs.coef * rs.c0 : -rs.c0);
+      const f2_t nc0 = splat2(sizeof(TIn) == 2 ? -coef * c0 : -c0);
       const int64_t yat = (int64_t)m.y + span.shift;                     // counted from piece 0
+      const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
       const int ypiece = y_valid ? (int)(yat / N - piece0) : -1;         // slice-relative
       char* gp = static_cast<char*>(p.grad) +
                  ((size_t)m.r * p.ld_grad - span.shift + (size_t)(piece0 + tid) * N) * sizeof(TOut);
@@ -387,8 +431,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
               for (int e = 0; e < NP; ++e) {
                 float lo, hi;
                 upk2(G[e], lo, hi);
-                if (ye == 2 * e) lo = rs.gy;
-                if (ye == 2 * e + 1) hi = rs.gy;
+                if (ye == 2 * e) lo = gy;
+                if (ye == 2 * e + 1) hi = gy;
                 G[e] = pk2(lo, hi);
               }
             }
@@ -417,8 +461,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       int k0 = 0;
       for (; (k0 + kU) * nt <= span.pieces; k0 += kU) group(std::true_type{}, k0);
       for (; k0 < plan.steps; k0 += kU) group(std::false_type{}, k0);
-      q_prev = lane_sum(hsum2(Q));
-      r_prev = m.r;
+      q_prev = hsum2(Q);
     }
   }
   if (TM) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -460,7 +503,7 @@ bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
   plan.per_rank = (int)((pieces + sh.cl - 1) / sh.cl);
   const int need = (plan.per_rank + sh.nt - 1) / sh.nt;
   plan.steps = (need + kU - 1) / kU * kU;
-  const int smem = kSmemPerSm / sh.ctas - kSmemReserved - kRowsCtrlBytes;
+  const int smem = kSmemPerSm / sh.ctas - kSmemReserved - rows_ctrl_bytes(sh.nt);
   const int sm_steps = smem / (32 * sh.nt) / kU * kU;
   // a lane group's columns are shared by its warps (every fourth); a piece pair takes 8 columns
   const int tm_most = sh.tm_cols ? sh.tm_cols / ((sh.nt + 127) / 128) / 8 / kU * kU : 0;
@@ -470,7 +513,7 @@ bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
 }
 
 int rows_smem(const RowsPlan& plan) {
-  return kRowsCtrlBytes + (plan.steps - plan.tm_steps) * 32 * plan.nt;
+  return rows_ctrl_bytes(plan.nt) + (plan.steps - plan.tm_steps) * 32 * plan.nt;
 }
 
 bool rows_plan(int64_t pieces, bool bf16, RowsPlan& plan) {
