@@ -20,10 +20,6 @@
 #include <mutex>
 #include <type_traits>
 #include <vector>
-#ifdef ADWIN_ROWS_TUNE
-#include <cstdio>
-#include <cstdlib>
-#endif
 
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
@@ -33,10 +29,8 @@ namespace adwin {
 namespace {
 
 constexpr int kRowsThreads = 352;     // threads of a CTA that hold pieces, at most
-#ifndef ROWS_U
-#define ROWS_U 2
-#endif
-constexpr int kU = ROWS_U;            // piece pairs in flight per thread
+constexpr int kRowsRegs = 80;         // registers per thread: 819 threads on an SM
+constexpr int kU = 2;                 // piece pairs in flight per thread
 constexpr int kRowsMaxCl = 4;
 constexpr float kSumLimit = 1.2676506e30f;   // 2^100: beyond it the shared reference is unsafe
 constexpr int kMetaDepth = 4;
@@ -95,7 +89,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 // offsets in the instructions.  A group of kU steps in which every thread has a piece takes the path
 // without tests (FULL below).
 template <typename TIn, typename TOut, int NT, bool TM, bool RAG>
-__global__ void __launch_bounds__(NT + 32, 65536 / 80 / (NT + 32))
+__global__ void __launch_bounds__(NT + 32, 65536 / kRowsRegs / (NT + 32))
 kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   constexpr int N = Elem<TIn>::N;
   constexpr int NP = Pairs<TIn>::NP;
@@ -478,23 +472,25 @@ constexpr int kSmemPerSm = 233472, kSmemReserved = 1024;   // bytes per SM, and 
 
 struct RowsShape {
   int ctas, nt, tm_cols, cl;
+  int most_kb;        // bytes of a row (both arrays) up to which the shape is taken, in KB
 };
-// From many small CTAs to two large ones, then clusters; the first that holds the row is taken: the
-// most CTAs per SM, because their number is what hides one row's exchange behind the others'
-// streaming.  Tensor memory is shared out in powers of two.  Measured over 2.4 GB of logits and
-// gradient (367 us at the copy rate; staged kernel / two sweeps over memory / this kernel):
-//   bf16  V =   4 096  2488 /  993 / 622 us  {8, 64}       fp32  V =   4 096  1247 / 599 / 439 us  {5, 128}
-//             16 384   993 /  625 / 555     {3, 224}              16 384   600 / 679 / 433      {2, 352}
-//             32 000   726 /  822 / 513     {2, 352}              32 000   510 / 733 / 444      {3, 224} x 2
-//             50 264   638 /  980 / 529     {2, 352}              50 264   597 / 772 / 478      {2, 352} x 2
-//            100 000   656 / 1019 / 547     {2, 352} x 2         100 000   547 / 781 / 485      {2, 352} x 4
-//            151 936   573 / 1012 / 586 (x 3), 595 (x 4)
-// bf16 rows are bound by arithmetic (28 issue slots per entry), fp32 rows by memory.  Clusters beyond
-// two CTAs leave SMs over, which costs bf16 rows more than the overlap gives: those go to the staged
-// kernel.
-constexpr RowsShape kShapes[] = {{8, 64, 0, 1}, {5, 128, 0, 1}, {3, 224, 128, 1}, {2, 352, 256, 1},
-                                 {3, 224, 128, 2}, {2, 352, 256, 2}, {2, 352, 256, 4}};
-constexpr int kMaxClBf16 = 2;
+// From many small CTAs to two large ones, then clusters; the first that takes the row and holds it
+// is used: the most CTAs per SM, because their number is what hides one row's exchange behind the
+// others' streaming.  Tensor memory is shared out in powers of two.  Measured over 2.4 GB of logits
+// and gradient (367 us at the copy rate; staged kernel / two sweeps over memory / this kernel):
+//   bf16  V =   4 096  2488 /  993 / 476 us  {8, 64}       fp32  V =   4 096  1247 / 599 / 411 us  {5, 128}
+//              8 192  1353 /  755 / 445     {5, 128}               12 000   790 / 604 / 421      {3, 224}
+//             16 384   993 /  625 / 484     {3, 224}               16 384   600 / 679 / 421      {2, 352}
+//             32 000   726 /  822 / 473     {2, 352}               32 000   510 / 733 / 459      {2, 352} x 2
+//             50 264   638 /  980 / 500     {2, 352}               50 264   597 / 772 / 465      {2, 352} x 2
+//            100 000   656 / 1019 / 513     {2, 352} x 2           65 536   521 / 766 / 454      {2, 352} x 4
+//            151 936   573 / 1012 / 557     {2, 352} x 4
+// bf16 rows are bound by arithmetic and latency (19 issue slots per entry, the ex2 unit 57 % busy),
+// fp32 rows by memory.  Three or four steps in flight spill at 80 registers and lose, one step at 64
+// registers and a third more threads is slower except around 16 384 entries.
+constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 1 << 20},   {5, 128, 0, 1, 1 << 20},
+                                 {3, 224, 128, 1, 100},    {2, 352, 256, 1, 1 << 20},
+                                 {2, 352, 256, 2, 1 << 20}, {2, 352, 256, 4, 1 << 20}};
 
 bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
   plan.cl = sh.cl;
@@ -516,30 +512,18 @@ int rows_smem(const RowsPlan& plan) {
   return rows_ctrl_bytes(plan.nt) + (plan.steps - plan.tm_steps) * 32 * plan.nt;
 }
 
-bool rows_plan(int64_t pieces, bool bf16, RowsPlan& plan) {
+bool rows_plan(int64_t pieces, RowsPlan& plan) {
   if (pieces < 1 || pieces > (int64_t)1 << 24) return false;
-#ifdef ADWIN_ROWS_TUNE
-  if (getenv("ROWS_SHAPE")) {
-    RowsShape sh;
-    sscanf(getenv("ROWS_SHAPE"), "%d,%d,%d,%d", &sh.ctas, &sh.nt, &sh.tm_cols, &sh.cl);
-    return shape_plan(sh, pieces, plan);
-  }
-#endif
   for (const RowsShape& sh : kShapes)
-    if ((!bf16 || sh.cl <= kMaxClBf16) && shape_plan(sh, pieces, plan)) return true;
+    if (pieces * 32 <= (int64_t)sh.most_kb * 1024 && shape_plan(sh, pieces, plan)) return true;
   return false;
 }
 
 typedef void (*RowsKernel)(KlParams, RowsPlan);
 template <typename TIn, typename TOut, int NT>
 RowsKernel rows_kernel_nt(bool tm, bool ragged) {
-#ifdef ADWIN_ROWS_TUNE
-  if (ragged || sizeof(TIn) != sizeof(TOut)) return nullptr;
-  return tm ? kl_rows_kernel<TIn, TOut, NT, true, false> : kl_rows_kernel<TIn, TOut, NT, false, false>;
-#else
   if (tm) return ragged ? kl_rows_kernel<TIn, TOut, NT, true, true> : kl_rows_kernel<TIn, TOut, NT, true, false>;
   return ragged ? kl_rows_kernel<TIn, TOut, NT, false, true> : kl_rows_kernel<TIn, TOut, NT, false, false>;
-#endif
 }
 template <typename TIn, typename TOut>
 RowsKernel rows_kernel(int nt, bool tm, bool ragged) {
@@ -594,8 +578,7 @@ template <typename TIn, typename TOut>
 cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStream_t s) {
   constexpr int N = Elem<TIn>::N;
   RowsPlan plan = {};
-  if (!rows_plan(ragged ? (p.V + 2 * N - 2) / N : p.V / N, sizeof(TIn) == 2, plan))
-    return cudaErrorNotSupported;
+  if (!rows_plan(ragged ? (p.V + 2 * N - 2) / N : p.V / N, plan)) return cudaErrorNotSupported;
   const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, plan.tm_cols > 0, ragged);
   if (!kernel) return cudaErrorNotSupported;
   const int smem = rows_smem(plan);
@@ -611,9 +594,6 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   if (e != cudaSuccess) return e;
   const int64_t rows = p.B * p.T;
   if (plan.num_clusters > rows) plan.num_clusters = (int)rows;
-#ifdef ADWIN_ROWS_TUNE
-  if (getenv("ROWS_DBG")) fprintf(stderr, "rows cl %d nt %d ctas %d per %d steps %d tm %d cols %d clusters %d smem %d\n", plan.cl, plan.nt, plan.ctas, plan.per_rank, plan.steps, plan.tm_steps, plan.tm_cols, plan.num_clusters, smem);
-#endif
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(plan.cl * plan.num_clusters);
   cfg.blockDim = dim3(plan.nt + 32);
