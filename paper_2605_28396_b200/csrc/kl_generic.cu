@@ -12,17 +12,21 @@
 
 namespace adwin {
 
-// 128-thread CTAs, one row each, five pairs of 16-byte loads in flight per thread: small CTAs put
-// many independent rows on an SM, so one row's reduction overlaps the others' streaming (measured on
-// the read-only pass at V = 151 936 with scalar arithmetic: 256 threads x 1 load 74 %, 256 x 8 81 %,
-// 512 x 8 79 %, 128 x 16 78 %, 128 x 8 90 % of the measured copy bandwidth).  With sweep 1 on packed
-// pairs the kernel wants more registers per thread; 5 loads at 5 CTAs per SM (<= 96 registers, no
-// spills) measured best among 4..8 loads x 4..8 CTAs, 3 % faster than the scalar 128 x 8 form both
-// on a cold GPU and in a back-to-back series (where every form runs ~12 % slower).
+// 128-thread CTAs, one row each, four pairs of 16-byte loads in flight per thread: small CTAs put
+// many independent rows on an SM, so one row's reduction overlaps the others' streaming.  The
+// read-only pass is at the copy rate on a cool GPU (2.23 ms for 14.9 GB at V = 151 936); in a
+// back-to-back series the power cap lowers the clocks and every instruction costs, hence references
+// fixed by a thread's first group instead of a maximum per piece, and moments only where the norm
+// takes them (series: 2.96 ms before, 2.55 now).  Measured in a series, threads x loads x CTAs per SM:
+// 128x3x7 2.56, 128x4x6 2.55, 128x5x5 2.59, 128x6x4 2.67, 64x5x10 2.58, 256x4x3 2.64, 256x5x2 2.99 ms.
 constexpr int kGenericThreads = 128;
 constexpr int kGenericWarps = kGenericThreads / 32;
-constexpr int kGenericUnroll = 5;
-constexpr int kGenericMinBlocks = 5;   // CTAs per SM the register allocation leaves room for
+constexpr int kGenericUnroll = 4;
+constexpr int kGenericMinBlocks = 6;   // CTAs per SM the register allocation leaves room for
+
+// A thread's sums are good up to 2^48: e^2 delta^2, the largest term, stays below 2^128 then for
+// logits up to 2^16 apart.
+constexpr float kSafeSum = 281474976710656.f;
 
 struct BlockScratch {
   float wm[2][kGenericWarps];
@@ -33,8 +37,7 @@ struct BlockScratch {
 };
 
 // Sweep 1 on packed fp32 pairs: sm_100 issues add / mul / fma on two fp32 lanes of a 64-bit
-// register pair in one slot, which halves the issue slots of the element-wise part (the sweep is
-// bound by issue slots and the ex2 unit as much as by memory).  Even and odd entries of a piece
+// register pair in one slot, which halves the issue slots of the element-wise part.  Even and odd entries of a piece
 // accumulate separately; fold() adds the two lanes.
 typedef unsigned long long pair_t;
 __device__ __forceinline__ pair_t pair(float lo, float hi) {
@@ -93,8 +96,34 @@ struct PairAcc {
   }
 };
 
-// acc_piece<N, true> on pairs (N even).
-template <int N>
+// The sums of acc_piece<N, true> against the references that `a` holds, on pairs (N even).  MOM: all
+// three moments of the gradient norm, or only B0, which is all that the norm of a sampled-token
+// gradient takes.
+template <int N, bool MOM>
+__device__ __forceinline__ void acc_sums(const float (&z)[N], const float (&u)[N], float dref, PairAcc& a) {
+  const pair_t L2 = pair(kLog2e, kLog2e), NEG1 = pair(-1.f, -1.f);
+  const pair_t nms = pair(-a.m2s, -a.m2s), nmt = pair(-a.m2t, -a.m2t), ndref = pair(-dref, -dref);
+#pragma unroll
+  for (int i = 0; i < N; i += 2) {
+    const pair_t Z = pair(z[i], z[i + 1]), U = pair(u[i], u[i + 1]);
+    const pair_t E = pex2(pfma(Z, L2, nms));
+    const pair_t D = padd(pfma(U, NEG1, Z), ndref);
+    a.S = padd(a.S, E);
+    a.B0 = pfma(E, E, a.B0);
+    if (MOM) {
+      const pair_t ED = pmul(E, D);
+      a.A = padd(a.A, ED);
+      a.B1 = pfma(E, ED, a.B1);
+      a.B2 = pfma(ED, ED, a.B2);
+    } else {
+      a.A = pfma(E, D, a.A);
+    }
+    a.St = padd(a.St, pex2(pfma(U, L2, nmt)));
+  }
+}
+
+// The same after raising the references to the piece's maxima.
+template <int N, bool MOM>
 __device__ __forceinline__ void acc_piece_pairs(const float (&z)[N], const float (&u)[N], float dref,
                                                 PairAcc& a) {
   float zm = z[0], um = u[0];
@@ -110,8 +139,10 @@ __device__ __forceinline__ void acc_piece_pairs(const float (&z)[N], const float
     a.S = pmul(a.S, F);
     a.A = pmul(a.A, F);
     a.B0 = pmul(a.B0, F2);
-    a.B1 = pmul(a.B1, F2);
-    a.B2 = pmul(a.B2, F2);
+    if (MOM) {
+      a.B1 = pmul(a.B1, F2);
+      a.B2 = pmul(a.B2, F2);
+    }
     a.m2s = zl;
   }
   if (ul > a.m2t) {
@@ -119,22 +150,7 @@ __device__ __forceinline__ void acc_piece_pairs(const float (&z)[N], const float
     a.St = pmul(a.St, pair(f, f));
     a.m2t = ul;
   }
-  const pair_t L2 = pair(kLog2e, kLog2e), NEG1 = pair(-1.f, -1.f);
-  const pair_t nms = pair(-a.m2s, -a.m2s), nmt = pair(-a.m2t, -a.m2t), ndref = pair(-dref, -dref);
-#pragma unroll
-  for (int i = 0; i < N; i += 2) {
-    const pair_t Z = pair(z[i], z[i + 1]), U = pair(u[i], u[i + 1]);
-    const pair_t E = pex2(pfma(Z, L2, nms));
-    const pair_t D = padd(pfma(U, NEG1, Z), ndref);
-    a.S = padd(a.S, E);
-    a.A = pfma(E, D, a.A);
-    const pair_t E2 = pmul(E, E);
-    const pair_t E2D = pmul(E2, D);
-    a.B0 = padd(a.B0, E2);
-    a.B1 = padd(a.B1, E2D);
-    a.B2 = pfma(E2D, D, a.B2);
-    a.St = padd(a.St, pex2(pfma(U, L2, nmt)));
-  }
+  acc_sums<N, MOM>(z, u, dref, a);
 }
 
 // Combine the per-thread accumulators of a CTA; every thread returns the same totals.
@@ -184,7 +200,7 @@ __device__ __forceinline__ RowTotals block_combine(const RowAcc& a, BlockScratch
   return t;
 }
 
-template <typename TIn, typename TOut, bool VEC>
+template <typename TIn, typename TOut, bool VEC, bool MOM>
 __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic_kernel(KlParams p) {
   __shared__ BlockScratch sm;
   constexpr int N = VEC ? Elem<TIn>::N : 1;
@@ -228,33 +244,60 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
       // (no gradient) is streamed past the caches, otherwise sweep 2 should find it in L2
       const uint4* zs = reinterpret_cast<const uint4*>(zrow + head * sizeof(TIn));
       const uint4* us = reinterpret_cast<const uint4*>(urow + head * sizeof(TIn));
+      auto load = [&](int64_t i, uint4& zv, uint4& uv) {
+        zv = write_grad ? __ldg(zs + i) : __ldcs(zs + i);
+        uv = write_grad ? __ldg(us + i) : __ldcs(us + i);
+      };
+      // one piece at a time, the references raised before each
+      auto singly = [&](int64_t i, int64_t end) {
+        for (; i < end; i += kGenericThreads) {
+          float z[N], u[N];
+          uint4 zv, uv;
+          if (!ADWIN_CHK(head + (i + 1) * N <= p.V, p.status)) break;
+          load(i, zv, uv);
+          Elem<TIn>::unpack(zv, reinterpret_cast<float(&)[Elem<TIn>::N]>(z));
+          Elem<TIn>::unpack(uv, reinterpret_cast<float(&)[Elem<TIn>::N]>(u));
+          acc_piece_pairs<N, MOM>(z, u, dref, pa);
+        }
+      };
       int64_t i = tid;
+      bool first = true;
       for (; i + (kGenericUnroll - 1) * kGenericThreads < pieces;
            i += kGenericUnroll * kGenericThreads) {
         uint4 zv[kGenericUnroll], uv[kGenericUnroll];
         if (!ADWIN_CHK(head + (i + (kGenericUnroll - 1) * kGenericThreads + 1) * N <= p.V, p.status)) break;
 #pragma unroll
-        for (int h = 0; h < kGenericUnroll; ++h) {
-          zv[h] = write_grad ? __ldg(zs + i + h * kGenericThreads) : __ldcs(zs + i + h * kGenericThreads);
-          uv[h] = write_grad ? __ldg(us + i + h * kGenericThreads) : __ldcs(us + i + h * kGenericThreads);
+        for (int h = 0; h < kGenericUnroll; ++h) load(i + h * kGenericThreads, zv[h], uv[h]);
+        if (first) {   // the references of all whole groups: the maxima of the thread's first one
+          first = false;
+#pragma unroll
+          for (int h = 0; h < kGenericUnroll; ++h) {
+            float z[N], u[N];
+            Elem<TIn>::unpack(zv[h], reinterpret_cast<float(&)[Elem<TIn>::N]>(z));
+            Elem<TIn>::unpack(uv[h], reinterpret_cast<float(&)[Elem<TIn>::N]>(u));
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+              pa.m2s = fmaxf(pa.m2s, z[j]);
+              pa.m2t = fmaxf(pa.m2t, u[j]);
+            }
+          }
+          pa.m2s *= kLog2e;
+          pa.m2t *= kLog2e;
         }
 #pragma unroll
         for (int h = 0; h < kGenericUnroll; ++h) {
           float z[N], u[N];
           Elem<TIn>::unpack(zv[h], reinterpret_cast<float(&)[Elem<TIn>::N]>(z));
           Elem<TIn>::unpack(uv[h], reinterpret_cast<float(&)[Elem<TIn>::N]>(u));
-          acc_piece_pairs<N>(z, u, dref, pa);
+          acc_sums<N, MOM>(z, u, dref, pa);
         }
       }
-      for (; i < pieces; i += kGenericThreads) {
-        float z[N], u[N];
-        if (!ADWIN_CHK(head + (i + 1) * N <= p.V, p.status)) break;
-        const uint4 zv = write_grad ? __ldg(zs + i) : __ldcs(zs + i);
-        const uint4 uv = write_grad ? __ldg(us + i) : __ldcs(us + i);
-        Elem<TIn>::unpack(zv, reinterpret_cast<float(&)[Elem<TIn>::N]>(z));
-        Elem<TIn>::unpack(uv, reinterpret_cast<float(&)[Elem<TIn>::N]>(u));
-        acc_piece_pairs<N>(z, u, dref, pa);
+      // a sum that has outgrown its reference (or is no number): the groups again, against running maxima
+      if (!first && !(psum(pa.S) < kSafeSum && psum(pa.St) < kSafeSum)) {
+        pa.reset();
+        singly(tid, i);
       }
+      singly(i, pieces);
       a = pa.fold();
       if (edge >= 0) {
         const float z[1] = {Elem<TIn>::load1(zrow, edge)}, u[1] = {Elem<TIn>::load1(urow, edge)};
@@ -358,10 +401,12 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
 
 template <typename TIn, typename TOut>
 static cudaError_t launch_t(const KlParams& p, bool vec, int grid, cudaStream_t s) {
-  if (vec)
-    kl_generic_kernel<TIn, TOut, true><<<grid, kGenericThreads, 0, s>>>(p);
+  if (vec && p.mode == ADWIN_GRAD_FULL_KL)
+    kl_generic_kernel<TIn, TOut, true, true><<<grid, kGenericThreads, 0, s>>>(p);
+  else if (vec)
+    kl_generic_kernel<TIn, TOut, true, false><<<grid, kGenericThreads, 0, s>>>(p);
   else
-    kl_generic_kernel<TIn, TOut, false><<<grid, kGenericThreads, 0, s>>>(p);
+    kl_generic_kernel<TIn, TOut, false, true><<<grid, kGenericThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -570,3 +570,21 @@ def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
     for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
         run_and_check(batch, grad_dtype=g_dt, grad_mode=mode)
     run_and_check(batch, grad_dtype=g_dt, flags=api.RANGE_FULL)
+
+
+@pytest.mark.parametrize("in_dt,V", [(2, 4095), (2, 4096), (2, 4104), (2, 20001), (1, 2047), (1, 2052), (1, 9001)])
+@pytest.mark.parametrize("mode", [api.GRAD_FULL_KL, api.GRAD_SAMPLED])
+def test_read_only_rows_that_outgrow_their_first_entries(in_dt, V, mode):
+    """Rows without gradient are summed against the maximum of each thread's first entries: rows that
+    rise after them by less than the sums bear, and by more (summed once more against running
+    maxima), in the student, the teacher and both; row lengths around one whole group of loads."""
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=5, V=V)
+    batch.window = torch.tensor([5, 4], dtype=torch.int32, device=DEV)
+    part = 4 * 128 * (4 if in_dt == 1 else 8)       # entries of the first group of a row
+    for t, (rise_s, rise_t) in enumerate(((20.0, 20.0), (60.0, 0.0), (0.0, 60.0), (90.0, 80.0))):
+        batch.student[0, t, :part] -= rise_s
+        batch.teacher[0, t, :part] -= rise_t
+        for x in (batch.student, batch.teacher):    # keep the sampled token near the maximum
+            x[0, t, int(batch.tokens[0, t])] = x[0, t].float().max() - 1.0
+    run_and_check(batch, grad_dtype=None, grad_mode=mode)
+    run_and_check(batch, grad_dtype=None, grad_mode=mode, flags=api.RANGE_FULL)
