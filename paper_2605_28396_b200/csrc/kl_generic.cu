@@ -1,4 +1,5 @@
-// Shape-agnostic row kernel: one CTA per processed row, two sweeps over global memory.
+// Shape-agnostic row kernel: one CTA per processed row (a cluster, where a call has few rows and
+// writes no gradient), two sweeps over global memory.
 //
 // Sweep 1 streams z and u once and accumulates the online log-sum-exp statistics, sum e*delta
 // (reverse KL) and the moments of the single-sweep gradient norm.  Sweep 2 (only for rows whose
@@ -9,6 +10,7 @@
 // Calls without gradient come here, and layouts that the staged cluster kernel does not take.
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
+#include "kl_pairs.cuh"
 
 namespace adwin {
 
@@ -20,6 +22,7 @@ namespace adwin {
 // takes them (series: 2.96 ms before, 2.55 now).  Measured in a series, threads x loads x CTAs per SM:
 // 128x3x7 2.56, 128x4x6 2.55, 128x5x5 2.59, 128x6x4 2.67, 64x5x10 2.58, 256x4x3 2.64, 256x5x2 2.99 ms.
 constexpr int kGenericThreads = 128;
+constexpr int kGenericMaxCl = 4;
 constexpr int kGenericWarps = kGenericThreads / 32;
 constexpr int kGenericUnroll = 4;
 constexpr int kGenericMinBlocks = 6;   // CTAs per SM the register allocation leaves room for
@@ -32,51 +35,16 @@ struct BlockScratch {
   float wm[2][kGenericWarps];
   float ws[6][kGenericWarps];
   float wq[kGenericWarps];
+  float xtot[2][kGenericMaxCl][8];   // per row parity, the totals of the row's CTAs (in the first one)
   RowScalars rs;
-  RowTotals tot;
 };
 
 // Sweep 1 on packed fp32 pairs: sm_100 issues add / mul / fma on two fp32 lanes of a 64-bit
 // register pair in one slot, which halves the issue slots of the element-wise part.  Even and odd entries of a piece
 // accumulate separately; fold() adds the two lanes.
-typedef unsigned long long pair_t;
-__device__ __forceinline__ pair_t pair(float lo, float hi) {
-  pair_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpair(pair_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ pair_t pfma(pair_t a, pair_t b, pair_t c) {
-  pair_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ pair_t padd(pair_t a, pair_t b) {
-  pair_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ pair_t pmul(pair_t a, pair_t b) {
-  pair_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ pair_t pex2(pair_t x) {
-  float a, b;
-  unpair(x, a, b);
-  return pair(ex2f(a), ex2f(b));
-}
-__device__ __forceinline__ float psum(pair_t v) {
-  float a, b;
-  unpair(v, a, b);
-  return a + b;
-}
-
 struct PairAcc {
   float m2s, m2t;                  // running references, as in RowAcc
-  pair_t S, A, B0, B1, B2, St;     // the sums of RowAcc, even / odd entries apart
+  f2_t S, A, B0, B1, B2, St;     // the sums of RowAcc, even / odd entries apart
   __device__ __forceinline__ void reset() {
     m2s = -INFINITY;
     m2t = -INFINITY;
@@ -86,39 +54,40 @@ struct PairAcc {
     RowAcc a;
     a.m2s = m2s;
     a.m2t = m2t;
-    a.S = psum(S);
-    a.A = psum(A);
-    a.B0 = psum(B0);
-    a.B1 = psum(B1);
-    a.B2 = psum(B2);
-    a.St = psum(St);
+    a.S = hsum2(S);
+    a.A = hsum2(A);
+    a.B0 = hsum2(B0);
+    a.B1 = hsum2(B1);
+    a.B2 = hsum2(B2);
+    a.St = hsum2(St);
     return a;
   }
 };
 
 // The sums of acc_piece<N, true> against the references that `a` holds, on pairs (N even).  MOM: all
 // three moments of the gradient norm, or only B0, which is all that the norm of a sampled-token
-// gradient takes.
+// gradient takes.  That norm subtracts p_y^2 from B0 / S^2, which only agree to the last bits for a
+// token with most of the mass when its exponent is taken near zero: it keeps to running maxima.
 template <int N, bool MOM>
 __device__ __forceinline__ void acc_sums(const float (&z)[N], const float (&u)[N], float dref, PairAcc& a) {
-  const pair_t L2 = pair(kLog2e, kLog2e), NEG1 = pair(-1.f, -1.f);
-  const pair_t nms = pair(-a.m2s, -a.m2s), nmt = pair(-a.m2t, -a.m2t), ndref = pair(-dref, -dref);
+  const f2_t L2 = splat2(kLog2e), NEG1 = splat2(-1.f);
+  const f2_t nms = splat2(-a.m2s), nmt = splat2(-a.m2t), ndref = splat2(-dref);
 #pragma unroll
   for (int i = 0; i < N; i += 2) {
-    const pair_t Z = pair(z[i], z[i + 1]), U = pair(u[i], u[i + 1]);
-    const pair_t E = pex2(pfma(Z, L2, nms));
-    const pair_t D = padd(pfma(U, NEG1, Z), ndref);
-    a.S = padd(a.S, E);
-    a.B0 = pfma(E, E, a.B0);
+    const f2_t Z = pk2(z[i], z[i + 1]), U = pk2(u[i], u[i + 1]);
+    const f2_t E = ex2_2(fma2(Z, L2, nms));
+    const f2_t D = add2(fma2(U, NEG1, Z), ndref);
+    a.S = add2(a.S, E);
+    a.B0 = fma2(E, E, a.B0);
     if (MOM) {
-      const pair_t ED = pmul(E, D);
-      a.A = padd(a.A, ED);
-      a.B1 = pfma(E, ED, a.B1);
-      a.B2 = pfma(ED, ED, a.B2);
+      const f2_t ED = mul2(E, D);
+      a.A = add2(a.A, ED);
+      a.B1 = fma2(E, ED, a.B1);
+      a.B2 = fma2(ED, ED, a.B2);
     } else {
-      a.A = pfma(E, D, a.A);
+      a.A = fma2(E, D, a.A);
     }
-    a.St = padd(a.St, pex2(pfma(U, L2, nmt)));
+    a.St = add2(a.St, ex2_2(fma2(U, L2, nmt)));
   }
 }
 
@@ -135,22 +104,50 @@ __device__ __forceinline__ void acc_piece_pairs(const float (&z)[N], const float
   const float zl = zm * kLog2e, ul = um * kLog2e;
   if (zl > a.m2s) {
     const float f = ex2f(a.m2s - zl);
-    const pair_t F = pair(f, f), F2 = pmul(F, F);
-    a.S = pmul(a.S, F);
-    a.A = pmul(a.A, F);
-    a.B0 = pmul(a.B0, F2);
+    const f2_t F = splat2(f), F2 = mul2(F, F);
+    a.S = mul2(a.S, F);
+    a.A = mul2(a.A, F);
+    a.B0 = mul2(a.B0, F2);
     if (MOM) {
-      a.B1 = pmul(a.B1, F2);
-      a.B2 = pmul(a.B2, F2);
+      a.B1 = mul2(a.B1, F2);
+      a.B2 = mul2(a.B2, F2);
     }
     a.m2s = zl;
   }
   if (ul > a.m2t) {
     const float f = ex2f(a.m2t - ul);
-    a.St = pmul(a.St, pair(f, f));
+    a.St = mul2(a.St, splat2(f));
     a.m2t = ul;
   }
   acc_sums<N, MOM>(z, u, dref, a);
+}
+
+// Partial sums against references of their own, in the order given.
+template <int MAX>
+__device__ __forceinline__ RowTotals combine_parts(const RowAcc (&part)[MAX], int n) {
+  RowTotals t;
+  t.M2s = t.M2t = -INFINITY;
+  t.S = t.A = t.B0 = t.B1 = t.B2 = t.St = 0.f;
+#pragma unroll
+  for (int w = 0; w < MAX; ++w) {
+    if (w >= n) break;
+    t.M2s = fmaxf(t.M2s, part[w].m2s);
+    t.M2t = fmaxf(t.M2t, part[w].m2t);
+  }
+#pragma unroll
+  for (int w = 0; w < MAX; ++w) {
+    if (w >= n) break;
+    const float gs = (part[w].m2s == -INFINITY) ? 0.f : ex2f(part[w].m2s - t.M2s);
+    const float gt = (part[w].m2t == -INFINITY) ? 0.f : ex2f(part[w].m2t - t.M2t);
+    const float gs2 = gs * gs;
+    t.S += part[w].S * gs;
+    t.A += part[w].A * gs;
+    t.B0 += part[w].B0 * gs2;
+    t.B1 += part[w].B1 * gs2;
+    t.B2 += part[w].B2 * gs2;
+    t.St += part[w].St * gt;
+  }
+  return t;
 }
 
 // Combine the per-thread accumulators of a CTA; every thread returns the same totals.
@@ -170,49 +167,39 @@ __device__ __forceinline__ RowTotals block_combine(const RowAcc& a, BlockScratch
     for (int i = 0; i < 6; ++i) sm.ws[i][warp] = v[i];
   }
   __syncthreads();
-  RowTotals t;
-  t.M2s = -INFINITY;
-  t.M2t = -INFINITY;
+  RowAcc part[kGenericWarps];
 #pragma unroll
   for (int w = 0; w < kGenericWarps; ++w) {
-    t.M2s = fmaxf(t.M2s, sm.wm[0][w]);
-    t.M2t = fmaxf(t.M2t, sm.wm[1][w]);
+    part[w].m2s = sm.wm[0][w];
+    part[w].m2t = sm.wm[1][w];
+    part[w].S = sm.ws[0][w];
+    part[w].A = sm.ws[1][w];
+    part[w].B0 = sm.ws[2][w];
+    part[w].B1 = sm.ws[3][w];
+    part[w].B2 = sm.ws[4][w];
+    part[w].St = sm.ws[5][w];
   }
-  float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int w = 0; w < kGenericWarps; ++w) {
-    const float gs = (sm.wm[0][w] == -INFINITY) ? 0.f : ex2f(sm.wm[0][w] - t.M2s);
-    const float gt = (sm.wm[1][w] == -INFINITY) ? 0.f : ex2f(sm.wm[1][w] - t.M2t);
-    const float gs2 = gs * gs;
-    acc[0] += sm.ws[0][w] * gs;
-    acc[1] += sm.ws[1][w] * gs;
-    acc[2] += sm.ws[2][w] * gs2;
-    acc[3] += sm.ws[3][w] * gs2;
-    acc[4] += sm.ws[4][w] * gs2;
-    acc[5] += sm.ws[5][w] * gt;
-  }
-  t.S = acc[0];
-  t.A = acc[1];
-  t.B0 = acc[2];
-  t.B1 = acc[3];
-  t.B2 = acc[4];
-  t.St = acc[5];
-  return t;
+  return combine_parts<kGenericWarps>(part, kGenericWarps);
 }
 
-template <typename TIn, typename TOut, bool VEC, bool MOM>
-__global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic_kernel(KlParams p) {
+// SPLIT: read-only rows, each over a cluster of CTAs that take a run of its pieces.
+template <typename TIn, typename TOut, bool VEC, bool MOM, bool SPLIT>
+__global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic_kernel(KlParams p, int clusters_of) {
   __shared__ BlockScratch sm;
   constexpr int N = VEC ? Elem<TIn>::N : 1;
   const int64_t rows = p.B * p.T;
   const int tid = threadIdx.x;
 
-  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+  const int cl = SPLIT ? clusters_of : 1, rank = SPLIT ? (int)cluster_rank() : 0;
+  int par = 0;
+  if (SPLIT) cluster_sync_all();   // every CTA runs before another one stores into it
+
+  for (int64_t r = blockIdx.x / cl; r < rows; r += gridDim.x / cl) {
     const int64_t b = r / p.T;
     const int t = (int)(r - b * p.T);
     if (t >= p.range[b]) continue;  // past the window: the row is never touched
     if (p.skip_below && t < p.skip_below[b]) continue;
-    const bool write_grad = (p.grad != nullptr) && (t < p.ewin[b]);
+    const bool write_grad = !SPLIT && (p.grad != nullptr) && (t < p.ewin[b]);
 
     const char* zrow = static_cast<const char*>(p.student) + (size_t)r * p.ld * sizeof(TIn);
     const char* urow = static_cast<const char*>(p.teacher) + (size_t)r * p.ld * sizeof(TIn);
@@ -232,9 +219,14 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
       if (head > p.V) head = (int)p.V;
       tail = (int)((p.V - head) % N);
     }
-    const int64_t pieces = VEC ? (p.V - head) / N : p.V;
+    int64_t pieces = VEC ? (p.V - head) / N : p.V, from = 0;
+    if (SPLIT) {
+      const int64_t part = ((pieces + cl - 1) / cl + 7) / 8 * 8;   // (whole 128-byte lines)
+      from = min(rank * part, pieces);
+      pieces = min(from + part, pieces);
+    }
     // the entry before or after the pieces that this thread looks after, or -1
-    const int64_t edge = !VEC ? -1
+    const int64_t edge = !VEC || rank != 0 ? -1
                          : tid < head ? tid
                          : (tid >= 32 && tid - 32 < tail) ? p.V - tail + (tid - 32) : -1;
     if (VEC) {
@@ -260,7 +252,7 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
           acc_piece_pairs<N, MOM>(z, u, dref, pa);
         }
       };
-      int64_t i = tid;
+      int64_t i = from + tid;
       bool first = true;
       for (; i + (kGenericUnroll - 1) * kGenericThreads < pieces;
            i += kGenericUnroll * kGenericThreads) {
@@ -268,7 +260,7 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
         if (!ADWIN_CHK(head + (i + (kGenericUnroll - 1) * kGenericThreads + 1) * N <= p.V, p.status)) break;
 #pragma unroll
         for (int h = 0; h < kGenericUnroll; ++h) load(i + h * kGenericThreads, zv[h], uv[h]);
-        if (first) {   // the references of all whole groups: the maxima of the thread's first one
+        if (MOM && first) {   // the references of all whole groups: the maxima of the thread's first one
           first = false;
 #pragma unroll
           for (int h = 0; h < kGenericUnroll; ++h) {
@@ -289,13 +281,14 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
           float z[N], u[N];
           Elem<TIn>::unpack(zv[h], reinterpret_cast<float(&)[Elem<TIn>::N]>(z));
           Elem<TIn>::unpack(uv[h], reinterpret_cast<float(&)[Elem<TIn>::N]>(u));
-          acc_sums<N, MOM>(z, u, dref, pa);
+          if (MOM) acc_sums<N, true>(z, u, dref, pa);
+          else acc_piece_pairs<N, false>(z, u, dref, pa);
         }
       }
       // a sum that has outgrown its reference (or is no number): the groups again, against running maxima
-      if (!first && !(psum(pa.S) < kSafeSum && psum(pa.St) < kSafeSum)) {
+      if (MOM && !first && !(hsum2(pa.S) < kSafeSum && hsum2(pa.St) < kSafeSum)) {
         pa.reset();
-        singly(tid, i);
+        singly(from + tid, i);
       }
       singly(i, pieces);
       a = pa.fold();
@@ -304,7 +297,7 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
         acc_piece<1, true>(z, u, dref, a);
       }
     } else {
-      for (int64_t i = tid; i < pieces; i += kGenericThreads) {
+      for (int64_t i = from + tid; i < pieces; i += kGenericThreads) {
         float z[N], u[N];
         if (!ADWIN_CHK(i < p.ld, p.status)) break;
         z[0] = Elem<TIn>::load1(zrow, i);
@@ -312,7 +305,27 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
         acc_piece<N, true>(z, u, dref, a);
       }
     }
-    const RowTotals tot = block_combine(a, sm);
+    RowTotals tot = block_combine(a, sm);
+    if (SPLIT) {
+      if (tid == 0) {
+        const uint32_t dst = map_to_rank(smem_u32(sm.xtot[par][rank]), 0);
+        remote_store4(dst, tot.M2s, tot.M2t, tot.S, tot.A);
+        remote_store4(dst + 16, tot.B0, tot.B1, tot.B2, tot.St);
+      }
+      cluster_sync_all();
+      if (rank != 0) {
+        par ^= 1;
+        continue;
+      }
+      RowAcc part[kGenericMaxCl];
+#pragma unroll
+      for (int j = 0; j < kGenericMaxCl; ++j) {
+        const float* x = sm.xtot[par][j];
+        if (j < cl) part[j] = {x[0], x[2], x[3], x[4], x[5], x[6], x[1], x[7]};
+      }
+      tot = combine_parts<kGenericMaxCl>(part, cl);
+      par ^= 1;
+    }
     if (tid == 0)
       sm.rs = finish_row(tot, zy, uy, y_valid, dref, p.alpha, p.mode,
                          p.row_coef ? p.row_coef + r : nullptr);
@@ -400,28 +413,65 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
 }
 
 template <typename TIn, typename TOut>
-static cudaError_t launch_t(const KlParams& p, bool vec, int grid, cudaStream_t s) {
-  if (vec && p.mode == ADWIN_GRAD_FULL_KL)
-    kl_generic_kernel<TIn, TOut, true, true><<<grid, kGenericThreads, 0, s>>>(p);
-  else if (vec)
-    kl_generic_kernel<TIn, TOut, true, false><<<grid, kGenericThreads, 0, s>>>(p);
+static cudaError_t launch_t(const KlParams& p, bool vec, int cl, int clusters, cudaStream_t s) {
+  const bool mom = p.mode == ADWIN_GRAD_FULL_KL;
+  void (*kernel)(KlParams, int);
+  if (cl > 1)
+    kernel = !vec ? kl_generic_kernel<TIn, TIn, false, true, true>
+             : mom ? kl_generic_kernel<TIn, TIn, true, true, true> : kl_generic_kernel<TIn, TIn, true, false, true>;
   else
-    kl_generic_kernel<TIn, TOut, false, true><<<grid, kGenericThreads, 0, s>>>(p);
-  return cudaGetLastError();
+    kernel = !vec ? kl_generic_kernel<TIn, TOut, false, true, false>
+             : mom ? kl_generic_kernel<TIn, TOut, true, true, false> : kl_generic_kernel<TIn, TOut, true, false, false>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(clusters * cl);
+  cfg.blockDim = dim3(kGenericThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cl > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, p, cl);
+}
+
+// CTAs per row of a read-only call.  A call of few rows leaves SMs idle or fills its last wave badly; a
+// cluster per row makes shorter waves, at a price (one cluster barrier and one more start per row)
+// that weighs the more the shorter the row.  Both are put in waves of whole rows; the price was
+// fitted to these times (us, one / two / four CTAs per row; `rows` is all the call may hold, the
+// lengths are on the device):
+//   bf16 V = 151 936:  64 rows 46 / 29 / 20   300 56 / 45 / 46   900 117 / 108 / 107   1500 154 / 158 / 167
+//   fp32 V =  93 534: 100 rows 69 / 41 / 26   300 73 / 50 / 54   600  88 /  96 /  87    945 164 / 145 / 136
+//   bf16 V =  32 000:  64 rows 17 / 15 / 13   300 19 / 18 / 23   900  34 /  39 /  50   4000  95 / 126 / 185
+static int split_rows(int64_t rows, int64_t row_bytes, int sm_count) {
+  const int64_t slots = (int64_t)sm_count * kGenericMinBlocks;
+  const double price = 0.15 * (512 << 10) / (double)row_bytes;
+  int best = 1;
+  double cost = 0.0;
+  for (int cl = 1, lg = 0; cl <= kGenericMaxCl; cl *= 2, ++lg) {
+    const double c = (double)((rows * cl + slots - 1) / slots) / cl * (1.0 + price * lg);
+    if (cl == 1 || c < cost) {
+      best = cl;
+      cost = c;
+    }
+  }
+  return best;
 }
 
 cudaError_t launch_kl_generic(const KlParams& p, int dtype, int grad_dtype, bool vec, int sm_count,
                               cudaStream_t s) {
   const int64_t rows = p.B * p.T;
   if (rows == 0) return cudaSuccess;
+  const int cl = p.grad ? 1 : split_rows(rows, 2 * p.V * (dtype == ADWIN_F32 ? 4 : 2), sm_count);
   const int64_t cap = (int64_t)sm_count * 64;
   const int grid = (int)(rows < cap ? rows : cap);
   if (dtype == ADWIN_F32) {
-    return grad_dtype == ADWIN_F32 ? launch_t<float, float>(p, vec, grid, s)
-                                   : launch_t<float, __nv_bfloat16>(p, vec, grid, s);
+    return grad_dtype == ADWIN_F32 ? launch_t<float, float>(p, vec, cl, grid, s)
+                                   : launch_t<float, __nv_bfloat16>(p, vec, cl, grid, s);
   }
-  return grad_dtype == ADWIN_F32 ? launch_t<__nv_bfloat16, float>(p, vec, grid, s)
-                                 : launch_t<__nv_bfloat16, __nv_bfloat16>(p, vec, grid, s);
+  return grad_dtype == ADWIN_F32 ? launch_t<__nv_bfloat16, float>(p, vec, cl, grid, s)
+                                 : launch_t<__nv_bfloat16, __nv_bfloat16>(p, vec, cl, grid, s);
 }
 
 }  // namespace adwin

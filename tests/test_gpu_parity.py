@@ -588,3 +588,16 @@ def test_read_only_rows_that_outgrow_their_first_entries(in_dt, V, mode):
             x[0, t, int(batch.tokens[0, t])] = x[0, t].float().max() - 1.0
     run_and_check(batch, grad_dtype=None, grad_mode=mode)
     run_and_check(batch, grad_dtype=None, grad_mode=mode, flags=api.RANGE_FULL)
+
+
+@pytest.mark.parametrize("in_dt,V,rows", [(2, 120000, 20), (2, 120001, 20), (2, 32003, 300), (1, 33, 6), (1, 93534, 20),
+                                          (1, 150001, 160)])
+def test_read_only_rows_split_over_a_cluster(in_dt, V, rows):
+    """Calls of few rows, read only: four, two and one CTAs per row (the lengths leave some clusters
+    without a row), rows off 16-byte boundaries, the last CTA's share shorter than the others'."""
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=rows // 2 + 1, V=V)
+    batch.window = torch.tensor([min(rows // 2, 8), 3], dtype=torch.int32, device=DEV)
+    for t, y in enumerate((0, V // 4 + 1, V - 1)):
+        batch.tokens[1, t] = y
+    for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
+        run_and_check(batch, grad_dtype=None, grad_mode=mode)
