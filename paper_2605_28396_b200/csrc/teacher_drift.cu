@@ -5,12 +5,17 @@
 //   rank[b,t] = 1 + #{k : u_k > u_y}             (rank of the sampled token under the teacher)
 // The entropy is accumulated against a running maximum m as  H = log S + B/S  with
 // S = sum e^(u-m) and B = sum e^(u-m) (m-u): both terms are non-negative, so nothing cancels.
-// The row is read exactly once (2*V bytes of bf16), 16-byte loads, eight in flight per thread.
+// The row is read exactly once (2*V bytes of bf16), 16-byte loads, eight in flight per thread, eight
+// CTAs per SM.  Alone the kernel reads at more than the copy rate; in a series the power cap makes
+// it pay for every instruction, so a group of eight pieces raises the maximum once, maxima and
+// comparisons run on packed bf16 and the sums on packed fp32 (V = 151 936, 12 300 rows of bf16:
+// 617 -> 532 us alone, 720 -> 630 in a series; four loads at twelve CTAs 638, twelve at six 633).
 //
 // worst_rank_kernel / drift_curves_kernel: the running worst rank of every rollout and, from it,
 // the per-position survival fraction S_T^(k) and the mean branching factor.
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
+#include "kl_pairs.cuh"
 
 namespace adwin {
 namespace {
@@ -18,42 +23,94 @@ namespace {
 constexpr int kDriftThreads = 128;
 constexpr int kDriftWarps = kDriftThreads / 32;
 constexpr int kDriftUnroll = 8;
+constexpr int kDriftMinBlocks = 8;   // CTAs per SM the register allocation leaves room for
 constexpr float kLn2 = 0.69314718055994531f;
 
 struct DriftAcc {
-  float m2;   // running maximum of u*log2(e)
-  float S;    // sum 2^(u2 - m2)
-  float Bq;   // sum 2^(u2 - m2) * (m2 - u2)      (in units of log2)
-  int cnt;    // entries strictly above the sampled token's logit
+  float m2;     // running maximum of u*log2(e)
+  f2_t S;       // sum 2^(u2 - m2)                     (even / odd entries apart, as below)
+  f2_t Bq;      // sum 2^(u2 - m2) * (m2 - u2)         (in units of log2)
+  f2_t cnt;     // entries strictly above the sampled token's logit (whole numbers below 2^24)
   __device__ __forceinline__ void reset() {
     m2 = -INFINITY;
-    S = 0.f;
-    Bq = 0.f;
-    cnt = 0;
+    S = Bq = cnt = 0ull;   // the bit pattern of {0.f, 0.f}
+  }
+  // Move the reference up to pm: S' = f S,  B' = f (B + S (m' - m)).
+  __device__ __forceinline__ void raise(float pm) {
+    if (pm > m2) {
+      const f2_t f = splat2((m2 == -INFINITY) ? 0.f : ex2f(m2 - pm));
+      const f2_t shift = splat2((m2 == -INFINITY) ? 0.f : pm - m2);
+      Bq = mul2(f, fma2(S, shift, Bq));
+      S = mul2(S, f);
+      m2 = pm;
+    }
+  }
+  __device__ __forceinline__ void add(f2_t u) {
+    const f2_t d = fma2(u, splat2(-kLog2e), splat2(m2));   // m2 - u2 >= 0
+    float dl, dh;
+    upk2(d, dl, dh);
+    const f2_t e = pk2(ex2f(-dl), ex2f(-dh));
+    S = add2(S, e);
+    Bq = fma2(e, d, Bq);
   }
 };
 
-template <int N>
-__device__ __forceinline__ void drift_piece(const float (&u)[N], float uy, DriftAcc& a) {
-  float pm = u[0];
+// U pieces, the maximum and the comparisons with the sampled token on packed bf16 where the logits
+// are: one slot for two entries.  (Counts of up to 4 U = 32 per half are whole numbers in bf16.)
+template <int U>
+__device__ __forceinline__ void drift_group(const uint4 (&v)[U], float uy, __nv_bfloat16*, DriftAcc& a) {
+  const __nv_bfloat162 y2 = __float2bfloat162_rn(uy);
+  __nv_bfloat162 m = __float2bfloat162_rn(-INFINITY), c = __float2bfloat162_rn(0.f);
 #pragma unroll
-  for (int i = 1; i < N; ++i) pm = fmaxf(pm, u[i]);
-  pm *= kLog2e;
-  if (pm > a.m2) {   // move the reference: S' = f S,  B' = f (B + S (m' - m))
-    const float f = (a.m2 == -INFINITY) ? 0.f : ex2f(a.m2 - pm);
-    const float shift = (a.m2 == -INFINITY) ? 0.f : pm - a.m2;
-    a.Bq = f * fmaf(a.S, shift, a.Bq);
-    a.S *= f;
-    a.m2 = pm;
-  }
+  for (int k = 0; k < U; ++k) {
+    const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    const float d = fmaf(-u[i], kLog2e, a.m2);   // m2 - u2 >= 0
-    const float e = ex2f(-d);
-    a.S += e;
-    a.Bq = fmaf(e, d, a.Bq);
-    a.cnt += (u[i] > uy) ? 1 : 0;
+    for (int j = 0; j < 4; ++j) {
+      const __nv_bfloat162 x = reinterpret_cast<const __nv_bfloat162&>(w[j]);
+      m = __hmax2(m, x);
+      c = __hadd2(c, __hgt2(x, y2));
+    }
   }
+  a.cnt = add2(a.cnt, pk2(__low2float(c), __high2float(c)));
+  a.raise(fmaxf(__low2float(m), __high2float(m)) * kLog2e);
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    f2_t u[4];
+    Pairs<__nv_bfloat16>::make(v[k], u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a.add(u[j]);
+  }
+}
+template <int U>
+__device__ __forceinline__ void drift_group(const uint4 (&v)[U], float uy, float*, DriftAcc& a) {
+  float m = -INFINITY;
+  int c = 0;
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      m = fmaxf(m, __uint_as_float(w[j]));
+      c += __uint_as_float(w[j]) > uy ? 1 : 0;
+    }
+  }
+  a.cnt = add2(a.cnt, pk2((float)c, 0.f));
+  a.raise(m * kLog2e);
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    f2_t u[2];
+    Pairs<float>::make(v[k], u);
+    a.add(u[0]);
+    a.add(u[1]);
+  }
+}
+// One entry.
+__device__ __forceinline__ void drift_entry(float u, float uy, DriftAcc& a) {
+  a.raise(u * kLog2e);
+  const float d = fmaf(u, -kLog2e, a.m2), e = ex2f(-d);
+  a.S = add2(a.S, pk2(e, 0.f));
+  a.Bq = add2(a.Bq, pk2(e * d, 0.f));
+  a.cnt = add2(a.cnt, pk2(u > uy ? 1.f : 0.f, 0.f));
 }
 
 struct DriftScratch {
@@ -62,7 +119,7 @@ struct DriftScratch {
 };
 
 template <typename TIn, bool VEC>
-__global__ void __launch_bounds__(kDriftThreads) teacher_drift_kernel(
+__global__ void __launch_bounds__(kDriftThreads, kDriftMinBlocks) teacher_drift_kernel(
     const void* __restrict__ teacher, int64_t B, int64_t T, int64_t V, int64_t ld,
     const int32_t* __restrict__ tokens, const int32_t* __restrict__ rollout_len,
     float* __restrict__ entropy, int32_t* __restrict__ rank, int32_t* __restrict__ status) {
@@ -103,10 +160,7 @@ __global__ void __launch_bounds__(kDriftThreads) teacher_drift_kernel(
     const int64_t pieces = VEC ? (V - head) / N : V;
     if (VEC) {
       const int64_t edge = tid < head ? tid : (tid >= 32 && tid - 32 < tail) ? V - tail + (tid - 32) : -1;
-      if (edge >= 0) {
-        const float u[1] = {Elem<TIn>::load1(urow, edge)};
-        drift_piece<1>(u, uy, a);
-      }
+      if (edge >= 0) drift_entry(Elem<TIn>::load1(urow, edge), uy, a);
       const uint4* src = reinterpret_cast<const uint4*>(urow + head * sizeof(TIn));
       int64_t i = tid;
       for (; i + (kDriftUnroll - 1) * kDriftThreads < pieces; i += kDriftUnroll * kDriftThreads) {
@@ -114,32 +168,26 @@ __global__ void __launch_bounds__(kDriftThreads) teacher_drift_kernel(
         if (!ADWIN_CHK(head + (i + (kDriftUnroll - 1) * kDriftThreads + 1) * N <= V, status)) break;
 #pragma unroll
         for (int k = 0; k < kDriftUnroll; ++k) v[k] = __ldcs(src + i + k * kDriftThreads);
-#pragma unroll
-        for (int k = 0; k < kDriftUnroll; ++k) {
-          float u[Elem<TIn>::N];
-          Elem<TIn>::unpack(v[k], u);
-          drift_piece<Elem<TIn>::N>(u, uy, a);
-        }
+        drift_group(v, uy, static_cast<TIn*>(nullptr), a);
       }
       for (; i < pieces; i += kDriftThreads) {
-        float u[Elem<TIn>::N];
         if (!ADWIN_CHK(head + (i + 1) * N <= V, status)) break;
-        Elem<TIn>::unpack(__ldcs(src + i), u);
-        drift_piece<Elem<TIn>::N>(u, uy, a);
+        const uint4 v[1] = {__ldcs(src + i)};
+        drift_group(v, uy, static_cast<TIn*>(nullptr), a);
       }
     } else {
       for (int64_t i = tid; i < pieces; i += kDriftThreads) {
         if (!ADWIN_CHK(i < ld, status)) break;
-        float u[1] = {Elem<TIn>::load1(urow, i)};
-        drift_piece<1>(u, uy, a);
+        drift_entry(Elem<TIn>::load1(urow, i), uy, a);
       }
     }
     // warp, then block: bring the partial sums to the common maximum, fixed order
     const float wm = warp_max(a.m2);
     const float f = (a.m2 == -INFINITY) ? 0.f : ex2f(a.m2 - wm);
     const float sh = (a.m2 == -INFINITY) ? 0.f : wm - a.m2;
-    float s = a.S * f, bq = f * fmaf(a.S, sh, a.Bq);
-    int c = a.cnt;
+    const float S = hsum2(a.S);
+    float s = S * f, bq = f * fmaf(S, sh, hsum2(a.Bq));
+    int c = (int)hsum2(a.cnt);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       s += __shfl_xor_sync(0xffffffffu, s, o);

@@ -66,6 +66,20 @@ def test_drift_on_odd_vocabularies_and_strides(V):
     _check(batch, ks=(1, 3))
 
 
+@pytest.mark.parametrize("cfg,V", [(2, 8191), (2, 8192), (2, 8200), (2, 40963), (1, 4095), (1, 4100), (1, 20487)])
+def test_drift_over_whole_groups_of_pieces(cfg, V):
+    """Row lengths around one and several whole groups of loads: rows that rise or fall throughout (the
+    reference moves in every group or never), a token below every other entry (the largest count) and
+    one above them all."""
+    batch = synth.make_batch(cfg, device=DEV, B=2, T=4, V=V)
+    batch.rollout_len = torch.tensor([4, 4], dtype=torch.int32, device=DEV)
+    ramp = torch.linspace(-30.0, 20.0, V, device=DEV).to(batch.teacher.dtype)
+    batch.teacher[0, 0], batch.teacher[0, 1] = ramp, ramp.flip(0)
+    batch.teacher[1, 0, 5], batch.teacher[1, 1, V - 3] = -50.0, 30.0
+    batch.tokens[0, 0], batch.tokens[0, 1], batch.tokens[1, 0], batch.tokens[1, 1] = 0, V // 2, 5, V - 3
+    _check(batch)
+
+
 def test_drift_with_ties_peaks_and_a_token_out_of_range():
     batch = synth.make_batch(2, device=DEV, B=2, T=5, V=8192)
     batch.teacher[0, 0, :] = 1.5                               # uniform: H = log V, every rank 1
