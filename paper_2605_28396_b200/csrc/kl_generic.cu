@@ -185,6 +185,7 @@ __device__ __forceinline__ RowTotals block_combine(const RowAcc& a, BlockScratch
 // SPLIT: read-only rows, each over a cluster of CTAs that take a run of its pieces.
 template <typename TIn, typename TOut, bool VEC, bool MOM, bool SPLIT>
 __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic_kernel(KlParams p, int clusters_of) {
+  chain();
   __shared__ BlockScratch sm;
   constexpr int N = VEC ? Elem<TIn>::N : 1;
   const int64_t rows = p.B * p.T;
@@ -422,18 +423,7 @@ static cudaError_t launch_t(const KlParams& p, bool vec, int cl, int clusters, c
   else
     kernel = !vec ? kl_generic_kernel<TIn, TOut, false, true, false>
              : mom ? kl_generic_kernel<TIn, TOut, true, true, false> : kl_generic_kernel<TIn, TOut, true, false, false>;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(clusters * cl);
-  cfg.blockDim = dim3(kGenericThreads);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cl;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = cl > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, p, cl);
+  return launch_chained(kernel, (unsigned)(clusters * cl), kGenericThreads, 0, cl, s, p, cl);
 }
 
 // CTAs per row of a read-only call.  A call of few rows leaves SMs idle or fills its last wave badly; a

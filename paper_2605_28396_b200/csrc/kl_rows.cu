@@ -91,6 +91,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 template <typename TIn, typename TOut, int NT, bool TM, bool RAG>
 __global__ void __launch_bounds__(NT + 32, 65536 / kRowsRegs / (NT + 32))
 kl_rows_kernel(const KlParams p, const RowsPlan plan) {
+  chain();
   constexpr int N = Elem<TIn>::N;
   constexpr int NP = Pairs<TIn>::NP;
   constexpr int nt = NT, nw = NT / 32, all = NT + 32;
@@ -594,19 +595,8 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   if (e != cudaSuccess) return e;
   const int64_t rows = p.B * p.T;
   if (plan.num_clusters > rows) plan.num_clusters = (int)rows;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(plan.cl * plan.num_clusters);
-  cfg.blockDim = dim3(plan.nt + 32);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = plan.cl;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = plan.cl > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, p, plan);
+  return launch_chained(kernel, (unsigned)(plan.cl * plan.num_clusters), plan.nt + 32, (size_t)smem, plan.cl, s,
+                        p, plan);
 }
 
 }  // namespace

@@ -260,6 +260,7 @@ __device__ __forceinline__ int resident_slot(int j, int nres, int nch) {
 
 template <typename TIn, typename TOut, bool TM, bool RAG>
 __global__ void __launch_bounds__(kThreads, 1) kl_staged_kernel(KlParams p, StagedPlan plan) {
+  chain();
   constexpr int N = Elem<TIn>::N;
   constexpr int NP = Pairs<TIn>::NP;
   extern __shared__ __align__(128) char smem[];
@@ -1077,22 +1078,10 @@ cudaError_t launch_staged_t(const KlParams& p, int dtype, int grad_dtype, bool r
 
   StagedKernel kernel = staged_kernel<TIn, TOut>(plan, ragged);
   const int smem = plan_smem_bytes(plan);
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = plan.cl;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   const int64_t rows = p.B * p.T;
   if (plan.num_clusters > rows) plan.num_clusters = (int)rows;
   plan.wait_limit_ns = handshake_wait_limit_ns();
-  cfg.gridDim = dim3(plan.cl * plan.num_clusters);
-  return cudaLaunchKernelEx(&cfg, kernel, p, plan);
+  return launch_chained(kernel, plan.cl * plan.num_clusters, kThreads, (size_t)smem, plan.cl, s, p, plan);
 }
 
 }  // namespace

@@ -138,6 +138,7 @@ struct SegPlan {
 __global__ void __launch_bounds__(1024) lm_plan_kernel(const int32_t* __restrict__ range,
                                                        const int32_t* __restrict__ ewin, int64_t B,
                                                        const SegPlan plan, int64_t* seg) {
+  chain();
   __shared__ int64_t part[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int64_t* out = seg + (int64_t)blockIdx.x * (B + 1);
@@ -220,6 +221,7 @@ __device__ __forceinline__ float copy_dot(const __nv_bfloat16* src, const __nv_b
 // almost surely the peak, where the centred difference is then exactly zero, which keeps the
 // single-sweep squared-norm moments well conditioned.
 __global__ void __launch_bounds__(kGatherThreads) lm_gather_kernel(const GatherParams p, const SegPlan plan) {
+  chain();
   __shared__ int64_t base[kMaxSeg + 1];
   __shared__ float red[2][kGatherThreads / 32];
   if (threadIdx.x == 0) {
@@ -343,6 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 lm_sweep_kernel(const __grid_constant__ CUtensorMap map_hs, const __grid_constant__ CUtensorMap map_ws,
                 const __grid_constant__ CUtensorMap map_ht, const __grid_constant__ CUtensorMap map_wt,
                 const SweepParams p) {
+  chain_wait();
   extern __shared__ uint8_t smem_raw[];
   __shared__ unsigned long long s_best;
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(smem_raw);
@@ -597,6 +600,7 @@ struct MergeParams {
 // why the records are spread over threads: 21 -> 5 us there against 8 threads per row.
 constexpr int kMergeRows = 32;
 __global__ void __launch_bounds__(1024) lm_merge_kernel(const MergeParams p) {
+  chain();
   __shared__ double red[6][32][kMergeRows];
   int64_t lo, hi;
   launch_tiles(p.hdr, p.tile0, p.tile_cap, p.rest, lo, hi);
@@ -714,6 +718,7 @@ struct GradParams {
 // as two full 32-byte sectors.  Bound by memory: 8 bytes read and 2 written per entry.
 template <bool NEED_U>
 __global__ void __launch_bounds__(256, 2) lm_grad_kernel(const GradParams p) {
+  chain();
   int64_t lo, hi;
   launch_tiles(p.hdr, p.tile0, p.tile_cap, 0, lo, hi);
   const int64_t tile = lo + blockIdx.x / p.n_groups;
@@ -791,6 +796,7 @@ __global__ void __launch_bounds__(256, 2) lm_grad_kernel(const GradParams p) {
 __global__ void __launch_bounds__(1024) lm_gsq_kernel(const LmHeader* hdr, const float* __restrict__ q,
                                                       const int32_t* __restrict__ rowdst,
                                                       int n_groups, float* gsq) {
+  chain();
   __shared__ double red[32][kMergeRows];
   const int64_t tile = blockIdx.x / (kBM / kMergeRows);
   if (tile >= hdr->grad_tiles) return;
@@ -868,8 +874,9 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
   gp.hs_c = hs_c;
   gp.ht_c = ht_c;
   gp.status = a.status;
-  lm_plan_kernel<<<plan.n_seg, 1024, 0, s>>>(gp.range, gp.ewin, a.B, plan, seg);
-  lm_gather_kernel<<<(int)(rows_cap < 16384 ? rows_cap : 16384), kGatherThreads, 0, s>>>(gp, plan);
+  launch_chained(lm_plan_kernel, plan.n_seg, 1024, 0, 1, s, gp.range, gp.ewin, a.B, plan, seg);
+  launch_chained(lm_gather_kernel, (unsigned)(rows_cap < 16384 ? rows_cap : 16384), kGatherThreads, 0, 1, s,
+                 gp, plan);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
   CUtensorMap m_hs, m_ws, m_ht, m_wt;
@@ -921,7 +928,7 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
         moments ? launch_pairs(lm_sweep_kernel<true>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp)
                 : launch_pairs(lm_sweep_kernel<false>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp);
     if (r != cudaSuccess) return r;
-    lm_merge_kernel<<<(unsigned)cap * (kBM / kMergeRows), 1024, 0, s>>>(mp);
+    launch_chained(lm_merge_kernel, (unsigned)cap * (kBM / kMergeRows), 1024, 0, 1, s, mp);
     return cudaGetLastError();
   };
   if (!a.want_grad) return statistics(0, L.max_tiles, 2, false, a.gsq != nullptr);
@@ -946,14 +953,14 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
     gr.tile0 = t0;
     gr.tile_cap = cap;
     const unsigned grid = (unsigned)(cap * L.grad_groups);
-    if (a.mode == ADWIN_GRAD_FULL_KL) lm_grad_kernel<true><<<grid, 256, 0, s>>>(gr);
-    else lm_grad_kernel<false><<<grid, 256, 0, s>>>(gr);
+    if (a.mode == ADWIN_GRAD_FULL_KL) launch_chained(lm_grad_kernel<true>, grid, 256, 0, 1, s, gr);
+    else launch_chained(lm_grad_kernel<false>, grid, 256, 0, 1, s, gr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (range_full && (e = statistics(0, L.max_tiles, 1, false, moments)) != cudaSuccess) return e;
   if (a.gsq)
-    lm_gsq_kernel<<<(unsigned)L.max_tiles * (kBM / kMergeRows), 1024, 0, s>>>(hdr, q, rowdst,
-                                                                             L.grad_groups, a.gsq);
+    launch_chained(lm_gsq_kernel, (unsigned)L.max_tiles * (kBM / kMergeRows), 1024, 0, 1, s, hdr, q,
+                   rowdst, L.grad_groups, a.gsq);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
   if (a.dH) {
@@ -1033,6 +1040,7 @@ constexpr int kGramFields = 2 * kMaxCand + 1;
 template <int NB>
 __global__ void __launch_bounds__(kGramThreads, 2) lm_gram_kernel(const float4* __restrict__ bins,
                                                                   int64_t n_vec, double* partial) {
+  chain();
   double acc[2 * NB - 1];
 #pragma unroll
   for (int i = 0; i < 2 * NB - 1; ++i) acc[i] = 0.0;
@@ -1080,8 +1088,8 @@ __global__ void __launch_bounds__(kGramThreads, 2) lm_gram_kernel(const float4* 
 template <int NB>
 void launch_gram(int nb, const float* bins, int64_t n_elem, double* partial, int blocks, cudaStream_t s) {
   if (nb == NB)
-    lm_gram_kernel<NB><<<blocks, kGramThreads, 0, s>>>(reinterpret_cast<const float4*>(bins),
-                                                       n_elem / 4, partial);
+    launch_chained(lm_gram_kernel<NB>, blocks, kGramThreads, 0, 1, s, reinterpret_cast<const float4*>(bins),
+                   n_elem / 4, partial);
   else if constexpr (NB < kMaxSeg)
     launch_gram<NB + 1>(nb, bins, n_elem, partial, blocks, s);
 }
@@ -1092,6 +1100,7 @@ __global__ void __launch_bounds__(1024) lm_align_finish_kernel(
     const double* __restrict__ partial, int n_blocks, CandList cand, double rho_star,
     const int32_t* __restrict__ rollout_len, int64_t B, int64_t T, double* batch_stats,
     int32_t* L_next, int32_t* flags_out) {
+  chain();
   __shared__ double tot[kGramFields];
   __shared__ double ntok[kMaxCand];
   const int K = cand.K, lane = threadIdx.x & 31;
@@ -1201,8 +1210,8 @@ cudaError_t launch_lmhead_weight_align(const void* hs, const void* ws, const voi
                           hdr->seg_kblock, status, sm_count, s);
   if (e != cudaSuccess) return e;
   launch_gram<2>(K + 1, bins, V * ds, partial, A.gram_blocks, s);   // (V and d_s are multiples of 8)
-  lm_align_finish_kernel<<<1, 1024, 0, s>>>(partial, A.gram_blocks, cand, rho_star, rollout_len, B, T,
-                                          batch_stats, L_next, flags_out);
+  launch_chained(lm_align_finish_kernel, 1, 1024, 0, 1, s, partial, A.gram_blocks, cand, rho_star,
+                 rollout_len, B, T, batch_stats, L_next, flags_out);
   return cudaGetLastError();
 }
 

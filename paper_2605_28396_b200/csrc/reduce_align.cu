@@ -110,6 +110,7 @@ __device__ __forceinline__ void window_batch(const WindowArgs& a) {
 }
 
 __global__ void __launch_bounds__(kRedThreads) window_reduce_kernel(const WindowArgs a) {
+  chain();
   __shared__ double sm[kRedWarps][3];
   for (int64_t b = blockIdx.x; b < a.B; b += gridDim.x) window_seq(a, b, sm);
   __syncthreads();
@@ -117,10 +118,11 @@ __global__ void __launch_bounds__(kRedThreads) window_reduce_kernel(const Window
   if (blockIdx.x == 0) window_batch(a);
 }
 __global__ void __launch_bounds__(kRedThreads) window_reduce_seq_kernel(const WindowArgs a) {
+  chain();
   __shared__ double sm[kRedWarps][3];
   for (int64_t b = blockIdx.x; b < a.B; b += gridDim.x) window_seq(a, b, sm);
 }
-__global__ void window_reduce_batch_kernel(const WindowArgs a) { window_batch(a); }
+__global__ void window_reduce_batch_kernel(const WindowArgs a) { chain(); window_batch(a); }
 
 // ---------------------------------------------------------------------------- alignment audit
 __constant__ int32_t kDefaultCandidates[6] = {64, 128, 256, 512, 1024, 2048};
@@ -223,6 +225,7 @@ __device__ __forceinline__ void align_batch(const AlignArgs& a, int* admissible,
 }
 
 __global__ void __launch_bounds__(kRedThreads) probe_align_kernel(const AlignArgs a) {
+  chain();
   __shared__ double sm[kRedWarps][3 * kSlots];
   __shared__ double full;
   __shared__ int admissible[65], degenerate;
@@ -232,11 +235,13 @@ __global__ void __launch_bounds__(kRedThreads) probe_align_kernel(const AlignArg
   if (blockIdx.x == 0) align_batch(a, admissible, &degenerate);
 }
 __global__ void __launch_bounds__(kRedThreads) probe_align_seq_kernel(const AlignArgs a) {
+  chain();
   __shared__ double sm[kRedWarps][3 * kSlots];
   __shared__ double full;
   for (int64_t b = blockIdx.x; b < a.B; b += gridDim.x) align_seq(a, b, sm, &full);
 }
 __global__ void probe_align_batch_kernel(const AlignArgs a) {
+  chain();
   __shared__ int admissible[65], degenerate;
   align_batch(a, admissible, &degenerate);
 }
@@ -247,21 +252,10 @@ cudaError_t launch_reduction(void (*fused)(Args), void (*seq)(Args), void (*batc
                              int batch_threads, const Args& a, cudaStream_t s) {
   if (a.B <= kFusedSeqs) {
     const int ctas = a.B < 1 ? 1 : (int)(a.B < kFusedCtas ? a.B : kFusedCtas);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(kRedThreads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fused, a);
+    return launch_chained(fused, ctas, kRedThreads, 0, ctas, s, a);
   }
-  seq<<<(int)(a.B < 4096 ? a.B : 4096), kRedThreads, 0, s>>>(a);
-  batch<<<1, batch_threads, 0, s>>>(a);
+  launch_chained(seq, (unsigned)(a.B < 4096 ? a.B : 4096), kRedThreads, 0, 1, s, a);
+  launch_chained(batch, 1, batch_threads, 0, 1, s, a);
   return cudaGetLastError();
 }
 

@@ -5,6 +5,7 @@
 // every thread folds a contiguous segment from its end, thread 0 chains the 256 segment results
 // from the last segment backwards, and every thread walks its segment again from the value at its
 // end.  All sums are fp64 in a fixed order, so the result does not depend on the launch.
+#include "adwin_common.cuh"
 #include "adwin_internal.h"
 
 namespace adwin {
@@ -16,6 +17,7 @@ __global__ void __launch_bounds__(kRtgThreads) return_to_go_kernel(
     const float* __restrict__ c, const int32_t* __restrict__ window,
     const int32_t* __restrict__ rollout_len, int64_t T, double gamma, int range_full,
     float* __restrict__ out) {
+  chain();
   __shared__ double seg_val[kRtgThreads];   // G at the segment start if G at its end were 0
   __shared__ double seg_mul[kRtgThreads];   // gamma^(segment length)
   __shared__ double seg_tail[kRtgThreads];  // G just past the segment's end
@@ -62,7 +64,7 @@ cudaError_t launch_return_to_go(const float* logratio, const int32_t* window,
                                 const int32_t* rollout_len, int64_t B, int64_t T, double gamma,
                                 int flags, float* rtg, cudaStream_t s) {
   if (B <= 0 || T <= 0) return cudaSuccess;
-  return_to_go_kernel<<<(unsigned)B, kRtgThreads, 0, s>>>(
+  launch_chained(return_to_go_kernel, (unsigned)B, kRtgThreads, 0, 1, s,
       logratio, window, rollout_len, T, gamma, (flags & ADWIN_RANGE_FULL) ? 1 : 0, rtg);
   return cudaGetLastError();
 }

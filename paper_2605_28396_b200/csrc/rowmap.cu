@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(kMapThreads) rowmap_kernel(
     const int32_t* __restrict__ window, const int32_t* __restrict__ rollout_len, int64_t B,
     int64_t T, int flags, int64_t* offsets, int64_t* offsets_win, int32_t* range, int32_t* ewin,
     float* kl, float* logratio, float* gsq, float* lse_s, float* lse_t, int32_t* status) {
+  chain();
   if (blockIdx.x == 0) {
     __shared__ int64_t part[kMapThreads];
     const int tid = threadIdx.x;
@@ -124,7 +125,7 @@ cudaError_t launch_rowmap(const int32_t* window, const int32_t* rollout_len, int
   int64_t fill_blocks = (n + kMapThreads - 1) / kMapThreads;
   if (fill_blocks > 1024) fill_blocks = 1024;
   if (fill_blocks < 1) fill_blocks = 1;
-  rowmap_kernel<<<(int)(1 + fill_blocks), kMapThreads, 0, s>>>(
+  launch_chained(rowmap_kernel, (unsigned)(1 + fill_blocks), kMapThreads, 0, 1, s,
       window, rollout_len, B, T, flags, reinterpret_cast<int64_t*>(base + w.off_offsets),
       with_window_offsets ? reinterpret_cast<int64_t*>(base + w.off_offsets_win) : nullptr,
       reinterpret_cast<int32_t*>(base + w.off_range), reinterpret_cast<int32_t*>(base + w.off_ewin),
@@ -135,6 +136,7 @@ cudaError_t launch_rowmap(const int32_t* window, const int32_t* rollout_len, int
 // ADWIN_ZERO_TAIL: zero-fill the gradient rows t >= E_b.
 template <typename TOut>
 __global__ void __launch_bounds__(256) zero_tail_kernel(KlParams p) {
+  chain();
   const int64_t rows = p.B * p.T;
   for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
     const int64_t b = r / p.T;
@@ -159,9 +161,9 @@ cudaError_t launch_zero_tail(const KlParams& p, int grad_dtype, cudaStream_t s) 
   if (rows == 0 || p.grad == nullptr) return cudaSuccess;
   const int grid = (int)(rows < 148 * 16 ? rows : 148 * 16);
   if (grad_dtype == ADWIN_F32)
-    zero_tail_kernel<float><<<grid, 256, 0, s>>>(p);
+    launch_chained(zero_tail_kernel<float>, grid, 256, 0, 1, s, p);
   else
-    zero_tail_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(p);
+    launch_chained(zero_tail_kernel<__nv_bfloat16>, grid, 256, 0, 1, s, p);
   return cudaGetLastError();
 }
 

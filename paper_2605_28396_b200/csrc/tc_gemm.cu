@@ -180,6 +180,7 @@ template <bool A_MN, bool B_MN>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const GemmParams p) {
+  chain_wait();
   extern __shared__ uint8_t smem_raw[];
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(smem_raw);
   const uint32_t stage0 = (smem_addr(smem_raw) + kCtrlBytes + 1023u) & ~1023u;
@@ -332,6 +333,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
 // Sums the pieces of the split tiles in order and stores C; a thread owns 8 columns of a row.
 __global__ void __launch_bounds__(128) gemm_reduce_kernel(const GemmParams p, int pairs) {
+  chain();
   const GemmWork w(p, pairs);
   if (w.split == 1) return;
   const int rest = w.m_pairs * p.n_tiles - w.whole;
@@ -371,7 +373,7 @@ cudaError_t launch_gemm(const void* A, int64_t lda, bool a_mn, const void* B, in
   const cudaError_t e = a_mn ? launch_pairs(tc_gemm_kernel<true, true>, sm_count, s, ma, mb, p)
                              : launch_pairs(tc_gemm_kernel<false, true>, sm_count, s, ma, mb, p);
   if (e != cudaSuccess || !p.pieces || p.k_blocks < 2 * kMinPiece) return e;   // (nothing is split)
-  gemm_reduce_kernel<<<sm_count * 4, 128, 0, s>>>(p, sm_count / 2);
+  launch_chained(gemm_reduce_kernel, sm_count * 4, 128, 0, 1, s, p, sm_count / 2);
   return cudaGetLastError();
 }
 

@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kDriftThreads, kDriftMinBlocks) teacher_drift_
     const void* __restrict__ teacher, int64_t B, int64_t T, int64_t V, int64_t ld,
     const int32_t* __restrict__ tokens, const int32_t* __restrict__ rollout_len,
     float* __restrict__ entropy, int32_t* __restrict__ rank, int32_t* __restrict__ status) {
+  chain();
   __shared__ DriftScratch sm;
   constexpr int N = VEC ? Elem<TIn>::N : 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(kDriftThreads, kDriftMinBlocks) teacher_drift_
 __global__ void __launch_bounds__(kDriftThreads) worst_rank_kernel(const int32_t* __restrict__ rank,
                                                                   int64_t T,
                                                                   int32_t* __restrict__ worst) {
+  chain();
   __shared__ int seg_max[kDriftThreads];
   __shared__ int seg_before[kDriftThreads];
   const int64_t b = blockIdx.x;
@@ -267,6 +269,7 @@ __global__ void __launch_bounds__(kDriftThreads) drift_curves_kernel(
     const int32_t* __restrict__ rollout_len, int64_t B, int64_t T, const int32_t* __restrict__ ks,
     int32_t K, double* __restrict__ survival, double* __restrict__ bf_mean,
     int32_t* __restrict__ n_active) {
+  chain();
   const int64_t t = (int64_t)blockIdx.x * kDriftThreads + threadIdx.x;
   if (t >= T) return;
   double bf = 0.0;
@@ -303,8 +306,8 @@ cudaError_t launch_teacher_drift(const void* teacher, int dtype, int64_t B, int6
   int64_t grid = (int64_t)sm_count * 64;
   if (grid > rows) grid = rows;
 #define ADWIN_DRIFT_LAUNCH(TIN, VEC)                                                      \
-  teacher_drift_kernel<TIN, VEC><<<(unsigned)grid, kDriftThreads, 0, s>>>(                \
-      teacher, B, T, V, ld, tokens, rollout_len, entropy, rank, status)
+  launch_chained(teacher_drift_kernel<TIN, VEC>, (unsigned)grid, kDriftThreads, 0, 1, s,   \
+                 teacher, B, T, V, ld, tokens, rollout_len, entropy, rank, status)
   if (dtype == ADWIN_F32) {
     if (vec) ADWIN_DRIFT_LAUNCH(float, true); else ADWIN_DRIFT_LAUNCH(float, false);
   } else {
@@ -319,12 +322,12 @@ cudaError_t launch_drift_curves(const float* entropy, const int32_t* rank,
                                 const int32_t* ks, int32_t K, int32_t* worst, double* survival,
                                 double* bf_mean, int32_t* n_active, cudaStream_t s) {
   if (T <= 0) return cudaSuccess;
-  if (B > 0) worst_rank_kernel<<<(unsigned)B, kDriftThreads, 0, s>>>(rank, T, worst);
+  if (B > 0) launch_chained(worst_rank_kernel, (unsigned)B, kDriftThreads, 0, 1, s, rank, T, worst);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((T + kDriftThreads - 1) / kDriftThreads);
-  drift_curves_kernel<<<blocks, kDriftThreads, 0, s>>>(entropy, worst, rollout_len, B, T, ks, K,
-                                                       survival, bf_mean, n_active);
+  launch_chained(drift_curves_kernel, blocks, kDriftThreads, 0, 1, s, entropy, worst, rollout_len, B, T, ks, K,
+                 survival, bf_mean, n_active);
   return cudaGetLastError();
 }
 

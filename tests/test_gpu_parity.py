@@ -601,3 +601,45 @@ def test_read_only_rows_split_over_a_cluster(in_dt, V, rows):
         batch.tokens[1, t] = y
     for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
         run_and_check(batch, grad_dtype=None, grad_mode=mode)
+
+
+@pytest.mark.parametrize("V,rows", [(4096, 40), (40000, 24)])
+def test_launches_that_overlap_their_predecessor(V, rows):
+    """Kernels of a call are set up while the one before drains: calls in a row over the same buffers and
+    workspace, on two streams and replayed from a graph, leave the bits that separate calls leave."""
+    batches = [synth.make_batch(2, device=DEV, seed=s, B=2, T=rows // 2, V=V) for s in (1, 2)]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+
+    def call(batch, o=None, ws=None):
+        grad = o.grad if o else torch.zeros_like(batch.student)
+        o = api.adwin_opd_kl_fwd_bwd(batch.student, batch.teacher, batch.tokens, batch.window,
+                                     batch.rollout_len, grad=grad, out=o, workspace=ws)
+        return o, api.adwin_window_reduce(o.kl, o.logratio, o.gsq, batch.window, batch.rollout_len)
+
+    def bits(o, red):
+        return [x.clone() for x in (o.kl, o.logratio, o.gsq, o.grad, *red)]
+
+    want = []
+    for b in batches:
+        want.append(bits(*call(b)))
+        torch.cuda.synchronize()
+    got = [[], []]
+    for i, s in enumerate(streams):
+        ws = torch.empty(1 << 16, dtype=torch.uint8, device=DEV)
+        with torch.cuda.stream(s):
+            s.wait_stream(torch.cuda.default_stream())
+            o = None
+            for n in range(12):           # the other batch first: its results are overwritten
+                o, red = call(batches[(n + i + 1) % 2], o, ws)
+            got[i] = bits(o, red)
+    torch.cuda.synchronize()
+    for i in (0, 1):
+        assert all(torch.equal(a, b) for a, b in zip(got[i], want[i]))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        o, red = call(batches[0])
+        o, red = call(batches[1], o)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(bits(o, red), want[1]))
