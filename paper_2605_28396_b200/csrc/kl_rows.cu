@@ -8,9 +8,9 @@
 // memory (tcgen05.st / tcgen05.ld) -- so between the sweeps the threads only exchange sums.  One more
 // warp does what is done once per row: it adds up the threads' sums, derives the row's scalars and
 // hands them back (the others would otherwise each spend ~300 issue slots on it, as much as a
-// tenth of a row of 32 000 entries), fetches the next row's metadata, and while the others are
-// in the second sweep it has the next row brought into L2 (cp.async.bulk.prefetch.L2), so that HBM
-// stays busy during both sweeps and the loads of the first sweep come from L2.
+// tenth of a row of 32 000 entries) and fetches the coming rows' metadata.  The next row is brought
+// into L2 meanwhile (cp.async.bulk.prefetch.L2), so that HBM stays busy during both sweeps and the
+// loads of the first sweep come from L2.
 //
 // Exponentials are taken against a reference that the whole row shares (the logit of the sampled
 // token), so partial sums add without rescaling.  If the sums overflow it (a sampled token more than
@@ -125,6 +125,21 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     return a;
   };
 
+  // The next row is brought into L2 ahead of its first sweep: bf16 rows by the row's warp, all at once
+  // when the second sweep of this row begins; fp32 rows, which memory bounds and not arithmetic, by
+  // thread 0 of the others, one array's part of a group at each group of either sweep, so that HBM has an
+  // even load (fp32 V = 32 000: 200 us before, 193 so; bf16, where thread 0's extra work holds its CTA
+  // up: 194 us against 202).
+  constexpr bool kSpread = sizeof(TIn) == 4;
+  auto prefetch = [&](int64_t r, const void* base, int from, int count) {
+    const RowSpan sn = span_of(r);
+    const int n = min(sn.pieces - from, count);
+    if (n > 0)
+      prefetch_l2(static_cast<const char*>(base) +
+                      ((size_t)r * p.ld - sn.shift + (size_t)(piece0 + from) * N) * sizeof(TIn),
+                  (uint32_t)n * 16u);
+  };
+
   if (TM) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (cl > 1) cluster_sync_all();   // peers run before anything is stored into them
   __syncthreads();
@@ -135,9 +150,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     RowCursor cur;
     cur.init(p);
     bool wg_unused;
-    int64_t r = 0;     // row i, then row i+1
     auto fetch = [&](int64_t i) {   // metadata of row i into its slot
-      r = cur.locate(p, cluster_id + i * plan.num_clusters, wg_unused);
+      const int64_t r = cur.locate(p, cluster_id + i * plan.num_clusters, wg_unused);
       if (lane == 0) {
         RowsMeta& m = ctrl.meta[i % kMetaDepth];
         const int y = p.tokens[r];
@@ -147,14 +161,14 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         m.w = p.row_coef ? p.row_coef[r] : 0.f;
       }
     };
-    if (my_rows > 0) fetch(0);
+    constexpr int kAheadRows = kSpread ? 2 : 1;
+    for (int64_t i = 0; i < kAheadRows && i < my_rows; ++i) fetch(i);
     __syncthreads();
     int64_t r_prev = 0;
     for (int64_t i = 0; i < iters; ++i) {
       const bool real = i < my_rows, more = i + 1 < my_rows;
       const int par = (int)(i & 1);
-      const int64_t ri = r;
-      if (more) fetch(i + 1);
+      if (i + kAheadRows < my_rows) fetch(i + kAheadRows);
       named_sync(kPosted, all);
       // fixed-order sums over the threads, then over the CTAs
       float v[4] = {0.f, 0.f, 0.f, 0.f};
@@ -178,6 +192,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = v[3];
       if (!real) break;
       const RowsMeta& m = ctrl.meta[i % kMetaDepth];
+      const int64_t ri = m.r;
       RowTotals t;
       t.M2s = m.zy * kLog2e;
       t.M2t = m.uy * kLog2e;
@@ -233,13 +248,9 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       }
       named_sync(kReady, all);
       if (lane == 0) {
-        if (more) {
-          const RowSpan sn = span_of(r);
-          const size_t off = ((size_t)r * p.ld - sn.shift + (size_t)piece0 * N) * sizeof(TIn);
-          if (sn.pieces > 0) {
-            prefetch_l2(static_cast<const char*>(p.student) + off, (uint32_t)sn.pieces * 16u);
-            prefetch_l2(static_cast<const char*>(p.teacher) + off, (uint32_t)sn.pieces * 16u);
-          }
+        if (!kSpread && more) {
+          prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, p.student, 0, plan.per_rank);
+          prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, p.teacher, 0, plan.per_rank);
         }
         if (rank == 0) {
           p.kl[ri] = rs.kl;
@@ -266,6 +277,13 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     for (int64_t i = 0; i < iters; ++i) {
       const bool real = i < my_rows;
       const RowsMeta& m = ctrl.meta[real ? i % kMetaDepth : 0];
+      const bool ahead = kSpread && tid == 0 && i + 1 < my_rows;
+      int part = 0;
+      auto prefetch_part = [&]() {
+        prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, (part & 1) ? p.teacher : p.student,
+                 (part >> 1) * kU * nt, kU * nt);
+        ++part;
+      };
       RowSpan span = {0, 0, -1, -1, N};
       Acc2 a;
       a.reset();
@@ -281,6 +299,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         auto group = [&](auto full, int k0) {
           constexpr bool FULL = decltype(full)::value;
           uint4 z[kU], u[kU];
+          if (ahead) prefetch_part();
 #pragma unroll
           for (int h = 0; h < kU; ++h) {
             if ((FULL || lp0 + h * nt < span.pieces) &&
@@ -389,6 +408,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       auto group = [&](auto full, int k0) {
         constexpr bool FULL = decltype(full)::value;
         uint4 z[kU], u[kU];
+        if (ahead) prefetch_part();
         if (TM && k0 < plan.tm_steps) {
 #pragma unroll
           for (int h = 0; h < kU; ++h) tm_load8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
