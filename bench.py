@@ -1,7 +1,7 @@
 #!/usr/bin/env python
 """Benchmark of the windowed OPD divergence hot path (one JSON line on stdout).
 
-A step = one pass of the whole path over one synthetic batch: row map, the staged fwd+bwd kernel
+A step = one pass of the whole path over one synthetic batch: row map, the fwd+bwd row kernel
 (log-sum-exp of both rows, reverse KL, sampled-token log-ratio, gradient, window skip), the
 windowed reductions and the alignment audit.  The workload is config 3 of the paper-shaped
 recipes in ``paper_2605_28396_b200/synth.py`` (Qwen3-scale vocabulary, reasoning-length rollouts).
@@ -32,7 +32,7 @@ UNIT = "tokens/s"
 WORKLOAD = ("config3: B=16 T=2048 V=151936 bf16 logits (student N(0,4)+10*Bern(0.05), teacher = "
             "student+N(0,2)), W_b in {256,512,1024,2048} x4, tokens ~ student softmax, "
             "FULL_KL gradient stored bf16, rows past the window skipped")
-LAUNCHES_PER_STEP = 7   # rowmap, staged kernel, 2 window-reduce kernels, 3 audit kernels
+LAUNCHES_PER_STEP = 4   # row map, row kernel, window reduce, audit
 
 
 def parse():
@@ -68,7 +68,7 @@ def measured_peak():
     return 6650.0, "fallback 6.65 TB/s (of fallback)"
 
 
-# DRAM bytes READ per processed row of the staged kernel, from the committed ncu capture of a
+# DRAM bytes READ per processed row of the row kernel, from the committed ncu capture of a
 # small case (960 rows), valid for the kernel source with this fingerprint.  The capture's write
 # counter is not scaled: the last ~56 MB of a launch's gradient are still in L2 when the kernel
 # ends, a residue bounded by the L2 size that does not grow with the rows, so at full size the
@@ -82,7 +82,7 @@ def recorded_traffic(rows, V):
     None once the kernel source has changed since the counters were taken."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("kl_staged.cu", "adwin_common.cuh"):
+    for f in ("kl_rows.cu", "kl_pairs.cuh", "adwin_common.cuh"):
         h.update((ROOT / "paper_2605_28396_b200" / "csrc" / f).read_bytes())
     if h.hexdigest()[:16] != TRAFFIC_KERNEL_SHA:
         return None
@@ -363,7 +363,7 @@ def run_ours(args):
                      "clocks": sus_clk}
 
     # ---- scalars for every t < R_b and the gradient inside the window, one call (default dispatch:
-    # the staged kernel over the window rows, the streaming kernel over the rest of every rollout)
+    # the row kernel over the window rows, the streaming kernel over the rest of every rollout)
     n2_line = None
     if side:
         ws2 = torch.empty(api.adwin_workspace_bytes(B, T, V), dtype=torch.uint8, device=dev)
@@ -383,7 +383,7 @@ def run_ours(args):
                    "frac_of_measured_peak": n2bytes / (n2ms * 1e-3) / 1e9 / peak_n2,
                    "launches_per_step": 3, "steps": 5,
                    "path": "adwin_opd_kl_fwd_bwd (RANGE_FULL with gradient: rowmap, "
-                           "kl_staged_kernel over t < E_b, kl_generic_kernel over E_b <= t < R_b)"}
+                           "kl_rows_kernel over t < E_b, kl_generic_kernel over E_b <= t < R_b)"}
 
     rtg_line = None
     if side:
@@ -450,7 +450,7 @@ def run_ours(args):
         probe_line = {"ms_per_step": pms, "positions": prows, "tokens_per_s": prows / (pms / 1e3),
                       "algorithmic_bytes": pbytes, "achieved_gbs": pbytes / (pms * 1e-3) / 1e9,
                       "frac_of_measured_peak": pbytes / (pms * 1e-3) / 1e9 / peak_p,
-                      "launches_per_step": 2 + 3, "steps": n_probe,
+                      "launches_per_step": 2 + 1, "steps": n_probe,
                       "path": "adwin_opd_kl_fwd_bwd (RANGE_FULL, no gradient: kl_generic_kernel) "
                               "-> adwin_probe_align (timed together)"}
         if int(status.item()):
@@ -512,7 +512,7 @@ def run_ours(args):
                      "tokens_per_s": c4rows / (c4ms / 1e3), "algorithmic_bytes": c4bytes,
                      "achieved_gbs": c4bytes / (c4ms * 1e-3) / 1e9,
                      "frac_of_measured_peak": c4bytes / (c4ms * 1e-3) / 1e9 / peak_4,
-                     "launches_per_step": 2 + 3, "steps": 5,
+                     "launches_per_step": 2 + 1, "steps": 5,
                      "path": "adwin_opd_kl_fwd_bwd (RANGE_FULL, no gradient: kl_generic_kernel) "
                              "-> adwin_probe_align (timed together)"}
         del b4, ws4, o4
@@ -649,7 +649,7 @@ def run_ours(args):
                    "parallelism": f"dp{world} (independent batches per rank, no collective)"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
-                     "kernel": "kl_staged_kernel<bf16,bf16> (timed with the row-map kernel it "
+                     "kernel": "kl_rows_kernel<bf16,bf16> (timed with the row-map kernel it "
                                "follows, < 0.5 % of the interval)",
                      "kernel_ms": kernel_ms, "algorithmic_bytes": alg_bytes,
                      "frac_of_nominal_8TBps": achieved / 8000.0},

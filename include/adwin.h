@@ -136,10 +136,10 @@ size_t adwin_workspace_bytes(int64_t B, int64_t T, int64_t V, int dtype, int fla
  * workspace    : >= adwin_workspace_bytes(...) bytes, 256-byte aligned; contents undefined after
  * dev_status   : one int32 the caller zeroed; bits are OR-ed in
  *
- * Two kernels do the work, with identical results up to rounding order.  Rows whose gradient is
- * written go to the staged cluster kernel (two sweeps with the row kept on chip), which needs
- * 16-byte aligned logits / gradient base pointers, row strides that are multiples of 16 bytes and
- * V*sizeof(element) a multiple of 16.  Rows without gradient (a call with grad_student == NULL,
+ * Several kernels do the work, with identical results up to rounding order.  Rows whose gradient is
+ * written are kept on chip between two sweeps (row kernel, staged cluster kernel beyond its sizes);
+ * that needs logits / gradient base pointers on 16-byte boundaries and, where ld_grad differs from
+ * ld, row strides that are multiples of 16 bytes.  Rows without gradient (a call with grad_student == NULL,
  * or the rows past the window of an ADWIN_RANGE_FULL call) and every other layout go to the
  * streaming kernel, one CTA per row.  ADWIN_FORCE_GENERIC / ADWIN_FORCE_STAGED override the choice.
  */

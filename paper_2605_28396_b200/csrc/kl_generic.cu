@@ -7,7 +7,7 @@
 // alignment.  VEC: the rows of all arrays share one offset from a 16-byte boundary (always so when
 // the arrays start on one and have one stride), and everything but the at most N - 1 entries before
 // the first boundary and after the last is moved 16 bytes at a time; otherwise entry by entry.
-// Calls without gradient come here, and layouts that the staged cluster kernel does not take.
+// Calls without gradient come here, and layouts that the row kernel does not take.
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
 #include "kl_pairs.cuh"
