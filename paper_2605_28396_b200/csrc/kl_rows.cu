@@ -499,13 +499,13 @@ struct RowsShape {
 // is used: the most CTAs per SM, because their number is what hides one row's exchange behind the
 // others' streaming.  Tensor memory is shared out in powers of two.  Measured over 2.4 GB of logits
 // and gradient (367 us at the copy rate; staged kernel / two sweeps over memory / this kernel):
-//   bf16  V =   4 096  2488 /  993 / 476 us  {8, 64}       fp32  V =   4 096  1247 / 599 / 411 us  {5, 128}
-//              8 192  1353 /  755 / 445     {5, 128}               12 000   790 / 604 / 421      {3, 224}
-//             16 384   993 /  625 / 484     {3, 224}               16 384   600 / 679 / 421      {2, 352}
-//             32 000   726 /  822 / 473     {2, 352}               32 000   510 / 733 / 459      {2, 352} x 2
-//             50 264   638 /  980 / 500     {2, 352}               50 264   597 / 772 / 465      {2, 352} x 2
-//            100 000   656 / 1019 / 513     {2, 352} x 2           65 536   521 / 766 / 454      {2, 352} x 4
-//            151 936   573 / 1012 / 557     {2, 352} x 4
+//   bf16  V =   4 096  2471 / 726 / 475 us  {8, 64}       fp32  V =   4 096  1245 / 454 / 398 us  {5, 128}
+//              8 192  1345 / 594 / 439     {5, 128}               12 000   784 / 606 / 401      {3, 224}
+//             16 384   987 / 556 / 480     {3, 224}               16 384   599 / 647 / 394      {2, 352}
+//             32 000   722 / 814 / 470     {2, 352}               32 000   500 / 686 / 429      {2, 352} x 2
+//             50 264   636 / 856 / 499     {2, 352}               50 264   597 / 719 / 474      {2, 352} x 2
+//            100 000   653 / 908 / 512     {2, 352} x 2           65 536   503 / 711 / 431      {2, 352} x 4
+//            151 936   568 / 852 / 550     {2, 352} x 4
 // bf16 rows are bound by arithmetic and latency (19 issue slots per entry, the ex2 unit 57 % busy),
 // fp32 rows by memory.  Three or four steps in flight spill at 80 registers and lose, one step at 64
 // registers and a third more threads is slower except around 16 384 entries.

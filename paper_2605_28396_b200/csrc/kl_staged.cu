@@ -1,6 +1,6 @@
 // Staged cluster kernel: each logit byte is read from HBM once.  It takes rows with gradient that are
-// too long for the row kernel's plans (kl_rows.cu, which is the faster one up to there: 473 us
-// against 726 for 2.4 GB at V = 32 000, 557 against 573 at 151 936), and, under
+// too long for the row kernel's plans (kl_rows.cu, which is the faster one up to there: 470 us
+// against 722 for 2.4 GB at V = 32 000, 550 against 568 at 151 936), and, under
 // ADWIN_FORCE_STAGED, every call.
 //
 // A thread-block cluster of CL CTAs (one CTA per SM) owns one processed row at a time; CTA `rank`
