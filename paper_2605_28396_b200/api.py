@@ -126,6 +126,8 @@ def _ptr(t):
 
 
 def _stream(device):
+    if device.type != "cuda":   # a host address must not reach a kernel
+        raise ValueError(f"Expected a cuda device, but got: {device}")
     i = device.index
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
 

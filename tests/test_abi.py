@@ -5,6 +5,7 @@ import re
 from pathlib import Path
 
 import pytest
+import torch
 
 from paper_2605_28396_b200 import api, build
 
@@ -165,3 +166,33 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(api, "LIB_PATH", tmp_path / "nope.so")
     with pytest.raises(FileNotFoundError):
         api.lib()
+
+
+def test_tensors_in_host_memory_are_refused_before_the_library_is_called(monkeypatch):
+    """Every entry point on device tensors, given tensors in host memory: an error, and no call that
+    would hand their addresses to a kernel."""
+    real = api.lib()
+
+    class Guard:      # sizes may be asked for; anything else is a call that should not happen
+        def __getattr__(self, name):
+            if name.endswith("_bytes"):
+                return getattr(real, name)
+            return lambda *a: pytest.fail(f"{name} called with host tensors")
+
+    monkeypatch.setattr(api, "_lib", Guard())
+    x = torch.zeros(2, 3)
+    n = torch.full((2,), 3, dtype=torch.int32)
+    y, z = torch.zeros(2, 3, dtype=torch.int32), torch.zeros(2, 3, 16)
+    h, w = torch.zeros(2, 3, 8, dtype=torch.bfloat16), torch.zeros(16, 8, dtype=torch.bfloat16)
+    status = torch.zeros(1, dtype=torch.int32)
+    calls = [lambda: api.adwin_window_reduce(x, x, x, n),
+             lambda: api.adwin_probe_align(x, x, x, n),
+             lambda: api.adwin_return_to_go(x, n),
+             lambda: api.adwin_drift_curves(x, y, ks=n),
+             lambda: api.adwin_opd_kl_fwd_bwd_no_alloc(z, z, y, n, n, grad=None, kl=x, logratio=x,
+                                                       gsq=x, dev_status=status),
+             lambda: api.adwin_opd_kl_lmhead_fwd_bwd(h, w, h, w, y, n),
+             lambda: api.adwin_lmhead_weight_align(h, w, h, w, y)]
+    for call in calls:
+        with pytest.raises(ValueError, match="cuda device"):
+            call()
