@@ -389,3 +389,16 @@ def test_rows_packed_across_sequences_at_tile_edges(windows):
     for flags, bound in ((0, rows), (api.RANGE_FULL, 0)):
         got = run(batch, flags=flags, max_rows=bound)
         check_all(batch, got, oracle(batch, api.GRAD_FULL_KL, flags), flags)
+
+
+@pytest.mark.parametrize("mode", [api.GRAD_FULL_KL, api.GRAD_SAMPLED])
+def test_large_logits_past_the_window_leave_the_weight_gradient_alone(mode):
+    """Rows without gradient share the last tile of those with: one whose logits are beyond what an
+    exponential in fp32 holds (all of them shifted, which changes neither policy) adds nothing to dW."""
+    batch = synth.make_lmhead_batch(DEV, B=2, T=40, V=1000, d_s=128, d_t=72, w_std=0.12)
+    batch.window = torch.tensor([20, 7], dtype=torch.int32, device=DEV)
+    batch.w_student[:, 0] = 1.0
+    batch.hidden_student[:, :, 0] = 0.0
+    batch.hidden_student[0, 25, 0], batch.hidden_student[1, 39, 0] = 150.0, 100.0
+    got = run(batch, mode=mode, flags=api.RANGE_FULL)
+    check_all(batch, got, oracle(batch, mode, api.RANGE_FULL), api.RANGE_FULL, mode=mode)
