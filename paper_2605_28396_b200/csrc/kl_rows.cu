@@ -24,6 +24,7 @@
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
 #include "kl_pairs.cuh"
+#include "tc_pipeline.cuh"
 
 namespace adwin {
 namespace {
@@ -513,14 +514,16 @@ constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 1 << 20},   {5, 128, 0, 1, 1 << 2
                                  {3, 224, 128, 1, 100},    {2, 352, 256, 1, 1 << 20},
                                  {2, 352, 256, 2, 1 << 20}, {2, 352, 256, 4, 1 << 20}};
 
-bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
+constexpr int shape_smem(int ctas) { return kSmemPerSm / ctas - kSmemReserved; }
+
+constexpr bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
   plan.cl = sh.cl;
   plan.nt = sh.nt;
   plan.ctas = sh.ctas;
   plan.per_rank = (int)((pieces + sh.cl - 1) / sh.cl);
   const int need = (plan.per_rank + sh.nt - 1) / sh.nt;
   plan.steps = (need + kU - 1) / kU * kU;
-  const int smem = kSmemPerSm / sh.ctas - kSmemReserved - rows_ctrl_bytes(sh.nt);
+  const int smem = shape_smem(sh.ctas) - rows_ctrl_bytes(sh.nt);
   const int sm_steps = smem / (32 * sh.nt) / kU * kU;
   // a lane group's columns are shared by its warps (every fourth); a piece pair takes 8 columns
   const int tm_most = sh.tm_cols ? sh.tm_cols / ((sh.nt + 127) / 128) / 8 / kU * kU : 0;
@@ -529,9 +532,33 @@ bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
   return plan.steps - plan.tm_steps <= sm_steps;
 }
 
-int rows_smem(const RowsPlan& plan) {
+constexpr int rows_smem(const RowsPlan& plan) {
   return rows_ctrl_bytes(plan.nt) + (plan.steps - plan.tm_steps) * 32 * plan.nt;
 }
+
+// Bytes a launch asks for.  The CTAs of a cluster hold tensor memory while they wait for one another,
+// and tcgen05.alloc waits without a limit: beside a tensor-core kernel of another stream (CTA pairs
+// with all 512 columns), a cluster and a pair could each hold an SM's columns and wait for the other's.
+// So the CTAs of a cluster take at least kClusterSmem: no CTA of tc_pipeline.cuh (199 KB), nor any
+// above 163 KB, fits on an SM beside one, and row CTAs among themselves never need more than 512
+// columns.  (A CTA without a cluster waits for nobody once it has its columns.)  Not the whole share of
+// an SM, which would leave 28 KB of L1 to the streaming kernel that follows in a call with scalars
+// over the rollout (update and audit on 3.8 GB of logits 1215 us so, 1164 with this).
+constexpr int kClusterSmem = 65536 - kSmemReserved;
+constexpr int launch_smem(const RowsPlan& plan) {
+  const int need = rows_smem(plan);
+  return plan.cl > 1 && plan.tm_cols > 0 && need < kClusterSmem ? kClusterSmem : need;
+}
+constexpr bool clusters_exclude_tensor_core_ctas() {
+  for (const RowsShape& sh : kShapes) {
+    RowsPlan plan = {};
+    for (int64_t pieces = sh.cl; sh.cl > 1 && shape_plan(sh, pieces, plan); pieces += sh.cl * sh.nt * kU)
+      if (plan.tm_cols > 0 && launch_smem(plan) + tc::kSmemBytes + 2 * kSmemReserved <= kSmemPerSm)
+        return false;
+  }
+  return true;
+}
+static_assert(clusters_exclude_tensor_core_ctas(), "a cluster could wait for a pair's tensor memory");
 
 bool rows_plan(int64_t pieces, RowsPlan& plan) {
   if (pieces < 1 || pieces > (int64_t)1 << 24) return false;
@@ -602,8 +629,8 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   if (!rows_plan(ragged ? (p.V + 2 * N - 2) / N : p.V / N, plan)) return cudaErrorNotSupported;
   const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, plan.tm_cols > 0, ragged);
   if (!kernel) return cudaErrorNotSupported;
-  const int smem = rows_smem(plan);
-  const int most = kSmemPerSm / plan.ctas - kSmemReserved;
+  const int smem = launch_smem(plan);
+  const int most = shape_smem(plan.ctas);
   plan.num_clusters = plan.ctas * sm_count;
   cudaError_t e;
   if (plan.cl > 1) {
