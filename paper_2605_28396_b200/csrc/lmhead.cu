@@ -595,7 +595,8 @@ struct MergeParams {
 // against common references (fixed order) and derive the per-token outputs and the gradient
 // coefficients:
 //   g_k = p_k (a1 (z_k - u_k) + a0) (+ gy at k = y),   p_k = 2^(z_k log2e - L2s);
-// a row without gradient has L2s = infinity.
+// a row without gradient has L2s = infinity: p_k, and g_k with a1 = a0 = gy = 0, are exactly zero
+// whatever its logits (with L2s = 0, p_k overflows beyond z = 88 and 0 * inf spreads over dW).
 // Records are read with the row as the fast index (whole 128-byte lines), reduced with the record
 // as the lane.  A short call has many records (126 for each of 225 rows at V = 32 000), which is
 // why the records are spread over threads: 21 -> 5 us there against 8 threads per row.
@@ -733,9 +734,6 @@ __global__ void __launch_bounds__(256, 2) lm_grad_kernel(const GradParams p) {
   int c0, c1;
   group_chunks(p.n_chunks, p.n_groups, g, c0, c1);
   const bool sectors = p.ldG % 16 == 0;   // 32 columns of a row are two whole 32-byte sectors
-  // Rows without gradient in a tile of rows with: their entries are exactly zero whatever their logits
-  // (2^(z log2e) overflows beyond z = 88, and 0 * inf would spread over dW), so these are not read.
-  const bool none = L2s == INFINITY;
   float q = 0.f;
   for (int c = c0; c < c1; ++c) {
     const float4* zp = p.keep + ((tile - lo) * p.n_chunks + c) * (2 * kKeepArray) +
@@ -748,8 +746,8 @@ __global__ void __launch_bounds__(256, 2) lm_grad_kernel(const GradParams p) {
       float4 z4[8], u4[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        z4[i] = none ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldcs(zp + (j * 8 + i) * kBM);
-        if (NEED_U) u4[i] = none ? z4[i] : __ldcs(zp + kKeepArray + (j * 8 + i) * kBM);
+        z4[i] = __ldcs(zp + (j * 8 + i) * kBM);
+        if (NEED_U) u4[i] = __ldcs(zp + kKeepArray + (j * 8 + i) * kBM);
       }
       float v[32];
 #pragma unroll
