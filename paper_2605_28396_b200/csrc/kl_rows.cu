@@ -19,7 +19,6 @@
 // CTA of the cluster.
 #include <mutex>
 #include <type_traits>
-#include <vector>
 
 #include "adwin_common.cuh"
 #include "adwin_internal.h"
@@ -585,23 +584,22 @@ RowsKernel rows_kernel(int nt, bool tm, bool ragged) {
 }
 
 // Clusters of `cl` CTAs that the GPU holds at a time (some SMs of a GPC are left over when `cl` does
-// not divide their number).  The occupancy query counts one CTA per SM for kernels that allocate
-// tensor memory, so it is asked about the same kernel without.
-cudaError_t resident_clusters(RowsKernel like, const RowsPlan& plan, int smem, int sm_count, int& n) {
-  struct Key {
-    int dev, nt, ctas, cl, n;
-  };
+// not divide their number), kept per device.  The occupancy query counts one CTA per SM for kernels
+// that allocate tensor memory, so it is asked about a kernel of the same shape without; which one does
+// not matter, their launch bounds leave all of them the shape's CTAs per SM.
+cudaError_t resident_clusters(const RowsPlan& plan, int sm_count, int& n) {
+  constexpr int kDevices = 64;
   static std::mutex mu;
-  static std::vector<Key> seen;
+  static int seen[kDevices][kRowsMaxCl + 1];   // (shapes with a cluster differ in `cl` alone)
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kDevices) return cudaErrorNotSupported;
   std::lock_guard<std::mutex> lock(mu);
-  for (const Key& k : seen)
-    if (k.dev == dev && k.nt == plan.nt && k.ctas == plan.ctas && k.cl == plan.cl) {
-      n = k.n;
-      return cudaSuccess;
-    }
+  n = seen[dev][plan.cl];
+  if (n > 0) return cudaSuccess;
+  const RowsKernel like = kl_rows_kernel<float, float, kRowsThreads, false, false>;
+  const int smem = shape_smem(plan.ctas);
   e = cudaFuncSetAttribute(like, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -618,9 +616,16 @@ cudaError_t resident_clusters(RowsKernel like, const RowsPlan& plan, int smem, i
   e = cudaOccupancyMaxActiveClusters(&n, like, &cfg);
   if (e != cudaSuccess) return e;
   if (n < 1) return cudaErrorNotSupported;
-  seen.push_back({dev, plan.nt, plan.ctas, plan.cl, n});
+  seen[dev][plan.cl] = n;
   return cudaSuccess;
 }
+constexpr bool cluster_shapes_differ_in_cl_alone() {
+  for (const RowsShape& a : kShapes)
+    for (const RowsShape& b : kShapes)
+      if (a.cl > 1 && b.cl > 1 && (a.nt != kRowsThreads || a.ctas != b.ctas)) return false;
+  return true;
+}
+static_assert(cluster_shapes_differ_in_cl_alone(), "resident_clusters keeps one number per cluster size");
 
 template <typename TIn, typename TOut>
 cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStream_t s) {
@@ -630,15 +635,15 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, plan.tm_cols > 0, ragged);
   if (!kernel) return cudaErrorNotSupported;
   const int smem = launch_smem(plan);
-  const int most = shape_smem(plan.ctas);
   plan.num_clusters = plan.ctas * sm_count;
   cudaError_t e;
   if (plan.cl > 1) {
-    e = resident_clusters(rows_kernel<TIn, TOut>(plan.nt, false, ragged), plan, most, sm_count,
-                          plan.num_clusters);
+    e = resident_clusters(plan, sm_count, plan.num_clusters);
     if (e != cudaSuccess) return e;
   }
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // the shape's whole share whatever this call needs: the limit belongs to the kernel, which launches of
+  // other threads with other row lengths use at the same time
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shape_smem(plan.ctas));
   if (e != cudaSuccess) return e;
   const int64_t rows = p.B * p.T;
   if (plan.num_clusters > rows) plan.num_clusters = (int)rows;

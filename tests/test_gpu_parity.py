@@ -1,5 +1,6 @@
 """GPU parity: the CUDA path (through the C ABI) against the float64 oracle, element by element."""
 import math
+import threading
 
 import numpy as np
 import pytest
@@ -643,3 +644,40 @@ def test_launches_that_overlap_their_predecessor(V, rows):
         graph.replay()
     torch.cuda.synchronize()
     assert all(torch.equal(a, b) for a, b in zip(bits(o, red), want[1]))
+
+
+def test_two_threads_with_vocabularies_of_their_own():
+    """Two host threads that call with different row lengths (the same kernel, different shared memory
+    per launch), each on its own stream: no launch may fail for what the other thread set up.  (Calls
+    of the library itself, back to back: it runs without the interpreter's lock.)"""
+    calls = {}
+    for V in (30000, 50000):
+        batch = synth.make_batch(2, device=DEV, seed=V, B=1, T=2, V=V)
+        batch.window = torch.tensor([2], dtype=torch.int32, device=DEV)
+        out = api.adwin_opd_kl_fwd_bwd(batch.student, batch.teacher, batch.tokens, batch.window,
+                                       batch.rollout_len, grad=torch.zeros_like(batch.student))
+        stream = torch.cuda.Stream()
+        args = (batch.student.data_ptr(), batch.teacher.data_ptr(), api.BF16, 1, 2, V, V,
+                batch.tokens.data_ptr(), batch.window.data_ptr(), batch.rollout_len.data_ptr(), 1.0,
+                api.GRAD_FULL_KL, 0, out.grad.data_ptr(), api.BF16, V, out.kl.data_ptr(),
+                out.logratio.data_ptr(), out.gsq.data_ptr(), None, None, out.workspace.data_ptr(),
+                out.workspace.numel(), out.dev_status.data_ptr(), stream.cuda_stream)
+        calls[V] = (batch, out, stream, args, out.grad.clone())
+    torch.cuda.synchronize()
+    failed = {}
+
+    def work(V):
+        torch.cuda.set_device(0)
+        call, args = api.lib().adwin_opd_kl_fwd_bwd, calls[V][3]
+        failed[V] = sum(call(*args) != api.OK for _ in range(20000))
+
+    threads = [threading.Thread(target=work, args=(V,)) for V in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert failed == {30000: 0, 50000: 0}
+    for batch, out, _, _, want in calls.values():
+        api.raise_on_dev_status(out.dev_status)
+        assert torch.equal(out.grad, want)
