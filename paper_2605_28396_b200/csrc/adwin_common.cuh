@@ -127,8 +127,14 @@ struct RowAcc {
   }
 };
 
-// Fold N consecutive vocabulary entries into the accumulators.
-template <int N, bool EXPAND>
+// The reference of a maximum, rounded up so that no entry's exponent is positive.  With masked entries
+// (-1e30, the type's lowest value, which overflows) rounding to nearest leaves the maximum itself an
+// exponent of any size: a thread that sees nothing else then sums to infinity, and its weight of zero
+// beside real entries does not help.
+__device__ __forceinline__ float reference_of(float maximum) { return __fmul_ru(maximum, kLog2e); }
+
+// Fold N consecutive vocabulary entries into the accumulators.  MASKED: there may be masked ones.
+template <int N, bool EXPAND, bool MASKED = true>
 __device__ __forceinline__ void acc_piece(const float (&z)[N], const float (&u)[N], float dref,
                                           RowAcc& a) {
   float zm = z[0], um = u[0];
@@ -137,7 +143,7 @@ __device__ __forceinline__ void acc_piece(const float (&z)[N], const float (&u)[
     zm = fmaxf(zm, z[i]);
     um = fmaxf(um, u[i]);
   }
-  const float zl = zm * kLog2e, ul = um * kLog2e;
+  const float zl = MASKED ? reference_of(zm) : zm * kLog2e, ul = MASKED ? reference_of(um) : um * kLog2e;
   if (zl > a.m2s) {
     const float f = ex2f(a.m2s - zl);
     a.S *= f;

@@ -101,7 +101,7 @@ __device__ __forceinline__ void acc_piece_pairs(const float (&z)[N], const float
     zm = fmaxf(zm, z[i]);
     um = fmaxf(um, u[i]);
   }
-  const float zl = zm * kLog2e, ul = um * kLog2e;
+  const float zl = reference_of(zm), ul = reference_of(um);
   if (zl > a.m2s) {
     const float f = ex2f(a.m2s - zl);
     const f2_t F = splat2(f), F2 = mul2(F, F);
@@ -274,8 +274,8 @@ __global__ void __launch_bounds__(kGenericThreads, kGenericMinBlocks) kl_generic
               pa.m2t = fmaxf(pa.m2t, u[j]);
             }
           }
-          pa.m2s *= kLog2e;
-          pa.m2t *= kLog2e;
+          pa.m2s = reference_of(pa.m2s);
+          pa.m2t = reference_of(pa.m2t);
         }
 #pragma unroll
         for (int h = 0; h < kGenericUnroll; ++h) {

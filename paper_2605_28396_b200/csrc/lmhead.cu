@@ -537,7 +537,7 @@ lm_sweep_kernel(const __grid_constant__ CUtensorMap map_hs, const __grid_constan
                 u[i] = kMasked;
               }
           }
-          acc_piece<32, MOMENTS>(z, u, dref, acc);
+          acc_piece<32, MOMENTS, false>(z, u, dref, acc);   // (kMasked: see there)
         }
         tc_fence_before_sync();
         __syncwarp();

@@ -27,7 +27,7 @@ constexpr int kDriftMinBlocks = 8;   // CTAs per SM the register allocation leav
 constexpr float kLn2 = 0.69314718055994531f;
 
 struct DriftAcc {
-  float m2;     // running maximum of u*log2(e)
+  float m2;     // running maximum of u*log2(e), rounded up
   f2_t S;       // sum 2^(u2 - m2)                     (even / odd entries apart, as below)
   f2_t Bq;      // sum 2^(u2 - m2) * (m2 - u2)         (in units of log2)
   f2_t cnt;     // entries strictly above the sampled token's logit (whole numbers below 2^24)
@@ -72,7 +72,7 @@ __device__ __forceinline__ void drift_group(const uint4 (&v)[U], float uy, __nv_
     }
   }
   a.cnt = add2(a.cnt, pk2(__low2float(c), __high2float(c)));
-  a.raise(fmaxf(__low2float(m), __high2float(m)) * kLog2e);
+  a.raise(reference_of(fmaxf(__low2float(m), __high2float(m))));
 #pragma unroll
   for (int k = 0; k < U; ++k) {
     f2_t u[4];
@@ -95,7 +95,7 @@ __device__ __forceinline__ void drift_group(const uint4 (&v)[U], float uy, float
     }
   }
   a.cnt = add2(a.cnt, pk2((float)c, 0.f));
-  a.raise(m * kLog2e);
+  a.raise(reference_of(m));
 #pragma unroll
   for (int k = 0; k < U; ++k) {
     f2_t u[2];
@@ -106,7 +106,7 @@ __device__ __forceinline__ void drift_group(const uint4 (&v)[U], float uy, float
 }
 // One entry.
 __device__ __forceinline__ void drift_entry(float u, float uy, DriftAcc& a) {
-  a.raise(u * kLog2e);
+  a.raise(reference_of(u));
   const float d = fmaf(u, -kLog2e, a.m2), e = ex2f(-d);
   a.S = add2(a.S, pk2(e, 0.f));
   a.Bq = add2(a.Bq, pk2(e * d, 0.f));

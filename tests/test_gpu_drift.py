@@ -140,3 +140,15 @@ def test_config3_full_size_drift_on_sampled_rows():
     assert (cur.n_active.cpu().numpy() == B).all()
     bf = np.exp(got.entropy.double().cpu().numpy()).mean(axis=0)
     np.testing.assert_allclose(cur.bf_mean.cpu().numpy(), bf, rtol=1e-12)
+
+
+@pytest.mark.parametrize("cfg", [1, 2])
+@pytest.mark.parametrize("V,masked", [(150, 3), (1001, 7), (1003, 293), (4099, 1), (50257, 300)])
+def test_drift_with_masked_entries(cfg, V, masked):
+    """Entries masked out at either end of the vocabulary, so that threads see nothing else or nothing
+    else first: they add nothing to the entropy."""
+    batch = synth.make_batch(cfg, device=DEV, B=2, T=4, V=V)
+    batch.rollout_len = torch.tensor([4, 3], dtype=torch.int32, device=DEV)
+    batch.teacher[0, :, V - masked:], batch.teacher[1, :, :masked] = -1e30, -1e9
+    batch.tokens[:] = V // 2
+    _check(batch)

@@ -681,3 +681,30 @@ def test_two_threads_with_vocabularies_of_their_own():
     for batch, out, _, _, want in calls.values():
         api.raise_on_dev_status(out.dev_status)
         assert torch.equal(out.grad, want)
+
+
+@pytest.mark.parametrize("path", PATHS)
+@pytest.mark.parametrize("in_dt", [1, 2])
+@pytest.mark.parametrize("V,masked,at", [(150, 3, "end"), (1001, 64, "end"), (1003, 293, "end"), (4099, 7, "start"),
+                                         (4096, 293, "start"), (50257, 300, "end")])
+@pytest.mark.parametrize("value", ["lowest", -1e30, -1e9])
+def test_masked_vocabulary_entries(path, in_dt, V, masked, at, value):
+    """Entries masked out in both policies, at either end of the vocabulary, so that some threads see
+    nothing else (or nothing else first): they count for nothing, as in the oracle.  One row whose token
+    is far below the maximum (summed against running maxima)."""
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=4, V=V)
+    batch.window = torch.tensor([4, 2], dtype=torch.int32, device=DEV)
+    where = slice(V - masked, V) if at == "end" else slice(0, masked)
+    value = torch.finfo(batch.student.dtype).min if value == "lowest" else value
+    for x in (batch.student, batch.teacher):
+        x[..., where] = value
+    # (the token with the largest log-ratio: the sampled gradient's norm is c^2 times a constant, and c, a
+    # difference of logits, is good to 1e-5, so that 1e-4 on the norm takes |c| > 0.2)
+    batch.tokens[:] = (batch.student.float() - batch.teacher.float()).argmax(dim=2)
+    y = int(batch.tokens[0, 2])
+    batch.student[0, 2, y] = batch.student[0, 2].float().max() - 98.0
+    batch.teacher[0, 2, y] = batch.teacher[0, 2].float().max() - 100.0
+    g_dt = batch.student.dtype
+    for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
+        for grad in (g_dt, None):
+            run_and_check(batch, grad_dtype=grad, grad_mode=mode, flags=PATHS[path])
