@@ -708,3 +708,48 @@ def test_masked_vocabulary_entries(path, in_dt, V, masked, at, value):
     for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
         for grad in (g_dt, None):
             run_and_check(batch, grad_dtype=grad, grad_mode=mode, flags=PATHS[path])
+
+
+@pytest.mark.parametrize("in_dt,V", [(2, 4096), (2, 4104), (2, 20001), (2, 120000), (1, 2052), (1, 9001)])
+@pytest.mark.parametrize("mode", [api.GRAD_FULL_KL, api.GRAD_SAMPLED])
+def test_read_only_rows_that_outgrow_first_entries_and_token(in_dt, V, mode):
+    """Read-only sums refer to the maximum of a thread's first entries and the sampled token: rows in which
+    both lie below the rest by less than the sums bear, and by more (summed once more against running
+    maxima).  Both policies alike, so that z - u at the token stays small (its magnitude times 2^-24 is the
+    error of every centred difference)."""
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=4, V=V)
+    batch.window = torch.tensor([4, 3], dtype=torch.int32, device=DEV)
+    part = 4 * 128 * (4 if in_dt == 1 else 8)       # entries of the first group of a row
+    for t, rise in enumerate((20.0, 60.0, 90.0)):
+        for x in (batch.student, batch.teacher):
+            x[0, t, :part] -= rise
+    # inside the lowered part, z - u near one: the sampled norm is c^2 times a constant, so c must not be
+    # near zero, and the one-sweep norm is centred on the token's z - u, whose distance from the others'
+    # (3 standard deviations for the largest one) enters its error squared
+    batch.tokens[:] = ((batch.student.float() - batch.teacher.float())[..., :part] - 1.0).abs().argmin(dim=2)
+    run_and_check(batch, grad_dtype=None, grad_mode=mode)
+    run_and_check(batch, grad_dtype=None, grad_mode=mode, flags=api.RANGE_FULL)
+
+
+def test_read_only_precision_of_references_and_running_maxima():
+    """kl and the log-ratio of a read-only row do not depend on the gradient mode, but the full-KL mode sums
+    against references fixed early and the sampled mode against running maxima: the first may not be
+    further from a 64-bit evaluation (10 % for the spread between two sets of 1100 rounding errors)."""
+    batch = synth.make_batch(3, device=DEV, B=2, T=550)
+    batch.rollout_len[:] = 550
+    args = (batch.student, batch.teacher, batch.tokens, batch.window, batch.rollout_len)
+    z, u = batch.student.flatten(0, 1), batch.teacher.flatten(0, 1)
+    y = batch.tokens.flatten().long()[:, None]
+    err = {}
+    for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
+        got = api.adwin_opd_kl_fwd_bwd(*args, grad_mode=mode, flags=api.RANGE_FULL)
+        kl, c = got.kl.double().flatten(), got.logratio.double().flatten()
+        sums = torch.zeros(2, dtype=torch.float64, device=DEV)
+        for r in range(0, len(y), 50):
+            d = torch.log_softmax(z[r:r + 50].double(), 1)
+            p = d.exp()
+            d -= torch.log_softmax(u[r:r + 50].double(), 1)
+            sums[0] += ((p * d).sum(1) - kl[r:r + 50]).square().sum()
+            sums[1] += (d.gather(1, y[r:r + 50])[:, 0] - c[r:r + 50]).square().sum()
+        err[mode] = sums.sqrt()
+    assert (err[api.GRAD_FULL_KL] <= 1.1 * err[api.GRAD_SAMPLED]).all(), err
