@@ -126,10 +126,12 @@ def _ptr(t):
 
 
 def _stream(device):
-    if device.type != "cuda":   # a host address must not reach a kernel
-        raise ValueError(f"Expected a cuda device, but got: {device}")
     i = device.index
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
+    if i is None:   # (so has a tensor in host memory, whose address must not reach a kernel)
+        if device.type != "cuda":
+            raise ValueError(f"Expected a cuda device, but got: {device}")
+        i = torch.cuda.current_device()
+    return torch._C._cuda_getCurrentRawStream(i)
 
 
 def _dtype_code(dt):
