@@ -125,6 +125,14 @@ cudaError_t launch_rowmap(const int32_t* window, const int32_t* rollout_len, int
   int64_t fill_blocks = (n + kMapThreads - 1) / kMapThreads;
   if (fill_blocks > 1024) fill_blocks = 1024;
   if (fill_blocks < 1) fill_blocks = 1;
+#ifdef ADWIN_CHECKED
+  // every block's own checks may OR a bit into the word, also before block 0 stores it
+  if (flags & ADWIN_STATUS_INIT) {
+    const cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int32_t), s);
+    if (e != cudaSuccess) return e;
+    flags &= ~ADWIN_STATUS_INIT;
+  }
+#endif
   launch_chained(rowmap_kernel, (unsigned)(1 + fill_blocks), kMapThreads, 0, 1, s,
       window, rollout_len, B, T, flags, reinterpret_cast<int64_t*>(base + w.off_offsets),
       with_window_offsets ? reinterpret_cast<int64_t*>(base + w.off_offsets_win) : nullptr,

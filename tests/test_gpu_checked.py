@@ -42,6 +42,10 @@ def test_degenerate_windows_padded_strides_and_overflow_fallback(checked_library
     G.test_config3_reduced_T_full_vocab(path, api.GRAD_FULL_KL)
 
 
+def test_status_word_collects_or_starts_fresh(checked_library):
+    G.test_status_word_collects_or_starts_fresh()
+
+
 def test_teacher_drift_and_return_to_go(checked_library):
     from tests import test_gpu_drift as D
     from tests import test_gpu_rtg as R
