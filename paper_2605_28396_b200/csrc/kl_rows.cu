@@ -102,6 +102,15 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   const int cl = plan.cl;
   float4* rec = reinterpret_cast<float4*>(smem + kRowsRec);
   char* stash = smem + rows_ctrl_bytes(NT) + tid * 16;   // [step][array][thread] 16 bytes
+#ifdef ADWIN_CHECKED
+  uint32_t smem_bytes;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(smem_bytes));
+  // a group's pieces from `at` on, and its columns of tensor memory (the same for a whole warp)
+  auto stash_ok = [&](const char* at) { return at + (2 * kU - 1) * array + 16 <= smem + smem_bytes; };
+  auto columns_ok = [&](int k0) {
+    return k0 + kU <= plan.tm_steps && ((tid >> 7) + 1) * plan.tm_steps * 8 <= plan.tm_cols;
+  };
+#endif
   const uint32_t rank = cl > 1 ? cluster_rank() : 0u;
   const int64_t cluster_id = blockIdx.x / cl;
   const int piece0 = (int)rank * plan.per_rank;
@@ -134,7 +143,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   auto prefetch = [&](int64_t r, const void* base, int from, int count) {
     const RowSpan sn = span_of(r);
     const int n = min(sn.pieces - from, count);
-    if (n > 0)
+    if (n > 0 && ADWIN_CHK(((int64_t)piece0 + from + n - (RAG ? 1 : 0)) * N <= p.V + sn.shift, p.status))
       prefetch_l2(static_cast<const char*>(base) +
                       ((size_t)r * p.ld - sn.shift + (size_t)(piece0 + from) * N) * sizeof(TIn),
                   (uint32_t)n * 16u);
@@ -152,7 +161,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     bool wg_unused;
     auto fetch = [&](int64_t i) {   // metadata of row i into its slot
       const int64_t r = cur.locate(p, cluster_id + i * plan.num_clusters, wg_unused);
-      if (lane == 0) {
+      if (lane == 0 && ADWIN_CHK(r >= 0 && r < p.B * p.T, p.status)) {
         RowsMeta& m = ctrl.meta[i % kMetaDepth];
         const int y = p.tokens[r];
         m.r = r;
@@ -180,7 +189,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
 #pragma unroll
       for (int f = 0; f < 4; ++f) v[f] = lane_sum(v[f]);
       if (cl > 1) {
-        if (lane < cl)
+        if (lane < cl && ADWIN_CHK(rank < (uint32_t)kRowsMaxCl, p.status))
           remote_store4(map_to_rank(smem_u32(ctrl.xrec[par][rank]), (uint32_t)lane), v[0], v[1], v[2], v[3]);
         cluster_sync_all();
         v[0] = v[1] = v[2] = v[3] = 0.f;
@@ -221,7 +230,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         };
         combine();
         if (cl > 1) {
-          if (lane < cl) {
+          if (lane < cl && ADWIN_CHK(rank < (uint32_t)kRowsMaxCl, p.status)) {
             const uint32_t dst = map_to_rank(smem_u32(ctrl.xsafe[rank]), (uint32_t)lane);
             remote_store4(dst, t.M2s, t.M2t, t.S, t.A);
             remote_store4(dst + 16, t.St, 0.f, 0.f, 0.f);
@@ -252,7 +261,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
           prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, p.student, 0, plan.per_rank);
           prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, p.teacher, 0, plan.per_rank);
         }
-        if (rank == 0) {
+        if (rank == 0 && ADWIN_CHK(ri >= 0 && ri < p.B * p.T, p.status)) {
           p.kl[ri] = rs.kl;
           p.logratio[ri] = rs.c;
           if (p.lse_s) p.lse_s[ri] = rs.lse_s;
@@ -317,12 +326,14 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
             }
           }
           if (TM && k0 < plan.tm_steps) {   // (every lane takes part)
+            if (ADWIN_CHK(columns_ok(k0), p.status)) {
 #pragma unroll
-            for (int h = 0; h < kU; ++h) tm_store8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
+              for (int h = 0; h < kU; ++h) tm_store8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
+            }
           } else {
 #pragma unroll
             for (int h = 0; h < kU; ++h) {
-              if (FULL || lp0 + h * nt < span.pieces) {
+              if ((FULL || lp0 + h * nt < span.pieces) && ADWIN_CHK(stash_ok(st), p.status)) {
                 *reinterpret_cast<uint4*>(st + 2 * h * array) = z[h];
                 *reinterpret_cast<uint4*>(st + (2 * h + 1) * array) = u[h];
               }
@@ -363,9 +374,11 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         for (int k = 0; k < plan.steps; ++k) {
           uint4 zv, uv;
           if (TM && k < plan.tm_steps) {
+            if (!ADWIN_CHK(columns_ok(k / kU * kU), p.status)) break;
             tm_load8(tm_lane + (uint32_t)(k * 8), zv, uv);
             tm_wait_ld();
           } else {
+            if (!ADWIN_CHK(stash_ok(st - (k % kU) * 2 * array), p.status)) break;
             zv = *reinterpret_cast<const uint4*>(st);
             uv = *reinterpret_cast<const uint4*>(st + array);
             st += 2 * array;
@@ -410,13 +423,15 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         uint4 z[kU], u[kU];
         if (ahead) prefetch_part();
         if (TM && k0 < plan.tm_steps) {
+          if (ADWIN_CHK(columns_ok(k0), p.status)) {
 #pragma unroll
-          for (int h = 0; h < kU; ++h) tm_load8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
-          tm_wait_ld();
+            for (int h = 0; h < kU; ++h) tm_load8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
+            tm_wait_ld();
+          }
         } else {
 #pragma unroll
           for (int h = 0; h < kU; ++h) {
-            if (FULL || lp0 + h * nt < span.pieces) {
+            if ((FULL || lp0 + h * nt < span.pieces) && ADWIN_CHK(stash_ok(st), p.status)) {
               z[h] = *reinterpret_cast<const uint4*>(st + 2 * h * array);
               u[h] = *reinterpret_cast<const uint4*>(st + (2 * h + 1) * array);
             }

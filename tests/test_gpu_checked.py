@@ -61,8 +61,36 @@ def test_teacher_drift_and_return_to_go(checked_library):
                 fn()
 
 
+@pytest.mark.parametrize("path", G.PATHS)
+def test_rows_off_16_byte_boundaries(checked_library, path):
+    for V in (33, 1001, 50257):
+        for in_dt, g_dt in ((1, torch.float32), (2, torch.bfloat16), (2, None)):
+            G.test_rows_that_start_and_end_off_16_byte_boundaries(path, in_dt, g_dt, V)
+    for V, ld, ld_grad in ((1001, 1008, 1024), (1001, 1003, 1005), (12000, 12004, 12004)):
+        G.test_odd_rows_at_a_padded_stride(path, V, ld, ld_grad)
+    G.test_arrays_that_start_off_a_16_byte_boundary()
+
+
+@pytest.mark.parametrize("v", G.SHAPE_ENDS)
+def test_ends_of_the_row_kernels_shapes(checked_library, v):
+    for V in (v - 7, v - 5, v, v + 8):
+        G.test_rows_held_by_one_cta_and_by_clusters(2, V)
+    for V in (v // 2 - 3, v // 2, v // 2 + 4):
+        G.test_rows_held_by_one_cta_and_by_clusters(1, V)
+
+
+def test_read_only_rows(checked_library):
+    for in_dt, V, rows in ((2, 120001, 20), (2, 32003, 300), (1, 93534, 20)):
+        G.test_read_only_rows_split_over_a_cluster(in_dt, V, rows)
+    for in_dt, V in ((2, 4104), (2, 20001), (1, 2052)):
+        for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
+            G.test_read_only_rows_that_outgrow_their_first_entries(in_dt, V, mode)
+
+
 def test_fused_lm_head_small_and_ragged(checked_library):
     L.test_small_case_modes_and_flags(api.GRAD_FULL_KL, api.RANGE_FULL)
+    for windows in ([127], [60, 69, 0, 128], [257, 3]):
+        L.test_rows_packed_across_sequences_at_tile_edges(windows)
     L.test_ragged_vocabulary_and_hidden_sizes(1000, 72, 200)
     L.test_all_windows_empty_gives_zero_gradients()
 

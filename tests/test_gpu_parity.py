@@ -552,13 +552,22 @@ def test_status_word_collects_or_starts_fresh():
     assert int(o.dev_status.item()) == api.DEV_TOKEN_RANGE | api.DEV_WINDOW
 
 
+# The longest rows of bf16 that the row kernel's shapes take (64, 128 and 224 threads; 352 threads with one,
+# two and four CTAs per row); half as many entries of fp32.  A row off 16-byte boundaries may lie in one
+# piece more than its length asks for.
+SHAPE_ENDS = (6144, 10240, 25600, 50688, 101376, 202752)
+
+
 @pytest.mark.parametrize("in_dt,V", [(2, 3584), (2, 3592), (2, 17920), (2, 36000), (2, 58880), (2, 70001),
-                                     (2, 117760), (1, 1792), (1, 33003), (1, 58900), (1, 118001)])
+                                     (2, 117760), (1, 1792), (1, 33003), (1, 58900), (1, 118001)] +
+                         [(2, v + more) for v in SHAPE_ENDS for more in (-7, -5, 0, 8)] +
+                         [(1, v // 2 + more) for v in SHAPE_ENDS for more in (-3, -1, 0, 4)])
 def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
     """The row kernel's shapes: rows of a few hundred pieces, rows that fill a CTA's shared memory and
-    run over into tensor memory, rows split over two and four CTAs; piece counts that fill every
-    group of steps and one more piece; a sampled token in every slice, and rows whose token is far
-    below the maximum (summed again from the copy on chip)."""
+    run over into tensor memory, rows split over two and four CTAs; at the end of every shape rows that
+    fill it and rows of one more piece, on and off 16-byte boundaries (the last go to the staged kernel); a
+    sampled token in every slice, and rows whose token is far below the maximum (summed again from the
+    copy on chip)."""
     batch = synth.make_batch(in_dt, device=DEV, B=2, T=6, V=V)
     batch.window = torch.tensor([6, 3], dtype=torch.int32, device=DEV)
     for t, y in enumerate((0, V // 4 + 1, V // 2 + 1, 3 * V // 4 + 1, V - 1)):
@@ -567,6 +576,10 @@ def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
         y = int(batch.tokens[b, t])
         batch.student[b, t, y] = batch.student[b, t].float().max() - 100.0
         batch.teacher[b, t, y] = batch.teacher[b, t].float().max() - 100.0
+    # z - u of one at the token: the sampled gradient is proportional to c, whose error of about 3e-7 (a
+    # difference of fp32 logits and logarithms) is within 1e-5 of it only for |c| > 0.03
+    y = batch.tokens.long()[..., None]
+    batch.teacher.scatter_(2, y, batch.student.gather(2, y) - 1.0)
     g_dt = torch.float32 if in_dt == 1 else torch.bfloat16
     for mode in (api.GRAD_FULL_KL, api.GRAD_SAMPLED):
         run_and_check(batch, grad_dtype=g_dt, grad_mode=mode)
