@@ -582,18 +582,25 @@ bool rows_plan(int64_t pieces, RowsPlan& plan) {
 }
 
 typedef void (*RowsKernel)(KlParams, RowsPlan);
+// Whether the shapes of NT threads use tensor memory (all of them or none; `steps` is never less than
+// kU, so a plan of such a shape always does).
+constexpr bool uses_tensor_memory(int nt) {
+  for (const RowsShape& sh : kShapes)
+    if (sh.nt == nt) return sh.tm_cols > 0;
+  return false;
+}
 template <typename TIn, typename TOut, int NT>
-RowsKernel rows_kernel_nt(bool tm, bool ragged) {
-  if (tm) return ragged ? kl_rows_kernel<TIn, TOut, NT, true, true> : kl_rows_kernel<TIn, TOut, NT, true, false>;
-  return ragged ? kl_rows_kernel<TIn, TOut, NT, false, true> : kl_rows_kernel<TIn, TOut, NT, false, false>;
+RowsKernel rows_kernel_nt(bool ragged) {
+  constexpr bool TM = uses_tensor_memory(NT);
+  return ragged ? kl_rows_kernel<TIn, TOut, NT, TM, true> : kl_rows_kernel<TIn, TOut, NT, TM, false>;
 }
 template <typename TIn, typename TOut>
-RowsKernel rows_kernel(int nt, bool tm, bool ragged) {
+RowsKernel rows_kernel(int nt, bool ragged) {
   switch (nt) {
-    case 64: return rows_kernel_nt<TIn, TOut, 64>(tm, ragged);
-    case 128: return rows_kernel_nt<TIn, TOut, 128>(tm, ragged);
-    case 224: return rows_kernel_nt<TIn, TOut, 224>(tm, ragged);
-    case 352: return rows_kernel_nt<TIn, TOut, 352>(tm, ragged);
+    case 64: return rows_kernel_nt<TIn, TOut, 64>(ragged);
+    case 128: return rows_kernel_nt<TIn, TOut, 128>(ragged);
+    case 224: return rows_kernel_nt<TIn, TOut, 224>(ragged);
+    case 352: return rows_kernel_nt<TIn, TOut, 352>(ragged);
     default: return nullptr;
   }
 }
@@ -647,7 +654,7 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   constexpr int N = Elem<TIn>::N;
   RowsPlan plan = {};
   if (!rows_plan(ragged ? (p.V + 2 * N - 2) / N : p.V / N, plan)) return cudaErrorNotSupported;
-  const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, plan.tm_cols > 0, ragged);
+  const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, ragged);
   if (!kernel) return cudaErrorNotSupported;
   const int smem = launch_smem(plan);
   plan.num_clusters = plan.ctas * sm_count;
