@@ -518,8 +518,8 @@ def run_ours(args):
         del b4, ws4, o4
         torch.cuda.empty_cache()
 
-    # ---- config 5: the fused LM-head variant (hidden states x output embeddings, logits never
-    # materialised), forward statistics + gradients with respect to H_s and W_s; tensor roofline
+    # ---- config 5: the fused LM-head variant (hidden states x output embeddings, no logits
+    # from the caller), forward statistics + gradients with respect to H_s and W_s; tensor roofline
     lm_line = None
     if side:
         lb = synth.make_lmhead_batch(dev, B=args.lmhead_seqs, T=args.lmhead_positions)

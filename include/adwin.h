@@ -254,8 +254,8 @@ int adwin_drift_curves(const float* entropy, const int32_t* rank, const int32_t*
 
 /*
  * The same divergence with both policies given as hidden states times an output embedding (the
- * form Eq. 2's policies have in a language model: pi = softmax(h W^T)), fused so that the logits
- * are never held in memory as a whole (a block of positions at a time, see workspace):
+ * form Eq. 2's policies have in a language model: pi = softmax(h W^T)), without logits
+ * from the caller (those of a block of positions pass through the workspace, see there):
  *     z[b,t,:] = hidden_student[b,t,:] W_s^T,      u[b,t,:] = hidden_teacher[b,t,:] W_t^T,
  * then kl, logratio, gsq, lse_student, lse_teacher exactly as adwin_opd_kl_fwd_bwd defines them on
  * (z, u), and the gradients of the windowed loss with respect to the student's hidden states and
@@ -281,7 +281,10 @@ int adwin_drift_curves(const float* entropy, const int32_t* rank, const int32_t*
  * workspace    : >= adwin_lmhead_workspace_bytes(...) bytes, 1024-byte aligned; it holds compact
  *                copies of the processed hidden states, partial row statistics and, when a
  *                gradient is requested, G in bf16 (2 V bytes per processed position) and the fp32
- *                logits of one block of positions at a time (8 V bytes each, 6 GB at most)
+ *                logits of one block of positions at a time (8 V bytes each; a block is 6 GB of them
+ *                or 256 positions, whichever is more, or all positions if they are fewer).
+ *                B = 16, T = 4096, V = 151 936, d = 2048 + 2560, 35 162 positions: 17.4 GB with
+ *                a gradient, 0.4 GB without
  * Errors as in adwin_opd_kl_fwd_bwd; shapes this path cannot take return ADWIN_ERR_UNSUPPORTED.
  */
 size_t adwin_lmhead_workspace_bytes(int64_t B, int64_t T, int64_t V, int64_t d_s, int64_t d_t,

@@ -523,7 +523,12 @@ struct RowsShape {
 //            151 936   568 / 852 / 550     {2, 352} x 4
 // bf16 rows are bound by arithmetic and latency (19 issue slots per entry, the ex2 unit 57 % busy),
 // fp32 rows by memory.  Three or four steps in flight spill at 80 registers and lose, one step at 64
-// registers and a third more threads is slower except around 16 384 entries.
+// registers and a third more threads is slower except around 16 384 entries.  (Rows off 16-byte
+// boundaries cost the 64-thread bf16 kernels 68 bytes of spills.)
+// {3, 224} could hold 126 KB but ends at 100 (25 600 entries of bf16).  {3, 224} / {2, 352}: bf16 12 000
+// entries 527 / 566 us, 16 384 487 / 483, 22 000 508 / 487, 25 600 489 / 480, 27 000 523 / 487, 32 000
+// 487 / 470; fp32 6 000 484 / 532, 8 192 392 / 400, 12 800 407 / 392, 14 336 413 / 394, 16 000 424 / 397.
+// So the line keeps the rows that lose 6 % out; the last of those below it still lose 2 to 4 %.
 constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 1 << 20},   {5, 128, 0, 1, 1 << 20},
                                  {3, 224, 128, 1, 100},    {2, 352, 256, 1, 1 << 20},
                                  {2, 352, 256, 2, 1 << 20}, {2, 352, 256, 4, 1 << 20}};
