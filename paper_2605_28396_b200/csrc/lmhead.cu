@@ -15,8 +15,8 @@
 //   dH, dW    dH_s = G W_s and dW_s = G^T H_s as two tensor-core GEMMs over G (tc_gemm.cu)
 //
 // Without a gradient, all that is ever in memory is one 128 x 256 tile of student logits per CTA (19 MB).
-// With one, the fp32 logits of a block of tiles are in the scratch buffer at a time (kKeepBytes: about
-// 5000 positions at V = 151 936; the logits of a call of no more are all there at once).  Keeping them for those few
+// With one, the fp32 logits of a block of tiles are in the scratch buffer at a time (kKeepBytes: 5120
+// positions at V = 151 936; the logits of a call of no more are all there at once).  Keeping them for those few
 // milliseconds replaces a second pass of both products: 8 bytes written and read again per logit
 // pair against 2 (d_s + d_t) operations.  A long run is bound by the board's 1 kW, so what counts is
 // energy: at 34 816 rows, V = 151 936, d = 2048 + 2560 a call takes 87 ms (sweep 38, gradient 10,
@@ -44,7 +44,7 @@ constexpr int kInfoFields = 8;   // L2s, a1, a0, gy, y (bits), unused x3
 constexpr float kMasked = -1.0e6f;
 // Scratch for the logits of one block of tiles, or of one pair of tiles where that is more (V above
 // 3 million).  Large enough that a block fills the GPU several
-// times over (38 tiles at V = 151 936: 8 blocks for 34 816 rows), small beside G.
+// times over (40 tiles at V = 151 936: 7 blocks for 34 816 rows), small beside G.
 constexpr size_t kKeepBytes = size_t(6) << 30;
 constexpr int kKeepArray = kBM * kBN / 4;            // float4 of one policy's 128 x 256 tile
 constexpr size_t kKeepTileChunk = (size_t)2 * kKeepArray * 16;

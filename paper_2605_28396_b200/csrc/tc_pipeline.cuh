@@ -287,9 +287,8 @@ __device__ __forceinline__ void load_operand_pair(uint32_t dst, const CUtensorMa
 // Keeps the pairs of a launch in step.  Pairs that work on neighbouring tiles read the same operand
 // slabs at about the same time, so all but the first read should hit L2; but a pipeline that is
 // never short of operands has nothing that pulls a pair back once it is ahead, and after a few
-// tiles the pairs had drifted further apart than L2 holds: 72 GB read from DRAM instead of 20 for
-// G W_s at 34 816 rows, V = 151 936, d_s = 2048 (28 GB with this; 1105 -> 1202 TFLOP/s sustained,
-// because DRAM traffic costs clock under the power limit).  Every kPaceStep k-blocks a pair adds to
+// tiles the pairs have drifted further apart than L2 holds (G W_s at 34 816 rows, V = 151 936, d_s = 2048:
+// 1105 TFLOP/s sustained without this, 1202 with it: DRAM traffic costs clock under the power limit).  Every kPaceStep k-blocks a pair adds to
 // a common counter and, if it is more than kPaceSlack steps ahead of the average, waits a little.
 // The wait is a courtesy: it ends by itself after kPaceTries looks, nothing depends on it.
 constexpr uint32_t kPaceStep = 16;     // k-blocks per step

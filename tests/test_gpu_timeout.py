@@ -1,7 +1,7 @@
 """The give-up path of the bounded on-chip waits, exercised without faulting anything.
 
-Every wait in the kernels has a time limit.  With the diagnostic limit of one nanosecond the first
-wait that is not already satisfied runs out: the kernel must raise ADWIN_DEV_TIMEOUT, let its own
+Every mbarrier wait in the kernels (staged and tensor-core; the others have none) has a time limit.
+With the diagnostic limit of one nanosecond the first wait that is not already satisfied runs out: the kernel must raise ADWIN_DEV_TIMEOUT, let its own
 copies land, free its tensor memory and return -- and the very next ordinary call on the same
 inputs must match the oracle, which shows that the context and the device state are intact.
 """
