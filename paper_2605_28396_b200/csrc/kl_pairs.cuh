@@ -24,6 +24,14 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
 }
+// The two halves of it, for a thread that publishes nothing itself: what it does between them overlaps its
+// peers' way to the barrier.
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -45,10 +53,18 @@ __device__ __forceinline__ void tm_store8(uint32_t taddr, const uint4& a, const 
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
                "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
 }
+__device__ __forceinline__ void tm_store4(uint32_t taddr, const uint4& a) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(a.x), "r"(a.y),
+               "r"(a.z), "r"(a.w) : "memory");
+}
 __device__ __forceinline__ void tm_load8(uint32_t taddr, uint4& a, uint4& b) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
                : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tm_load4(uint32_t taddr, uint4& a) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tm_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -209,6 +225,21 @@ __device__ __forceinline__ void acc_grad(const f2_t (&Z)[NP], const f2_t (&U)[NP
     a.A = fma2(E, D, a.A);
     const f2_t xt = fma2(U[i], L2, nreft);
     a.St = add2(a.St, (i < PT) ? ex2_poly2(xt) : ex2_2(xt));
+  }
+}
+
+// The same with delta centred on -ndref.
+template <int NP>
+__device__ __forceinline__ void acc_grad_centred(const f2_t (&Z)[NP], const f2_t (&U)[NP], f2_t nrefs, f2_t nreft,
+                                                 f2_t ndref, Acc2& a) {
+  const f2_t L2 = splat2(kLog2e), NEG1 = splat2(-1.f);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    const f2_t E = ex2_2(fma2(Z[i], L2, nrefs));
+    const f2_t D = add2(fma2(U[i], NEG1, Z[i]), ndref);
+    a.S = add2(a.S, E);
+    a.A = fma2(E, D, a.A);
+    a.St = add2(a.St, ex2_2(fma2(U[i], L2, nreft)));
   }
 }
 

@@ -1,16 +1,21 @@
-// Row kernel for calls with gradient: a row (or a cluster's slice of it) is read from HBM once, kept on
-// chip between the two sweeps, several CTAs per SM.
+// Row kernel for calls with gradient: a row (or a cluster's slice of it) is read from HBM once and kept on
+// chip between its two sweeps; a row's second sweep and the next row's first run together.
 //
-// Two to eight small CTAs share an SM, each on a row of its own, so that one CTA's exchange and
-// row scalars overlap the other CTAs' streaming.  There are no roles and no hand-shakes: every
-// thread loads its own 16-byte pieces with plain coalesced loads, folds them into its sums and
-// puts them where only it will look for them again -- shared memory, or the otherwise idle tensor
-// memory (tcgen05.st / tcgen05.ld) -- so between the sweeps the threads only exchange sums.  One more
-// warp does what is done once per row: it adds up the threads' sums, derives the row's scalars and
-// hands them back (the others would otherwise each spend ~300 issue slots on it, as much as a
-// tenth of a row of 32 000 entries) and fetches the coming rows' metadata.  The next row is brought
-// into L2 meanwhile (cp.async.bulk.prefetch.L2), so that HBM stays busy during both sweeps and the
-// loads of the first sweep come from L2.
+// A row needs its sums before its gradient can be formed, so a CTA that finished one row before it began the
+// next would leave HBM idle during the exchange and the arithmetic of the second sweep.  Here every thread goes
+// through one stream of 16-byte pieces: for each group of pieces it forms the gradient of the row that has its
+// sums, puts the next row's pieces into the places that fall free, folds them into that row's sums and asks for the
+// group after (so loads are always one group ahead in registers).  The places are a ring of groups in
+// tensor memory (tcgen05.st / tcgen05.ld; no MMA runs here) and shared memory, each thread's its own: no
+// hand-shakes over data.  The ring has room for one or two groups more than a row, which are taken while
+// the row's sums travel, so the exchange costs no idle time either.  Rows are brought into L2 three groups
+// ahead (cp.async.bulk.prefetch.L2).  (All at once a row ahead is too early: rows of 100 000 bf16 entries were
+// pushed out of L2 again, 609 us against 489 for 2.4 GB.)
+//
+// One more warp does what is done once per row: it adds up the threads' sums, derives the row's scalars and
+// hands them back, fetches the coming rows' metadata, and looks after the few entries before a row's first
+// and after its last whole piece.  Pieces are counted from the 128-byte line in which a row starts: a warp's
+// loads and stores are whole lines whatever the row's offset (fp32, rows of 50 264 entries: 435 us before, 380 so).
 //
 // Exponentials are taken against a reference that the whole row shares (the logit of the sampled
 // token), so partial sums add without rescaling.  If the sums overflow it (a sampled token more than
@@ -28,34 +33,92 @@
 namespace adwin {
 namespace {
 
-constexpr int kRowsThreads = 352;     // threads of a CTA that hold pieces, at most
-constexpr int kRowsRegs = 80;         // registers per thread: 819 threads on an SM
-constexpr int kU = 2;                 // piece pairs in flight per thread
+constexpr int kRowsThreads = 512;     // threads of a CTA that hold pieces, at most
+// Steps of a group: the piece pairs that a thread has in flight.  One: 540 us where two take 430 (32 000
+// entries of bf16; the ring's bookkeeping is per group); four spill.
+constexpr int kU = 2;
 constexpr int kRowsMaxCl = 4;
 constexpr float kSumLimit = 1.2676506e30f;   // 2^100: beyond it the shared reference is unsafe
-constexpr int kMetaDepth = 4;
+constexpr int kMetaDepth = 8;
+constexpr int kMostEarly = 3;         // groups from a piece's way into L2 to its load, at most
+constexpr int kLine = 128;
+constexpr int kEdges = 16;            // entries beside a row's whole pieces: less than 8 on each side
+constexpr float kMaskedEdge = -1e30f;
 
 struct RowsPlan {
   int cl;             // CTAs per row
-  int nt;             // threads per CTA that hold pieces (one more warp looks ahead)
+  int nt;             // threads per CTA that hold pieces (one more warp does the row's own work)
   int ctas;           // CTAs per SM
   int per_rank;       // 16-byte pieces of a slice (per array)
-  int steps;          // piece pairs per thread, rounded up to a multiple of kU
-  int tm_steps;       // of these, in tensor memory (a multiple of kU; the first ones)
+  int groups;         // groups of kU steps (a piece of every thread each) that a slice takes
+  int early;          // groups between a piece's way into L2 and its first sweep (at most `groups`)
+  int ahead;          // groups of the next row that are taken before this row's second sweep
+  int tm_groups;      // groups kept in tensor memory (the ring's first ones); the rest in shared memory
   int tm_cols;        // tensor-memory columns per CTA (0: none)
   int num_clusters;
 };
+
+struct RowsShape {
+  int ctas, nt, tm_cols, cl;
+  int most;           // pieces of a row up to which the shape is taken
+};
+// The first that takes the row is used: the more and smaller CTAs, the less of a group lies idle at a row's
+// end; beyond 57 000 entries of bf16 one CTA per SM and not two in clusters (151 936 entries: two CTAs in clusters of
+// four, of which 71 fit on 148 SMs, 496 us; this 421).  Registers allow 20 warps of 96 (or 24 of 80, which is what
+// the 64-thread kernels take): 22 warps of 80 in {2, 352} 443 us where {2, 256} took 422 (32 000 entries).
+// Tensor memory is shared out in powers of two.  Measured over 2.4 GB of logits and gradient (367 us at the
+// copy rate; a kernel that ended one row before it began the next, on {8, 64} to {2, 352} x 4 / this one):
+//   bf16  V =   4 096  478 / 448 us  {8, 64}       fp32  V =   4 096  402 / 376 us  {4, 128}
+//              8 192  444 / 433     {4, 128}               5 001  481 / 381     {4, 128}
+//             16 384  484 / 414     {4, 128}              50 264  483 / 373     {1, 512}
+//             32 000  471 / 420     {2, 256}             100 000  497 / 381     {1, 512} x 2
+//             50 257  508 / 417     {2, 256}        bf16, sampled-token estimator
+//             80 000  512 / 397     {1, 512}              32 000  472 / 420     {2, 256}
+//            151 936  556 / 421     {1, 512} x 2          64 000  496 / 398     {1, 512}
+//            262 144  614 / 440     {1, 512} x 4         151 936  551 / 392     {1, 512}
+// fp32 rows are at the copy rate.  bf16 rows (163 issue slots and 24 of ex2 for eight entries, where the copy
+// rate leaves 273 clocks) are bound by arithmetic, short ones also by what is done once per row (5 000
+// entries 514 us, 507 before).
+// (The small shapes hold twice as much of a row whose second sweep takes the student alone, but are slower there:
+// 10 309 entries on {8, 64} 140 us where {4, 128} takes 131.)
+constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 768}, {4, 128, 128, 1, 3584}, {2, 256, 256, 1, 7168},
+                                 {1, kRowsThreads, 512, 1, 1 << 24}, {1, kRowsThreads, 512, 2, 1 << 24},
+                                 {1, kRowsThreads, 512, 4, 1 << 24}};
+// CTAs per SM of the shapes with nt threads, and whether they use tensor memory (the same for all of them).
+constexpr int ctas_of(int nt) {
+  for (const RowsShape& sh : kShapes)
+    if (sh.nt == nt) return sh.ctas;
+  return 1;
+}
+constexpr bool uses_tensor_memory(int nt) {
+  for (const RowsShape& sh : kShapes)
+    if (sh.nt == nt) return sh.tm_cols > 0;
+  return false;
+}
 
 struct __align__(16) RowsMeta {
   int64_t r;
   int y;
   float w;            // caller-supplied row coefficient (0 when there is none)
   float zy, uy;
+  float dref;         // z - u at the sampled token
+  float pad;
+  // as pairs and negated: the references of the student's and the teacher's sums, the centre of delta, which
+  // is exactly zero then at the peak of most peaked rows (it is the sampled token): beside a term of that size
+  // the rest of the row would lose the bits that the difference from the mean is made of
+  float nref[8];
+  float edge[kEdges][2];   // logits of the entries beside the row's whole pieces (kMaskedEdge where there is none)
 };
+// A row's constants stay in shared memory and are read with every group: both sweeps' would take ten
+// registers that the loads in flight need.
+__device__ __forceinline__ void row_pairs(const float* at, f2_t& a, f2_t& b) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(smem_u32(at)));
+}
 
-// What sweep 2 needs of a row.
+// What the second sweep needs of a row, as pairs: -m2s, the coefficient, the (scaled) centre.
 struct __align__(16) RowsScalars {
-  float m2s, coef, c0, gy;
+  float nm2s[2], coef[2];
+  float nc0[2], gy;
   int again;          // the sums overflowed: sum the row once more against running maxima
 };
 
@@ -85,67 +148,87 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// A row in a CTA's slice.  Pieces are counted from the 128-byte line that the student's row starts in, so
+// that a warp's 512 bytes are whole lines.
+struct RowSlice {
+  int begin, pieces;   // the slice's pieces [begin, pieces) are the row's
+  int shift;           // entries from the line's start to the row's
+};
+
 // NT: threads that hold pieces, a template constant so that the strides between a thread's pieces are
-// offsets in the instructions.  A group of kU steps in which every thread has a piece takes the path
-// without tests (FULL below).
-template <typename TIn, typename TOut, int NT, bool TM, bool RAG>
-__global__ void __launch_bounds__(NT + 32, 65536 / kRowsRegs / (NT + 32))
+// offsets in the instructions.  A group of kU steps in which every thread has whole pieces takes the path
+// without tests (FULL below).  FULLKL: the gradient of Eq. 2; without it, of Eq. 4, whose second sweep
+// takes the student's logits alone, so only they are kept.
+template <typename TIn, typename TOut, int NT, bool TM, bool RAG, bool FULLKL>
+__global__ void __launch_bounds__(NT + 32, ctas_of(NT))
 kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   chain();
   constexpr int N = Elem<TIn>::N;
   constexpr int NP = Pairs<TIn>::NP;
   constexpr int nt = NT, nw = NT / 32, all = NT + 32;
   constexpr uint32_t array = NT * 16u;
+  constexpr int kKept = FULLKL ? 2 : 1;             // arrays kept
+  // delta is summed about a centre (RowsMeta::dref) and the coefficient chosen for the product with the mean (see
+  // there) where a thread's chain of additions is longest; fp32 rows keep to delta itself, whose
+  // tolerance a centre far from the mean would cost.  (2.4 GB of rows of 32 000 entries 420 -> 424 us with both, where
+  // shorter ones would pay more: 8 192 436 -> 453, 5 000 519 -> 539.)
+  constexpr bool kCentred = sizeof(TIn) == 2 && NT >= 256;
+  constexpr uint32_t group_bytes = kU * kKept * array;
+  constexpr int group_cols = kU * kKept * 4;
   extern __shared__ __align__(128) char smem[];
   RowsCtrl& ctrl = *reinterpret_cast<RowsCtrl*>(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cl = plan.cl;
   float4* rec = reinterpret_cast<float4*>(smem + kRowsRec);
-  char* stash = smem + rows_ctrl_bytes(NT) + tid * 16;   // [step][array][thread] 16 bytes
+  char* stash = smem + rows_ctrl_bytes(NT) + tid * 16;   // [group][step][array][thread] 16 bytes
 #ifdef ADWIN_CHECKED
   uint32_t smem_bytes;
   asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(smem_bytes));
   // a group's pieces from `at` on, and its columns of tensor memory (the same for a whole warp)
-  auto stash_ok = [&](const char* at) { return at + (2 * kU - 1) * array + 16 <= smem + smem_bytes; };
-  auto columns_ok = [&](int k0) {
-    return k0 + kU <= plan.tm_steps && ((tid >> 7) + 1) * plan.tm_steps * 8 <= plan.tm_cols;
+  auto stash_ok = [&](const char* at) {
+    return at >= stash && at + (kU * kKept - 1) * array + 16 <= smem + smem_bytes;
+  };
+  auto columns_ok = [&](int pos) {
+    return pos >= 0 && pos < plan.tm_groups && ((tid >> 7) + 1) * plan.tm_groups * group_cols <= plan.tm_cols;
   };
 #endif
   const uint32_t rank = cl > 1 ? cluster_rank() : 0u;
   const int64_t cluster_id = blockIdx.x / cl;
   const int piece0 = (int)rank * plan.per_rank;
   const int64_t total_rows = p.offsets[p.B];
-  const int64_t my_rows =
-      cluster_id < total_rows ? (total_rows - cluster_id + plan.num_clusters - 1) / plan.num_clusters : 0;
+  const int my_rows =
+      cluster_id < total_rows ? (int)((total_rows - cluster_id + plan.num_clusters - 1) / plan.num_clusters) : 0;
 
   if (TM && warp == nw) tm_alloc(smem_u32(&ctrl.tmem_base), (uint32_t)plan.tm_cols);
 
-  // where row r lies in this CTA's slice (base pointers are 16-byte aligned)
-  auto span_of = [&](int64_t r) -> RowSpan {
-    RowSpan a = {0, 0, -1, -1, N};
-    if (RAG) a.shift = (int)((r * p.ld) & (N - 1));
-    const int64_t end = a.shift + p.V, total = (end + N - 1) / N, left = total - piece0;
-    a.pieces = (int)(left < 0 ? 0 : (left > plan.per_rank ? plan.per_rank : left));
+  // where row r lies in this CTA's slice (base pointers are 16-byte aligned; without RAG rows are lines).
+  // The at most N - 1 entries before its first and after its last whole piece are its own warp's.
+  auto slice_of = [&](int64_t r) -> RowSlice {
+    RowSlice a = {0, 0, 0};
     if (RAG) {
-      a.first = (a.shift > 0 && piece0 == 0) ? 0 : -1;
-      a.last_n = (int)(end - (total - 1) * N);
-      a.last = (a.last_n < N && left > 0 && left <= plan.per_rank) ? (int)left - 1 : -1;
+      a.shift = (int)((reinterpret_cast<uintptr_t>(p.student) / sizeof(TIn) + r * p.ld) & (kLine / sizeof(TIn) - 1));
+      if (piece0 == 0) a.begin = (a.shift + N - 1) / N;
     }
+    const int64_t left = (a.shift + p.V) / N - piece0;
+    a.pieces = (int)(left < 0 ? 0 : (left > plan.per_rank ? plan.per_rank : left));
     return a;
   };
+  // its groups [full_from, full_to) have a piece for every thread in every step
+  auto full_from = [&](const RowSlice& a) { return RAG && a.begin > 0 ? 1 : 0; };
+  auto full_to = [&](const RowSlice& a) { return a.pieces / (kU * nt); };
+  auto holds = [&](const RowSlice& a, int lp) { return lp < a.pieces && (!RAG || lp >= a.begin); };
+  [[maybe_unused]] auto inside = [&](const RowSlice& a, int lp) {
+    return lp >= a.begin && ((int64_t)piece0 + lp + 1) * N <= a.shift + p.V;
+  };
 
-  // The next row is brought into L2 ahead of its first sweep: bf16 rows by the row's warp, all at once
-  // when the second sweep of this row begins; fp32 rows, which memory bounds and not arithmetic, by
-  // thread 0 of the others, one array's part of a group at each group of either sweep, so that HBM has an
-  // even load (fp32 V = 32 000: 200 us before, 193 so; bf16, where thread 0's extra work holds its CTA
-  // up: 194 us against 202).
-  constexpr bool kSpread = sizeof(TIn) == 4;
+  // Rows are brought into L2 a few groups (plan.early) ahead of their first sweep, each group's pieces by
+  // one thread of the warp whose turn it is.
   auto prefetch = [&](int64_t r, const void* base, int from, int count) {
-    const RowSpan sn = span_of(r);
-    const int n = min(sn.pieces - from, count);
-    if (n > 0 && ADWIN_CHK(((int64_t)piece0 + from + n - (RAG ? 1 : 0)) * N <= p.V + sn.shift, p.status))
+    const RowSlice sn = slice_of(r);
+    const int lo = max(from, sn.begin), n = min(sn.pieces, from + count) - lo;
+    if (n > 0 && ADWIN_CHK(inside(sn, lo) && inside(sn, lo + n - 1), p.status))
       prefetch_l2(static_cast<const char*>(base) +
-                      ((size_t)r * p.ld - sn.shift + (size_t)(piece0 + from) * N) * sizeof(TIn),
+                      ((size_t)r * p.ld - sn.shift + (size_t)(piece0 + lo) * N) * sizeof(TIn),
                   (uint32_t)n * 16u);
   };
 
@@ -153,38 +236,103 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   if (cl > 1) cluster_sync_all();   // peers run before anything is stored into them
   __syncthreads();
   if (TM) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const int64_t iters = my_rows > 0 ? my_rows + 1 : 0;   // + one exchange for the last norm
   if (warp == nw) {
     // ------------------------------------------------------------------ the row's own warp
     RowCursor cur;
     cur.init(p);
     bool wg_unused;
-    auto fetch = [&](int64_t i) {   // metadata of row i into its slot
-      const int64_t r = cur.locate(p, cluster_id + i * plan.num_clusters, wg_unused);
-      if (lane == 0 && ADWIN_CHK(r >= 0 && r < p.B * p.T, p.status)) {
-        RowsMeta& m = ctrl.meta[i % kMetaDepth];
-        const int y = p.tokens[r];
-        m.r = r;
-        m.y = y;
-        fetch_logits_at<TIn>(p, r, y, m.zy, m.uy);
-        m.w = p.row_coef ? p.row_coef[r] : 0.f;
-      }
+    // the entry beside row r's whole pieces that this lane looks after (lanes 0-7 before, 8-15 behind), or -1
+    const bool edges = RAG && rank == 0 && (p.ld % N != 0 || p.V % N != 0);   // (rows of whole pieces have none)
+    auto edge_of = [&](int64_t r) -> int64_t {
+      if (!edges) return -1;
+      const int shift = slice_of(r).shift, head = (N - shift % N) % N;
+      if (lane < 8) return lane < head && lane < p.V ? lane : -1;
+      const int64_t k = ((shift + p.V) / N) * N - shift + (lane - 8);   // (rows have several pieces)
+      return lane < 16 && k < p.V ? k : -1;
     };
-    constexpr int kAheadRows = kSpread ? 2 : 1;
-    for (int64_t i = 0; i < kAheadRows && i < my_rows; ++i) fetch(i);
+    auto fill = [&](int i, int64_t r) {    // row i's metadata into its slot
+      if (!ADWIN_CHK(r >= 0 && r < p.B * p.T, p.status)) return;
+      RowsMeta& m = ctrl.meta[i % kMetaDepth];
+      const int y = p.tokens[r];
+      m.r = r;
+      m.y = y;
+      float zy, uy;
+      fetch_logits_at<TIn>(p, r, y, zy, uy);
+      m.zy = zy;
+      m.uy = uy;
+      m.nref[0] = m.nref[1] = -zy * kLog2e;
+      m.nref[2] = m.nref[3] = -uy * kLog2e;
+      // (a token far from the others' differences, or masked in one policy, is no centre)
+      const float dref = kCentred && fabsf(zy - uy) <= 16.f ? zy - uy : 0.f;
+      m.dref = dref;
+      m.nref[4] = m.nref[5] = -dref;
+      m.nref[6] = m.nref[7] = 0.f;
+      m.w = p.row_coef ? p.row_coef[r] : 0.f;
+    };
+    auto fill_edges = [&](int i, int64_t r) {
+      if (!edges || lane >= kEdges) return;
+      const int64_t k = edge_of(r);
+      float* at = ctrl.meta[i % kMetaDepth].edge[lane];
+      const bool has = k >= 0 && ADWIN_CHK(k < p.V && r < p.B * p.T, p.status);
+      at[0] = has ? Elem<TIn>::load1(p.student, r * p.ld + k) : kMaskedEdge;
+      at[1] = has ? Elem<TIn>::load1(p.teacher, r * p.ld + k) : kMaskedEdge;
+    };
+    auto row_of = [&](int i) { return cur.locate(p, cluster_id + (int64_t)i * plan.num_clusters, wg_unused); };
+    auto fetch = [&](int i) {
+      const int64_t r = row_of(i);
+      if (lane == 0) fill(i, r);
+      fill_edges(i, r);
+    };
+    // The first three rows at once, a lane each (one after another they are nine round trips to memory), and
+    // the first row on its way into L2 before its metadata.
+    constexpr int kFirst = 3;
+    {
+      const int n = min(kFirst, my_rows);
+      const int64_t r = row_of(min(lane, max(n - 1, 0)));
+      if (lane == 0 && n > 0) {
+        prefetch(r, p.student, 0, plan.per_rank);
+        prefetch(r, p.teacher, 0, plan.per_rank);
+      }
+      if (lane < n) fill(lane, r);
+      for (int i = 0; i < n; ++i) fill_edges(i, __shfl_sync(0xffffffffu, r, i));
+    }
     __syncthreads();
     int64_t r_prev = 0;
-    for (int64_t i = 0; i < iters; ++i) {
-      const bool real = i < my_rows, more = i + 1 < my_rows;
-      const int par = (int)(i & 1);
-      if (i + kAheadRows < my_rows) fetch(i + kAheadRows);
+    float q_edge = 0.f;   // this lane's share of the previous row's squared norm
+    float q_scale = 1.f;  // and what the norm is to be scaled by
+    // one more exchange than rows, for the last norm
+    for (int i = 0; i <= my_rows && my_rows > 0; ++i) {
+      const bool real = i < my_rows;
+      const int par = i & 1;
+      // (the others are at rows i - 1 and i, and take up i + 1 after this exchange)
+      if (i + 3 < my_rows) fetch(i + 3);
       named_sync(kPosted, all);
       // fixed-order sums over the threads, then over the CTAs
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      float4 x4[nw];
 #pragma unroll
-      for (int w = 0; w < nw; ++w) {
-        const float4 x = rec[w * 32 + lane];
-        v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+      for (int w = 0; w < nw; ++w) x4[w] = rec[w * 32 + lane];
+#pragma unroll
+      for (int n = nw / 2; n > 0; n /= 2) {
+#pragma unroll
+        for (int w = 0; w < n; ++w) {
+          x4[w].x += x4[w + n].x; x4[w].y += x4[w + n].y; x4[w].z += x4[w + n].z; x4[w].w += x4[w + n].w;
+        }
+      }
+      float v[4] = {x4[0].x, x4[0].y, x4[0].z, x4[0].w};
+      float ze = kMaskedEdge, ue = kMaskedEdge;
+      if (edges) {
+        v[3] += q_edge;
+        if (real) {
+          const RowsMeta& m = ctrl.meta[i % kMetaDepth];
+          if (lane < kEdges) {
+            ze = m.edge[lane][0];
+            ue = m.edge[lane][1];
+          }
+          const float e = ex2f(fmaf(ze, kLog2e, m.nref[0]));
+          v[0] += e;
+          v[1] = fmaf(e, (ze - ue) + m.nref[4], v[1]);
+          v[2] += ex2f(fmaf(ue, kLog2e, m.nref[2]));
+        }
       }
 #pragma unroll
       for (int f = 0; f < 4; ++f) v[f] = lane_sum(v[f]);
@@ -198,7 +346,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
           v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
         }
       }
-      if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = v[3];
+      if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = v[3] * q_scale;
       if (!real) break;
       const RowsMeta& m = ctrl.meta[i % kMetaDepth];
       const int64_t ri = m.r;
@@ -218,6 +366,13 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         if (lane < nw) {
 #pragma unroll
           for (int f = 0; f < 5; ++f) x[f] = ctrl.safe[lane][f];
+        }
+        if (edges && edge_of(ri) >= 0) {   // this lane's entry beside the pieces
+          RowAcc ra;
+          ra.m2s = x[0]; ra.m2t = x[1]; ra.S = x[2]; ra.A = x[3]; ra.St = x[4];
+          const float z1[1] = {ze}, u1[1] = {ue};
+          acc_piece<1, false>(z1, u1, m.dref, ra);
+          x[0] = ra.m2s; x[1] = ra.m2t; x[2] = ra.S; x[3] = ra.A; x[4] = ra.St;
         }
         auto combine = [&]() {
           t.M2s = warp_max(x[0]);
@@ -246,21 +401,64 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         }
       }
       const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
-      const RowScalars rs = finish_row(t, m.zy, m.uy, y_valid, 0.f, p.alpha, p.mode,
-                                       p.row_coef ? &m.w : nullptr);
-      if (lane == 0) {
-        ctrl.out.m2s = t.M2s;
-        ctrl.out.coef = rs.coef;
-        ctrl.out.c0 = rs.c0;
-        ctrl.out.gy = rs.gy;
-        ctrl.out.again = 0;
-      }
-      named_sync(kReady, all);
-      if (lane == 0) {
-        if (!kSpread && more) {
-          prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, p.student, 0, plan.per_rank);
-          prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, p.teacher, 0, plan.per_rank);
+      const float inv = 1.f / t.S;
+      // the mean of delta over the row, as a sum of two floats
+      const float about = t.A * inv, mean = about + m.dref, back = mean - about;
+      const float rest = (about - (mean - back)) + (m.dref - back);
+      float coef = p.alpha * inv, nc0 = -mean;
+      q_scale = 1.f;
+      if constexpr (FULLKL && sizeof(TIn) == 2) {
+        // bf16 logits: g = e * (coef*delta - coef*mean) saves one operation per pair; its rounding
+        // (relative to coef*delta, not to the difference) is far inside that dtype's tolerance.  But that of
+        // coef*mean is common to the row, and a peaked row's norm, all of it from a delta beside the mean, is off
+        // by twice the rounding times mean / (delta - mean).  A bf16 gradient does not see 2^-20 of its
+        // coefficient, so of the 32 nearest the one whose product with the mean needs the least rounding is
+        // taken, and the norm scaled back.  (With the centre: over 15 360 rows of 151 936 entries the norm's
+        // error is 3.5e-7 in the root mean square and 1.7e-5 at most, 2.2e-6 and 9.9e-5 without both.)
+        if (kCentred && sizeof(TOut) == 2 && fabsf(coef) > 1e-30f && fabsf(coef) < 1e30f) {
+          const float c = __int_as_float(__float_as_int(coef) + lane - 16);
+          const float prod = c * mean, low = fmaf(c, rest, fmaf(c, mean, -prod)), near = prod + low;
+          const float off = fabsf(low - (near - prod));
+          const unsigned best = __reduce_min_sync(0xffffffffu, (__float_as_uint(off) & ~31u) | (unsigned)lane) & 31u;
+          const float taken = __shfl_sync(0xffffffffu, c, (int)best);
+          nc0 = -__shfl_sync(0xffffffffu, near, (int)best);
+          q_scale = coef / taken;
+          q_scale *= q_scale;
+          coef = taken;
+        } else {
+          nc0 = -coef * mean;
         }
+      }
+      auto publish = [&](float gy) {
+        if (lane == 0) {
+          ctrl.out.nm2s[0] = ctrl.out.nm2s[1] = -t.M2s;
+          ctrl.out.coef[0] = ctrl.out.coef[1] = coef;
+          ctrl.out.nc0[0] = ctrl.out.nc0[1] = nc0;
+          ctrl.out.gy = gy;
+          ctrl.out.again = 0;
+        }
+        named_sync(kReady, all);
+      };
+      // what the second sweep of Eq. 2's gradient takes needs no logarithm (as finish_row has it)
+      if constexpr (FULLKL) publish(0.f);
+      const RowScalars rs = finish_row(t, m.zy, m.uy, y_valid, m.dref, p.alpha, FULLKL ? ADWIN_GRAD_FULL_KL : ADWIN_GRAD_SAMPLED,
+                                       p.row_coef ? &m.w : nullptr);
+      if constexpr (!FULLKL) {
+        coef = rs.coef;
+        publish(rs.gy);
+      }
+      if (edges) {   // the gradient of the edge entries, as in the second sweep
+        const int64_t k = edge_of(ri);
+        const float e = ex2f(fmaf(ze, kLog2e, -t.M2s));
+        float g;
+        if (!FULLKL) g = k == m.y ? rs.gy : e * coef;
+        else if (sizeof(TIn) == 2) g = e * fmaf(ze - ue, coef, nc0);
+        else g = e * ((ze - ue + nc0) * coef);
+        q_edge = k >= 0 ? g * g : 0.f;
+        if (k >= 0 && ADWIN_CHK(k < p.V && ri < p.B * p.T, p.status))
+          Elem<TOut>::store1(p.grad, ri * p.ld_grad + k, g);
+      }
+      if (lane == 0) {
         if (rank == 0 && ADWIN_CHK(ri >= 0 && ri < p.B * p.T, p.status)) {
           p.kl[ri] = rs.kl;
           p.logratio[ri] = rs.c;
@@ -276,118 +474,247 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       r_prev = ri;
     }
   } else {
-    __syncthreads();   // the first row's metadata
+    __syncthreads();   // the first rows' metadata
     // this thread's tensor-memory columns: its lane, the columns split between the warps of a lane group
     const uint32_t tm_lane = TM ? ctrl.tmem_base + ((uint32_t)((warp & 3) * 32) << 16) +
-                                      (uint32_t)((warp >> 2) * plan.tm_steps * 8)
+                                      (uint32_t)((warp >> 2) * plan.tm_groups * group_cols)
                                 : 0u;
-    const bool full_mode = (p.mode == ADWIN_GRAD_FULL_KL);
-    float q_prev = 0.f;       // this thread's share of the previous row's squared norm
-    for (int64_t i = 0; i < iters; ++i) {
-      const bool real = i < my_rows;
-      const RowsMeta& m = ctrl.meta[real ? i % kMetaDepth : 0];
-      const bool ahead = kSpread && tid == 0 && i + 1 < my_rows;
-      int part = 0;
-      auto prefetch_part = [&]() {
-        prefetch(ctrl.meta[(i + 1) % kMetaDepth].r, (part & 1) ? p.teacher : p.student,
-                 (part >> 1) * kU * nt, kU * nt);
-        ++part;
-      };
-      RowSpan span = {0, 0, -1, -1, N};
-      Acc2 a;
+    const int ring = plan.groups + plan.ahead;
+    int pos = 0;              // the ring's group that comes next
+
+    // ---- loads: the pieces of the first sweep's next group, always one group ahead of it
+    uint4 zn[kU], un[kU];
+    const char* zp = nullptr;   // the next piece of the student's row to be loaded
+    int left = 0;               // pieces of the slice from it on
+    bool before = false;        // (the piece belongs to the row before: only the first one may)
+    int load_row = -1, load_group = 0;
+    const ptrdiff_t to_teacher = static_cast<const char*>(p.teacher) - static_cast<const char*>(p.student);
+    auto load = [&](int h) {
+      if (left > h * nt && !(RAG && h == 0 && before) &&
+          ADWIN_CHK((zp - static_cast<const char*>(p.student)) + (h * nt + 1) * 16 <=
+                        ((p.B * p.T - 1) * p.ld + p.V) * (int64_t)sizeof(TIn), p.status)) {
+        zn[h] = __ldcs(reinterpret_cast<const uint4*>(zp) + h * nt);
+        un[h] = __ldcs(reinterpret_cast<const uint4*>(zp + to_teacher) + h * nt);
+      }
+    };
+    auto next_load_row = [&]() {
+      ++load_row;
+      load_group = 0;
+      left = 0;
+      if (load_row < my_rows) {
+        const int64_t r = ctrl.meta[load_row % kMetaDepth].r;
+        const RowSlice sn = slice_of(r);
+        zp = static_cast<const char*>(p.student) +
+             ((size_t)r * p.ld - sn.shift + (size_t)(piece0 + tid) * N) * sizeof(TIn);
+        left = sn.pieces - tid;
+        if (RAG) before = tid < sn.begin;
+      }
+    };
+    auto loaded = [&]() {       // a whole group has been asked for
+      zp += kU * array;
+      left -= kU * nt;
+      before = false;
+      if (++load_group == plan.groups) next_load_row();
+    };
+
+    // ---- first sweep: the row's sums and copies
+    RowSlice sp1 = slice_of(0);   // (without RAG the same for all rows)
+    const float* refs = nullptr;
+    Acc2 a;
+    auto begin_sums = [&](int i) {
+      const RowsMeta& m = ctrl.meta[i % kMetaDepth];
+      if (RAG) sp1 = slice_of(m.r);
+      refs = m.nref;
       a.reset();
-      if (real) {
-        // ------------------------------------------------------------ sweep 1
-        span = span_of(m.r);
-        const size_t off = ((size_t)m.r * p.ld - span.shift + (size_t)piece0 * N) * sizeof(TIn);
-        const uint4* zp = reinterpret_cast<const uint4*>(static_cast<const char*>(p.student) + off) + tid;
-        const uint4* up = reinterpret_cast<const uint4*>(static_cast<const char*>(p.teacher) + off) + tid;
-        const f2_t nrefs = splat2(-m.zy * kLog2e), nreft = splat2(-m.uy * kLog2e);
-        char* st = stash;
-        int lp0 = tid;     // this thread's piece in the group's first step
-        auto group = [&](auto full, int k0) {
-          constexpr bool FULL = decltype(full)::value;
-          uint4 z[kU], u[kU];
-          if (ahead) prefetch_part();
+    };
+    // ---- second sweep: what it takes of its row
+    RowSlice sp2 = sp1;
+    f2_t Q = 0ull;
+    float gy = 0.f;
+    int yleft = -1;           // pieces from this thread's next one to the sampled token's (< 0: passed, or elsewhere)
+    int ye = 0;
+    char* gp = nullptr;
+
+    // One group: the second sweep's group g2 (TWO) and the first sweep's group g1 of the row after (ONE),
+    // which takes its place in the ring.
+    auto group = [&](auto one_, auto two_, auto full_, int g1, int g2) __attribute__((always_inline)) {
+      constexpr bool ONE = decltype(one_)::value, TWO = decltype(two_)::value, FULL = decltype(full_)::value;
+      const bool in_tm = TM && pos < plan.tm_groups;
+      const uint32_t tm_at = TM ? tm_lane + (uint32_t)(pos * group_cols) : 0u;
+      char* st = stash + (size_t)((uint32_t)(pos - plan.tm_groups) * group_bytes);
+      const int l1 = tid + g1 * (kU * nt), l2 = tid + g2 * (kU * nt);   // this thread's pieces of the first step
+      const f2_t L2 = splat2(kLog2e), NEG1 = splat2(-1.f);
+      f2_t nM2s, coef2, nc0, nrefs, nreft, ndref, unused;
+      if constexpr (TWO) {
+        row_pairs(ctrl.out.nm2s, nM2s, coef2);
+        if constexpr (FULLKL) row_pairs(ctrl.out.nc0, nc0, unused);
+      }
+      if constexpr (ONE) {
+        row_pairs(refs, nrefs, nreft);
+        if constexpr (kCentred) row_pairs(refs + 4, ndref, unused);
+      }
 #pragma unroll
-          for (int h = 0; h < kU; ++h) {
-            if ((FULL || lp0 + h * nt < span.pieces) &&
-                ADWIN_CHK(((int64_t)piece0 + lp0 + h * nt + (RAG ? 0 : 1)) * N <= p.V + span.shift, p.status)) {
-              z[h] = __ldcs(zp + h * nt);
-              u[h] = __ldcs(up + h * nt);
+      for (int h = 0; h < kU; ++h) {
+        if constexpr (TWO) {
+          const int lp = l2 + h * nt;
+          uint4 z, u;
+          if (in_tm) {   // (every lane takes part)
+            if (ADWIN_CHK(columns_ok(pos), p.status)) {
+              if constexpr (FULLKL) tm_load8(tm_at + (uint32_t)(h * 8), z, u);
+              else tm_load4(tm_at + (uint32_t)(h * 4), z);
+              tm_wait_ld();
             }
+          } else if ((FULL || holds(sp2, lp)) && ADWIN_CHK(stash_ok(st), p.status)) {
+            z = *reinterpret_cast<const uint4*>(st + kKept * h * array);
+            if constexpr (FULLKL) u = *reinterpret_cast<const uint4*>(st + (kKept * h + 1) * array);
           }
-          if (RAG) {
+          if (FULL || holds(sp2, lp)) {
+            f2_t Z[NP], U[NP], G[NP];
+            Pairs<TIn>::make(z, Z);
+            if constexpr (FULLKL) Pairs<TIn>::make(u, U);
 #pragma unroll
-            for (int h = 0; h < kU; ++h) {
-              const int lp = lp0 + h * nt;
-              if (lp == span.first || lp == span.last)
-                mask_piece<TIn>(z[h], u[h], span.e0(lp), lp == span.last ? span.last_n : N);
-            }
-          }
-          if (TM && k0 < plan.tm_steps) {   // (every lane takes part)
-            if (ADWIN_CHK(columns_ok(k0), p.status)) {
-#pragma unroll
-              for (int h = 0; h < kU; ++h) tm_store8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
-            }
-          } else {
-#pragma unroll
-            for (int h = 0; h < kU; ++h) {
-              if ((FULL || lp0 + h * nt < span.pieces) && ADWIN_CHK(stash_ok(st), p.status)) {
-                *reinterpret_cast<uint4*>(st + 2 * h * array) = z[h];
-                *reinterpret_cast<uint4*>(st + (2 * h + 1) * array) = u[h];
+            for (int e = 0; e < NP; ++e) {
+              const f2_t E = ex2_2(fma2(Z[e], L2, nM2s));
+              if constexpr (FULLKL) {
+                if (sizeof(TIn) == 2) G[e] = mul2(E, fma2(fma2(U[e], NEG1, Z[e]), coef2, nc0));
+                else G[e] = mul2(E, mul2(add2(fma2(U[e], NEG1, Z[e]), nc0), coef2));
+              } else {
+                G[e] = mul2(E, coef2);
               }
             }
-            st += 2 * kU * array;
-          }
+            if constexpr (!FULLKL) {
+              if (yleft == h * nt) {
 #pragma unroll
-          for (int h = 0; h < kU; ++h) {
-            if (FULL || lp0 + h * nt < span.pieces) {
-              f2_t Z[NP], U[NP];
-              Pairs<TIn>::make(z[h], Z);
-              Pairs<TIn>::make(u[h], U);
-              acc_grad<NP, 0>(Z, U, nrefs, nreft, a);
+                for (int e = 0; e < NP; ++e) {
+                  float lo, hi;
+                  upk2(G[e], lo, hi);
+                  if (ye == 2 * e) lo = gy;
+                  if (ye == 2 * e + 1) hi = gy;
+                  G[e] = pk2(lo, hi);
+                }
+              }
+            }
+#pragma unroll
+            for (int e = 0; e < NP; ++e) Q = fma2(G[e], G[e], Q);
+            char* dst = gp + (size_t)h * nt * N * sizeof(TOut);
+            if (ADWIN_CHK(inside(sp2, lp), p.status)) {
+              store_pairs<TOut, NP>(dst, G);
             }
           }
-          zp += kU * nt;
-          up += kU * nt;
-          lp0 += kU * nt;
-        };
-        int k0 = 0;
-        for (; (k0 + kU) * nt <= span.pieces; k0 += kU) group(std::true_type{}, k0);
-        for (; k0 < plan.steps; k0 += kU) group(std::false_type{}, k0);
-        if (TM) tm_wait_st();
+        }
+        if constexpr (ONE) {
+          const int lp = l1 + h * nt;
+          if (in_tm) {   // (every lane takes part)
+            if (ADWIN_CHK(columns_ok(pos), p.status)) {
+              if constexpr (FULLKL) tm_store8(tm_at + (uint32_t)(h * 8), zn[h], un[h]);
+              else tm_store4(tm_at + (uint32_t)(h * 4), zn[h]);
+            }
+          } else if ((FULL || holds(sp1, lp)) && ADWIN_CHK(stash_ok(st), p.status)) {
+            *reinterpret_cast<uint4*>(st + kKept * h * array) = zn[h];
+            if constexpr (FULLKL) *reinterpret_cast<uint4*>(st + (kKept * h + 1) * array) = un[h];
+          }
+          if (FULL || holds(sp1, lp)) {
+            f2_t Z[NP], U[NP];
+            Pairs<TIn>::make(zn[h], Z);
+            Pairs<TIn>::make(un[h], U);
+            if constexpr (kCentred) acc_grad_centred<NP>(Z, U, nrefs, nreft, ndref, a);
+            else acc_grad<NP, 0>(Z, U, nrefs, nreft, a);
+          }
+          load(h);
+        }
       }
-
-      // -------------------------------------------------------------- exchange
-      rec[tid] = make_float4(hsum2(a.S), hsum2(a.A), hsum2(a.St), q_prev);
+      if constexpr (TWO) {
+        gp += (size_t)kU * nt * N * sizeof(TOut);
+        if constexpr (!FULLKL) yleft -= kU * nt;
+      }
+      if constexpr (ONE) loaded();
+      pos = pos + 1 == ring ? 0 : pos + 1;
+    };
+    constexpr std::true_type yes{};
+    constexpr std::false_type no{};
+    // the group `plan.early` groups behind group g of row i in the order of the first sweeps
+    auto early = [&](int i, int g) {
+      if (warp == g % nw && lane == 0) {
+        g += plan.early;
+        if (g >= plan.groups) {
+          g -= plan.groups;
+          ++i;
+        }
+        if (i < my_rows) {
+          const int64_t r = ctrl.meta[i % kMetaDepth].r;
+          prefetch(r, p.student, g * kU * nt, kU * nt);
+          prefetch(r, p.teacher, g * kU * nt, kU * nt);
+        }
+      }
+    };
+    auto post = [&](float q) {
+      rec[tid] = make_float4(hsum2(a.S), hsum2(a.A), hsum2(a.St), q);
       named_arrive(kPosted, all);
-      if (cl > 1) cluster_sync_all();
-      if (!real) break;
+      if (cl > 1) cluster_arrive_relaxed();
+    };
+
+    next_load_row();
+#pragma unroll
+    for (int h = 0; h < kU; ++h) load(h);
+    loaded();
+#pragma unroll 1
+    for (int i = -1; i < my_rows; ++i) {
+      const bool next = i + 1 < my_rows;
+      if (RAG) sp2 = sp1;
+      // the next row's first groups (all of them for the first row), into the part of the ring that this
+      // row does not take: this row's sums travel meanwhile
+      if (next) {
+        begin_sums(i + 1);
+        const int to = i < 0 ? plan.groups : plan.ahead;
+        if (i >= 0) pos = pos + plan.groups >= ring ? pos - plan.ahead : pos + plan.groups;
+#pragma unroll 1
+        for (int g = 0; g < to; ++g) {
+          early(i + 1, g);
+          group(yes, no, no, g, 0);
+        }
+      }
+      if (i < 0) {
+        pos = 0;
+        if (next) post(0.f);
+        continue;
+      }
+      const RowsMeta& m = ctrl.meta[i % kMetaDepth];
+      if (cl > 1) cluster_wait();
       named_sync(kReady, all);
+      if (TM) tm_wait_st();
 
       // -------------------------------------------------------------- overflow: running maxima
       if (ctrl.out.again) {
         RowAcc ra;
         ra.reset();
-        const char* st = stash;
-        for (int k = 0; k < plan.steps; ++k) {
-          uint4 zv, uv;
-          if (TM && k < plan.tm_steps) {
-            if (!ADWIN_CHK(columns_ok(k / kU * kU), p.status)) break;
-            tm_load8(tm_lane + (uint32_t)(k * 8), zv, uv);
+        const uint4* uq = nullptr;
+        if (!FULLKL)
+          uq = reinterpret_cast<const uint4*>(
+                   static_cast<const char*>(p.teacher) +
+                   ((size_t)m.r * p.ld - sp2.shift + (size_t)piece0 * N) * sizeof(TIn)) + tid;
+#pragma unroll 1
+        for (int k = 0; k < plan.groups * kU; ++k) {
+          const int at = pos + k / kU >= ring ? pos + k / kU - ring : pos + k / kU;
+          const int lp = tid + k * nt;
+          uint4 zv = make_uint4(0u, 0u, 0u, 0u), uv = zv;
+          if (TM && at < plan.tm_groups) {
+            if (!ADWIN_CHK(columns_ok(at), p.status)) break;
+            const uint32_t col = tm_lane + (uint32_t)(at * group_cols + k % kU * kKept * 4);
+            if (FULLKL) tm_load8(col, zv, uv);
+            else tm_load4(col, zv);
             tm_wait_ld();
-          } else {
-            if (!ADWIN_CHK(stash_ok(st - (k % kU) * 2 * array), p.status)) break;
-            zv = *reinterpret_cast<const uint4*>(st);
-            uv = *reinterpret_cast<const uint4*>(st + array);
-            st += 2 * array;
+          } else if (holds(sp2, lp)) {
+            const char* st = stash + (size_t)((uint32_t)(at - plan.tm_groups) * group_bytes);
+            if (!ADWIN_CHK(stash_ok(st), p.status)) break;
+            zv = *reinterpret_cast<const uint4*>(st + k % kU * kKept * array);
+            if (FULLKL) uv = *reinterpret_cast<const uint4*>(st + (k % kU * kKept + 1) * array);
           }
-          if (tid + k * nt < span.pieces) {
+          if (holds(sp2, lp)) {
+            if (!FULLKL && ADWIN_CHK(inside(sp2, lp), p.status)) uv = __ldg(uq + k * nt);
             float z[N], u[N];
             Elem<TIn>::unpack(zv, z);
             Elem<TIn>::unpack(uv, u);
-            acc_piece<N, false>(z, u, 0.f, ra);
+            acc_piece<N, false>(z, u, m.dref, ra);
           }
         }
         const float wms = warp_max(ra.m2s), wmt = warp_max(ra.m2t);
@@ -403,96 +730,35 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         named_sync(kReady, all);
       }
 
-      // -------------------------------------------------------------- sweep 2
-      const f2_t L2 = splat2(kLog2e), NEG1 = splat2(-1.f);
-      const float coef = ctrl.out.coef, c0 = ctrl.out.c0, gy = ctrl.out.gy;
-      const f2_t nM2s = splat2(-ctrl.out.m2s), coef2 = splat2(coef);
-      // bf16 logits: g = e * (coef*delta - coef*c0) saves one operation per pair; its rounding
-      // (relative to coef*delta, not to the difference) is far inside that dtype's tolerance.
-      const f2_t nc0 = splat2(sizeof(TIn) == 2 ? -coef * c0 : -c0);
-      const int64_t yat = (int64_t)m.y + span.shift;                     // counted from piece 0
-      const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
-      const int ypiece = y_valid ? (int)(yat / N - piece0) : -1;         // slice-relative
-      char* gp = static_cast<char*>(p.grad) +
-                 ((size_t)m.r * p.ld_grad - span.shift + (size_t)(piece0 + tid) * N) * sizeof(TOut);
-      f2_t Q = 0ull;
-      const char* st = stash;
-      int lp0 = tid;
-      auto group = [&](auto full, int k0) {
-        constexpr bool FULL = decltype(full)::value;
-        uint4 z[kU], u[kU];
-        if (ahead) prefetch_part();
-        if (TM && k0 < plan.tm_steps) {
-          if (ADWIN_CHK(columns_ok(k0), p.status)) {
-#pragma unroll
-            for (int h = 0; h < kU; ++h) tm_load8(tm_lane + (uint32_t)((k0 + h) * 8), z[h], u[h]);
-            tm_wait_ld();
-          }
+      // -------------------------------------------------------------- second sweep, next row's first
+      {
+        gy = ctrl.out.gy;
+        const int64_t yat = (int64_t)m.y + sp2.shift;                     // counted from piece 0
+        const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
+        yleft = y_valid ? (int)(yat / N - piece0) - tid : -1;             // (slice-relative)
+        ye = (int)(yat % N);
+        gp = static_cast<char*>(p.grad) +
+             ((size_t)m.r * p.ld_grad - sp2.shift + (size_t)(piece0 + tid) * N) * sizeof(TOut);
+        Q = 0ull;
+      }
+      const int groups = plan.groups, both = next ? groups - plan.ahead : 0;
+      // whole groups of both rows
+      const int lo = max(full_from(sp2), full_from(sp1) - plan.ahead), hi = min(full_to(sp2), full_to(sp1) - plan.ahead);
+#pragma unroll 1
+      for (int g = 0; g < groups; ++g) {
+        const int g1 = g + plan.ahead;
+        if (g >= both) {
+          group(no, yes, no, 0, g);
         } else {
-#pragma unroll
-          for (int h = 0; h < kU; ++h) {
-            if ((FULL || lp0 + h * nt < span.pieces) && ADWIN_CHK(stash_ok(st), p.status)) {
-              z[h] = *reinterpret_cast<const uint4*>(st + 2 * h * array);
-              u[h] = *reinterpret_cast<const uint4*>(st + (2 * h + 1) * array);
-            }
-          }
-          st += 2 * kU * array;
+          early(i + 1, g1);
+          if (g >= lo && g < hi) group(yes, yes, yes, g1, g);
+          else group(yes, yes, no, g1, g);
         }
-#pragma unroll
-        for (int h = 0; h < kU; ++h) {
-          const int lp = lp0 + h * nt;
-          if (FULL || lp < span.pieces) {
-            f2_t Z[NP], U[NP], G[NP];
-            Pairs<TIn>::make(z[h], Z);
-            Pairs<TIn>::make(u[h], U);
-#pragma unroll
-            for (int e = 0; e < NP; ++e) {
-              const f2_t E = ex2_2(fma2(Z[e], L2, nM2s));
-              if (full_mode) {
-                if (sizeof(TIn) == 2) G[e] = mul2(E, fma2(fma2(U[e], NEG1, Z[e]), coef2, nc0));
-                else G[e] = mul2(E, mul2(add2(fma2(U[e], NEG1, Z[e]), nc0), coef2));
-              } else {
-                G[e] = mul2(E, coef2);
-              }
-            }
-            if (!full_mode && lp == ypiece) {
-              const int ye = (int)(yat % N);
-#pragma unroll
-              for (int e = 0; e < NP; ++e) {
-                float lo, hi;
-                upk2(G[e], lo, hi);
-                if (ye == 2 * e) lo = gy;
-                if (ye == 2 * e + 1) hi = gy;
-                G[e] = pk2(lo, hi);
-              }
-            }
-#pragma unroll
-            for (int e = 0; e < NP; ++e) Q = fma2(G[e], G[e], Q);
-            if (ADWIN_CHK(((int64_t)piece0 + lp + (RAG ? 0 : 1)) * N <= p.V + span.shift && m.r < p.B * p.T, p.status)) {
-              char* dst = gp + (size_t)h * nt * N * sizeof(TOut);
-              if (RAG && (lp == span.first || lp == span.last)) {   // the row's own entries only
-                const int e0 = span.e0(lp), e1 = lp == span.last ? span.last_n : N;
-#pragma unroll
-                for (int e = 0; e < NP; ++e) {
-                  float lo, hi;
-                  upk2(G[e], lo, hi);
-                  if (2 * e >= e0 && 2 * e < e1) Elem<TOut>::store1(dst, 2 * e, lo);
-                  if (2 * e + 1 >= e0 && 2 * e + 1 < e1) Elem<TOut>::store1(dst, 2 * e + 1, hi);
-                }
-              } else {
-                store_pairs<TOut, NP>(dst, G);
-              }
-            }
-          }
-        }
-        gp += (size_t)kU * nt * N * sizeof(TOut);
-        lp0 += kU * nt;
-      };
-      int k0 = 0;
-      for (; (k0 + kU) * nt <= span.pieces; k0 += kU) group(std::true_type{}, k0);
-      for (; k0 < plan.steps; k0 += kU) group(std::false_type{}, k0);
-      q_prev = hsum2(Q);
+      }
+      if (!next) a.reset();
+      post(hsum2(Q));
     }
+    if (cl > 1 && my_rows > 0) cluster_wait();
   }
   if (TM) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (cl > 1) cluster_sync_all();   // no CTA leaves while a peer may still store into it
@@ -506,106 +772,86 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
 // ---------------------------------------------------------------------------- host side
 constexpr int kSmemPerSm = 233472, kSmemReserved = 1024;   // bytes per SM, and taken by every CTA
 
-struct RowsShape {
-  int ctas, nt, tm_cols, cl;
-  int most_kb;        // bytes of a row (both arrays) up to which the shape is taken, in KB
-};
-// From many small CTAs to two large ones, then clusters; the first that takes the row and holds it
-// is used: the most CTAs per SM, because their number is what hides one row's exchange behind the
-// others' streaming.  Tensor memory is shared out in powers of two.  Measured over 2.4 GB of logits
-// and gradient (367 us at the copy rate; staged kernel / two sweeps over memory / this kernel):
-//   bf16  V =   4 096  2471 / 726 / 475 us  {8, 64}       fp32  V =   4 096  1245 / 454 / 398 us  {5, 128}
-//              8 192  1345 / 594 / 439     {5, 128}               12 000   784 / 606 / 401      {3, 224}
-//             16 384   987 / 556 / 480     {3, 224}               16 384   599 / 647 / 394      {2, 352}
-//             32 000   722 / 814 / 470     {2, 352}               32 000   500 / 686 / 429      {2, 352} x 2
-//             50 264   636 / 856 / 499     {2, 352}               50 264   597 / 719 / 474      {2, 352} x 2
-//            100 000   653 / 908 / 512     {2, 352} x 2           65 536   503 / 711 / 431      {2, 352} x 4
-//            151 936   568 / 852 / 550     {2, 352} x 4
-// bf16 rows are bound by arithmetic and latency (19 issue slots per entry, the ex2 unit 57 % busy),
-// fp32 rows by memory.  Three or four steps in flight spill at 80 registers and lose, one step at 64
-// registers and a third more threads is slower except around 16 384 entries.  (Rows off 16-byte
-// boundaries cost the 64-thread bf16 kernels 68 bytes of spills.)
-// {3, 224} could hold 126 KB but ends at 100 (25 600 entries of bf16).  {3, 224} / {2, 352}: bf16 12 000
-// entries 527 / 566 us, 16 384 487 / 483, 22 000 508 / 487, 25 600 489 / 480, 27 000 523 / 487, 32 000
-// 487 / 470; fp32 6 000 484 / 532, 8 192 392 / 400, 12 800 407 / 392, 14 336 413 / 394, 16 000 424 / 397.
-// So the line keeps the rows that lose 6 % out; the last of those below it still lose 2 to 4 %.
-constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 1 << 20},   {5, 128, 0, 1, 1 << 20},
-                                 {3, 224, 128, 1, 100},    {2, 352, 256, 1, 1 << 20},
-                                 {2, 352, 256, 2, 1 << 20}, {2, 352, 256, 4, 1 << 20}};
-
 constexpr int shape_smem(int ctas) { return kSmemPerSm / ctas - kSmemReserved; }
 
-constexpr bool shape_plan(const RowsShape& sh, int64_t pieces, RowsPlan& plan) {
+// kept: arrays of which the second sweep needs a copy (2, or the student's alone).
+constexpr bool shape_plan(const RowsShape& sh, int64_t pieces, int kept, RowsPlan& plan) {
   plan.cl = sh.cl;
   plan.nt = sh.nt;
   plan.ctas = sh.ctas;
-  plan.per_rank = (int)((pieces + sh.cl - 1) / sh.cl);
-  const int need = (plan.per_rank + sh.nt - 1) / sh.nt;
-  plan.steps = (need + kU - 1) / kU * kU;
-  const int smem = shape_smem(sh.ctas) - rows_ctrl_bytes(sh.nt);
-  const int sm_steps = smem / (32 * sh.nt) / kU * kU;
-  // a lane group's columns are shared by its warps (every fourth); a piece pair takes 8 columns
-  const int tm_most = sh.tm_cols ? sh.tm_cols / ((sh.nt + 127) / 128) / 8 / kU * kU : 0;
-  plan.tm_steps = plan.steps < tm_most ? plan.steps : tm_most;
-  plan.tm_cols = plan.tm_steps ? sh.tm_cols : 0;
-  return plan.steps - plan.tm_steps <= sm_steps;
+  plan.per_rank = (int)((pieces + sh.cl - 1) / sh.cl + kLine / 16 - 1) / (kLine / 16) * (kLine / 16);   // whole lines
+  plan.groups = (plan.per_rank + sh.nt * kU - 1) / (sh.nt * kU);
+  plan.early = plan.groups < kMostEarly ? plan.groups : kMostEarly;
+  const int sm_groups = (shape_smem(sh.ctas) - rows_ctrl_bytes(sh.nt)) / (kU * kept * 16 * sh.nt);
+  // a lane group's columns are shared by its warps (every fourth); a piece takes 4 columns
+  const int tm_groups = sh.tm_cols ? sh.tm_cols / ((sh.nt + 127) / 128) / (kU * kept * 4) : 0;
+  const int spare = sm_groups + tm_groups - plan.groups;
+  if (spare < 0) return false;
+  // one group covers a CTA's own exchange, a cluster's takes two (151 936 entries 426 us with one, 412 with
+  // two); more only run the sweeps apart (32 000 entries 422 with one, 430 with three)
+  const int most = sh.cl > 1 ? 2 : 1;
+  plan.ahead = spare < most ? spare : most;
+  if (plan.ahead > plan.groups) plan.ahead = plan.groups;
+  const int ring = plan.groups + plan.ahead;
+  plan.tm_groups = ring < tm_groups ? ring : tm_groups;
+  plan.tm_cols = plan.tm_groups ? sh.tm_cols : 0;
+  return true;
 }
 
-constexpr int rows_smem(const RowsPlan& plan) {
-  return rows_ctrl_bytes(plan.nt) + (plan.steps - plan.tm_steps) * 32 * plan.nt;
+constexpr int rows_smem(const RowsPlan& plan, int kept) {
+  return rows_ctrl_bytes(plan.nt) +
+         (plan.groups + plan.ahead - plan.tm_groups) * kU * kept * 16 * plan.nt;
 }
 
 // Bytes a launch asks for.  The CTAs of a cluster hold tensor memory while they wait for one another,
 // and tcgen05.alloc waits without a limit: beside a tensor-core kernel of another stream (CTA pairs
 // with all 512 columns), a cluster and a pair could each hold an SM's columns and wait for the other's.
 // So the CTAs of a cluster take at least kClusterSmem: no CTA of tc_pipeline.cuh (199 KB), nor any
-// above 163 KB, fits on an SM beside one, and row CTAs among themselves never need more than 512
-// columns.  (A CTA without a cluster waits for nobody once it has its columns.)  Not the whole share of
-// an SM, which would leave 28 KB of L1 to the streaming kernel that follows in a call with scalars
-// over the rollout (update and audit on 3.8 GB of logits 1215 us so, 1164 with this).
-constexpr int kClusterSmem = 65536 - kSmemReserved;
-constexpr int launch_smem(const RowsPlan& plan) {
-  const int need = rows_smem(plan);
+// above 112 KB, and no other cluster's fits on an SM beside one.  (A CTA without a cluster waits for
+// nobody once it has its columns.)  Not the whole share of an SM, which would leave 28 KB of L1 to the
+// streaming kernel that follows in a call with scalars over the rollout (update and audit on 3.8 GB of
+// logits 1215 us so, 1164 with less).
+constexpr int kClusterSmem = kSmemPerSm / 2;
+constexpr int launch_smem(const RowsPlan& plan, int kept) {
+  const int need = rows_smem(plan, kept);
   return plan.cl > 1 && plan.tm_cols > 0 && need < kClusterSmem ? kClusterSmem : need;
 }
-constexpr bool clusters_exclude_tensor_core_ctas() {
+constexpr bool clusters_exclude_one_another_and_tensor_core_ctas() {
   for (const RowsShape& sh : kShapes) {
     RowsPlan plan = {};
-    for (int64_t pieces = sh.cl; sh.cl > 1 && shape_plan(sh, pieces, plan); pieces += sh.cl * sh.nt * kU)
-      if (plan.tm_cols > 0 && launch_smem(plan) + tc::kSmemBytes + 2 * kSmemReserved <= kSmemPerSm)
-        return false;
+    for (int kept = 1; kept <= 2; ++kept)
+      for (int64_t pieces = sh.cl; sh.cl > 1 && shape_plan(sh, pieces, kept, plan); pieces += sh.cl * sh.nt * kU)
+        if (plan.tm_cols > 0 &&
+            (launch_smem(plan, kept) + tc::kSmemBytes + 2 * kSmemReserved <= kSmemPerSm ||
+             2 * (launch_smem(plan, kept) + kSmemReserved) <= kSmemPerSm))
+          return false;
   }
   return true;
 }
-static_assert(clusters_exclude_tensor_core_ctas(), "a cluster could wait for a pair's tensor memory");
+static_assert(clusters_exclude_one_another_and_tensor_core_ctas(), "a cluster could wait for another's tensor memory");
 
-bool rows_plan(int64_t pieces, RowsPlan& plan) {
+bool rows_plan(int64_t pieces, int kept, RowsPlan& plan) {
   if (pieces < 1 || pieces > (int64_t)1 << 24) return false;
   for (const RowsShape& sh : kShapes)
-    if (pieces * 32 <= (int64_t)sh.most_kb * 1024 && shape_plan(sh, pieces, plan)) return true;
+    if (pieces <= sh.most && shape_plan(sh, pieces, kept, plan)) return true;
   return false;
 }
 
 typedef void (*RowsKernel)(KlParams, RowsPlan);
-// Whether the shapes of NT threads use tensor memory (all of them or none; `steps` is never less than
-// kU, so a plan of such a shape always does).
-constexpr bool uses_tensor_memory(int nt) {
-  for (const RowsShape& sh : kShapes)
-    if (sh.nt == nt) return sh.tm_cols > 0;
-  return false;
-}
 template <typename TIn, typename TOut, int NT>
-RowsKernel rows_kernel_nt(bool ragged) {
+RowsKernel rows_kernel_nt(bool ragged, bool full_kl) {
   constexpr bool TM = uses_tensor_memory(NT);
-  return ragged ? kl_rows_kernel<TIn, TOut, NT, TM, true> : kl_rows_kernel<TIn, TOut, NT, TM, false>;
+  if (full_kl)
+    return ragged ? kl_rows_kernel<TIn, TOut, NT, TM, true, true> : kl_rows_kernel<TIn, TOut, NT, TM, false, true>;
+  return ragged ? kl_rows_kernel<TIn, TOut, NT, TM, true, false> : kl_rows_kernel<TIn, TOut, NT, TM, false, false>;
 }
 template <typename TIn, typename TOut>
-RowsKernel rows_kernel(int nt, bool ragged) {
+RowsKernel rows_kernel(int nt, bool ragged, bool full_kl) {
   switch (nt) {
-    case 64: return rows_kernel_nt<TIn, TOut, 64>(ragged);
-    case 128: return rows_kernel_nt<TIn, TOut, 128>(ragged);
-    case 224: return rows_kernel_nt<TIn, TOut, 224>(ragged);
-    case 352: return rows_kernel_nt<TIn, TOut, 352>(ragged);
+    case 64: return rows_kernel_nt<TIn, TOut, 64>(ragged, full_kl);
+    case 128: return rows_kernel_nt<TIn, TOut, 128>(ragged, full_kl);
+    case 256: return rows_kernel_nt<TIn, TOut, 256>(ragged, full_kl);
+    case kRowsThreads: return rows_kernel_nt<TIn, TOut, kRowsThreads>(ragged, full_kl);
     default: return nullptr;
   }
 }
@@ -625,7 +871,7 @@ cudaError_t resident_clusters(const RowsPlan& plan, int sm_count, int& n) {
   std::lock_guard<std::mutex> lock(mu);
   n = seen[dev][plan.cl];
   if (n > 0) return cudaSuccess;
-  const RowsKernel like = kl_rows_kernel<float, float, kRowsThreads, false, false>;
+  const RowsKernel like = kl_rows_kernel<float, float, kRowsThreads, false, false, true>;
   const int smem = shape_smem(plan.ctas);
   e = cudaFuncSetAttribute(like, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -658,10 +904,15 @@ template <typename TIn, typename TOut>
 cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStream_t s) {
   constexpr int N = Elem<TIn>::N;
   RowsPlan plan = {};
-  if (!rows_plan(ragged ? (p.V + 2 * N - 2) / N : p.V / N, plan)) return cudaErrorNotSupported;
-  const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, ragged);
+  const bool full_kl = p.mode == ADWIN_GRAD_FULL_KL;
+  const int kept = full_kl ? 2 : 1;
+  // rows that do not all start on the same 16-byte boundary of a line
+  ragged = ragged || (p.ld * sizeof(TIn)) % kLine != 0 || reinterpret_cast<uintptr_t>(p.student) % kLine != 0;
+  const int64_t lead = ragged ? kLine / (int64_t)sizeof(TIn) - 1 : 0;   // entries of a line before the row, at most
+  if (!rows_plan((lead + p.V + N - 1) / N, kept, plan)) return cudaErrorNotSupported;
+  const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, ragged, full_kl);
   if (!kernel) return cudaErrorNotSupported;
-  const int smem = launch_smem(plan);
+  const int smem = launch_smem(plan, kept);
   plan.num_clusters = plan.ctas * sm_count;
   cudaError_t e;
   if (plan.cl > 1) {

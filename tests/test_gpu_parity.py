@@ -586,6 +586,30 @@ def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
     run_and_check(batch, grad_dtype=g_dt, flags=api.RANGE_FULL)
 
 
+# Several rows for every CTA of a launch, so that a row's second sweep runs beside the next row's first and
+# the ring of kept pieces turns over: the longest rows of each shape (bf16; half of that fp32), rows of whole
+# lines and rows that start anywhere in one, and the first of a cluster of two and of four.
+@pytest.mark.parametrize("in_dt,V,rows", [(2, 4099, 2500), (2, 4096, 2500), (2, 28665, 1250), (2, 57341, 620), (2, 57344, 620),
+                                          (2, 114681, 310), (2, 114752, 170), (2, 262144, 80), (1, 2050, 2500),
+                                          (1, 14331, 1250), (1, 57341, 310), (1, 57349, 170)])
+def test_rows_one_after_another(in_dt, V, rows):
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=rows // 2, V=V)
+    batch.window = torch.tensor([rows // 2, rows // 2 - 3], dtype=torch.int32, device=DEV)
+    # sampled tokens in the partial pieces of a row and between; every seventh far below the maximum, which
+    # sums the row again.  z - u of eight there: c is a difference of fp32 logits and logarithms of up to 16, off by
+    # 2e-6, and twice that over |c| has to stay below 1e-4 (the norm of the sampled gradient)
+    for k, y in enumerate((0, 3, V - 1, V - 4, V // 2)):
+        batch.tokens[:, k::6] = y
+    y = batch.tokens.long()[..., None]
+    z = batch.student.gather(2, y)
+    z[:, ::7] = batch.student[:, ::7].float().amax(2, keepdim=True).to(z.dtype) - 100.0
+    batch.student.scatter_(2, y, z)
+    batch.teacher.scatter_(2, y, z - 8.0)
+    g_dt = torch.float32 if in_dt == 1 else torch.bfloat16
+    run_and_check(batch, grad_dtype=g_dt, grad_mode=api.GRAD_FULL_KL)
+    run_and_check(batch, grad_dtype=g_dt, grad_mode=api.GRAD_SAMPLED)
+
+
 @pytest.mark.parametrize("in_dt,V", [(2, 4095), (2, 4096), (2, 4104), (2, 20001), (1, 2047), (1, 2052), (1, 9001)])
 @pytest.mark.parametrize("mode", [api.GRAD_FULL_KL, api.GRAD_SAMPLED])
 def test_read_only_rows_that_outgrow_their_first_entries(in_dt, V, mode):
