@@ -222,15 +222,47 @@ __device__ __forceinline__ float copy_dot(const __nv_bfloat16* src, const __nv_b
 // their difference is the value the sweep centres z - u on: on a peaked row the sampled token is
 // almost surely the peak, where the centred difference is then exactly zero, which keeps the
 // single-sweep squared-norm moments well conditioned.
+// OWN: every block forms the prefix sums itself, in shared memory, which for a short call costs less than a
+// launch of lm_plan_kernel and round trips to memory for the search below (225 rows: 7.5 us where the two kernels
+// take 11.5; 4 400 rows in seven segments 54 us where they take 40).
+constexpr int kGatherSeqs = 128;
+constexpr int64_t kGatherOwnRows = 2048;
+template <bool OWN>
 __global__ void __launch_bounds__(kGatherThreads) lm_gather_kernel(const GatherParams p, const SegPlan plan) {
   chain();
   __shared__ int64_t base[kMaxSeg + 1];
   __shared__ float red[2][kGatherThreads / 32];
+  __shared__ int64_t own[OWN ? kMaxSeg : 1][OWN ? kGatherSeqs + 1 : 1];
+  if (OWN) {
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < plan.n_seg; i += kGatherThreads / 32) {   // a warp per segment
+      int64_t before = 0;
+      for (int b0 = 0; b0 < p.B; b0 += 32) {
+        int64_t n = 0;
+        if (b0 + lane < p.B) {
+          int lo, hi;
+          plan.range(i, p.ewin[b0 + lane], p.range[b0 + lane], lo, hi);
+          n = hi - lo;
+        }
+        int64_t x = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (b0 + lane < p.B) own[i][b0 + lane] = before + x - n;
+        before += __shfl_sync(0xffffffffu, x, 31);
+      }
+      if (lane == 0) own[i][p.B] = before;
+    }
+    __syncthreads();
+  }
+  auto offsets = [&](int i) { return OWN ? own[i] : p.seg + (int64_t)i * (p.B + 1); };
   if (threadIdx.x == 0) {
     int64_t o = 0;
     for (int i = 0; i < plan.n_seg; ++i) {
       base[i] = o;
-      o += (p.seg[(int64_t)i * (p.B + 1) + p.B] + plan.pad - 1) / plan.pad * plan.pad;
+      o += (offsets(i)[p.B] + plan.pad - 1) / plan.pad * plan.pad;
     }
     base[plan.n_seg] = o;
   }
@@ -255,7 +287,7 @@ __global__ void __launch_bounds__(kGatherThreads) lm_gather_kernel(const GatherP
     if (r < rows) {
       int i = 0;
       while (r >= base[i + 1]) ++i;
-      const int64_t* off = p.seg + (int64_t)i * (p.B + 1);
+      const int64_t* off = offsets(i);
       const int64_t k = r - base[i];
       if (k < off[p.B]) {
         int64_t b = 0, e = p.B;   // the last sequence with off[b] <= k
@@ -599,40 +631,51 @@ struct MergeParams {
 //   g_k = p_k (a1 (z_k - u_k) + a0) (+ gy at k = y),   p_k = 2^(z_k log2e - L2s);
 // a row without gradient has L2s = infinity: p_k, and g_k with a1 = a0 = gy = 0, are exactly zero
 // whatever its logits (with L2s = 0, p_k overflows beyond z = 88 and 0 * inf spreads over dW).
-// Records are read with the row as the fast index (whole 128-byte lines), reduced with the record
+// Records are read with the row as the fast index (whole 32-byte sectors at least), reduced with the record
 // as the lane.  A short call has many records (126 for each of 225 rows at V = 32 000), which is
-// why the records are spread over threads: 21 -> 5 us there against 8 threads per row.
+// why the records are spread over threads, and the more the fewer tiles there are: ROWS = 8 up to
+// kMergeFewTiles (225 rows: 8 blocks of 32 rows, four records a thread, took 14.5 us).
 constexpr int kMergeRows = 32;
+constexpr int kMergeFewTiles = 8;
+template <int ROWS>
 __global__ void __launch_bounds__(1024) lm_merge_kernel(const MergeParams p) {
   chain();
-  __shared__ double red[6][32][kMergeRows];
+  constexpr int kRecs = 1024 / ROWS;   // threads per row
+  __shared__ double red[6][32][ROWS];  // a value per warp and row
   int64_t lo, hi;
   launch_tiles(p.hdr, p.tile0, p.tile_cap, p.rest, lo, hi);
-  const int64_t tile = lo + blockIdx.x / (kBM / kMergeRows);
+  const int64_t tile = lo + blockIdx.x / (kBM / ROWS);
   if (tile >= hi) return;
-  const int first = blockIdx.x % (kBM / kMergeRows) * kMergeRows;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int first = blockIdx.x % (kBM / ROWS) * ROWS;
+  const int row = threadIdx.x % ROWS, mine = threadIdx.x / ROWS;
   const int n = p.hdr->n_groups * 2;
-  // while reading: lane = row, warp = record
-  const float* rec = p.part + ((tile - lo) * n * kRecFields) * kBM + first + lane;
+  const float* rec = p.part + ((tile - lo) * n * kRecFields) * kBM + first + row;
   auto f = [&](int i, int k) { return (double)rec[((int64_t)i * kRecFields + k) * kBM]; };
   double M2s = -INFINITY, M2t = -INFINITY;
-  for (int i = warp; i < n; i += 32) {
+  for (int i = mine; i < n; i += kRecs) {
     M2s = fmax(M2s, f(i, 0));
     M2t = fmax(M2t, f(i, 6));
   }
-  red[0][warp][lane] = M2s;
-  red[1][warp][lane] = M2t;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o >= ROWS; o >>= 1) {
+    M2s = fmax(M2s, __shfl_xor_sync(0xffffffffu, M2s, o));
+    M2t = fmax(M2t, __shfl_xor_sync(0xffffffffu, M2t, o));
+  }
+  if (lane < ROWS) {
+    red[0][warp][lane] = M2s;
+    red[1][warp][lane] = M2t;
+  }
   __syncthreads();
-  M2s = red[0][0][lane];
-  M2t = red[1][0][lane];
+  M2s = red[0][0][row];
+  M2t = red[1][0][row];
   for (int w = 1; w < 32; ++w) {
-    M2s = fmax(M2s, red[0][w][lane]);
-    M2t = fmax(M2t, red[1][w][lane]);
+    M2s = fmax(M2s, red[0][w][row]);
+    M2t = fmax(M2t, red[1][w][row]);
   }
   __syncthreads();
   double v[6] = {0, 0, 0, 0, 0, 0};   // S, Ac, B0, B1, B2, St
-  for (int i = warp; i < n; i += 32) {
+  for (int i = mine; i < n; i += kRecs) {
     const double w = exp2(f(i, 0) - M2s), w2 = w * w;
     v[0] += w * f(i, 1);
     v[1] += w * f(i, 2);
@@ -642,15 +685,22 @@ __global__ void __launch_bounds__(1024) lm_merge_kernel(const MergeParams p) {
     v[5] += exp2(f(i, 6) - M2t) * f(i, 7);
   }
 #pragma unroll
-  for (int k = 0; k < 6; ++k) red[k][warp][lane] = v[k];
-  __syncthreads();
-  if (warp < 6) {   // one field per warp, lane = row
-    double t = 0.0;
-    for (int w = 0; w < 32; ++w) t += red[warp][w][lane];
-    red[warp][0][lane] = t;
+  for (int k = 0; k < 6; ++k) {
+#pragma unroll
+    for (int o = 16; o >= ROWS; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane < ROWS) red[k][warp][lane] = v[k];
   }
   __syncthreads();
-  if (warp != 0) return;
+  if (warp < 6) {   // one field per warp, 32 / ROWS lanes per row
+    double t = 0.0;
+    for (int w = lane / ROWS; w < 32; w += 32 / ROWS) t += red[warp][w][lane % ROWS];
+#pragma unroll
+    for (int o = 16; o >= ROWS; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    __syncwarp();
+    if (lane < ROWS) red[warp][0][lane] = t;
+  }
+  __syncthreads();
+  if (warp != 0 || lane >= ROWS) return;
   const int64_t crow = tile * kBM + first + lane;
   const double S = red[0][0][lane], Ac = red[1][0][lane], B0 = red[2][0][lane];
   const double B1 = red[3][0][lane], B2 = red[4][0][lane], St = red[5][0][lane];
@@ -878,9 +928,13 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
   gp.hs_c = hs_c;
   gp.ht_c = ht_c;
   gp.status = a.status;
-  launch_chained(lm_plan_kernel, plan.n_seg, 1024, 0, 1, s, gp.range, gp.ewin, a.B, plan, seg);
-  launch_chained(lm_gather_kernel, (unsigned)(rows_cap < 16384 ? rows_cap : 16384), kGatherThreads, 0, 1, s,
-                 gp, plan);
+  const unsigned gather_grid = (unsigned)(rows_cap < 16384 ? rows_cap : 16384);
+  if (a.B <= kGatherSeqs && rows_cap <= kGatherOwnRows) {
+    launch_chained(lm_gather_kernel<true>, gather_grid, kGatherThreads, 0, 1, s, gp, plan);
+  } else {
+    launch_chained(lm_plan_kernel, plan.n_seg, 1024, 0, 1, s, gp.range, gp.ewin, a.B, plan, seg);
+    launch_chained(lm_gather_kernel<false>, gather_grid, kGatherThreads, 0, 1, s, gp, plan);
+  }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
   CUtensorMap m_hs, m_ws, m_ht, m_wt;
@@ -932,7 +986,8 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
         moments ? launch_pairs(lm_sweep_kernel<true>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp)
                 : launch_pairs(lm_sweep_kernel<false>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp);
     if (r != cudaSuccess) return r;
-    launch_chained(lm_merge_kernel, (unsigned)cap * (kBM / kMergeRows), 1024, 0, 1, s, mp);
+    if (cap <= kMergeFewTiles) launch_chained(lm_merge_kernel<8>, (unsigned)cap * (kBM / 8), 1024, 0, 1, s, mp);
+    else launch_chained(lm_merge_kernel<32>, (unsigned)cap * (kBM / 32), 1024, 0, 1, s, mp);
     return cudaGetLastError();
   };
   if (!a.want_grad) return statistics(0, L.max_tiles, 2, false, a.gsq != nullptr);
