@@ -19,8 +19,8 @@
 //
 // Exponentials are taken against a reference that the whole row shares (the logit of the sampled
 // token), so partial sums add without rescaling.  If the sums overflow it (a sampled token more than
-// ~69 nats below the row maximum) the row is summed once more, from its on-chip copy, against
-// running maxima.  Rows too long for one CTA are split over a cluster; the CTAs' sums then go to every
+// ~69 nats below the row maximum) the row is summed once more, from its on-chip copy (the teacher's
+// pieces from memory where only the student's are kept), against running maxima.  Rows too long for one CTA are split over a cluster; the CTAs' sums then go to every
 // CTA of the cluster.
 #include <mutex>
 #include <type_traits>
