@@ -391,6 +391,17 @@ def test_rows_packed_across_sequences_at_tile_edges(windows):
         check_all(batch, got, oracle(batch, api.GRAD_FULL_KL, flags), flags)
 
 
+@pytest.mark.parametrize("B,T", [(33, 9), (128, 8), (129, 8), (40, 27), (40, 60)])
+def test_many_short_sequences(B, T):
+    """The prefix sums over the sequences formed by the gather kernel's blocks (up to 128 sequences and 2048
+    rows) and by a kernel of their own; the partial records merged 8 rows a block (up to 8 tiles) and 32."""
+    batch = synth.make_lmhead_batch(DEV, B=B, T=T, V=520, d_s=64, d_t=72, w_std=0.1)
+    rng = np.random.default_rng(B + T)
+    batch.window = torch.from_numpy(rng.integers(0, T + 1, B).astype(np.int32)).to(DEV)
+    got = run(batch, flags=api.RANGE_FULL)
+    check_all(batch, got, oracle(batch, api.GRAD_FULL_KL, api.RANGE_FULL), api.RANGE_FULL)
+
+
 @pytest.mark.parametrize("mode", [api.GRAD_FULL_KL, api.GRAD_SAMPLED])
 def test_large_logits_past_the_window_leave_the_weight_gradient_alone(mode):
     """Rows without gradient share the last tile of those with: one whose logits are beyond what an
