@@ -39,6 +39,11 @@ constexpr int kRowsThreads = 512;     // threads of a CTA that hold pieces, at m
 constexpr int kU = 2;
 constexpr int kRowsMaxCl = 4;
 constexpr float kSumLimit = 1.2676506e30f;   // 2^100: beyond it the shared reference is unsafe
+// Rows' metadata: the row's own warp has written that of row i + kMetaAhead when it gives out row i's scalars
+// (kReady), and the other threads may look at no row beyond before they are through the next kReady.  A load is one group
+// ahead of its sweep, which itself runs `ahead` groups into row i + 1 before row i's kReady: rows of one group
+// are asked for two rows after i + 1.  metadata_precedes_its_readers() holds every plan against this.
+constexpr int kMetaAhead = 4;
 constexpr int kMetaDepth = 8;
 constexpr int kMostEarly = 3;         // groups from a piece's way into L2 to its load, at most
 constexpr int kLine = 128;
@@ -283,11 +288,10 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       if (lane == 0) fill(i, r);
       fill_edges(i, r);
     };
-    // The first three rows at once, a lane each (one after another they are nine round trips to memory), and
+    // The first rows at once, a lane each (one after another they are three round trips to memory each), and
     // the first row on its way into L2 before its metadata.
-    constexpr int kFirst = 3;
     {
-      const int n = min(kFirst, my_rows);
+      const int n = min(kMetaAhead, my_rows);
       const int64_t r = row_of(min(lane, max(n - 1, 0)));
       if (lane == 0 && n > 0) {
         prefetch(r, p.student, 0, plan.per_rank);
@@ -304,8 +308,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     for (int i = 0; i <= my_rows && my_rows > 0; ++i) {
       const bool real = i < my_rows;
       const int par = i & 1;
-      // (the others are at rows i - 1 and i, and take up i + 1 after this exchange)
-      if (i + 3 < my_rows) fetch(i + 3);
+      // (the others have begun no row before i - 1 ended, and read no further than kMetaAhead says)
+      if (i + kMetaAhead < my_rows) fetch(i + kMetaAhead);
       named_sync(kPosted, all);
       // fixed-order sums over the threads, then over the CTAs
       float4 x4[nw];
@@ -829,6 +833,21 @@ constexpr bool clusters_exclude_one_another_and_tensor_core_ctas() {
   return true;
 }
 static_assert(clusters_exclude_one_another_and_tensor_core_ctas(), "a cluster could wait for another's tensor memory");
+
+constexpr bool metadata_precedes_its_readers() {
+  for (const RowsShape& sh : kShapes) {
+    RowsPlan plan = {};
+    for (int kept = 1; kept <= 2; ++kept)
+      for (int64_t pieces = 1; shape_plan(sh, pieces, kept, plan); pieces += sh.cl * sh.nt * kU) {
+        // the last rows, counted from i, that are loaded from and brought into L2 before row i's kReady
+        const int loaded = 1 + (plan.ahead + 1) / plan.groups;
+        const int prefetched = plan.ahead ? 1 + (plan.ahead - 1 + plan.early) / plan.groups : 1;
+        if (loaded >= kMetaAhead || prefetched >= kMetaAhead) return false;
+      }
+  }
+  return kMetaAhead + 1 < kMetaDepth;   // row i - 1 is in use while that of row i + kMetaAhead is written
+}
+static_assert(metadata_precedes_its_readers(), "a row's metadata could be read before it is written");
 
 bool rows_plan(int64_t pieces, int kept, RowsPlan& plan) {
   if (pieces < 1 || pieces > (int64_t)1 << 24) return false;

@@ -79,6 +79,12 @@ def test_ends_of_the_row_kernels_shapes(checked_library, v):
         G.test_rows_held_by_one_cta_and_by_clusters(1, V)
 
 
+@pytest.mark.parametrize("in_dt,V", [(2, 33), (2, 961), (2, 1024), (2, 1032), (1, 481)])
+def test_short_rows_one_after_another(checked_library, in_dt, V):
+    G.test_short_rows_one_after_another(in_dt, V, 2, 3500)
+    G.test_short_rows_one_after_another(in_dt, V, 900, 16)
+
+
 def test_read_only_rows(checked_library):
     for in_dt, V, rows in ((2, 120001, 20), (2, 32003, 300), (1, 93534, 20)):
         G.test_read_only_rows_split_over_a_cluster(in_dt, V, rows)

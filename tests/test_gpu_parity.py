@@ -595,9 +595,14 @@ def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
 def test_rows_one_after_another(in_dt, V, rows):
     batch = synth.make_batch(in_dt, device=DEV, B=2, T=rows // 2, V=V)
     batch.window = torch.tensor([rows // 2, rows // 2 - 3], dtype=torch.int32, device=DEV)
+    check_rows_one_after_another(batch)
+
+
+def check_rows_one_after_another(batch, second=False):
     # sampled tokens in the partial pieces of a row and between; every seventh far below the maximum, which
     # sums the row again.  z - u of eight there: c is a difference of fp32 logits and logarithms of up to 16, off by
     # 2e-6, and twice that over |c| has to stay below 1e-4 (the norm of the sampled gradient)
+    V = batch.shape[2]
     for k, y in enumerate((0, 3, V - 1, V - 4, V // 2)):
         batch.tokens[:, k::6] = y
     y = batch.tokens.long()[..., None]
@@ -605,9 +610,31 @@ def test_rows_one_after_another(in_dt, V, rows):
     z[:, ::7] = batch.student[:, ::7].float().amax(2, keepdim=True).to(z.dtype) - 100.0
     batch.student.scatter_(2, y, z)
     batch.teacher.scatter_(2, y, z - 8.0)
-    g_dt = torch.float32 if in_dt == 1 else torch.bfloat16
+    if second:
+        # In a short row the peak may have nearly all of the mass, and a gradient that is the rounding of z - u less its mean.
+        # So an entry beside the peak gets 1/21 of its mass, at z - u = -16, eight and more from the peak's: 2^-24 * 16 a
+        # rounding against 8 / 21 and more, 5e-6 of the norm, of which its tolerance of 1e-4 bears twenty.
+        z, at = batch.student.max(2, keepdim=True)
+        at = torch.where((at + 1) % V == y, at + 2, at + 1) % V
+        z = (z.float() - 3.0).to(z.dtype)
+        batch.student.scatter_(2, at, z)
+        batch.teacher.scatter_(2, at, z + 16.0)
+    g_dt = batch.student.dtype
     run_and_check(batch, grad_dtype=g_dt, grad_mode=api.GRAD_FULL_KL)
     run_and_check(batch, grad_dtype=g_dt, grad_mode=api.GRAD_SAMPLED)
+
+
+# Rows of one and two groups of loads, several for every CTA of the 64-thread shape (1184 CTAs on 148 SMs): the
+# loads run two rows ahead of the row whose sums are out, and so do its metadata.  Two long sequences, and
+# many so short that a CTA's next row is several sequences on.
+@pytest.mark.parametrize("in_dt,V", [(2, 33), (2, 64), (2, 961), (2, 1024), (2, 1032), (1, 33), (1, 481), (1, 512)])
+@pytest.mark.parametrize("B,T", [(2, 3500), (900, 16)])
+def test_short_rows_one_after_another(in_dt, V, B, T):
+    batch = synth.make_batch(in_dt, device=DEV, B=B, T=T, V=V)
+    rng = np.random.default_rng(V + B)
+    batch.window = torch.from_numpy(rng.integers(T - 3 if B == 2 else 1, T + 1, B).astype(np.int32)).to(DEV)
+    batch.rollout_len[:] = T
+    check_rows_one_after_another(batch, second=True)
 
 
 @pytest.mark.parametrize("in_dt,V", [(2, 4095), (2, 4096), (2, 4104), (2, 20001), (1, 2047), (1, 2052), (1, 9001)])
