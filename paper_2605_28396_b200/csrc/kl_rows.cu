@@ -162,7 +162,8 @@ struct RowSlice {
 
 // NT: threads that hold pieces, a template constant so that the strides between a thread's pieces are
 // offsets in the instructions.  A group of kU steps in which every thread has whole pieces takes the path
-// without tests (FULL below).  FULLKL: the gradient of Eq. 2; without it, of Eq. 4, whose second sweep
+// without tests (FULL below), also where one sweep runs alone: with one row a CTA nothing else runs (280 rows of
+// 32 000 entries of bf16, 23.4 us with the tests there, 20.9 without).  FULLKL: the gradient of Eq. 2; without it, of Eq. 4, whose second sweep
 // takes the student's logits alone, so only they are kept.
 template <typename TIn, typename TOut, int NT, bool TM, bool RAG, bool FULLKL>
 __global__ void __launch_bounds__(NT + 32, ctas_of(NT))
@@ -674,7 +675,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
 #pragma unroll 1
         for (int g = 0; g < to; ++g) {
           early(i + 1, g);
-          group(yes, no, no, g, 0);
+          if (g >= full_from(sp1) && g < full_to(sp1)) group(yes, no, yes, g, 0);
+          else group(yes, no, no, g, 0);
         }
       }
       if (i < 0) {
@@ -752,7 +754,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       for (int g = 0; g < groups; ++g) {
         const int g1 = g + plan.ahead;
         if (g >= both) {
-          group(no, yes, no, 0, g);
+          if (g >= full_from(sp2) && g < full_to(sp2)) group(no, yes, yes, 0, g);
+          else group(no, yes, no, 0, g);
         } else {
           early(i + 1, g1);
           if (g >= lo && g < hi) group(yes, yes, yes, g1, g);
