@@ -289,14 +289,16 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       if (lane == 0) fill(i, r);
       fill_edges(i, r);
     };
-    // The first rows at once, a lane each (one after another they are three round trips to memory each), and
-    // the first row on its way into L2 before its metadata.
+    // The first rows at once, a lane each (one after another they are three round trips to memory each).  Before
+    // them the first row's first groups set out for L2; the rest follows as in every row.  (All of the row at once, and
+    // its groups once more as their turn came: one row a CTA, 280 rows of 32 000 entries of bf16, 20.9 us, 19.6 so;
+    // of 50 257 entries 27.6 and 25.5.)
     {
       const int n = min(kMetaAhead, my_rows);
       const int64_t r = row_of(min(lane, max(n - 1, 0)));
       if (lane == 0 && n > 0) {
-        prefetch(r, p.student, 0, plan.per_rank);
-        prefetch(r, p.teacher, 0, plan.per_rank);
+        prefetch(r, p.student, 0, plan.early * kU * nt);
+        prefetch(r, p.teacher, 0, plan.early * kU * nt);
       }
       if (lane < n) fill(lane, r);
       for (int i = 0; i < n; ++i) fill_edges(i, __shfl_sync(0xffffffffu, r, i));
