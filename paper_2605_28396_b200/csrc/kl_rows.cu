@@ -275,19 +275,25 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       m.nref[6] = m.nref[7] = 0.f;
       m.w = p.row_coef ? p.row_coef[r] : 0.f;
     };
-    auto fill_edges = [&](int i, int64_t r) {
-      if (!edges || lane >= kEdges) return;
+    auto edge_logits = [&](int64_t r, float& z, float& u) {
       const int64_t k = edge_of(r);
-      float* at = ctrl.meta[i % kMetaDepth].edge[lane];
       const bool has = k >= 0 && ADWIN_CHK(k < p.V && r < p.B * p.T, p.status);
-      at[0] = has ? Elem<TIn>::load1(p.student, r * p.ld + k) : kMaskedEdge;
-      at[1] = has ? Elem<TIn>::load1(p.teacher, r * p.ld + k) : kMaskedEdge;
+      z = has ? Elem<TIn>::load1(p.student, r * p.ld + k) : kMaskedEdge;
+      u = has ? Elem<TIn>::load1(p.teacher, r * p.ld + k) : kMaskedEdge;
+    };
+    auto put_edges = [&](int i, float z, float u) {
+      if (!edges || lane >= kEdges) return;
+      float* at = ctrl.meta[i % kMetaDepth].edge[lane];
+      at[0] = z;
+      at[1] = u;
     };
     auto row_of = [&](int i) { return cur.locate(p, cluster_id + (int64_t)i * plan.num_clusters, wg_unused); };
     auto fetch = [&](int i) {
       const int64_t r = row_of(i);
       if (lane == 0) fill(i, r);
-      fill_edges(i, r);
+      float z, u;
+      edge_logits(r, z, u);
+      put_edges(i, z, u);
     };
     // The first rows at once, a lane each (one after another they are three round trips to memory each).  Before
     // them the first row's first groups set out for L2; the rest follows as in every row.  (All of the row at once, and
@@ -300,8 +306,16 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         prefetch(r, p.student, 0, plan.early * kU * nt);
         prefetch(r, p.teacher, 0, plan.early * kU * nt);
       }
+      float z[kMetaAhead], u[kMetaAhead];   // (all asked for before the first is stored)
+#pragma unroll
+      for (int i = 0; i < kMetaAhead; ++i) {
+        const int64_t ri = __shfl_sync(0xffffffffu, r, i);
+        if (i < n) edge_logits(ri, z[i], u[i]);
+      }
       if (lane < n) fill(lane, r);
-      for (int i = 0; i < n; ++i) fill_edges(i, __shfl_sync(0xffffffffu, r, i));
+#pragma unroll
+      for (int i = 0; i < kMetaAhead; ++i)
+        if (i < n) put_edges(i, z[i], u[i]);
     }
     __syncthreads();
     int64_t r_prev = 0;
