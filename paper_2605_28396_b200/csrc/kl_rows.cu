@@ -510,7 +510,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     bool before = false;        // (the piece belongs to the row before: only the first one may)
     int load_row = -1, load_group = 0;
     const ptrdiff_t to_teacher = static_cast<const char*>(p.teacher) - static_cast<const char*>(p.student);
-    auto load = [&](int h) {
+    auto load = [&](int h, uint4 (&zn)[kU], uint4 (&un)[kU]) {
       if (left > h * nt && !(RAG && h == 0 && before) &&
           ADWIN_CHK((zp - static_cast<const char*>(p.student)) + (h * nt + 1) * 16 <=
                         ((p.B * p.T - 1) * p.ld + p.V) * (int64_t)sizeof(TIn), p.status)) {
@@ -557,9 +557,11 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     char* gp = nullptr;
 
     // One group: the second sweep's group g2 (TWO) and the first sweep's group g1 of the row after (ONE),
-    // which takes its place in the ring.
-    auto group = [&](auto one_, auto two_, auto full_, int g1, int g2) __attribute__((always_inline)) {
+    // which takes its place in the ring.  g1's pieces are in zn and un; with LOAD the next in line replace them.
+    auto group_of = [&](auto one_, auto two_, auto full_, auto load_, int g1, int g2, uint4 (&zn)[kU],
+                        uint4 (&un)[kU]) __attribute__((always_inline)) {
       constexpr bool ONE = decltype(one_)::value, TWO = decltype(two_)::value, FULL = decltype(full_)::value;
+      constexpr bool LOAD = decltype(load_)::value;
       const bool in_tm = TM && pos < plan.tm_groups;
       const uint32_t tm_at = TM ? tm_lane + (uint32_t)(pos * group_cols) : 0u;
       char* st = stash + (size_t)((uint32_t)(pos - plan.tm_groups) * group_bytes);
@@ -641,18 +643,21 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
             if constexpr (kCentred) acc_grad_centred<NP>(Z, U, nrefs, nreft, ndref, a);
             else acc_grad<NP, 0>(Z, U, nrefs, nreft, a);
           }
-          load(h);
+          if constexpr (LOAD) load(h, zn, un);
         }
       }
       if constexpr (TWO) {
         gp += (size_t)kU * nt * N * sizeof(TOut);
         if constexpr (!FULLKL) yleft -= kU * nt;
       }
-      if constexpr (ONE) loaded();
+      if constexpr (ONE && LOAD) loaded();
       pos = pos + 1 == ring ? 0 : pos + 1;
     };
     constexpr std::true_type yes{};
     constexpr std::false_type no{};
+    auto group = [&](auto one, auto two, auto full, int g1, int g2) __attribute__((always_inline)) {
+      group_of(one, two, full, yes, g1, g2, zn, un);
+    };
     // the group `plan.early` groups behind group g of row i in the order of the first sweeps
     auto early = [&](int i, int g) {
       if (warp == g % nw && lane == 0) {
@@ -676,7 +681,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
 
     next_load_row();
 #pragma unroll
-    for (int h = 0; h < kU; ++h) load(h);
+    for (int h = 0; h < kU; ++h) load(h, zn, un);
     loaded();
 #pragma unroll 1
     for (int i = -1; i < my_rows; ++i) {
@@ -688,8 +693,27 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         begin_sums(i + 1);
         const int to = i < 0 ? plan.groups : plan.ahead;
         if (i >= 0) pos = pos + plan.groups >= ring ? pos - plan.ahead : pos + plan.groups;
+        int g = 0;
+        // The first row has no second sweep beside it to fill the time of a load: two groups are in flight.  Clusters of
+        // two, 60 rows of 151 936 entries of bf16: 23.6 us with one, 22.7 with two; 1400 rows 226 and 220.  (Not in the other
+        // kernels: {2, 256} and rows off the lines pay for the registers in the loop below, 700 rows of 50 257 entries
+        // 49.0 -> 53.5 us; fp32 rows, which have less to do per byte, gain nothing.)
+        if constexpr (sizeof(TIn) == 2 && NT == kRowsThreads && !RAG) {
+          const int whole = i < 0 ? min(to, full_to(sp1)) : 0;
 #pragma unroll 1
-        for (int g = 0; g < to; ++g) {
+          for (; g + 2 <= whole; g += 2) {
+            early(i + 1, g);
+            early(i + 1, g + 1);
+            uint4 z2[kU], u2[kU];
+#pragma unroll
+            for (int h = 0; h < kU; ++h) load(h, z2, u2);
+            loaded();
+            group_of(yes, no, yes, yes, g, 0, zn, un);
+            group_of(yes, no, yes, no, g + 1, 0, z2, u2);
+          }
+        }
+#pragma unroll 1
+        for (; g < to; ++g) {
           early(i + 1, g);
           if (g >= full_from(sp1) && g < full_to(sp1)) group(yes, no, yes, g, 0);
           else group(yes, no, no, g, 0);
