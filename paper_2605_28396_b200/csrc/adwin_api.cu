@@ -37,16 +37,6 @@ int sm_count_of_current_device() {
   return cached[dev];
 }
 
-// Shared body of the two forward+backward entry points (row_coef is null for the plain one).
-int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, int dtype,
-                        int64_t B, int64_t T, int64_t V, int64_t ld, const int32_t* tokens,
-                        const int32_t* window, const int32_t* rollout_len, float grad_scale,
-                        int grad_mode, int flags, void* grad_student, int grad_dtype,
-                        int64_t ld_grad, float* kl, float* logratio, float* gsq,
-                        float* lse_student, float* lse_teacher, void* workspace,
-                        size_t workspace_bytes, int32_t* dev_status, void* cuda_stream,
-                        const float* row_coef);
-
 }  // namespace
 }  // namespace adwin
 
@@ -91,7 +81,7 @@ int adwin_opd_kl_fwd_bwd(const void* student_logits, const void* teacher_logits,
   return opd_kl_fwd_bwd_impl(student_logits, teacher_logits, dtype, B, T, V, ld, tokens, window,
                              rollout_len, grad_scale, grad_mode, flags, grad_student, grad_dtype,
                              ld_grad, kl, logratio, gsq, lse_student, lse_teacher, workspace,
-                             workspace_bytes, dev_status, cuda_stream, nullptr);
+                             workspace_bytes, dev_status, cuda_stream, nullptr, B * T);
 }
 
 int adwin_opd_kl_fwd_bwd_weighted(const void* student_logits, const void* teacher_logits,
@@ -108,7 +98,7 @@ int adwin_opd_kl_fwd_bwd_weighted(const void* student_logits, const void* teache
   return opd_kl_fwd_bwd_impl(student_logits, teacher_logits, dtype, B, T, V, ld, tokens, window,
                              rollout_len, grad_scale, ADWIN_GRAD_SAMPLED, flags, grad_student,
                              grad_dtype, ld_grad, kl, logratio, gsq, lse_student, lse_teacher,
-                             workspace, workspace_bytes, dev_status, cuda_stream, row_coef);
+                             workspace, workspace_bytes, dev_status, cuda_stream, row_coef, B * T);
 }
 
 int adwin_return_to_go(const float* logratio, const int32_t* window, const int32_t* rollout_len,
@@ -170,7 +160,6 @@ int adwin_drift_curves(const float* entropy, const int32_t* rank, const int32_t*
 }  // extern "C"
 
 namespace adwin {
-namespace {
 
 int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, int dtype,
                         int64_t B, int64_t T, int64_t V, int64_t ld, const int32_t* tokens,
@@ -179,7 +168,7 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
                         int64_t ld_grad, float* kl, float* logratio, float* gsq,
                         float* lse_student, float* lse_teacher, void* workspace,
                         size_t workspace_bytes, int32_t* dev_status, void* cuda_stream,
-                        const float* row_coef) {
+                        const float* row_coef, int64_t plan_rows) {
   if (dtype != ADWIN_F32 && dtype != ADWIN_BF16) return ADWIN_ERR_DTYPE;
   if (grad_mode != ADWIN_GRAD_FULL_KL && grad_mode != ADWIN_GRAD_SAMPLED) return ADWIN_ERR_DTYPE;
   if (flags & ~kKnownFlags) return ADWIN_ERR_DTYPE;
@@ -224,6 +213,7 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
   p.range = reinterpret_cast<const int32_t*>(wbase + wl.off_range);
   p.ewin = reinterpret_cast<const int32_t*>(wbase + wl.off_ewin);
   p.row_coef = row_coef;
+  p.plan_rows = plan_rows;
   p.skip_below = nullptr;
 
   // Layout.  vec: row r of every array has the same offset from a 16-byte boundary (the gradient in
@@ -296,7 +286,6 @@ int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, 
   return ADWIN_OK;
 }
 
-}  // namespace
 }  // namespace adwin
 
 extern "C" {

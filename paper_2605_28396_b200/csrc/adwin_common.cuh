@@ -57,6 +57,7 @@ struct KlParams {
   // SAMPLED mode only: per-position coefficient that takes the place of c_t (the discounted
   // return-to-go of Eq. 3); null for the token-local estimator of Eq. 4
   const float* row_coef;
+  int64_t plan_rows;   // row kernel only: rows of the caller's call, of which this may be a part
   // streaming kernel only: when set, positions t < skip_below[b] are left to another launch
   const int32_t* skip_below;
 };

@@ -50,6 +50,18 @@ struct WorkspaceLayout {
 };
 WorkspaceLayout workspace_layout(int64_t B);
 
+// Shared body of the forward+backward entry points.  row_coef: null for the plain ones.  plan_rows: the rows of
+// the caller's call, of which this may be a part: the row kernel's shape goes by it, so that the
+// parts leave the bits that the whole would.
+int opd_kl_fwd_bwd_impl(const void* student_logits, const void* teacher_logits, int dtype,
+                        int64_t B, int64_t T, int64_t V, int64_t ld, const int32_t* tokens,
+                        const int32_t* window, const int32_t* rollout_len, float grad_scale,
+                        int grad_mode, int flags, void* grad_student, int grad_dtype,
+                        int64_t ld_grad, float* kl, float* logratio, float* gsq,
+                        float* lse_student, float* lse_teacher, void* workspace,
+                        size_t workspace_bytes, int32_t* dev_status, void* cuda_stream,
+                        const float* row_coef, int64_t plan_rows);
+
 cudaError_t launch_rowmap(const int32_t* window, const int32_t* rollout_len, int64_t B, int64_t T,
                           int flags, void* workspace, bool with_window_offsets, float* kl,
                           float* logratio, float* gsq, float* lse_s, float* lse_t, int32_t* status,

@@ -166,7 +166,7 @@ int adwin_opd_kl_fwd_bwd_host(const void* student_host, const void* teacher_host
       set_lengths_kernel<<<1, 1, 0, user>>>(reinterpret_cast<int32_t*>(base + L.off_win),
                                             reinterpret_cast<int32_t*>(base + L.off_rl),
                                             (int32_t)wrows, (int32_t)rows);
-      const int rc = adwin_opd_kl_fwd_bwd(
+      const int rc = opd_kl_fwd_bwd_impl(
           base + L.off_z, base + L.off_u, dtype, 1, rows, V, L.pitch_in,
           reinterpret_cast<const int32_t*>(base + L.off_tok),
           reinterpret_cast<const int32_t*>(base + L.off_win),
@@ -174,7 +174,7 @@ int adwin_opd_kl_fwd_bwd_host(const void* student_host, const void* teacher_host
           flags & ~(ADWIN_ZERO_TAIL | ADWIN_STATUS_INIT), has_grad ? base + L.off_grad : nullptr, gd, L.pitch_out,
           reinterpret_cast<float*>(base + L.off_kl), reinterpret_cast<float*>(base + L.off_c),
           reinterpret_cast<float*>(base + L.off_q), nullptr, nullptr, base + L.off_ws,
-          workspace_layout(1).total_ext, dev_status, user);
+          workspace_layout(1).total_ext, dev_status, user, nullptr, B * T);
       if (rc != ADWIN_OK) return rc;
       cudaEventRecord(pl->comp_done[s], user);
 

@@ -22,6 +22,7 @@
 // ~69 nats below the row maximum) the row is summed once more, from its on-chip copy (the teacher's
 // pieces from memory where only the student's are kept), against running maxima.  Rows too long for one CTA are split over a cluster; the CTAs' sums then go to every
 // CTA of the cluster.
+#include <iterator>
 #include <mutex>
 #include <type_traits>
 
@@ -66,6 +67,7 @@ struct RowsPlan {
 struct RowsShape {
   int ctas, nt, tm_cols, cl;
   int most;           // pieces of a row up to which the shape is taken
+  int few;            // and, where a call has no more rows than the GPU holds at a time so, from which (0: never)
 };
 // The first that takes the row is used: the more and smaller CTAs, the less of a group lies idle at a row's
 // end; beyond 57 000 entries of bf16 one CTA per SM and not two in clusters (151 936 entries: two CTAs in clusters of
@@ -86,9 +88,20 @@ struct RowsShape {
 // entries 514 us, 507 before).
 // (The small shapes hold twice as much of a row whose second sweep takes the student alone, but are slower there:
 // 10 309 entries on {8, 64} 140 us where {4, 128} takes 131.)
-constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 768}, {4, 128, 128, 1, 3584}, {2, 256, 256, 1, 7168},
-                                 {1, kRowsThreads, 512, 1, 1 << 24}, {1, kRowsThreads, 512, 2, 1 << 24},
-                                 {1, kRowsThreads, 512, 4, 1 << 24}};
+// A call of so few rows that each gets a CTA or cluster of its own anyway takes the last (widest) shape for
+// which that holds, from `few` pieces on.  B * T counts as its rows, which is what the host knows of them, so a
+// shape is never too wide for the rows there are.  Device time of a call (the shape by length alone / this one /
+// a kernel with up to four CTAs of 352 threads a row that did not join the sweeps):
+//   bf16  13 rows of 151 936   21.2 / 15.1 / 17.4 us  x 4    64 rows  24.2 / 22.9 / 22.6 us  x 2
+//                     80 000   18.9 / 12.1 / 17.8     x 4             20.7 / 17.0 / 18.9     x 2
+//                     50 257   18.2 / 11.6 / 18.3     x 4             18.8 / 15.3 / 19.4     x 2
+//                     16 384   10.8 /  9.0 /  9.9     {1, 512}        12.0 /  9.7 / 12.3     {1, 512}
+//                      4 096    7.8 /  7.2 /  7.8     {2, 256}         8.0 /  7.2 /  8.2     {2, 256}
+// With a piece or two per thread a row's exchange costs more than its sweeps: 16 384 entries, 8 rows, four
+// CTAs 9.3, two 9.6, one 9.05; 24 576 entries 9.5, 10.5, 10.2; 4 096 entries {1, 512} 7.65, {2, 256} 7.2.
+constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 768, 0}, {4, 128, 128, 1, 3584, 0}, {2, 256, 256, 1, 7168, 512},
+                                 {1, kRowsThreads, 512, 1, 1 << 24, 1024}, {1, kRowsThreads, 512, 2, 1 << 24, 3584},
+                                 {1, kRowsThreads, 512, 4, 1 << 24, 3584}};
 // CTAs per SM of the shapes with nt threads, and whether they use tensor memory (the same for all of them).
 constexpr int ctas_of(int nt) {
   for (const RowsShape& sh : kShapes)
@@ -892,13 +905,6 @@ constexpr bool metadata_precedes_its_readers() {
 }
 static_assert(metadata_precedes_its_readers(), "a row's metadata could be read before it is written");
 
-bool rows_plan(int64_t pieces, int kept, RowsPlan& plan) {
-  if (pieces < 1 || pieces > (int64_t)1 << 24) return false;
-  for (const RowsShape& sh : kShapes)
-    if (pieces <= sh.most && shape_plan(sh, pieces, kept, plan)) return true;
-  return false;
-}
-
 typedef void (*RowsKernel)(KlParams, RowsPlan);
 template <typename TIn, typename TOut, int NT>
 RowsKernel rows_kernel_nt(bool ragged, bool full_kl) {
@@ -962,6 +968,27 @@ constexpr bool cluster_shapes_differ_in_cl_alone() {
 }
 static_assert(cluster_shapes_differ_in_cl_alone(), "resident_clusters keeps one number per cluster size");
 
+// The plan of a call of at most `rows` rows, and how many rows the GPU holds at a time so.
+cudaError_t rows_plan(int64_t pieces, int kept, int64_t rows, int sm_count, RowsPlan& plan) {
+  if (pieces < 1 || pieces > (int64_t)1 << 24) return cudaErrorNotSupported;
+  const RowsShape* by_length = std::begin(kShapes);
+  while (!(pieces <= by_length->most && shape_plan(*by_length, pieces, kept, plan)))
+    if (++by_length == std::end(kShapes)) return cudaErrorNotSupported;
+  for (const RowsShape* sh = std::end(kShapes) - 1;; --sh) {
+    plan.num_clusters = sh->ctas * sm_count / sh->cl;
+    const bool wider = sh != by_length;
+    if (wider && (!sh->few || pieces < sh->few || rows > plan.num_clusters)) continue;
+    if (!shape_plan(*sh, pieces, kept, plan)) continue;
+    if (plan.cl > 1) {
+      const cudaError_t e = resident_clusters(plan, sm_count, plan.num_clusters);
+      if (wider && e == cudaErrorNotSupported) continue;
+      if (e != cudaSuccess) return e;
+    }
+    if (wider && rows > plan.num_clusters) continue;
+    return cudaSuccess;
+  }
+}
+
 template <typename TIn, typename TOut>
 cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStream_t s) {
   constexpr int N = Elem<TIn>::N;
@@ -971,22 +998,16 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   // rows that do not all start on the same 16-byte boundary of a line
   ragged = ragged || (p.ld * sizeof(TIn)) % kLine != 0 || reinterpret_cast<uintptr_t>(p.student) % kLine != 0;
   const int64_t lead = ragged ? kLine / (int64_t)sizeof(TIn) - 1 : 0;   // entries of a line before the row, at most
-  if (!rows_plan((lead + p.V + N - 1) / N, kept, plan)) return cudaErrorNotSupported;
+  cudaError_t e = rows_plan((lead + p.V + N - 1) / N, kept, p.plan_rows, sm_count, plan);
+  if (e != cudaSuccess) return e;
+  if (plan.num_clusters > p.B * p.T) plan.num_clusters = (int)(p.B * p.T);
   const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, ragged, full_kl);
   if (!kernel) return cudaErrorNotSupported;
   const int smem = launch_smem(plan, kept);
-  plan.num_clusters = plan.ctas * sm_count;
-  cudaError_t e;
-  if (plan.cl > 1) {
-    e = resident_clusters(plan, sm_count, plan.num_clusters);
-    if (e != cudaSuccess) return e;
-  }
   // the shape's whole share whatever this call needs: the limit belongs to the kernel, which launches of
   // other threads with other row lengths use at the same time
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shape_smem(plan.ctas));
   if (e != cudaSuccess) return e;
-  const int64_t rows = p.B * p.T;
-  if (plan.num_clusters > rows) plan.num_clusters = (int)rows;
   return launch_chained(kernel, (unsigned)(plan.cl * plan.num_clusters), plan.nt + 32, (size_t)smem, plan.cl, s,
                         p, plan);
 }

@@ -637,6 +637,19 @@ def test_short_rows_one_after_another(in_dt, V, B, T):
     check_rows_one_after_another(batch, second=True)
 
 
+# Calls with a CTA or cluster for every row take wider shapes than the row's length alone asks for: at the piece
+# counts where each is first taken (512, 1024 and 3584 pieces) and one piece below, on and off the lines, with as many
+# rows as clusters of four and of two and one or two CTAs per SM hold at a time, and a few more than that.
+@pytest.mark.parametrize("in_dt,V", [(2, 4088), (2, 4096), (2, 8184), (2, 8192), (2, 8131), (2, 28664), (2, 28672), (2, 50257),
+                                     (1, 2048), (1, 4095), (1, 14332), (1, 14336), (1, 20001)])
+@pytest.mark.parametrize("rows", [33, 37, 70, 78, 148, 150, 296, 298])
+def test_calls_of_few_rows(in_dt, V, rows):
+    batch = synth.make_batch(in_dt, device=DEV, B=1, T=rows, V=V)
+    batch.window[:] = rows
+    batch.rollout_len[:] = rows
+    check_rows_one_after_another(batch)
+
+
 @pytest.mark.parametrize("in_dt,V", [(2, 4095), (2, 4096), (2, 4104), (2, 20001), (1, 2047), (1, 2052), (1, 9001)])
 @pytest.mark.parametrize("mode", [api.GRAD_FULL_KL, api.GRAD_SAMPLED])
 def test_read_only_rows_that_outgrow_their_first_entries(in_dt, V, mode):
