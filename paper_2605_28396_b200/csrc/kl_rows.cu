@@ -175,8 +175,10 @@ struct RowSlice {
 
 // NT: threads that hold pieces, a template constant so that the strides between a thread's pieces are
 // offsets in the instructions.  A group of kU steps in which every thread has whole pieces takes the path
-// without tests (FULL below), also where one sweep runs alone: with one row a CTA nothing else runs (280 rows of
-// 32 000 entries of bf16, 23.4 us with the tests there, 20.9 without).  FULLKL: the gradient of Eq. 2; without it, of Eq. 4, whose second sweep
+// without tests (FULL below), kWholeAlone: also where one sweep runs alone, as with one row a CTA (280 rows of
+// 32 000 entries of bf16, 23.4 us with the tests there, 20.9 without).  Not in the small kernels of rows off the
+// lines, which such calls do not take and whose loop comes out slower beside that code (2.4 GB of rows of 9 001 entries
+// 506 us, 564 with it; of 5 000 513, 570).  FULLKL: the gradient of Eq. 2; without it, of Eq. 4, whose second sweep
 // takes the student's logits alone, so only they are kept.
 template <typename TIn, typename TOut, int NT, bool TM, bool RAG, bool FULLKL>
 __global__ void __launch_bounds__(NT + 32, ctas_of(NT))
@@ -192,6 +194,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   // tolerance a centre far from the mean would cost.  (2.4 GB of rows of 32 000 entries 420 -> 424 us with both, where
   // shorter ones would pay more: 8 192 436 -> 453, 5 000 519 -> 539.)
   constexpr bool kCentred = sizeof(TIn) == 2 && NT >= 256;
+  constexpr bool kWholeAlone = !RAG || NT >= 256;
   constexpr uint32_t group_bytes = kU * kKept * array;
   constexpr int group_cols = kU * kKept * 4;
   extern __shared__ __align__(128) char smem[];
@@ -728,8 +731,11 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
 #pragma unroll 1
         for (; g < to; ++g) {
           early(i + 1, g);
-          if (g >= full_from(sp1) && g < full_to(sp1)) group(yes, no, yes, g, 0);
-          else group(yes, no, no, g, 0);
+          if (kWholeAlone && g >= full_from(sp1) && g < full_to(sp1)) {
+            if constexpr (kWholeAlone) group(yes, no, yes, g, 0);
+          } else {
+            group(yes, no, no, g, 0);
+          }
         }
       }
       if (i < 0) {
@@ -807,8 +813,11 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       for (int g = 0; g < groups; ++g) {
         const int g1 = g + plan.ahead;
         if (g >= both) {
-          if (g >= full_from(sp2) && g < full_to(sp2)) group(no, yes, yes, 0, g);
-          else group(no, yes, no, 0, g);
+          if (kWholeAlone && g >= full_from(sp2) && g < full_to(sp2)) {
+            if constexpr (kWholeAlone) group(no, yes, yes, 0, g);
+          } else {
+            group(no, yes, no, 0, g);
+          }
         } else {
           early(i + 1, g1);
           if (g >= lo && g < hi) group(yes, yes, yes, g1, g);
