@@ -48,6 +48,7 @@ constexpr int kMetaAhead = 4;
 constexpr int kMetaDepth = 8;
 constexpr int kMostEarly = 3;         // groups from a piece's way into L2 to its load, at most
 constexpr int kLine = 128;
+constexpr int64_t kShortRow = 14336;  // entries
 constexpr int kEdges = 16;            // entries beside a row's whole pieces: less than 8 on each side
 constexpr float kMaskedEdge = -1e30f;
 
@@ -166,8 +167,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// A row in a CTA's slice.  Pieces are counted from the 128-byte line that the student's row starts in, so
-// that a warp's 512 bytes are whole lines.
+// A row in a CTA's slice.  With RAG pieces are counted from the 128-byte line that the student's row starts in, so
+// that a warp's 512 bytes are whole lines; without, from the row's start (a line's, but for short rows).
 struct RowSlice {
   int begin, pieces;   // the slice's pieces [begin, pieces) are the row's
   int shift;           // entries from the line's start to the row's
@@ -223,7 +224,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
 
   if (TM && warp == nw) tm_alloc(smem_u32(&ctrl.tmem_base), (uint32_t)plan.tm_cols);
 
-  // where row r lies in this CTA's slice (base pointers are 16-byte aligned; without RAG rows are lines).
+  // where row r lies in this CTA's slice (base pointers are 16-byte aligned; without RAG rows are whole pieces).
   // The at most N - 1 entries before its first and after its last whole piece are its own warp's.
   auto slice_of = [&](int64_t r) -> RowSlice {
     RowSlice a = {0, 0, 0};
@@ -1004,8 +1005,11 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   RowsPlan plan = {};
   const bool full_kl = p.mode == ADWIN_GRAD_FULL_KL;
   const int kept = full_kl ? 2 : 1;
-  // rows that do not all start on the same 16-byte boundary of a line
-  ragged = ragged || (p.ld * sizeof(TIn)) % kLine != 0 || reinterpret_cast<uintptr_t>(p.student) % kLine != 0;
+  // Rows of whole pieces off the lines: pieces are counted from the line (see RowSlice) except in short bf16 rows, which
+  // lose more by the groups that are then partial at both ends.  2.4 GB, from the line / from the row: 4 104 entries 572 /
+  // 537 us, 5 000 513 / 495, 7 000 518 / 484, 9 000 493 / 466, 20 008 436 / 440, 50 264 427 / 443; fp32 2 500 395 / 431.
+  const bool off_lines = (p.ld * sizeof(TIn)) % kLine != 0 || reinterpret_cast<uintptr_t>(p.student) % kLine != 0;
+  ragged = ragged || (off_lines && (sizeof(TIn) == 4 || p.V > kShortRow));
   const int64_t lead = ragged ? kLine / (int64_t)sizeof(TIn) - 1 : 0;   // entries of a line before the row, at most
   cudaError_t e = rows_plan((lead + p.V + N - 1) / N, kept, p.plan_rows, sm_count, plan);
   if (e != cudaSuccess) return e;

@@ -588,8 +588,9 @@ def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
 
 # Several rows for every CTA of a launch, so that a row's second sweep runs beside the next row's first and
 # the ring of kept pieces turns over: the longest rows of each shape (bf16; half of that fp32), rows of whole
-# lines and rows that start anywhere in one, and the first of a cluster of two and of four.
+# lines, of whole pieces and rows that start anywhere in one, and the first of a cluster of two and of four.
 @pytest.mark.parametrize("in_dt,V,rows", [(2, 4099, 2500), (2, 4096, 2500), (2, 28665, 1250), (2, 57341, 620), (2, 57344, 620),
+                                          (2, 5000, 2500), (2, 14328, 2500), (2, 14344, 2500),
                                           (2, 114681, 310), (2, 114752, 170), (2, 262144, 80), (1, 2050, 2500),
                                           (1, 14331, 1250), (1, 57341, 310), (1, 57349, 170)])
 def test_rows_one_after_another(in_dt, V, rows):
