@@ -337,7 +337,6 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     __syncthreads();
     int64_t r_prev = 0;
     float q_edge = 0.f;   // this lane's share of the previous row's squared norm
-    float q_scale = 1.f;  // and what the norm is to be scaled by
     // one more exchange than rows, for the last norm
     for (int i = 0; i <= my_rows && my_rows > 0; ++i) {
       const bool real = i < my_rows;
@@ -384,7 +383,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
           v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
         }
       }
-      if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = v[3] * q_scale;
+      if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = v[3];
       if (!real) break;
       const RowsMeta& m = ctrl.meta[i % kMetaDepth];
       const int64_t ri = m.r;
@@ -443,33 +442,31 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       // the mean of delta over the row, as a sum of two floats
       const float about = t.A * inv, mean = about + m.dref, back = mean - about;
       const float rest = (about - (mean - back)) + (m.dref - back);
-      float coef = p.alpha * inv, nc0 = -mean;
-      q_scale = 1.f;
+      float coef = p.alpha * inv, nc0 = -mean, nm2s = -t.M2s;
       if constexpr (FULLKL && sizeof(TIn) == 2) {
         // bf16 logits: g = e * (coef*delta - coef*mean) saves one operation per pair; its rounding
         // (relative to coef*delta, not to the difference) is far inside that dtype's tolerance.  But that of
         // coef*mean is common to the row, and a peaked row's norm, all of it from a delta beside the mean, is off
-        // by twice the rounding times mean / (delta - mean).  A bf16 gradient does not see 2^-20 of its
-        // coefficient, so of the 32 nearest the one whose product with the mean needs the least rounding is
-        // taken, and the norm scaled back.  (With the centre: over 15 360 rows of 151 936 entries the norm's
-        // error is 3.5e-7 in the root mean square and 1.7e-5 at most, 2.2e-6 and 9.9e-5 without both.)
-        if (kCentred && sizeof(TOut) == 2 && fabsf(coef) > 1e-30f && fabsf(coef) < 1e30f) {
-          const float c = __int_as_float(__float_as_int(coef) + lane - 16);
+        // by twice the rounding times mean / (delta - mean).  Another reference for e makes another coefficient: of 32
+        // references 2^-16 apart the one whose coefficient needs the least rounding in its product with
+        // the mean is taken.  (2^-s = 1 - x + x^2 / 2 with x = s ln 2 < 2e-4; the next term is 2^-39.)
+        // An infinite mean, of a teacher's entry masked by -infinity, has no rounding to look after.
+        if (kCentred && fabsf(coef) > 1e-30f && fabsf(coef) < 1e30f && fabsf(mean) < 1e30f) {
+          const float ref = nm2s + (float)(lane - 16) * 0x1p-16f;     // (rounded: the step is the difference below)
+          const float x = (ref - nm2s) * 0.69314718f, c = fmaf(coef, x * fmaf(x, 0.5f, -1.f), coef);
           const float prod = c * mean, low = fmaf(c, rest, fmaf(c, mean, -prod)), near = prod + low;
           const float off = fabsf(low - (near - prod));
           const unsigned best = __reduce_min_sync(0xffffffffu, (__float_as_uint(off) & ~31u) | (unsigned)lane) & 31u;
-          const float taken = __shfl_sync(0xffffffffu, c, (int)best);
+          nm2s = __shfl_sync(0xffffffffu, ref, (int)best);
           nc0 = -__shfl_sync(0xffffffffu, near, (int)best);
-          q_scale = coef / taken;
-          q_scale *= q_scale;
-          coef = taken;
+          coef = __shfl_sync(0xffffffffu, c, (int)best);
         } else {
           nc0 = -coef * mean;
         }
       }
       auto publish = [&](float gy) {
         if (lane == 0) {
-          ctrl.out.nm2s[0] = ctrl.out.nm2s[1] = -t.M2s;
+          ctrl.out.nm2s[0] = ctrl.out.nm2s[1] = nm2s;
           ctrl.out.coef[0] = ctrl.out.coef[1] = coef;
           ctrl.out.nc0[0] = ctrl.out.nc0[1] = nc0;
           ctrl.out.gy = gy;
@@ -487,7 +484,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       }
       if (edges) {   // the gradient of the edge entries, as in the second sweep
         const int64_t k = edge_of(ri);
-        const float e = ex2f(fmaf(ze, kLog2e, -t.M2s));
+        const float e = ex2f(fmaf(ze, kLog2e, nm2s));
         float g;
         if (!FULLKL) g = k == m.y ? rs.gy : e * coef;
         else if (sizeof(TIn) == 2) g = e * fmaf(ze - ue, coef, nc0);

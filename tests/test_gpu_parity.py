@@ -788,6 +788,24 @@ def test_masked_vocabulary_entries(path, in_dt, V, masked, at, value):
             run_and_check(batch, grad_dtype=grad, grad_mode=mode, flags=PATHS[path])
 
 
+@pytest.mark.parametrize("in_dt,V", [(2, 4096), (2, 32000), (2, 50257), (2, 151936), (1, 20001)])
+@pytest.mark.parametrize("rows", [6, 310])
+def test_entries_that_only_the_teacher_masks(in_dt, V, rows):
+    """Entries at -infinity in the teacher alone, where the student has mass: the divergence is infinite and so
+    is the gradient (towards minus infinity, -p_k times it), with no entry of it undefined but the masked ones."""
+    batch = synth.make_batch(in_dt, device=DEV, B=1, T=rows, V=V)
+    batch.window[:] = batch.rollout_len[:] = rows
+    batch.teacher[..., 100:140] = batch.student[..., 100:140] = float("-inf")
+    batch.tokens[:] = batch.student.argmax(dim=2)
+    batch.student[..., 100:140] = batch.student.float().amax(dim=2, keepdim=True) - 2.0
+    grad = torch.zeros_like(batch.student)
+    got = api.adwin_opd_kl_fwd_bwd(batch.student, batch.teacher, batch.tokens, batch.window, batch.rollout_len, grad=grad)
+    torch.cuda.synchronize()
+    assert (got.kl == float("inf")).all() and torch.isfinite(got.logratio).all()
+    grad[..., 100:140] = float("-inf")
+    assert (grad == float("-inf")).all()
+
+
 @pytest.mark.parametrize("in_dt,V", [(2, 4096), (2, 4104), (2, 20001), (2, 120000), (1, 2052), (1, 9001)])
 @pytest.mark.parametrize("mode", [api.GRAD_FULL_KL, api.GRAD_SAMPLED])
 def test_read_only_rows_that_outgrow_first_entries_and_token(in_dt, V, mode):
