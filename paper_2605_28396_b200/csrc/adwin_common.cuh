@@ -186,6 +186,7 @@ struct RowTotals {
 
 struct RowScalars {
   float kl, c, lse_s, lse_t, gsq_expanded;
+  float lse_diff;   // lse_s - lse_t
   float c0;      // E_p[delta] (centred): A/S
   float coef;    // alpha / S      (FULL_KL)   or  -alpha*c / S   (SAMPLED)
   float gy;      // SAMPLED: gradient entry at the sampled token, alpha*c*(1-p_y)
@@ -214,6 +215,7 @@ __device__ __forceinline__ RowScalars finish_row(const RowTotals& t, float zy, f
   const float delta = ((t.M2s - t.M2t) + log2f(t.S / t.St)) * kLn2f;
   const float inv_s = 1.f / t.S;
   r.c0 = t.A * inv_s;
+  r.lse_diff = delta;
   r.kl = (r.c0 + dref) - delta;
   r.c = y_valid ? (zy - uy) - delta : __int_as_float(0x7fc00000);
   if (mode == ADWIN_GRAD_FULL_KL) {

@@ -174,6 +174,34 @@ __device__ __forceinline__ float hsum2(f2_t v) {
   return a + b;
 }
 
+// Sums of pairs with what their additions round off (Knuth's two-sum); plain ones without EXACT.
+template <bool EXACT>
+struct ExactSum {
+  f2_t hi, lo;
+  __device__ __forceinline__ void set(f2_t x) {
+    hi = x;
+    lo = 0ull;
+  }
+  __device__ __forceinline__ void add(f2_t x) {
+    const f2_t s = add2(hi, x);
+    if (EXACT) {
+      const f2_t c = sub2(s, hi);
+      lo = add2(lo, add2(sub2(hi, sub2(s, c)), sub2(x, c)));
+    }
+    hi = s;
+  }
+  __device__ __forceinline__ void add(const ExactSum& x) {
+    if (EXACT) lo = add2(lo, x.lo);
+    add(x.hi);
+  }
+  __device__ __forceinline__ ExactSum of_lane_xor(int o) const {
+    ExactSum x;
+    x.hi = __shfl_xor_sync(0xffffffffu, hi, o);
+    x.lo = EXACT ? __shfl_xor_sync(0xffffffffu, lo, o) : 0ull;
+    return x;
+  }
+};
+
 // A 16-byte piece as NP pairs of consecutive vocabulary entries.
 template <typename T>
 struct Pairs;

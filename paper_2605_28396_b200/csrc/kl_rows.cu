@@ -93,11 +93,10 @@ struct RowsShape {
 // which that holds, from `few` pieces on.  B * T counts as its rows, which is what the host knows of them, so a
 // shape is never too wide for the rows there are.  Device time of a call (the shape by length alone / this one /
 // a kernel with up to four CTAs of 352 threads a row that did not join the sweeps):
-//   bf16  13 rows of 151 936   21.2 / 15.1 / 17.4 us  x 4    64 rows  24.2 / 22.9 / 22.6 us  x 2
-//                     80 000   18.9 / 12.1 / 17.8     x 4             20.7 / 17.0 / 18.9     x 2
-//                     50 257   18.2 / 11.6 / 18.3     x 4             18.8 / 15.3 / 19.4     x 2
-//                     16 384   10.8 /  9.0 /  9.9     {1, 512}        12.0 /  9.7 / 12.3     {1, 512}
-//                      4 096    7.8 /  7.2 /  7.8     {2, 256}         8.0 /  7.2 /  8.2     {2, 256}
+//   bf16  13 rows of 151 936   21.1 / 15.7 / 17.4 us  x 4    64 rows  25.0 / 23.2 / 22.8 us  x 2
+//                     80 000   19.0 / 12.7 / 17.8     x 4             21.7 / 17.6 / 19.0     x 2
+//                     50 257   19.2 / 12.2 / 18.3     x 4             21.2 / 15.9 / 19.4     x 2
+//                      4 096    8.2 /  7.5 /  7.9     {2, 256}         8.3 /  7.5 /  8.0     {2, 256}
 // With a piece or two per thread a row's exchange costs more than its sweeps: 16 384 entries, 8 rows, four
 // CTAs 9.3, two 9.6, one 9.05; 24 576 entries 9.5, 10.5, 10.2; 4 096 entries {1, 512} 7.65, {2, 256} 7.2.
 constexpr RowsShape kShapes[] = {{8, 64, 0, 1, 768, 0}, {4, 128, 128, 1, 3584, 0}, {2, 256, 256, 1, 7168, 512},
@@ -143,7 +142,7 @@ struct __align__(16) RowsScalars {
 
 struct __align__(16) RowsCtrl {
   float safe[kRowsThreads / 32][8];    // the warps' records of the running-maximum pass
-  float xrec[2][kRowsMaxCl][4];    // per row parity, one record per CTA of the cluster
+  float xrec[2][kRowsMaxCl][8];    // per row parity, one record per CTA of the cluster
   float xsafe[kRowsMaxCl][8];
   RowsScalars out;
   RowsMeta meta[kMetaDepth];
@@ -190,11 +189,23 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   constexpr int nt = NT, nw = NT / 32, all = NT + 32;
   constexpr uint32_t array = NT * 16u;
   constexpr int kKept = FULLKL ? 2 : 1;             // arrays kept
-  // delta is summed about a centre (RowsMeta::dref) and the coefficient chosen for the product with the mean (see
-  // there) where a thread's chain of additions is longest; fp32 rows keep to delta itself, whose
+  // delta is summed about a centre (RowsMeta::dref) and the reference chosen for the coefficient's product with the
+  // mean (see there) where a thread's chain of additions is longest; fp32 rows keep to delta itself, whose
   // tolerance a centre far from the mean would cost.  (2.4 GB of rows of 32 000 entries 420 -> 424 us with both, where
   // shorter ones would pay more: 8 192 436 -> 453, 5 000 519 -> 539.)
   constexpr bool kCentred = sizeof(TIn) == 2 && NT >= 256;
+  // Where a thread's chains of additions are longer, and rows are added up over more threads, than in the kernel that
+  // did not join the sweeps: what the additions over the threads round off is kept (S and A over all of them, the teacher's
+  // sum and the norm over lanes and CTAs), and a thread's norm is two sums.  Median errors against a 64-bit
+  // evaluation, of that kernel / of plain sums / of these:
+  //   tokens drawn uniformly, 50 248 entries   KL 1.06e-7 / 1.16e-7 / 0.94e-7   log-ratio 0.54e-7 / 0.53e-7 / 0.48e-7
+  //                                            squared norm 1.48e-7 / 1.60e-7 / 1.29e-7
+  //   spikes, 151 936 entries                  KL 0.73e-7 / 0.84e-7 / 0.66e-7   log-ratio 0.87e-7 / 0.87e-7 / 0.82e-7
+  //                                            squared norm 1.24e-7 / 1.59e-7 / 1.24e-7
+  // (2.4 GB: rows of 32 000 entries 405 us with plain sums and so, 151 936 402 and 412, 50 257 429 and 434.  All four
+  // sums over all threads: 151 936 440.)
+  constexpr bool kExact = NT >= 256;
+  constexpr int kNorms = kExact && FULLKL ? kU : 1;
   constexpr bool kWholeAlone = !RAG || NT >= 256;
   constexpr uint32_t group_bytes = kU * kKept * array;
   constexpr int group_cols = kU * kKept * 4;
@@ -344,21 +355,28 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       // (the others have begun no row before i - 1 ended, and read no further than kMetaAhead says)
       if (i + kMetaAhead < my_rows) fetch(i + kMetaAhead);
       named_sync(kPosted, all);
-      // fixed-order sums over the threads, then over the CTAs
-      float4 x4[nw];
+      // fixed-order sums over the threads, then over the CTAs: S and A, St and the norm (what kReady waits for
+      // beside the others' issue slots: every operation counts here)
+      ExactSum<kExact> sa[nw], tq[nw];
 #pragma unroll
-      for (int w = 0; w < nw; ++w) x4[w] = rec[w * 32 + lane];
+      for (int w = 0; w < nw; ++w) {
+        f2_t x, y;
+        row_pairs(&rec[w * 32 + lane].x, x, y);
+        sa[w].set(x);
+        tq[w].set(y);
+      }
 #pragma unroll
       for (int n = nw / 2; n > 0; n /= 2) {
 #pragma unroll
         for (int w = 0; w < n; ++w) {
-          x4[w].x += x4[w + n].x; x4[w].y += x4[w + n].y; x4[w].z += x4[w + n].z; x4[w].w += x4[w + n].w;
+          sa[w].add(sa[w + n]);
+          tq[w].hi = add2(tq[w].hi, tq[w + n].hi);
         }
       }
-      float v[4] = {x4[0].x, x4[0].y, x4[0].z, x4[0].w};
+      ExactSum<kExact> SA = sa[0], TQ = tq[0];
       float ze = kMaskedEdge, ue = kMaskedEdge;
       if (edges) {
-        v[3] += q_edge;
+        float e_t = 0.f;
         if (real) {
           const RowsMeta& m = ctrl.meta[i % kMetaDepth];
           if (lane < kEdges) {
@@ -366,35 +384,54 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
             ue = m.edge[lane][1];
           }
           const float e = ex2f(fmaf(ze, kLog2e, m.nref[0]));
-          v[0] += e;
-          v[1] = fmaf(e, (ze - ue) + m.nref[4], v[1]);
-          v[2] += ex2f(fmaf(ue, kLog2e, m.nref[2]));
+          SA.add(pk2(e, e * ((ze - ue) + m.nref[4])));
+          e_t = ex2f(fmaf(ue, kLog2e, m.nref[2]));
         }
+        TQ.add(pk2(e_t, q_edge));
       }
 #pragma unroll
-      for (int f = 0; f < 4; ++f) v[f] = lane_sum(v[f]);
+      for (int o = 16; o > 0; o >>= 1) {
+        SA.add(SA.of_lane_xor(o));
+        TQ.add(TQ.of_lane_xor(o));
+      }
       if (cl > 1) {
-        if (lane < cl && ADWIN_CHK(rank < (uint32_t)kRowsMaxCl, p.status))
-          remote_store4(map_to_rank(smem_u32(ctrl.xrec[par][rank]), (uint32_t)lane), v[0], v[1], v[2], v[3]);
+        if (lane < cl && ADWIN_CHK(rank < (uint32_t)kRowsMaxCl, p.status)) {
+          const uint32_t dst = map_to_rank(smem_u32(ctrl.xrec[par][rank]), (uint32_t)lane);
+          float v[8];
+          upk2(SA.hi, v[0], v[1]);
+          upk2(TQ.hi, v[2], v[3]);
+          upk2(SA.lo, v[4], v[5]);
+          upk2(TQ.lo, v[6], v[7]);
+          remote_store4(dst, v[0], v[1], v[2], v[3]);
+          remote_store4(dst + 16, v[4], v[5], v[6], v[7]);
+        }
         cluster_sync_all();
-        v[0] = v[1] = v[2] = v[3] = 0.f;
+        SA.set(0ull);
+        TQ.set(0ull);
         for (int j = 0; j < cl; ++j) {
-          const float4 x = *reinterpret_cast<const float4*>(ctrl.xrec[par][j]);
-          v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+          ExactSum<kExact> x, y;
+          row_pairs(ctrl.xrec[par][j], x.hi, y.hi);
+          row_pairs(ctrl.xrec[par][j] + 4, x.lo, y.lo);
+          SA.add(x);
+          TQ.add(y);
         }
       }
-      if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = v[3];
+      RowTotals t;
+      float S_off, A_off, St_off, q, q_off;
+      upk2(SA.hi, t.S, t.A);
+      upk2(SA.lo, S_off, A_off);
+      upk2(TQ.hi, t.St, q);
+      upk2(TQ.lo, St_off, q_off);
+      t.St += St_off;
+      if (rank == 0 && lane == 0 && i > 0 && p.gsq) p.gsq[r_prev] = isfinite(q) ? q + q_off : q;
       if (!real) break;
       const RowsMeta& m = ctrl.meta[i % kMetaDepth];
       const int64_t ri = m.r;
-      RowTotals t;
       t.M2s = m.zy * kLog2e;
       t.M2t = m.uy * kLog2e;
-      t.S = v[0];
-      t.A = v[1];
-      t.St = v[2];
       t.B0 = t.B1 = t.B2 = 0.f;
-      // (the totals are identical in every CTA of the cluster, so this branch is too)
+      // (the totals are identical in every CTA of the cluster, so this branch is too; an infinite sum's St_off is
+      // not a number)
       if (!(t.S < kSumLimit) || !(t.St < kSumLimit)) {
         if (lane == 0) ctrl.out.again = 1;
         named_sync(kReady, all);
@@ -436,12 +473,20 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
           }
           combine();
         }
+        S_off = A_off = 0.f;
       }
       const bool y_valid = m.y >= 0 && (int64_t)m.y < p.V;
-      const float inv = 1.f / t.S;
+      const float inv0 = 1.f / t.S, inv = kExact ? fmaf(-S_off * inv0, inv0, inv0) : inv0;
       // the mean of delta over the row, as a sum of two floats
-      const float about = t.A * inv, mean = about + m.dref, back = mean - about;
-      const float rest = (about - (mean - back)) + (m.dref - back);
+      const float about = t.A * inv;
+      const float about_off = (fmaf(-about, t.S, t.A) + fmaf(-about, S_off, A_off)) * inv;
+      const float near_mean = about + m.dref, back = near_mean - about;
+      const float near_off = ((about - (near_mean - back)) + (m.dref - back)) + about_off;
+      float mean = near_mean + near_off, rest = near_off - (mean - near_mean);
+      if (!isfinite(mean)) {   // (a difference of logits that is: no rounding to look after)
+        mean = near_mean;
+        rest = 0.f;
+      }
       float coef = p.alpha * inv, nc0 = -mean, nm2s = -t.M2s;
       if constexpr (FULLKL && sizeof(TIn) == 2) {
         // bf16 logits: g = e * (coef*delta - coef*mean) saves one operation per pair; its rounding
@@ -495,7 +540,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       }
       if (lane == 0) {
         if (rank == 0 && ADWIN_CHK(ri >= 0 && ri < p.B * p.T, p.status)) {
-          p.kl[ri] = rs.kl;
+          p.kl[ri] = (mean - rs.lse_diff) + rest;
           p.logratio[ri] = rs.c;
           if (p.lse_s) p.lse_s[ri] = rs.lse_s;
           if (p.lse_t) p.lse_t[ri] = rs.lse_t;
@@ -564,7 +609,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
     };
     // ---- second sweep: what it takes of its row
     RowSlice sp2 = sp1;
-    f2_t Q = 0ull;
+    f2_t Q[kNorms] = {};
     float gy = 0.f;
     int yleft = -1;           // pieces from this thread's next one to the sampled token's (< 0: passed, or elsewhere)
     int ye = 0;
@@ -632,7 +677,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
               }
             }
 #pragma unroll
-            for (int e = 0; e < NP; ++e) Q = fma2(G[e], G[e], Q);
+            for (int e = 0; e < NP; ++e) Q[h % kNorms] = fma2(G[e], G[e], Q[h % kNorms]);
             char* dst = gp + (size_t)h * nt * N * sizeof(TOut);
             if (ADWIN_CHK(inside(sp2, lp), p.status)) {
               store_pairs<TOut, NP>(dst, G);
@@ -802,7 +847,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         ye = (int)(yat % N);
         gp = static_cast<char*>(p.grad) +
              ((size_t)m.r * p.ld_grad - sp2.shift + (size_t)(piece0 + tid) * N) * sizeof(TOut);
-        Q = 0ull;
+        Q[0] = Q[kNorms - 1] = 0ull;
       }
       const int groups = plan.groups, both = next ? groups - plan.ahead : 0;
       // whole groups of both rows
@@ -823,7 +868,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
         }
       }
       if (!next) a.reset();
-      post(hsum2(Q));
+      post(hsum2(kNorms > 1 ? add2(Q[0], Q[kNorms - 1]) : Q[0]));
     }
     if (cl > 1 && my_rows > 0) cluster_wait();
   }
@@ -854,9 +899,10 @@ constexpr bool shape_plan(const RowsShape& sh, int64_t pieces, int kept, RowsPla
   const int tm_groups = sh.tm_cols ? sh.tm_cols / ((sh.nt + 127) / 128) / (kU * kept * 4) : 0;
   const int spare = sm_groups + tm_groups - plan.groups;
   if (spare < 0) return false;
-  // one group covers a CTA's own exchange, a cluster's takes two (151 936 entries 426 us with one, 412 with
-  // two); more only run the sweeps apart (32 000 entries 422 with one, 430 with three)
-  const int most = sh.cl > 1 ? 2 : 1;
+  // one group covers the exchange of two CTAs on an SM, of one CTA two, a cluster's takes three (151 936 entries
+  // 418 us with two, 410 with three; 80 000 entries 395 with one, 391 with two); more only run the sweeps apart
+  // (32 000 entries 404 with one, 409 with two)
+  const int most = sh.cl > 1 ? 3 : sh.ctas == 1 ? 2 : 1;
   plan.ahead = spare < most ? spare : most;
   if (plan.ahead > plan.groups) plan.ahead = plan.groups;
   const int ring = plan.groups + plan.ahead;

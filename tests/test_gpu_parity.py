@@ -849,3 +849,32 @@ def test_read_only_precision_of_references_and_running_maxima():
             sums[1] += (d.gather(1, y[r:r + 50])[:, 0] - c[r:r + 50]).square().sum()
         err[mode] = sums.sqrt()
     assert (err[api.GRAD_FULL_KL] <= 1.1 * err[api.GRAD_SAMPLED]).all(), err
+
+
+def test_precision_of_rows_with_gradient():
+    """The row kernel adds a row up over more entries per thread than the staged kernel, and about the sampled token's
+    z - u: its scalars may not be further from a 64-bit evaluation for it, with tokens drawn uniformly, which are
+    poor centres (10 % for the spread between two sets of 2048 rounding errors)."""
+    T, V = 2048, 50248
+    z, u = (torch.zeros((1, T, V), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+    tokens = torch.zeros((1, T), dtype=torch.int32, device=DEV)
+    gen = torch.Generator(device=DEV).manual_seed(7)
+    synth.fill_sequence(z[0], u[0], tokens[0], s_std=2.0, mix=1.0, t_std=1.0, spike_p=0.0, tokens="uniform", gen=gen)
+    window = torch.tensor([T], dtype=torch.int32, device=DEV)
+    grad = torch.zeros_like(z)
+    got = {flags: api.adwin_opd_kl_fwd_bwd(z, u, tokens, window, window, flags=flags, grad=grad)
+           for flags in (0, api.FORCE_STAGED)}
+    sums = {flags: torch.zeros(3, dtype=torch.float64, device=DEV) for flags in got}
+    for r in range(0, T, 64):
+        rows = slice(r, r + 64)
+        d = torch.log_softmax(z[0, rows].double(), 1)
+        p = d.exp()
+        d -= torch.log_softmax(u[0, rows].double(), 1)
+        kl = (p * d).sum(1)
+        gsq = (p * (d - kl[:, None])).square().sum(1)
+        c = d.gather(1, tokens[0, rows].long()[:, None])[:, 0]
+        for flags, o in got.items():
+            sums[flags] += torch.stack([((o.kl[0, rows].double() - kl) / kl).square().sum(),
+                                        (o.logratio[0, rows].double() - c).square().sum(),
+                                        ((o.gsq[0, rows].double() - gsq) / gsq).square().sum()])
+    assert (sums[0].sqrt() <= 1.1 * sums[api.FORCE_STAGED].sqrt()).all(), sums
