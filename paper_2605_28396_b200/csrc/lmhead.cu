@@ -223,10 +223,14 @@ __device__ __forceinline__ float copy_dot(const __nv_bfloat16* src, const __nv_b
 // almost surely the peak, where the centred difference is then exactly zero, which keeps the
 // single-sweep squared-norm moments well conditioned.
 // OWN: every block forms the prefix sums itself, in shared memory, which for a short call costs less than a
-// launch of lm_plan_kernel and round trips to memory for the search below (225 rows: 7.5 us where the two kernels
-// take 11.5; 4 400 rows in seven segments 54 us where they take 40).
+// launch of lm_plan_kernel and round trips to memory for the search below, but each block pays for every segment
+// of every sequence, and beyond about ten blocks per SM they take turns.  Whole calls at V = 8 192, d = 512, by the two
+// kernels / so: two segments of 2 sequences, 512 rows 82.0 / 80.4 us, 1 400 121.6 / 119.3, 1 536 125.6 / 126.4; of 128
+// sequences, 512 rows 83.5 / 82.0, 1 280 120.5 / 119.3; seven segments of 16 sequences, 640 rows 127.0 / 123.7, 1 440
+// 154.4 / 155.5; of 64, 1 280 rows 149.9 / 153.2; of 128, 512 rows 119.7 / 123.1, 1 280 157.7 / 170.2.
 constexpr int kGatherSeqs = 128;
-constexpr int64_t kGatherOwnRows = 2048;
+constexpr int64_t kGatherOwnRows = 1408;      // (without the segments' padding)
+constexpr int64_t kGatherOwnSums = 256;       // segments times sequences
 template <bool OWN>
 __global__ void __launch_bounds__(kGatherThreads) lm_gather_kernel(const GatherParams p, const SegPlan plan) {
   chain();
@@ -929,7 +933,8 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
   gp.ht_c = ht_c;
   gp.status = a.status;
   const unsigned gather_grid = (unsigned)(rows_cap < 16384 ? rows_cap : 16384);
-  if (a.B <= kGatherSeqs && rows_cap <= kGatherOwnRows) {
+  if (a.B <= kGatherSeqs && plan.n_seg * a.B <= kGatherOwnSums &&
+      rows_cap - (int64_t)plan.n_seg * (plan.pad - 1) <= kGatherOwnRows) {
     launch_chained(lm_gather_kernel<true>, gather_grid, kGatherThreads, 0, 1, s, gp, plan);
   } else {
     launch_chained(lm_plan_kernel, plan.n_seg, 1024, 0, 1, s, gp.range, gp.ewin, a.B, plan, seg);
