@@ -629,7 +629,7 @@ struct MergeParams {
   int32_t* status;
 };
 
-// Block = 32 compact rows, 32 threads per row: combine the partial records of the row in float64
+// Block = ROWS compact rows, 1024 / ROWS threads per row: combine the partial records of the row in float64
 // against common references (fixed order) and derive the per-token outputs and the gradient
 // coefficients:
 //   g_k = p_k (a1 (z_k - u_k) + a0) (+ gy at k = y),   p_k = 2^(z_k log2e - L2s);
@@ -637,10 +637,12 @@ struct MergeParams {
 // whatever its logits (with L2s = 0, p_k overflows beyond z = 88 and 0 * inf spreads over dW).
 // Records are read with the row as the fast index (whole 32-byte sectors at least), reduced with the record
 // as the lane.  A short call has many records (126 for each of 225 rows at V = 32 000), which is
-// why the records are spread over threads, and the more the fewer tiles there are: ROWS = 8 up to
-// kMergeFewTiles (225 rows: 8 blocks of 32 rows, four records a thread, took 14.5 us).
+// why the records are spread over threads, and more so with few tiles: ROWS = 8 up to two, and of many chunks
+// of the vocabulary up to four.  Whole calls with 32 rows a block / with 8: V = 32 000, 128 rows
+// 165.7 / 164.1 us, 256 176.9 / 175.2, 384 214.8 / 213.9, 512 226.6 / 227.2, 600 270.1 / 272.2; V = 16 000, 128 rows 91.7 /
+// 90.1, 512 113.6 / 112.7; V = 8 192, 128 rows 69.1 / 67.8, 256 72.9 / 72.2, 512 77.8 / 80.4.
 constexpr int kMergeRows = 32;
-constexpr int kMergeFewTiles = 8;
+bool merge_by_8(int64_t tiles, int n_chunks) { return tiles <= 2 || (tiles <= 4 && n_chunks >= 48); }
 template <int ROWS>
 __global__ void __launch_bounds__(1024) lm_merge_kernel(const MergeParams p) {
   chain();
@@ -850,7 +852,7 @@ __global__ void __launch_bounds__(256, 2) lm_grad_kernel(const GradParams p) {
 
 // Squared gradient norm of the rows whose gradient was formed: the sum of g_k^2 over the entries
 // themselves (fixed order, float64), which replaces the single-sweep moment value there.  Block = 32
-// compact rows, 32 threads per row, as in lm_merge_kernel.
+// compact rows, 32 threads per row, as in lm_merge_kernel<32>.
 __global__ void __launch_bounds__(1024) lm_gsq_kernel(const LmHeader* hdr, const float* __restrict__ q,
                                                       const int32_t* __restrict__ rowdst,
                                                       int n_groups, float* gsq) {
@@ -991,7 +993,7 @@ cudaError_t run_lmhead(const LmCall& a, const LmLayout& L, const SegPlan& plan, 
         moments ? launch_pairs(lm_sweep_kernel<true>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp)
                 : launch_pairs(lm_sweep_kernel<false>, a.sm_count, s, m_hs, m_ws, m_ht, m_wt, sp);
     if (r != cudaSuccess) return r;
-    if (cap <= kMergeFewTiles) launch_chained(lm_merge_kernel<8>, (unsigned)cap * (kBM / 8), 1024, 0, 1, s, mp);
+    if (merge_by_8(cap, L.n_chunks)) launch_chained(lm_merge_kernel<8>, (unsigned)cap * (kBM / 8), 1024, 0, 1, s, mp);
     else launch_chained(lm_merge_kernel<32>, (unsigned)cap * (kBM / 32), 1024, 0, 1, s, mp);
     return cudaGetLastError();
   };

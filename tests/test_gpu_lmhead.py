@@ -391,11 +391,13 @@ def test_rows_packed_across_sequences_at_tile_edges(windows):
         check_all(batch, got, oracle(batch, api.GRAD_FULL_KL, flags), flags)
 
 
-@pytest.mark.parametrize("B,T", [(33, 9), (128, 8), (129, 8), (40, 27), (40, 60)])
-def test_many_short_sequences(B, T):
-    """The prefix sums over the sequences formed by the gather kernel's blocks (up to 128 sequences and 2048
-    rows) and by a kernel of their own; the partial records merged 8 rows a block (up to 8 tiles) and 32."""
-    batch = synth.make_lmhead_batch(DEV, B=B, T=T, V=520, d_s=64, d_t=72, w_std=0.1)
+@pytest.mark.parametrize("B,T,V", [(33, 9, 520), (128, 8, 520), (129, 8, 520), (40, 27, 520), (40, 36, 520), (40, 60, 520),
+                                   (33, 9, 12288), (11, 46, 12288), (11, 48, 12280)])
+def test_many_short_sequences(B, T, V):
+    """The prefix sums over the sequences formed by the gather kernel's blocks (up to 128 sequences and 1408
+    rows) and by a kernel of their own; the partial records merged 8 rows a block (up to 2 tiles, and
+    up to 4 from 48 chunks of 256 entries on) and 32."""
+    batch = synth.make_lmhead_batch(DEV, B=B, T=T, V=V, d_s=64, d_t=72, w_std=0.1)
     rng = np.random.default_rng(B + T)
     batch.window = torch.from_numpy(rng.integers(0, T + 1, B).astype(np.int32)).to(DEV)
     got = run(batch, flags=api.RANGE_FULL)
