@@ -71,12 +71,24 @@ def test_rows_off_16_byte_boundaries(checked_library, path):
     G.test_arrays_that_start_off_a_16_byte_boundary()
 
 
-@pytest.mark.parametrize("v", G.SHAPE_ENDS)
-def test_ends_of_the_row_kernels_shapes(checked_library, v):
-    for V in (v - 7, v - 5, v, v + 8):
-        G.test_rows_held_by_one_cta_and_by_clusters(2, V)
-    for V in (v // 2 - 3, v // 2, v // 2 + 4):
-        G.test_rows_held_by_one_cta_and_by_clusters(1, V)
+@pytest.mark.parametrize("v,rows", G.SHAPE_ENDS)
+def test_ends_of_the_row_kernels_shapes(checked_library, v, rows):
+    for V in (v - 63, v - 61, v, v + 8):
+        G.test_rows_held_by_one_cta_and_by_clusters(2, V, rows)
+    for V in (v // 2 - 31, v // 2, v // 2 + 4):
+        G.test_rows_held_by_one_cta_and_by_clusters(1, V, rows)
+
+
+@pytest.mark.parametrize("in_dt,V,rows", [(2, 4099, 2500), (2, 6144, 2500), (2, 28609, 1250), (2, 57281, 620), (2, 114625, 310),
+                                          (2, 151936, 160), (2, 229376, 160), (2, 262144, 80), (2, 458752, 80), (1, 2050, 2500),
+                                          (1, 57341, 310)])
+def test_rows_one_after_another(checked_library, in_dt, V, rows):
+    G.test_rows_one_after_another(in_dt, V, rows)
+
+
+@pytest.mark.parametrize("in_dt,V,rows", [(2, 8192, 33), (2, 28672, 70), (2, 50257, 37), (2, 50257, 148), (1, 4095, 296)])
+def test_calls_of_few_rows(checked_library, in_dt, V, rows):
+    G.test_calls_of_few_rows(in_dt, V, rows)
 
 
 @pytest.mark.parametrize("in_dt,V", [(2, 33), (2, 961), (2, 1024), (2, 1032), (1, 481)])

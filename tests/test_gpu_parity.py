@@ -552,24 +552,29 @@ def test_status_word_collects_or_starts_fresh():
     assert int(o.dev_status.item()) == api.DEV_TOKEN_RANGE | api.DEV_WINDOW
 
 
-# The longest rows of bf16 that the row kernel's shapes take (64, 128 and 224 threads; 352 threads with one,
-# two and four CTAs per row); half as many entries of fp32.  A row off 16-byte boundaries may lie in one
-# piece more than its length asks for.
-SHAPE_ENDS = (6144, 10240, 25600, 50688, 101376, 202752)
+# The longest bf16 rows that the row kernel's shapes take (64, 128, 256 threads; 512 threads with one, two and four CTAs
+# per row; half as many entries of fp32), and how many rows of them a call has to be for so that the shape goes by the
+# length alone.  The sampled-token estimator keeps the student alone: twice as much on 512 threads.  Rows off the lines
+# may lie in as much as 63 entries more (31 of fp32) than they have; bf16 rows of whole pieces up to 14 336 do not.
+SHAPE_ENDS = ((6144, 298), (28672, 298), (57344, 150), (114688, 76), (229376, 38), (458752, 2), (237568, 76), (475136, 38),
+              (950272, 2))
 
 
-@pytest.mark.parametrize("in_dt,V", [(2, 3584), (2, 3592), (2, 17920), (2, 36000), (2, 58880), (2, 70001),
-                                     (2, 117760), (1, 1792), (1, 33003), (1, 58900), (1, 118001)] +
-                         [(2, v + more) for v in SHAPE_ENDS for more in (-7, -5, 0, 8)] +
-                         [(1, v // 2 + more) for v in SHAPE_ENDS for more in (-3, -1, 0, 4)])
-def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
+@pytest.mark.parametrize("in_dt,V,rows", [(2, v, 12) for v in (3584, 3592, 10240, 17920, 25600, 36000, 50688, 58880, 70001,
+                                                               101376, 117760, 202752)] +
+                         [(1, v, 12) for v in (1792, 5119, 33003, 50689, 58900, 101373, 118001)] +
+                         [(2, v + more, rows) for v, rows in SHAPE_ENDS for more in (-63, -61, 0, 8, 64)] +
+                         [(1, v // 2 + more, rows) for v, rows in SHAPE_ENDS for more in (-31, -29, 0, 4)])
+def test_rows_held_by_one_cta_and_by_clusters(in_dt, V, rows):
     """The row kernel's shapes: rows of a few hundred pieces, rows that fill a CTA's shared memory and
     run over into tensor memory, rows split over two and four CTAs; at the end of every shape rows that
-    fill it and rows of one more piece, on and off 16-byte boundaries (the last go to the staged kernel); a
+    fill it and rows of one more piece, on and off the lines (the last of each estimator go to the staged kernel); a
     sampled token in every slice, and rows whose token is far below the maximum (summed again from the
-    copy on chip)."""
-    batch = synth.make_batch(in_dt, device=DEV, B=2, T=6, V=V)
+    copy on chip).  Few rows of a call have a gradient, whatever it is for."""
+    T = max(6, rows // 2)
+    batch = synth.make_batch(in_dt, device=DEV, B=2, T=T, V=V)
     batch.window = torch.tensor([6, 3], dtype=torch.int32, device=DEV)
+    batch.rollout_len = torch.tensor([6, 6], dtype=torch.int32, device=DEV)
     for t, y in enumerate((0, V // 4 + 1, V // 2 + 1, 3 * V // 4 + 1, V - 1)):
         batch.tokens[0, t] = y
     for b, t in ((0, 1), (0, 4), (1, 2)):     # (both policies, see the test of odd rows)
@@ -587,10 +592,15 @@ def test_rows_held_by_one_cta_and_by_clusters(in_dt, V):
 
 
 # Several rows for every CTA of a launch, so that a row's second sweep runs beside the next row's first and
-# the ring of kept pieces turns over: the longest rows of each shape (bf16; half of that fp32), rows of whole
-# lines, of whole pieces and rows that start anywhere in one, and the first of a cluster of two and of four.
+# the ring of kept pieces turns over: the longest rows of each shape (bf16; half of that fp32), whose ring has no room
+# beside a row, and rows that leave one and two groups; rows of whole lines, of whole pieces and rows that start anywhere
+# in one; the first of a cluster of two and of four.
 @pytest.mark.parametrize("in_dt,V,rows", [(2, 4099, 2500), (2, 4096, 2500), (2, 28665, 1250), (2, 57341, 620), (2, 57344, 620),
-                                          (2, 5000, 2500), (2, 14328, 2500), (2, 14344, 2500),
+                                          (2, 5000, 2500), (2, 6081, 2500), (2, 6144, 2500), (2, 14328, 2500), (2, 14344, 2500),
+                                          (2, 28609, 1250), (2, 28672, 1250), (2, 57281, 620), (2, 114625, 310), (2, 114688, 310),
+                                          (2, 196609, 160), (2, 212992, 160), (2, 229376, 160), (2, 393217, 80), (2, 425984, 80),
+                                          (2, 458752, 80), (2, 237568, 310), (2, 475136, 160), (2, 950272, 80), (1, 3072, 2500),
+                                          (1, 28672, 620), (1, 57344, 310), (1, 114688, 160), (1, 229376, 80),
                                           (2, 114681, 310), (2, 114752, 170), (2, 262144, 80), (1, 2050, 2500),
                                           (1, 14331, 1250), (1, 57341, 310), (1, 57349, 170)])
 def test_rows_one_after_another(in_dt, V, rows):
@@ -682,7 +692,9 @@ def test_read_only_rows_split_over_a_cluster(in_dt, V, rows):
         run_and_check(batch, grad_dtype=None, grad_mode=mode)
 
 
-@pytest.mark.parametrize("V,rows", [(4096, 40), (40000, 24)])
+# (clusters of four for few rows; 151 936 entries also clusters of two, several rows each, more of them than the GPU
+# holds at a time)
+@pytest.mark.parametrize("V,rows", [(4096, 40), (40000, 24), (151936, 20), (151936, 180)])
 def test_launches_that_overlap_their_predecessor(V, rows):
     """Kernels of a call are set up while the one before drains: calls in a row over the same buffers and
     workspace, on two streams and replayed from a graph, leave the bits that separate calls leave."""
