@@ -175,12 +175,9 @@ struct RowSlice {
 
 // NT: threads that hold pieces, a template constant so that the strides between a thread's pieces are
 // offsets in the instructions.  A group of kU steps in which every thread has whole pieces takes the path
-// without tests (FULL below), kWholeAlone: also where one sweep runs alone, as with one row a CTA (280 rows of
-// 32 000 entries of bf16, 23.4 us with the tests there, 20.9 without).  Not in the small kernels of rows off the
-// lines, which such calls do not take and whose loop comes out slower beside that code (2.4 GB of rows of 9 001 entries
-// 506 us, 564 with it; of 5 000 513, 570).  FULLKL: the gradient of Eq. 2; without it, of Eq. 4, whose second sweep
+// without tests (FULL below), with ALONE also where one sweep runs alone (see lone_sweeps).  FULLKL: the gradient of Eq. 2; without it, of Eq. 4, whose second sweep
 // takes the student's logits alone, so only they are kept.
-template <typename TIn, typename TOut, int NT, bool TM, bool RAG, bool FULLKL>
+template <typename TIn, typename TOut, int NT, bool TM, bool RAG, bool FULLKL, bool ALONE>
 __global__ void __launch_bounds__(NT + 32, ctas_of(NT))
 kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   chain();
@@ -206,7 +203,6 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
   // sums over all threads: 151 936 440.)
   constexpr bool kExact = NT >= 256;
   constexpr int kNorms = kExact && FULLKL ? kU : 1;
-  constexpr bool kWholeAlone = !RAG || NT >= 256;
   constexpr uint32_t group_bytes = kU * kKept * array;
   constexpr int group_cols = kU * kKept * 4;
   extern __shared__ __align__(128) char smem[];
@@ -774,8 +770,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
 #pragma unroll 1
         for (; g < to; ++g) {
           early(i + 1, g);
-          if (kWholeAlone && g >= full_from(sp1) && g < full_to(sp1)) {
-            if constexpr (kWholeAlone) group(yes, no, yes, g, 0);
+          if (ALONE && g >= full_from(sp1) && g < full_to(sp1)) {
+            if constexpr (ALONE) group(yes, no, yes, g, 0);
           } else {
             group(yes, no, no, g, 0);
           }
@@ -856,8 +852,8 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       for (int g = 0; g < groups; ++g) {
         const int g1 = g + plan.ahead;
         if (g >= both) {
-          if (kWholeAlone && g >= full_from(sp2) && g < full_to(sp2)) {
-            if constexpr (kWholeAlone) group(no, yes, yes, 0, g);
+          if (ALONE && g >= full_from(sp2) && g < full_to(sp2)) {
+            if constexpr (ALONE) group(no, yes, yes, 0, g);
           } else {
             group(no, yes, no, 0, g);
           }
@@ -959,20 +955,33 @@ constexpr bool metadata_precedes_its_readers() {
 static_assert(metadata_precedes_its_readers(), "a row's metadata could be read before it is written");
 
 typedef void (*RowsKernel)(KlParams, RowsPlan);
-template <typename TIn, typename TOut, int NT>
-RowsKernel rows_kernel_nt(bool ragged, bool full_kl) {
+// ALONE: a call of one row a CTA has lone sweeps only (280 rows of 32 000 entries of bf16 23.4 us with the tests
+// there, 20.9 without), one of many rows a group or two a row, beside whose code the loop of both sweeps comes out faster
+// or slower.  2.4 GB without / with it: bf16 rows on the lines 4 096 entries 451 / 446 us, 20 032 452 / 437, 80 000 449 /
+// 420; fp32 4 096 376 / 382; off the lines 5 000 513 / 570, 9 001 506 / 564, 33 001 447 / 456, 50 257 415 / 424, 80 001 408 /
+// 414, sampled 421 / 414.  Calls of few rows do not take the small shapes; those of 256 threads have both.
+constexpr bool lone_sweeps(int nt, bool ragged, bool few, size_t entry) {
+  return nt > 256 || (ragged ? nt == 256 && few : nt == 256 || entry == 2);
+}
+template <typename TIn, typename TOut, int NT, bool RAG, bool FULLKL>
+RowsKernel rows_kernel_of(bool few) {
   constexpr bool TM = uses_tensor_memory(NT);
-  if (full_kl)
-    return ragged ? kl_rows_kernel<TIn, TOut, NT, TM, true, true> : kl_rows_kernel<TIn, TOut, NT, TM, false, true>;
-  return ragged ? kl_rows_kernel<TIn, TOut, NT, TM, true, false> : kl_rows_kernel<TIn, TOut, NT, TM, false, false>;
+  constexpr bool kFew = lone_sweeps(NT, RAG, true, sizeof(TIn)), kMany = lone_sweeps(NT, RAG, false, sizeof(TIn));
+  return few ? kl_rows_kernel<TIn, TOut, NT, TM, RAG, FULLKL, kFew>
+             : kl_rows_kernel<TIn, TOut, NT, TM, RAG, FULLKL, kMany>;
+}
+template <typename TIn, typename TOut, int NT>
+RowsKernel rows_kernel_nt(bool ragged, bool full_kl, bool few) {
+  if (full_kl) return ragged ? rows_kernel_of<TIn, TOut, NT, true, true>(few) : rows_kernel_of<TIn, TOut, NT, false, true>(few);
+  return ragged ? rows_kernel_of<TIn, TOut, NT, true, false>(few) : rows_kernel_of<TIn, TOut, NT, false, false>(few);
 }
 template <typename TIn, typename TOut>
-RowsKernel rows_kernel(int nt, bool ragged, bool full_kl) {
+RowsKernel rows_kernel(int nt, bool ragged, bool full_kl, bool few) {
   switch (nt) {
-    case 64: return rows_kernel_nt<TIn, TOut, 64>(ragged, full_kl);
-    case 128: return rows_kernel_nt<TIn, TOut, 128>(ragged, full_kl);
-    case 256: return rows_kernel_nt<TIn, TOut, 256>(ragged, full_kl);
-    case kRowsThreads: return rows_kernel_nt<TIn, TOut, kRowsThreads>(ragged, full_kl);
+    case 64: return rows_kernel_nt<TIn, TOut, 64>(ragged, full_kl, few);
+    case 128: return rows_kernel_nt<TIn, TOut, 128>(ragged, full_kl, few);
+    case 256: return rows_kernel_nt<TIn, TOut, 256>(ragged, full_kl, few);
+    case kRowsThreads: return rows_kernel_nt<TIn, TOut, kRowsThreads>(ragged, full_kl, few);
     default: return nullptr;
   }
 }
@@ -992,7 +1001,7 @@ cudaError_t resident_clusters(const RowsPlan& plan, int sm_count, int& n) {
   std::lock_guard<std::mutex> lock(mu);
   n = seen[dev][plan.cl];
   if (n > 0) return cudaSuccess;
-  const RowsKernel like = kl_rows_kernel<float, float, kRowsThreads, false, false, true>;
+  const RowsKernel like = kl_rows_kernel<float, float, kRowsThreads, false, false, true, false>;
   const int smem = shape_smem(plan.ctas);
   e = cudaFuncSetAttribute(like, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -1056,9 +1065,9 @@ cudaError_t launch_rows_t(const KlParams& p, bool ragged, int sm_count, cudaStre
   const int64_t lead = ragged ? kLine / (int64_t)sizeof(TIn) - 1 : 0;   // entries of a line before the row, at most
   cudaError_t e = rows_plan((lead + p.V + N - 1) / N, kept, p.plan_rows, sm_count, plan);
   if (e != cudaSuccess) return e;
-  if (plan.num_clusters > p.B * p.T) plan.num_clusters = (int)(p.B * p.T);
-  const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, ragged, full_kl);
+  const RowsKernel kernel = rows_kernel<TIn, TOut>(plan.nt, ragged, full_kl, p.B * p.T <= plan.num_clusters);
   if (!kernel) return cudaErrorNotSupported;
+  if (plan.num_clusters > p.B * p.T) plan.num_clusters = (int)(p.B * p.T);
   const int smem = launch_smem(plan, kept);
   // the shape's whole share whatever this call needs: the limit belongs to the kernel, which launches of
   // other threads with other row lengths use at the same time
