@@ -200,16 +200,19 @@ struct RowScalars {
 //   KL = E_p[delta] - Delta;   c = (z_y - u_y) - Delta
 // The expanded squared norm sum p^2 (delta - E_p delta)^2 = (B2 - 2 c0 B1 + c0^2 B0) / S^2 is only
 // used for rows whose gradient is not written.
+// nonfinite: whether either log-sum-exp is; they themselves only with want_lse.
 // w: SAMPLED mode only, null or the address of a caller-supplied coefficient that takes the place
 // of c (Eq. 3); it is read only on that branch.
 __device__ __forceinline__ RowScalars finish_row(const RowTotals& t, float zy, float uy,
                                                  bool y_valid, float dref, float alpha, int mode,
-                                                 const float* w = nullptr) {
+                                                 const float* w = nullptr, bool want_lse = true) {
   constexpr float kLn2f = 0.69314718055994531f;
   RowScalars r;
-  const float l2s = log2f(t.S), l2t = log2f(t.St);
-  r.lse_s = (t.M2s + l2s) * kLn2f;
-  r.lse_t = (t.M2t + l2t) * kLn2f;
+  r.lse_s = r.lse_t = 0.f;
+  if (want_lse) {
+    r.lse_s = (t.M2s + log2f(t.S)) * kLn2f;
+    r.lse_t = (t.M2t + log2f(t.St)) * kLn2f;
+  }
   // log2 S - log2 St as one logarithm of the ratio: both sums can be large against a shared
   // reference, and their separate logarithms would each carry an absolute error of an ulp of ~20.
   const float delta = ((t.M2s - t.M2t) + log2f(t.S / t.St)) * kLn2f;
@@ -231,7 +234,7 @@ __device__ __forceinline__ RowScalars finish_row(const RowTotals& t, float zy, f
     r.coef = -ac * inv_s;
     r.gy = ac * (1.f - py);
   }
-  r.nonfinite = !(isfinite(r.lse_s) && isfinite(r.lse_t));
+  r.nonfinite = !(isfinite(t.M2s) && t.S > 0.f && isfinite(t.S) && isfinite(t.M2t) && t.St > 0.f && isfinite(t.St));
   return r;
 }
 

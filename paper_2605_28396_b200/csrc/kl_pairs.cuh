@@ -182,6 +182,14 @@ struct ExactSum {
     hi = x;
     lo = 0ull;
   }
+  __device__ __forceinline__ void set(f2_t x, f2_t y) {
+    hi = add2(x, y);
+    lo = 0ull;
+    if (EXACT) {
+      const f2_t c = sub2(hi, x);
+      lo = add2(sub2(x, sub2(hi, c)), sub2(y, c));
+    }
+  }
   __device__ __forceinline__ void add(f2_t x) {
     const f2_t s = add2(hi, x);
     if (EXACT) {

@@ -353,23 +353,26 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       named_sync(kPosted, all);
       // fixed-order sums over the threads, then over the CTAs: S and A, St and the norm (what kReady waits for
       // beside the others' issue slots: every operation counts here)
-      ExactSum<kExact> sa[nw], tq[nw];
+      ExactSum<kExact> sa[nw / 2], TQ;
+      f2_t tq[nw / 2];
 #pragma unroll
-      for (int w = 0; w < nw; ++w) {
-        f2_t x, y;
+      for (int w = 0; w < nw / 2; ++w) {
+        f2_t x, y, x2, y2;
         row_pairs(&rec[w * 32 + lane].x, x, y);
-        sa[w].set(x);
-        tq[w].set(y);
+        row_pairs(&rec[(w + nw / 2) * 32 + lane].x, x2, y2);
+        sa[w].set(x, x2);
+        tq[w] = add2(y, y2);
       }
 #pragma unroll
-      for (int n = nw / 2; n > 0; n /= 2) {
+      for (int n = nw / 4; n > 0; n /= 2) {
 #pragma unroll
         for (int w = 0; w < n; ++w) {
           sa[w].add(sa[w + n]);
-          tq[w].hi = add2(tq[w].hi, tq[w + n].hi);
+          tq[w] = add2(tq[w], tq[w + n]);
         }
       }
-      ExactSum<kExact> SA = sa[0], TQ = tq[0];
+      ExactSum<kExact> SA = sa[0];
+      TQ.set(tq[0]);
       float ze = kMaskedEdge, ue = kMaskedEdge;
       if (edges) {
         float e_t = 0.f;
@@ -518,7 +521,7 @@ kl_rows_kernel(const KlParams p, const RowsPlan plan) {
       // what the second sweep of Eq. 2's gradient takes needs no logarithm (as finish_row has it)
       if constexpr (FULLKL) publish(0.f);
       const RowScalars rs = finish_row(t, m.zy, m.uy, y_valid, m.dref, p.alpha, FULLKL ? ADWIN_GRAD_FULL_KL : ADWIN_GRAD_SAMPLED,
-                                       p.row_coef ? &m.w : nullptr);
+                                       p.row_coef ? &m.w : nullptr, p.lse_s || p.lse_t);
       if constexpr (!FULLKL) {
         coef = rs.coef;
         publish(rs.gy);
