@@ -962,14 +962,17 @@ typedef void (*RowsKernel)(KlParams, RowsPlan);
 // there, 20.9 without), one of many rows a group or two a row, beside whose code the loop of both sweeps comes out faster
 // or slower.  2.4 GB without / with it: bf16 rows on the lines 4 096 entries 451 / 446 us, 20 032 452 / 437, 80 000 449 /
 // 420; fp32 4 096 376 / 382; off the lines 5 000 513 / 570, 9 001 506 / 564, 33 001 447 / 456, 50 257 415 / 424, 80 001 408 /
-// 414, sampled 421 / 414.  Calls of few rows do not take the small shapes; those of 256 threads have both.
-constexpr bool lone_sweeps(int nt, bool ragged, bool few, size_t entry) {
-  return nt > 256 || (ragged ? nt == 256 && few : nt == 256 || entry == 2);
+// 414, sampled 421 / 414; sampled 32 000 413 / 435.  Calls of few rows do not take the small shapes; most of those of 256
+// threads are built both ways.
+constexpr bool lone_sweeps(int nt, bool ragged, bool full_kl, bool few, size_t entry) {
+  if (nt == 256) return few || (full_kl && !ragged);
+  return nt > 256 || (!ragged && entry == 2);
 }
 template <typename TIn, typename TOut, int NT, bool RAG, bool FULLKL>
 RowsKernel rows_kernel_of(bool few) {
   constexpr bool TM = uses_tensor_memory(NT);
-  constexpr bool kFew = lone_sweeps(NT, RAG, true, sizeof(TIn)), kMany = lone_sweeps(NT, RAG, false, sizeof(TIn));
+  constexpr bool kFew = lone_sweeps(NT, RAG, FULLKL, true, sizeof(TIn));
+  constexpr bool kMany = lone_sweeps(NT, RAG, FULLKL, false, sizeof(TIn));
   return few ? kl_rows_kernel<TIn, TOut, NT, TM, RAG, FULLKL, kFew>
              : kl_rows_kernel<TIn, TOut, NT, TM, RAG, FULLKL, kMany>;
 }
