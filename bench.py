@@ -73,8 +73,8 @@ def measured_peak():
 # counter is not scaled: the last ~56 MB of a launch's gradient are still in L2 when the kernel
 # ends, a residue bounded by the L2 size that does not grow with the rows, so at full size the
 # writes are taken as the gradient bytes themselves.
-TRAFFIC_READ_BYTES_PER_ROW = 607887
-TRAFFIC_KERNEL_SHA = "c351889fc7deaf3a"
+TRAFFIC_READ_BYTES_PER_ROW = 607965
+TRAFFIC_KERNEL_SHA = "7c1ca67b56909b37"
 
 
 def recorded_traffic(rows, V):

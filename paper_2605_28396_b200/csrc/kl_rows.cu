@@ -7,8 +7,8 @@
 // sums, puts the next row's pieces into the places that fall free, folds them into that row's sums and asks for the
 // group after (so loads are always one group ahead in registers).  The places are a ring of groups in
 // tensor memory (tcgen05.st / tcgen05.ld; no MMA runs here) and shared memory, each thread's its own: no
-// hand-shakes over data.  The ring has room for one or two groups more than a row, which are taken while
-// the row's sums travel, so the exchange costs no idle time either.  Rows are brought into L2 three groups
+// hand-shakes over data.  The ring has room for up to three groups more than a row, which are taken while
+// the row's sums travel, so the exchange costs no idle time either (the longest rows of a shape leave none).  Rows are brought into L2 three groups
 // ahead (cp.async.bulk.prefetch.L2).  (All at once a row ahead is too early: rows of 100 000 bf16 entries were
 // pushed out of L2 again, 609 us against 489 for 2.4 GB.)
 //
@@ -20,8 +20,8 @@
 // Exponentials are taken against a reference that the whole row shares (the logit of the sampled
 // token), so partial sums add without rescaling.  If the sums overflow it (a sampled token more than
 // ~69 nats below the row maximum) the row is summed once more, from its on-chip copy (the teacher's
-// pieces from memory where only the student's are kept), against running maxima.  Rows too long for one CTA are split over a cluster; the CTAs' sums then go to every
-// CTA of the cluster.
+// pieces from memory where only the student's are kept), against running maxima.  Rows too long for one CTA, and
+// the rows of calls with few, are split over a cluster; the CTAs' sums then go to every CTA of the cluster.
 #include <iterator>
 #include <mutex>
 #include <type_traits>
@@ -72,21 +72,25 @@ struct RowsShape {
 };
 // The first that takes the row is used: the more and smaller CTAs, the less of a group lies idle at a row's
 // end; beyond 57 000 entries of bf16 one CTA per SM and not two in clusters (151 936 entries: two CTAs in clusters of
-// four, of which 71 fit on 148 SMs, 496 us; this 421).  Registers allow 20 warps of 96 (or 24 of 80, which is what
+// four, of which 71 fit on 148 SMs, 496 us where this took 421).  Registers allow 20 warps of 96 (or 24 of 80, which is what
 // the 64-thread kernels take): 22 warps of 80 in {2, 352} 443 us where {2, 256} took 422 (32 000 entries).
 // Tensor memory is shared out in powers of two.  Measured over 2.4 GB of logits and gradient (367 us at the
 // copy rate; a kernel that ended one row before it began the next, on {8, 64} to {2, 352} x 4 / this one):
-//   bf16  V =   4 096  478 / 448 us  {8, 64}       fp32  V =   4 096  402 / 376 us  {4, 128}
-//              8 192  444 / 433     {4, 128}               5 001  481 / 381     {4, 128}
-//             16 384  484 / 414     {4, 128}              50 264  483 / 373     {1, 512}
-//             32 000  471 / 420     {2, 256}             100 000  497 / 381     {1, 512} x 2
-//             50 257  508 / 417     {2, 256}        bf16, sampled-token estimator
-//             80 000  512 / 397     {1, 512}              32 000  472 / 420     {2, 256}
-//            151 936  556 / 421     {1, 512} x 2          64 000  496 / 398     {1, 512}
-//            262 144  614 / 440     {1, 512} x 4         151 936  551 / 392     {1, 512}
+//   bf16  V =   4 096  477 / 440 us  {8, 64}       fp32  V =   4 096  416 / 376 us  {4, 128}
+//              5 000  506 / 491     {8, 64}                5 001  479 / 379     {4, 128}
+//              8 192  443 / 430     {4, 128}              50 264  480 / 372     {1, 512}
+//             16 384  486 / 411     {4, 128}             100 000  495 / 380     {1, 512} x 2
+//             32 000  470 / 407     {2, 256}        bf16, sampled-token estimator
+//             50 257  508 / 415     {2, 256}              32 000  466 / 411     {2, 256}
+//             57 344  512 / 395     {2, 256}              64 000  498 / 387     {1, 512}
+//             80 000  515 / 394     {1, 512}             151 936  547 / 382     {1, 512}
+//            114 688  560 / 394     {1, 512}
+//            151 936  555 / 411     {1, 512} x 2
+//            229 376  631 / 414     {1, 512} x 2
+//            262 144  614 / 441     {1, 512} x 4
+// (57 344, 114 688 and 229 376 fill their shapes, whose ring then has no group to spare for the exchange.)
 // fp32 rows are at the copy rate.  bf16 rows (163 issue slots and 24 of ex2 for eight entries, where the copy
-// rate leaves 273 clocks) are bound by arithmetic, short ones also by what is done once per row (5 000
-// entries 514 us, 507 before).
+// rate leaves 273 clocks) are bound by arithmetic, short ones also by what is done once per row.
 // (The small shapes hold twice as much of a row whose second sweep takes the student alone, but are slower there:
 // 10 309 entries on {8, 64} 140 us where {4, 128} takes 131.)
 // A call of so few rows that each gets a CTA or cluster of its own anyway takes the last (widest) shape for
@@ -958,6 +962,8 @@ constexpr bool metadata_precedes_its_readers() {
 static_assert(metadata_precedes_its_readers(), "a row's metadata could be read before it is written");
 
 typedef void (*RowsKernel)(KlParams, RowsPlan);
+// (72 kernels: two types in and out, four thread counts, on and off the lines, both estimators -- the sampled-token
+// one keeps half as much, 151 936 entries on one CTA and not two -- and some with ALONE both ways.)
 // ALONE: a call of one row a CTA has lone sweeps only (280 rows of 32 000 entries of bf16 23.4 us with the tests
 // there, 20.9 without), one of many rows a group or two a row, beside whose code the loop of both sweeps comes out faster
 // or slower.  2.4 GB without / with it: bf16 rows on the lines 4 096 entries 451 / 446 us, 20 032 452 / 437, 80 000 449 /
